@@ -52,6 +52,7 @@ void free_csr(DevCsr& c) {
     cudaFree(c.rp);
     cudaFree(c.col);
     cudaFree(c.info);
+    cudaFree(c.walk);
     cudaFree(c.seg);
     cudaFree(c.long_rows);
     cudaFree(c.long_first);
@@ -158,10 +159,12 @@ esim_status upload_csr(int64_t n, const std::vector<uint32_t>& rp, const std::ve
     ESIM_CUDA_TRY(cudaMemcpy(d.long_first, long_first.data(), sizeof(int32_t) * long_first.size(), cudaMemcpyHostToDevice),
                   "upload long first");
     if (with_info) {
-        std::vector<uint2> info((size_t)n);
-        for (int64_t r = 0; r < n; ++r) info[r] = make_uint2(rp[r], rp[r + 1] - rp[r]);
+        // filled on the device (launch_walk_table); the tail past m is never used as a position
+        const size_t entries = (size_t)std::max(m, n);
         if (dev_alloc(&d.info, (size_t)n) != cudaSuccess) return fail(ESIM_ENOMEM, "cudaMalloc(row info)");
-        ESIM_CUDA_TRY(cudaMemcpy(d.info, info.data(), sizeof(uint2) * (size_t)n, cudaMemcpyHostToDevice), "upload row info");
+        if (dev_alloc(&d.walk, entries) != cudaSuccess) return fail(ESIM_ENOMEM, "cudaMalloc(walk table)");
+        if ((int64_t)entries > m)
+            ESIM_CUDA_TRY(cudaMemset(d.walk + m, 0, sizeof(uint2) * (entries - (size_t)m)), "clear walk table tail");
     }
     return ESIM_OK;
 }
@@ -1342,7 +1345,14 @@ esim_status esim_load_graph(int64_t n, const int64_t* in_rowptr, const int32_t* 
     }
     g.scan_blocks = nb;
     g.stream = g.own_stream;
-    cudaMemset(g.status, 0, sizeof(Status));
+    cudaError_t we = cudaMemset(g.status, 0, sizeof(Status));
+    if (we == cudaSuccess) we = launch_walk_table(g);
+    if (we == cudaSuccess) we = cudaStreamSynchronize(g.stream);
+    if (we != cudaSuccess) {
+        release(g);
+        delete h;
+        return cuda_fail(we, "walk table");
+    }
     *out = h;
     return ESIM_OK;
 }

@@ -20,6 +20,13 @@ enum : int {
     kErrCapacity = 4, // the sparse history outgrew its (pigeonhole) capacity
 };
 
+// Chunk counter of one sampler launch: zero before and after it.
+struct SampleWork {
+    unsigned long long next;  // chunks taken beyond every warp's first
+    unsigned int done;        // blocks that have finished
+    unsigned int pad;
+};
+
 // Per-query device status block (one per graph handle).
 struct Status {
     unsigned long long sum_R;
@@ -29,6 +36,7 @@ struct Status {
     unsigned int ticket;             // last-block ticket of the sparse-history compaction
     unsigned long long hist_count;   // sparse history entries so far
     unsigned long long pair_steps_side;  // pair-steps of the side-stream sampler launch
+    SampleWork work[2];              // the sampler on the query's stream, and the side launch
 };
 
 // Sparse history of one query (sparse linearization): entries [lvl[l], lvl[l+1]) are
@@ -53,7 +61,8 @@ struct Segment {
 struct DevCsr {
     uint32_t* rp = nullptr;      // n+1
     int32_t* col = nullptr;      // m
-    uint2* info = nullptr;       // n: (rp[i], rp[i+1] - rp[i]), one 8-byte load per row (walks)
+    uint2* info = nullptr;       // n: (first in-edge, din), or (i, 0) without in-edges (walks)
+    uint2* walk = nullptr;       // max(m, n): info of the node behind each in-edge (walks)
     Segment* seg = nullptr;      // nseg
     int32_t* long_rows = nullptr;  // nlong row ids
     int32_t* long_first = nullptr; // nlong+1: first segment of each long row
@@ -184,6 +193,8 @@ cudaError_t launch_reverse_sparse(const Graph& g, const SparseHist& h, int32_t L
                                   double* s_out, double* sa);
 
 // sample.cu
+// fills in.info and in.walk from the uploaded in-edge CSR
+cudaError_t launch_walk_table(const Graph& g);
 int64_t allocate_blocks(int64_t n);
 cudaError_t launch_allocate(const Graph& g, const double* hist, int32_t L, double R_b, int mode, double* pi_out,
                             uint64_t* R_out, uint64_t* off);

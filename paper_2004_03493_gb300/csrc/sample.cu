@@ -257,127 +257,350 @@ __device__ __forceinline__ uint32_t segment_node(unsigned long long seg, unsigne
     return (uint32_t)(seg < n_nodes ? seg : seg % n_nodes);
 }
 
-// State of one walk pair stream: the thread's current node k, pair r of R(k)
-// (rk), the two walk positions, the step t, and the pairs still to run.
-// A segment is the run of pairs of one (column, node): in a single query segment k
-// is node k; in a batch of B columns segment q*n + k is node k of column q.
-struct PairState {
-    unsigned long long r, rk, left, cnt, g_end, seg;
-    uint32_t k, xa, xb, t, d;  // d: Algorithm 3 depth of node k (0: Algorithm 2)
+// ---------------------------------------------------------------- sampler
+//
+// Graph form: a walk's position is the pair (first in-edge, din) of its node, and
+// walk[p] holds that pair for the node behind in-edge p, so a step is one dependent
+// 8-byte load per walk.  A node without in-edges has (node id, 0): (first, din) is unique
+// per node either way, so two walks meet iff both words agree, and reading walk[first] of
+// such a node stays inside the array (it has max(m, n) entries).
+//
+// A warp takes a chunk of consecutive pair indices at a time from a counter (the first
+// one by its own number).  A segment is the run of pairs of one (column, node): in a
+// single query segment k is node k; in a batch of B columns segment q*n + k is node k of
+// column q; with shared walks segment k*B + i is interval i of node k.
+//
+// Long runs of one segment (run_one): node, depth and the first Philox round are the
+// warp's, a lane whose pair ended takes the next pair number by a ballot and a prefix
+// count, and the counts are added once per run.  Short segments (run_many): the lanes hold
+// the offsets of 32 consecutive segments and find their pair's segment by shuffles; the
+// window moves on while other lanes' pairs still run.
+//
+// What bounds it: the generator.  A Philox block is 20 wide multiplies, 4 cycles each on a
+// scheduler's multiply pipe, and 40 three-input XORs, 2 cycles each on its integer pipe;
+// alone it reaches 426 G blocks/s on this chip.  run_one needs 17 of the multiplies, 103
+// instructions per warp and step in all, and runs at 270 G pair-steps/s (9.5e8 pairs on the
+// n = 2000 graph at the paper's kappa: 8.4 ms; the multiply pipe 75 % busy).  One pair
+// stream per thread over a (rowptr, col) CSR, which this replaces, took 130 instructions and
+// two dependent loads per walk and step, and a fixed share of the pairs per thread: 11.8 ms
+// there, and 207 against 122 ms on a batch of 64 sources.
+// Six blocks of 256 threads per SM measured as 5 (8.4 against 8.5 ms) and leave the side
+// launch's register share as it was.
+constexpr uint32_t kRunMin = 128;        // shortest run of one segment that gets a loop of its own
+constexpr uint32_t kChunkMin = 256;      // pairs per chunk where there are many
+constexpr uint32_t kChunkMax = 16384;    // few enough that the warps finish together
+constexpr uint32_t kChunksPerWarp = 8;
+constexpr uint32_t kPhiloxM0 = 0xD2511F53u, kPhiloxM1 = 0xCD9E8D57u;
+
+struct WalkArgs {
+    const uint2* __restrict__ row;    // n: (first in-edge, din), or (node, 0); positions times 8 if narrow
+    const uint2* __restrict__ walk;   // max(m, n): the same of the node behind each in-edge
+    const uint64_t* __restrict__ off; // nseg + 1
+    const uint8_t* __restrict__ depth;
+    unsigned long long* __restrict__ counts;
+    uint64_t nseg;
+    uint64_t n;
+    SharedSegs sh;
+    uint32_t T;
 };
 
-// One step of the current pair (branch-free apart from the rare Lemire
-// rejection and the change of node): both walks' rows and chosen in-neighbours
-// are loaded whether or not the walks move (an index into a row without
-// in-edges is clamped to entry 0), and the outcome is applied with selects.
-__device__ __forceinline__ void pair_step(PairState& S, const uint2* __restrict__ row,
-                                          const int32_t* __restrict__ col, const uint64_t* __restrict__ off,
-                                          uint32_t T, const PhiloxKeys& K, unsigned long long* __restrict__ nonmeet,
-                                          unsigned long long& steps, unsigned long long n_nodes,
-                                          const uint8_t* __restrict__ depth, const SharedSegs& sh) {
-    const uint32_t rlo = (uint32_t)S.r, rhi = (uint32_t)(S.r >> 32);
-    const uint4 w = philox4x32_10(make_uint4(rlo, rhi, S.k, S.t), K);
-    const uint2 ra = __ldg(row + S.xa), rb = __ldg(row + S.xb);  // (first in-edge, din)
-    // Algorithm 3's special pairs move without the continuation draw for their first d steps
-    const bool forced = S.t < S.d;
-    const bool cont = (forced | ((w.x < T) & (w.z < T))) & (ra.y != 0u) & (rb.y != 0u);
-    const unsigned long long ma = (unsigned long long)w.y * ra.y;
-    const unsigned long long mb = (unsigned long long)w.w * rb.y;
-    uint32_t ia = (uint32_t)(ma >> 32), ib = (uint32_t)(mb >> 32);
-    if (__builtin_expect(cont & (((uint32_t)ma < ra.y) | ((uint32_t)mb < rb.y)), 0)) {
-        if ((uint32_t)ma < ra.y) ia = pick_redraw(ra.y, ma, rlo, rhi, S.k, 0x80000000u | S.t, K);
-        if ((uint32_t)mb < rb.y) ib = pick_redraw(rb.y, mb, rlo, rhi, S.k, 0xC0000000u | S.t, K);
-    }
-    const uint32_t na = (uint32_t)__ldg(col + (ra.y ? ra.x + ia : 0u));
-    const uint32_t nb = (uint32_t)__ldg(col + (rb.y ? rb.x + ib : 0u));
-    const bool meet = cont & (na == nb);
-    const bool ended = !cont | meet | (S.t + 1u >= kWalkMaxSteps);
-    S.xa = ended ? S.k : na;
-    S.xb = ended ? S.k : nb;
-    if (!ended) {
-        ++S.t;
-        return;
-    }
-    steps += S.t + 1u;
-    // Algorithm 2 counts pairs that never meet; Algorithm 3 counts pairs that first
-    // meet after their d forced steps
-    S.cnt += S.d ? ((meet & (S.t >= S.d)) ? 1ull : 0ull) : (meet ? 0ull : 1ull);
-    S.t = 0;
-    if (--S.left == 0) {
-        if (S.cnt) atomicAdd(nonmeet + S.seg, S.cnt);
-        S.cnt = 0;
-        return;
-    }
-    if (++S.r == S.rk) {  // segment done: flush and move to the next segment with pairs
-        if (S.cnt) atomicAdd(nonmeet + S.seg, S.cnt);
-        S.cnt = 0;
-        const unsigned long long g = S.g_end - S.left;
-        do {
-            ++S.seg;
-            if (sh.B) {  // shared layout: a node's empty intervals are its last ones; skip them at once
-                const unsigned long long i = S.seg % (unsigned long long)sh.B;
-                if (i != 0 && __ldg(off + S.seg + 1) == __ldg(off + S.seg)) S.seg += (unsigned long long)sh.B - 1 - i;
-            }
-        } while (__ldg(off + S.seg + 1) <= g);
-        S.r = sh.rbase ? __ldg(sh.rbase + S.seg) : 0ull;
-        S.rk = S.r + (__ldg(off + S.seg + 1) - __ldg(off + S.seg));
-        S.k = segment_node(S.seg, n_nodes, sh);
-        S.d = depth ? depth[S.k] : 0u;
-        S.xa = S.xb = S.k;
-    }
+__device__ __forceinline__ uint32_t lanes_below() {
+    uint32_t m;
+    asm("mov.u32 %0, %%lanemask_lt;" : "=r"(m));
+    return m;
 }
 
-// Persistent walk-pair sampler.  Thread t takes a contiguous run of global pair
-// indices (about total / #threads of them) and advances its current pair by one
-// step per loop iteration, so a lane whose pair ended starts its next pair at
-// once and lanes stay busy.  Counts stay in registers while the node does not
-// change and are flushed with one atomic add per (thread, node).
-__global__ void __launch_bounds__(kBlock, 6) sample_pairs_kernel(int64_t n, int64_t nseg, const uint2* __restrict__ row,
-                                                                 const int32_t* __restrict__ col,
-                                                                 const uint64_t* __restrict__ off, uint32_t T,
-                                                                 const __grid_constant__ PhiloxKeys K, double budget,
-                                                                 unsigned long long* __restrict__ nonmeet,
+// Rounds first..9 of Philox-4x32-10.
+template <int kFirst>
+__device__ __forceinline__ uint4 philox_rounds(uint4 x, const PhiloxKeys& K) {
+#pragma unroll
+    for (int i = kFirst; i < 10; ++i) {
+        const unsigned long long p0 = (unsigned long long)kPhiloxM0 * x.x;
+        const unsigned long long p1 = (unsigned long long)kPhiloxM1 * x.z;
+        x = make_uint4((uint32_t)(p1 >> 32) ^ x.y ^ K.k0[i], (uint32_t)p1, (uint32_t)(p0 >> 32) ^ x.w ^ K.k1[i],
+                       (uint32_t)p0);
+    }
+    return x;
+}
+
+// The table entry i places after a row's first one.  kNarrow: positions are byte offsets
+// of 32 bits (a table below 4 GiB), which the load adds to its uniform base.
+template <bool kNarrow>
+__device__ __forceinline__ uint2 walk_entry(const uint2* __restrict__ walk, uint32_t first, uint32_t i) {
+    if constexpr (kNarrow)
+        return __ldg(reinterpret_cast<const uint2*>(reinterpret_cast<const char*>(walk) + (first + (i << 3))));
+    else return __ldg(walk + (first + i));
+}
+
+// Whether two walks stand on the same node.
+template <bool kNarrow>
+__device__ __forceinline__ bool same_node(uint2 A, uint2 B) {
+    return kNarrow ? A.x == B.x : A.x == B.x && A.y == B.y;
+}
+
+// The move of both walks on the words w of step t; false when the pair does not go on
+// (a walk stops or has nowhere to go).  forced: the step is taken without the draw.
+template <bool kNarrow>
+__device__ __forceinline__ bool walk_move(uint4 w, bool forced, uint32_t T, uint2& A, uint2& B, uint32_t rlo, uint32_t rhi,
+                                          uint32_t k, uint32_t t, const uint2* __restrict__ walk, const PhiloxKeys& K) {
+    const bool cont = (forced | ((w.x < T) & (w.z < T))) & (A.y != 0u) & (B.y != 0u);
+    const unsigned long long ma = (unsigned long long)w.y * A.y;
+    const unsigned long long mb = (unsigned long long)w.w * B.y;
+    uint32_t ia = (uint32_t)(ma >> 32), ib = (uint32_t)(mb >> 32);
+    if (__builtin_expect(cont & (((uint32_t)ma < A.y) | ((uint32_t)mb < B.y)), 0)) {
+        if ((uint32_t)ma < A.y) ia = pick_redraw(A.y, ma, rlo, rhi, k, 0x80000000u | t, K);
+        if ((uint32_t)mb < B.y) ib = pick_redraw(B.y, mb, rlo, rhi, k, 0xC0000000u | t, K);
+    }
+    if (cont) {
+        A = walk_entry<kNarrow>(walk, A.x, ia);
+        B = walk_entry<kNarrow>(walk, B.x, ib);
+    }
+    return cont;
+}
+
+// len pairs (r0, r0 + 1, ...; no carry into the high word) of node k, depth d (kForced:
+// d > 0), by the whole warp.  Adds this lane's steps; returns its count: Algorithm 2 counts
+// pairs that never meet, Algorithm 3 pairs that first meet after their d forced steps.
+template <bool kForced, bool kNarrow>
+__device__ __forceinline__ uint32_t run_one(const WalkArgs& a, uint32_t k, uint2 home, uint32_t d, uint32_t rlo0,
+                                            uint32_t rhi, uint32_t len, const PhiloxKeys& K, uint32_t& steps) {
+    const uint32_t lane = threadIdx.x & 31;
+    // round 0 multiplies k and r only; of round 1 the product of the first word is the run's
+    const unsigned long long q1 = (unsigned long long)kPhiloxM1 * k;
+    const uint32_t x0 = (uint32_t)(q1 >> 32) ^ rhi ^ K.k0[0];
+    const uint32_t y0 = (uint32_t)q1 ^ K.k0[1];
+    const unsigned long long q0 = (unsigned long long)kPhiloxM0 * x0;
+    const uint32_t z1 = (uint32_t)(q0 >> 32) ^ K.k1[1], w1 = (uint32_t)q0;
+    uint32_t next = 32, rlo = rlo0 + lane, t = 0, cnt = 0;
+    unsigned long long p = (unsigned long long)kPhiloxM0 * rlo;
+    uint32_t ph = (uint32_t)(p >> 32) ^ K.k1[0], pl = (uint32_t)p ^ z1;
+    uint2 A = home, B = home;
+    auto words = [&]() {
+        const unsigned long long p1 = (unsigned long long)kPhiloxM1 * (ph ^ t);
+        return philox_rounds<2>(make_uint4((uint32_t)(p1 >> 32) ^ y0, (uint32_t)p1, pl, w1), K);
+    };
+    auto restart = [&](uint32_t i) {
+        rlo = rlo0 + i;
+        p = (unsigned long long)kPhiloxM0 * rlo;
+        ph = (uint32_t)(p >> 32) ^ K.k1[0];
+        pl = (uint32_t)p ^ z1;
+        t = 0;
+        A = B = home;
+    };
+    // While 32 more pairs are left every lane has one, and before iteration 65535 no pair is
+    // that long: neither is tested here.
+    uint32_t it = 0;
+    for (; next + 32 <= len && it < kWalkMaxSteps - 1; ++it) {
+        const uint4 w = words();
+        const bool cont = walk_move<kNarrow>(w, kForced && t < d, a.T, A, B, rlo, rhi, k, t, a.walk, K);
+        const bool go = cont & !same_node<kNarrow>(A, B);
+        if (kForced) cnt += (cont & !go & (t >= d)) ? 1u : 0u;
+        else cnt += cont ? 0u : 1u;
+        const uint32_t done = __ballot_sync(0xffffffffu, !go);
+        ++t;
+        if (!go) restart(next + __popc(done & lanes_below()));
+        next += __popc(done);
+    }
+    steps += it;
+    bool active = rlo - rlo0 < len;
+    while (__any_sync(0xffffffffu, active)) {
+        const uint4 w = words();
+        const bool cont = active && walk_move<kNarrow>(w, kForced && t < d, a.T, A, B, rlo, rhi, k, t, a.walk, K);
+        const bool meet = cont & same_node<kNarrow>(A, B);
+        const bool ended = active & !(cont & !meet & (t + 1u < kWalkMaxSteps));
+        steps += active ? 1u : 0u;
+        cnt += (ended & (kForced ? meet & (t >= d) : !meet)) ? 1u : 0u;
+        const uint32_t done = __ballot_sync(0xffffffffu, ended);
+        ++t;
+        if (ended) {
+            const uint32_t i = next + __popc(done & lanes_below());
+            active = i < len;
+            restart(i);
+        }
+        next += __popc(done);
+    }
+    return cnt;
+}
+
+// Index of the segment that holds pair g (off[seg] <= g < off[seg+1]), seg >= lo, by the
+// whole warp: each round splits the interval in 32.
+__device__ __forceinline__ uint64_t find_segment(const uint64_t* __restrict__ off, uint64_t lo, uint64_t hi,
+                                                 unsigned long long g) {
+    const uint32_t lane = threadIdx.x & 31;
+    while (hi - lo > 1) {  // off[lo] <= g < off[hi]
+        const uint64_t step = (hi - lo + 31) >> 5;
+        const uint64_t at = lo + (uint64_t)(lane + 1) * step;
+        const bool below = at < hi && __ldg(off + at) <= g;
+        const int c = __popc(__ballot_sync(0xffffffffu, below));  // the lanes below are the first c
+        const uint64_t nlo = lo + (uint64_t)c * step;
+        hi = nlo + step < hi ? nlo + step : hi;
+        lo = nlo;
+    }
+    return lo;
+}
+
+// The pairs from g on, up to g1 or to the first segment with kRunMin pairs or more of the
+// chunk, over many segments; seg holds g.  Returns where it stopped (seg likewise).
+template <bool kNarrow>
+__device__ __forceinline__ unsigned long long run_many(const WalkArgs& a, unsigned long long g, unsigned long long g1,
+                                                    uint64_t& seg_io, const PhiloxKeys& K, uint32_t& steps) {
+    const uint32_t lane = threadIdx.x & 31;
+    uint64_t wseg = seg_io;        // the window: segments wseg .. wseg + 31, one per lane
+    uint32_t wend = 0, next = 0;   // pairs g + [next, wend) of the window are not taken yet
+    uint32_t start = 0;            // pair number (from g) at which this lane's segment starts
+    bool last = false;             // no window after this one
+    bool active = false;
+    uint32_t k = 0, rlo = 0, rhi = 0, t = 0, d = 0;
+    uint64_t seg = 0;
+    uint2 A = make_uint2(0u, 0u), B = A;
+    bool first = true;
+    for (;;) {
+        const uint32_t idle = __ballot_sync(0xffffffffu, !active);
+        if (idle && next >= wend && !last) {  // the next window (uniform)
+            if (!first) {
+                wseg += 32;
+                g += wend;
+                next = wend = 0;
+            }
+            first = false;
+            if (g >= g1 || wseg >= a.nseg) {
+                last = true;
+            } else {
+                uint64_t e = wseg + lane + 1 <= a.nseg ? wseg + lane + 1 : a.nseg;
+                unsigned long long hi = __ldg(a.off + e);
+                if (!__any_sync(0xffffffffu, hi > g)) {  // a stretch without pairs: to the one that holds g
+                    wseg = find_segment(a.off, wseg + 32, a.nseg, g);
+                    e = wseg + lane + 1 <= a.nseg ? wseg + lane + 1 : a.nseg;
+                    hi = __ldg(a.off + e);
+                }
+                if (hi > g1) hi = g1;
+                if (hi < g) hi = g;
+                unsigned long long lo = __shfl_up_sync(0xffffffffu, hi, 1);
+                if (lane == 0) lo = g;
+                const uint32_t large = __ballot_sync(0xffffffffu, hi - lo >= kRunMin);
+                const int upto = large ? __ffs(large) - 1 : 32;  // segments of the window to run here
+                start = (uint32_t)(lo - g);
+                const uint32_t all = (uint32_t)(__shfl_sync(0xffffffffu, hi, 31) - g);
+                wend = upto < 32 ? __shfl_sync(0xffffffffu, start, upto & 31) : all;
+                if (upto < 32) {
+                    last = true;
+                    if ((int)lane >= upto) start = 0xffffffffu;
+                    seg_io = wseg + (uint32_t)upto;
+                }
+            }
+        }
+        // idle lanes take pairs: the segment is the last one that starts at or before it
+        if (idle) {
+            const uint32_t i = next + __popc(idle & lanes_below());
+            const bool take = !active && i < wend;
+            int j = 0;
+#pragma unroll
+            for (int s = 16; s > 0; s >>= 1) {
+                const uint32_t v = __shfl_sync(0xffffffffu, start, j + s);
+                if (v <= i) j += s;
+            }
+            const uint32_t sj = __shfl_sync(0xffffffffu, start, j);
+            next += __popc(idle);
+            if (next > wend) next = wend;
+            if (take) {
+                seg = wseg + (uint32_t)j;
+                k = segment_node(seg, a.n, a.sh);
+                // pair number inside the segment: g + sj is where the window's share of it starts
+                const unsigned long long r = (a.sh.rbase ? __ldg(a.sh.rbase + seg) : 0ull) + (g + i - __ldg(a.off + seg));
+                (void)sj;
+                rlo = (uint32_t)r;
+                rhi = (uint32_t)(r >> 32);
+                d = a.depth ? a.depth[k] : 0u;
+                A = B = __ldg(a.row + k);
+                t = 0;
+                active = true;
+            }
+        }
+        if (!__any_sync(0xffffffffu, active)) {
+            if (last) break;
+            continue;
+        }
+        const uint4 w = philox_rounds<0>(make_uint4(rlo, rhi, k, t), K);
+        const bool cont = active && walk_move<kNarrow>(w, t < d, a.T, A, B, rlo, rhi, k, t, a.walk, K);
+        const bool meet = cont & same_node<kNarrow>(A, B);
+        const bool go = cont & !meet & (t + 1u < kWalkMaxSteps);
+        steps += active ? 1u : 0u;
+        if (active & !go) {
+            if (d ? (meet & (t >= d)) : !meet) atomicAdd(a.counts + seg, 1ull);
+            active = false;
+        }
+        ++t;
+    }
+    return g + wend;
+}
+
+// Persistent walk-pair sampler (see above).  work: the chunk counter, zero before and
+// after the launch (the last block to finish clears it); ticket likewise.
+template <bool kNarrow>
+__global__ void __launch_bounds__(kBlock, 6) sample_pairs_kernel(const __grid_constant__ WalkArgs a, const __grid_constant__ PhiloxKeys K,
+                                                                 double budget,
                                                                  unsigned long long* __restrict__ steps_out,
-                                                                 Status* __restrict__ st,
-                                                                 const uint8_t* __restrict__ depth,
-                                                                 const SharedSegs sh) {
-    __shared__ unsigned long long red[kBlock / 32];
-    const unsigned long long total = off[nseg];
+                                                                 Status* __restrict__ st, SampleWork* __restrict__ work) {
+    __shared__ unsigned long long wsteps[kBlock / 32];
+    unsigned long long total = __ldg(a.off + a.nseg);
     if ((double)total > budget || (st->err & kErrBudget)) {
         if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&st->err, kErrBudget);
-        return;
+        total = 0ull;  // no walks; the block still counts itself in the ticket below
     }
-    const unsigned long long nthreads = (unsigned long long)gridDim.x * blockDim.x;
-    const unsigned long long tid = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const unsigned long long per = total / nthreads, rem = total % nthreads;
-    const unsigned long long g0 = tid * per + (tid < rem ? tid : rem);
-    const unsigned long long g1 = g0 + per + (tid < rem ? 1ull : 0ull);
-    PairState S;
-    S.left = g1 - g0;
-    S.g_end = g1;
-    S.cnt = 0;
-    S.t = 0;
-    unsigned long long steps = 0;
-    if (S.left) {
-        int64_t lo = 0, hi = nseg;  // segment of pair g0: off[seg] <= g0 < off[seg+1]
-        while (hi - lo > 1) {
-            const int64_t mid = (lo + hi) >> 1;
-            if (__ldg(off + mid) <= g0) lo = mid; else hi = mid;
+    const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const unsigned long long nwarps = (unsigned long long)gridDim.x * (kBlock / 32);
+    // A few pairs are spread over all warps, 32 or more each: the launch then lasts as long as
+    // its longest pair (18,000 pairs: the query takes 329 us, 370 with chunks of 256).  Many go
+    // in chunks of at least kChunkMin, which pay for the search for their segment, about
+    // kChunksPerWarp for each warp (24 instead of 8: 8.50 against 8.39 ms).
+    unsigned long long size = total / nwarps < kChunkMin ? total / nwarps : kChunkMin;
+    if (total / (nwarps * kChunksPerWarp) > size) size = total / (nwarps * kChunksPerWarp);
+    size = size < 32 ? 32 : (size > kChunkMax ? kChunkMax : size);
+    const unsigned long long nchunks = (total + size - 1) / size;
+    if (lane == 0) wsteps[wid] = 0ull;
+    // consecutive chunks go to different blocks, so that a few chunks use all SMs
+    unsigned long long c = (unsigned long long)wid * gridDim.x + blockIdx.x;
+    while (c < nchunks) {
+        unsigned long long g = c * size;
+        const unsigned long long g1 = g + size < total ? g + size : total;
+        uint64_t seg = find_segment(a.off, 0, a.nseg, g);
+        uint32_t steps = 0;
+        while (g < g1) {
+            const unsigned long long sb = __ldg(a.off + seg), se = __ldg(a.off + seg + 1);
+            unsigned long long end = se < g1 ? se : g1;
+            // a long run, or what is left of the chunk lies in one segment
+            if (end - g >= kRunMin || end == g1) {
+                const uint32_t k = segment_node(seg, a.n, a.sh);
+                const unsigned long long r = (a.sh.rbase ? __ldg(a.sh.rbase + seg) : 0ull) + (g - sb);
+                const unsigned long long carry = (1ull << 32) - (r & 0xffffffffull);  // pairs to the next high word
+                if (end - g > carry) end = g + carry;
+                const uint32_t d = a.depth ? a.depth[k] : 0u, len = (uint32_t)(end - g);
+                const uint2 home = __ldg(a.row + k);
+                uint32_t cnt = d ? run_one<true, kNarrow>(a, k, home, d, (uint32_t)r, (uint32_t)(r >> 32), len, K, steps)
+                                 : run_one<false, kNarrow>(a, k, home, 0u, (uint32_t)r, (uint32_t)(r >> 32), len, K, steps);
+                cnt = __reduce_add_sync(0xffffffffu, cnt);
+                if (lane == 0 && cnt) atomicAdd(a.counts + seg, (unsigned long long)cnt);
+                g = end;
+                if (g == se) ++seg;
+                if (g < g1 && __ldg(a.off + seg + 1) <= g) seg = find_segment(a.off, seg, a.nseg, g);
+            } else {
+                g = run_many<kNarrow>(a, g, g1, seg, K, steps);
+            }
         }
-        S.seg = (unsigned long long)lo;
-        S.k = segment_node(S.seg, (unsigned long long)n, sh);
-        S.d = depth ? depth[S.k] : 0u;
-        const unsigned long long rb = sh.rbase ? __ldg(sh.rbase + S.seg) : 0ull;
-        S.r = rb + (g0 - __ldg(off + S.seg));
-        S.rk = rb + (__ldg(off + S.seg + 1) - __ldg(off + S.seg));
-        S.xa = S.xb = S.k;
-        for (;;) {
-            if (!S.left) break;
-            pair_step(S, row, col, off, T, K, nonmeet, steps, (unsigned long long)n, depth, sh);
+        steps = __reduce_add_sync(0xffffffffu, steps);
+        if (lane == 0) {
+            wsteps[wid] += steps;
+            c = nwarps + atomicAdd(&work->next, 1ull);
         }
+        c = __shfl_sync(0xffffffffu, c, 0);
     }
-    steps = block_sum(steps, red);
-    if (threadIdx.x == 0 && steps) atomicAdd(steps_out, steps);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        unsigned long long s = 0;
+        for (int w = 0; w < kBlock / 32; ++w) s += wsteps[w];
+        if (s) atomicAdd(steps_out, s);
+        if (atomicInc(&work->done, gridDim.x - 1) == gridDim.x - 1) work->next = 0ull;  // every chunk was taken
+    }
 }
 
 __global__ void dhat_kernel(int64_t n, const uint64_t* __restrict__ nonmeet, const uint64_t* __restrict__ off,
@@ -421,10 +644,35 @@ __global__ void mark_kernel(const int32_t* __restrict__ ids, int count, uint8_t*
     for (int i = threadIdx.x; i < count; i += blockDim.x) mark[ids[i]] = 1u;
 }
 
+// (first in-edge, din) of every node, or (node, 0) without in-edges; positions times 8 in
+// a narrow table
+__global__ void walk_rows_kernel(int64_t n, const uint32_t* __restrict__ rp, int shift, uint2* __restrict__ row) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const uint32_t b = rp[i], d = rp[i + 1] - b;
+        row[i] = make_uint2(((d ? b : (uint32_t)i) << shift) | (d || !shift ? 0u : 4u), d);
+    }
+}
+
+// the same of the node behind every in-edge
+__global__ void walk_edges_kernel(int64_t m, const int32_t* __restrict__ col, const uint2* __restrict__ row,
+                                  uint2* __restrict__ walk) {
+    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < m; p += (int64_t)gridDim.x * blockDim.x)
+        walk[p] = row[col[p]];
+}
+
 static int eb_cap(const Graph& g, int64_t n) {
     int64_t b = (n + kBlock - 1) / kBlock;
     if (b > (int64_t)g.sm_count * 8) b = (int64_t)g.sm_count * 8;
     return (int)(b < 1 ? 1 : b);
+}
+
+// 32-bit byte offsets reach the whole walk table
+static bool walk_narrow(const Graph& g) { return (g.m > g.n ? g.m : g.n) < ((int64_t)1 << 29); }
+
+cudaError_t launch_walk_table(const Graph& g) {
+    walk_rows_kernel<<<eb_cap(g, g.n), kBlock, 0, g.stream>>>(g.n, g.in.rp, walk_narrow(g) ? 3 : 0, g.in.info);
+    walk_edges_kernel<<<eb_cap(g, g.m), kBlock, 0, g.stream>>>(g.m, g.in.col, g.in.info, g.in.walk);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_mask_R(const Graph& g, const uint64_t* R, const uint8_t* keep, uint8_t want_mask, uint64_t* R_out) {
@@ -469,17 +717,19 @@ cudaError_t launch_sample_segments(const Graph& g, int64_t nseg, const uint64_t*
     }
     if (g_sample_blocks_per_sm == 0) {
         int b = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, sample_pairs_kernel, kBlock, 0);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, sample_pairs_kernel<true>, kBlock, 0);
         if (e != cudaSuccess) return e;
         g_sample_blocks_per_sm = b > 0 ? b : 1;
     }
     const int per_sm = g.sample_block_cap > 0 && g.sample_block_cap < g_sample_blocks_per_sm ? g.sample_block_cap
                                                                                               : g_sample_blocks_per_sm;
     const unsigned blocks = (unsigned)(g.sm_count * per_sm);
-    sample_pairs_kernel<<<blocks, kBlock, 0, g.stream>>>(g.n, nseg, g.in.info, g.in.col, off, walk_threshold(c),
-                                                         philox_keys(seed), g.pair_budget,
-                                                         (unsigned long long*)nonmeet, steps, g.status, depth,
-                                                         SharedSegs{rbase ? shared_B : 0, rbase});
+    const WalkArgs a{g.in.info, g.in.walk, off, depth, (unsigned long long*)nonmeet, (uint64_t)nseg, (uint64_t)g.n,
+                     SharedSegs{rbase ? shared_B : 0, rbase}, walk_threshold(c)};
+    // the side launch may run beside a launch on the query's own stream: each has its counter
+    SampleWork* work = &g.status->work[steps == &g.status->pair_steps_side ? 1 : 0];
+    auto* kernel = walk_narrow(g) ? sample_pairs_kernel<true> : sample_pairs_kernel<false>;
+    kernel<<<blocks, kBlock, 0, g.stream>>>(a, philox_keys(seed), g.pair_budget, steps, g.status, work);
     return cudaGetLastError();
 }
 
