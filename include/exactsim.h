@@ -435,8 +435,8 @@ esim_status esim_select_topk(esim_graph* g, const double* scores, int64_t exclud
  * every node; slots beyond the eligible nodes get id -1 and score 0.  Needs no
  * graph handle; work is enqueued on `stream` (a cudaStream_t of the current
  * device, NULL for the legacy default stream) and the call returns without
- * waiting.  Scratch: a static device array of about 66 KB (the radix-select state
- * and 4096 candidates), resident on every GPU that loads the library until the
+ * waiting.  Scratch: a static device array of about 328 KB (the slices' maxima and
+ * the candidates), resident on every GPU that loads the library until the
  * process exits.  The first call on a device looks up that array's device address
  * (cudaGetSymbolAddress, with the device current); make that first call before
  * any stream capture.  The address is kept with the id of the CUDA context it was

@@ -671,7 +671,7 @@ esim_status plan_alg3(Graph& g, const Ws& w, double c, double R_b, int* launches
     double* vals_d = (double*)stage;
     int32_t* ids_d = (int32_t*)(stage + sizeof(double) * kTopkMax);
     ESIM_CUDA_TRY(launch_topk(g, w.pi, -1, K, ids_d, vals_d, g.topk_ws), "Algorithm 3 node selection");
-    *launches += 27;
+    *launches += 2;
     std::vector<int32_t> ids((size_t)K);
     std::vector<double> pis((size_t)K);
     ESIM_CUDA_TRY(cudaMemcpyAsync(ids.data(), ids_d, sizeof(int32_t) * K, cudaMemcpyDeviceToHost, g.stream), "copy ids");
@@ -900,12 +900,12 @@ esim_status run_query(Graph& g, int64_t u, double c, double eps, uint64_t seed, 
     const Status hs = *g.status_host;
     g.last_L = L;
     // kernels launched: forward init + per level (rows [+ long rows]), 3 allocation
-    // kernels, the sampler, D^, reverse init + per level, and 27 for top-k
+    // kernels, the sampler, D^, reverse init + per level, and 2 for top-k
     // the sparse history's sweeps sum in FP64 on the row kernel (long-row table nlong), the
     // others on the tile kernel (tnlong)
     const int fwd_per = 1 + (sparse ? (g.out.nlong > 0) : (g.out.tnlong > 0));
     const int rev_per = 1 + (sparse ? (g.in.nlong > 0) : (g.in.tnlong > 0));
-    g.last_launches = (1 + L * fwd_per) + 3 + 1 + 1 + (1 + L * rev_per) + (k > 0 ? 27 : 0) + extra_launches;
+    g.last_launches = (1 + L * fwd_per) + 3 + 1 + 1 + (1 + L * rev_per) + (k > 0 ? 2 : 0) + extra_launches;
     if (sparse) g.last_launches += 2 * (L + 1) + count_launches;  // compactions, scatters, counting pass
     g.last_hist_entries = sparse ? std::min<uint64_t>(hs.hist_count, cap) : (uint64_t)(L + 1) * (uint64_t)g.n;
     g.last_R_b = R_b;
@@ -1071,7 +1071,7 @@ esim_status run_batch(Graph& g, int32_t B, const int64_t* u, const double* eps, 
     const Status hs = *g.status_host;
     g.last_L = plan.Lmax;
     g.last_launches = 1 + plan.Lmax * (1 + (g.out.nlong > 0 ? 1 : 0)) + 1 + 3 + 1 + 1 + 1 +
-                      plan.Lmax * (1 + (g.in.nlong > 0 ? 1 : 0)) + (k > 0 ? 27 : 0) + (g.shared_walks ? 2 : 0);
+                      plan.Lmax * (1 + (g.in.nlong > 0 ? 1 : 0)) + (k > 0 ? 2 : 0) + (g.shared_walks ? 2 : 0);
     g.last_R_b = plan.Rb[0];
     g.last_kappa = kappa_of(g, c);
     g.last_norm2 = 0.0;

@@ -2,11 +2,21 @@
 //
 // Each candidate node i gets a 96-bit key (ordered(score) << 32 | ~i): a larger
 // key is a higher score, and among equal scores a smaller id.  Keys are unique,
-// so the top-k set is unique.  A most-significant-digit radix select (8-bit
-// digits, warp-aggregated shared-memory histograms) narrows a key prefix until
-// the bucket at the current depth holds exactly the number of keys still
-// needed; every key at or above that prefix is selected, and one block sorts
-// the <= 4096 winners (bitonic, shared memory).
+// so the top-k set is unique.
+//
+// Two launches read the scores once each.  The first cuts the nodes into slices (one
+// thread's or a group of lanes' elements, a few thousand in all) and keeps each slice's
+// largest key; its last block to finish finds the k-th largest of those by a radix select
+// over 8-bit digits.  The slices' maxima are k different keys, so the k-th largest of all
+// keys is no smaller: that is a bound below which nothing is selected.  The second launch
+// collects the keys at or above the bound, little more than k of them, and its last block
+// sorts them.  If they are more than its list holds (scores arranged so that a few slices
+// hold most of the large ones), that block selects over all scores by radix itself.
+//
+// What bounds it: two passes over n scores (8 MB at n = 2^20: 1.2 us each at the HBM rate)
+// and about five dependent small steps.  Histogram and select launches for every digit of
+// the key, most of them with nothing left to do, took 142 us there for k = 100; this takes
+// 30 (and 46 with the maxima read from L2 for every digit instead of once into registers).
 #include "common.cuh"
 #include "internal.h"
 #include "exactsim.h"
@@ -19,15 +29,16 @@ namespace esim {
 
 namespace {
 
+constexpr int kTopkThreads = 1024;
+constexpr int kMaxSlices = 16384;   // maxima per column
+constexpr int kCandMax = 8192;      // collected keys per column, at most
+
 struct TopkState {
-    unsigned long long pre_hi;
-    unsigned int pre_lo;
-    unsigned int k_rem;
-    int depth;      // number of 8-bit digits fixed in the prefix
-    int done;
-    unsigned int count;
-    unsigned int pad;
-    unsigned int hist[256];
+    unsigned long long bound_hi;
+    unsigned int bound_lo;
+    unsigned int count;       // keys collected
+    unsigned int ticket[2];   // blocks of the two launches that have finished
+    unsigned int pad[2];
 };
 
 struct Cand {
@@ -50,155 +61,291 @@ __device__ __forceinline__ unsigned digit_of(unsigned long long hi, unsigned lo,
     return d < 8 ? (unsigned)((hi >> (56 - 8 * d)) & 0xFFu) : (unsigned)((lo >> (24 - 8 * (d - 8))) & 0xFFu);
 }
 
-// Compare the top `depth` digits of (hi, lo) with the prefix: -1, 0, +1.
-__device__ __forceinline__ int cmp_prefix(unsigned long long hi, unsigned lo, const TopkState& s, int depth) {
+// The prefix of a radix select over the keys' 8-bit digits, most significant first.
+struct Prefix {
+    unsigned long long hi;
+    unsigned int lo;
+    unsigned int k_rem;   // keys still to select within the prefix
+    int done;
+    int depth;            // digits fixed
+};
+
+// Whether the top `depth` digits of the key are the prefix's (-1, 0, +1).
+__device__ __forceinline__ int cmp_prefix(unsigned long long hi, unsigned lo, const Prefix& s, int depth) {
     if (depth == 0) return 0;
     if (depth <= 8) {
         const int sh = 64 - 8 * depth;
-        const unsigned long long a = hi >> sh, b = s.pre_hi >> sh;
+        const unsigned long long a = hi >> sh, b = s.hi >> sh;
         return a < b ? -1 : (a > b ? 1 : 0);
     }
-    if (hi != s.pre_hi) return hi < s.pre_hi ? -1 : 1;
+    if (hi != s.hi) return hi < s.hi ? -1 : 1;
     const int sh = 32 - 8 * (depth - 8);
-    const unsigned a = sh >= 32 ? 0u : (lo >> sh), b = sh >= 32 ? 0u : (s.pre_lo >> sh);
+    const unsigned a = lo >> sh, b = s.lo >> sh;
     return a < b ? -1 : (a > b ? 1 : 0);
 }
 
-// Every kernel below handles one column per blockIdx.y (select/sort: blockIdx.x);
-// a single selection is the one-column case.
-__global__ void topk_init_kernel(TopkState* st, unsigned k) {
-    st += blockIdx.x;
-    const int t = threadIdx.x;
-    if (t == 0) {
-        st->pre_hi = 0;
-        st->pre_lo = 0;
-        st->k_rem = k;
-        st->depth = 0;
-        st->done = 0;
-        st->count = 0;
-    }
-    for (int b = t; b < 256; b += blockDim.x) st->hist[b] = 0;
-}
-
-__global__ void __launch_bounds__(kBlock) topk_hist_kernel(int64_t n, const double* __restrict__ scores,
-                                                           int64_t exclude, TopkState* __restrict__ st, int d,
-                                                           int64_t col_stride, const int64_t* __restrict__ excl) {
-    __shared__ unsigned int h[256];
-    scores += (int64_t)blockIdx.y * col_stride;
-    st += blockIdx.y;
-    if (excl) exclude = excl[blockIdx.y];
-    if (st->done) return;
-    for (int b = threadIdx.x; b < 256; b += blockDim.x) h[b] = 0;
-    __syncthreads();
-    const TopkState s = *st;
+// One block: fixes digits of `pre` until the keys of the prefix bucket are exactly those
+// still needed, or until at most `slack` more than k keys lie at or above the prefix.
+// key(i, hi, lo) gives key i < count, false where there is none.  Fewer than k keys in
+// all: the prefix stays empty (depth 0), which every key reaches.  kRegs > 0: count is at most
+// kRegs per thread, and the keys are read once, into registers.
+template <int kRegs, class Key>
+__device__ void radix_select(int64_t count, unsigned k, unsigned slack, Prefix& pre, unsigned* hist, const Key& key) {
     const int lane = threadIdx.x & 31;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    // warp-uniform loop so that every lane takes part in the match below
-    for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < n; base += stride) {
-        const int64_t i = base + lane;
-        unsigned dig = 256u;  // sentinel: not counted
-        if (i < n && i != exclude) {
-            const unsigned long long hi = ordered_bits(scores[i]);
-            const unsigned lo = ~(unsigned)i;
-            if (cmp_prefix(hi, lo, s, d) == 0) dig = digit_of(hi, lo, d);
+    if (threadIdx.x == 0) pre = Prefix{0ull, 0u, k, 0, 0};
+    unsigned long long rh[kRegs ? kRegs : 1];
+    unsigned rl[kRegs ? kRegs : 1];
+    bool there[kRegs ? kRegs : 1];
+    if constexpr (kRegs > 0) {
+#pragma unroll
+        for (int u = 0; u < kRegs; ++u) {
+            const int64_t i = threadIdx.x + (int64_t)u * blockDim.x;
+            there[u] = i < count && key(i, rh[u], rl[u]);
         }
-        // warp-aggregated increment: one shared atomic per distinct digit in the warp
-        const unsigned peers = __match_any_sync(0xffffffffu, dig);
-        if (dig < 256u && lane == __ffs(peers) - 1) atomicAdd(&h[dig], (unsigned)__popc(peers));
+    }
+    for (int d = 0; d < 12; ++d) {
+        for (int b = threadIdx.x; b < 256; b += blockDim.x) hist[b] = 0;
+        __syncthreads();
+        const Prefix s = pre;
+        if (s.done) break;
+        auto count_key = [&](bool is, unsigned long long hi, unsigned lo) {  // every lane takes part
+            const unsigned dig = is && cmp_prefix(hi, lo, s, d) == 0 ? digit_of(hi, lo, d) : 256u;
+            const unsigned peers = __match_any_sync(0xffffffffu, dig);
+            if (dig < 256u && lane == __ffs(peers) - 1) atomicAdd(&hist[dig], (unsigned)__popc(peers));
+        };
+        if constexpr (kRegs > 0) {
+#pragma unroll
+            for (int u = 0; u < kRegs; ++u) count_key(there[u], rh[u], rl[u]);
+        } else {
+            for (int64_t base = threadIdx.x & ~31; base < count; base += blockDim.x) {  // warp-uniform
+                unsigned long long hi = 0;
+                unsigned lo = 0;
+                const bool is = base + lane < count && key(base + lane, hi, lo);
+                count_key(is, hi, lo);
+            }
+        }
+        __syncthreads();
+        if (threadIdx.x < 32) {  // lane l: bins 255 - 8l down to 248 - 8l
+            unsigned mine = 0;
+            for (int j = 0; j < 8; ++j) mine += hist[255 - 8 * lane - j];
+            unsigned incl = mine;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned v = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += v;
+            }
+            const unsigned total = __shfl_sync(0xffffffffu, incl, 31);
+            if (d == 0 && total <= s.k_rem) {
+                if (lane == 0) pre.done = 1;
+            } else if (incl >= s.k_rem && incl - mine < s.k_rem) {  // exactly one lane
+                unsigned cum = incl - mine;
+                int B = 255 - 8 * lane;
+                while (cum + hist[B] < s.k_rem) cum += hist[B--];
+                if (d < 8) pre.hi |= (unsigned long long)B << (56 - 8 * d);
+                else pre.lo |= (unsigned)B << (24 - 8 * (d - 8));
+                pre.k_rem = s.k_rem - cum;
+                pre.depth = d + 1;
+                pre.done = hist[B] <= pre.k_rem + slack;
+            }
+        }
+        __syncthreads();
     }
     __syncthreads();
-    for (int b = threadIdx.x; b < 256; b += blockDim.x)
-        if (h[b]) atomicAdd(&st->hist[b], h[b]);
 }
 
-__global__ void topk_select_kernel(TopkState* st, int d) {
-    st += blockIdx.x;
-    if (threadIdx.x != 0 || st->done) return;
-    unsigned total = 0;
-    for (int b = 0; b < 256; ++b) total += st->hist[b];
-    if (d == 0 && total <= st->k_rem) {  // fewer candidates than k: take all
-        st->done = 1;
-        st->depth = 0;
-    } else {
-        unsigned cum = 0;
-        int B = 0;
-        for (int b = 255; b >= 0; --b) {
-            const unsigned c = st->hist[b];
-            if (cum + c >= st->k_rem) {
-                B = b;
-                break;
-            }
-            cum += c;
-        }
-        if (d < 8) st->pre_hi |= (unsigned long long)B << (56 - 8 * d);
-        else st->pre_lo |= (unsigned)B << (24 - 8 * (d - 8));
-        st->k_rem -= cum;
-        st->depth = d + 1;
-        if (st->hist[B] == st->k_rem) st->done = 1;
-    }
-    for (int b = 0; b < 256; ++b) st->hist[b] = 0;
+// Whether this block is the last of the column to get here (all threads call it); what the
+// other blocks wrote before is then visible.
+__device__ __forceinline__ bool last_block(unsigned* ticket) {
+    __shared__ bool last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (last) __threadfence();
+    return last;
 }
 
-__global__ void __launch_bounds__(kBlock) topk_gather_kernel(int64_t n, const double* __restrict__ scores,
-                                                             int64_t exclude, TopkState* __restrict__ st,
-                                                             Cand* __restrict__ cand, unsigned cap, int64_t col_stride,
-                                                             const int64_t* __restrict__ excl) {
+// Launch 1: the largest key of every slice (the elements of G consecutive threads of a
+// block); the last block's bound.  One column per blockIdx.y in both launches.
+__global__ void __launch_bounds__(kTopkThreads) topk_bound_kernel(int64_t n, const double* __restrict__ scores,
+                                                                  int64_t exclude, TopkState* __restrict__ st,
+                                                                  unsigned long long* __restrict__ max_hi,
+                                                                  unsigned* __restrict__ max_lo, int G, unsigned k,
+                                                                  int64_t col_stride, const int64_t* __restrict__ excl) {
+    __shared__ unsigned hist[256];
+    __shared__ Prefix pre;
     scores += (int64_t)blockIdx.y * col_stride;
     st += blockIdx.y;
-    cand += (size_t)blockIdx.y * cap;
+    max_hi += (size_t)blockIdx.y * kMaxSlices;
+    max_lo += (size_t)blockIdx.y * kMaxSlices;
     if (excl) exclude = excl[blockIdx.y];
-    const TopkState s = *st;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        if (i == exclude) continue;
-        const unsigned long long hi = ordered_bits(scores[i]);
-        const unsigned lo = ~(unsigned)i;
-        if (cmp_prefix(hi, lo, s, s.depth) < 0) continue;
-        const unsigned slot = atomicAdd(&st->count, 1u);
-        if (slot < cap) cand[slot] = Cand{hi, lo, 0u};
+    const int64_t tid = (int64_t)blockIdx.x * kTopkThreads + threadIdx.x;
+    const int64_t stride = (int64_t)gridDim.x * kTopkThreads;
+    unsigned long long hi = 0;
+    unsigned lo = 0;  // 0: no element yet (~i is never 0)
+    constexpr int kU = 4;  // loads in flight
+    for (int64_t i0 = tid; i0 < n; i0 += stride * kU) {
+        double v[kU];
+#pragma unroll
+        for (int u = 0; u < kU; ++u)
+            if (i0 + u * stride < n) v[u] = scores[i0 + u * stride];
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+            const int64_t i = i0 + u * stride;
+            if (i >= n || i == exclude) continue;
+            const unsigned long long h = ordered_bits(v[u]);
+            if (lo == 0u || h > hi) {  // ids ascend: among equal scores the first stays
+                hi = h;
+                lo = ~(unsigned)i;
+            }
+        }
+    }
+    auto larger = [&](unsigned long long h, unsigned l) {
+        if (h > hi || (h == hi && l > lo)) {
+            hi = h;
+            lo = l;
+        }
+    };
+    for (int o = 1; o < G && o < 32; o <<= 1) {
+        const unsigned long long h = __shfl_xor_sync(0xffffffffu, hi, o);
+        larger(h, __shfl_xor_sync(0xffffffffu, lo, o));
+    }
+    if (G > 32) {  // slices of several warps
+        __shared__ unsigned long long wh[kTopkThreads / 32];
+        __shared__ unsigned wl[kTopkThreads / 32];
+        if ((threadIdx.x & 31) == 0) {
+            wh[threadIdx.x >> 5] = hi;
+            wl[threadIdx.x >> 5] = lo;
+        }
+        __syncthreads();
+        if ((threadIdx.x & (G - 1)) == 0)
+            for (int w = 1; w < G / 32; ++w) larger(wh[(threadIdx.x >> 5) + w], wl[(threadIdx.x >> 5) + w]);
+    }
+    if ((threadIdx.x & (G - 1)) == 0) {
+        max_hi[tid / G] = hi;
+        max_lo[tid / G] = lo;
+    }
+    if (!last_block(&st->ticket[0])) return;
+    auto key = [&](int64_t i, unsigned long long& h, unsigned& l) {
+        h = __ldcg(max_hi + i);
+        l = __ldcg(max_lo + i);
+        return l != 0u;
+    };
+    const int64_t slices = stride / G;
+    if (slices <= 4 * kTopkThreads) radix_select<4>(slices, k, k / 8 + 32, pre, hist, key);
+    else radix_select<0>(slices, k, k / 8 + 32, pre, hist, key);
+    if (threadIdx.x == 0) {
+        st->bound_hi = pre.hi;
+        st->bound_lo = pre.lo;
     }
 }
 
-// One block of 1024 threads sorts the selected keys, descending.  P (a power of
-// two >= k) keys live in dynamic shared memory: P * 12 bytes <= 48 KB.
-__global__ void __launch_bounds__(1024) topk_sort_kernel(const TopkState* __restrict__ st,
-                                                         const Cand* __restrict__ cand, int k, int P,
-                                                         int32_t* __restrict__ ids_out, double* __restrict__ vals_out,
-                                                         unsigned cap) {
+// Launch 2: the keys at or above the bound into cand (cap of them at most); the last block
+// sorts them, descending, and writes the first k.  P, a power of two >= cap, keys fit its
+// dynamic shared memory.
+__global__ void __launch_bounds__(kTopkThreads) topk_pick_kernel(int64_t n, const double* __restrict__ scores,
+                                                                 int64_t exclude, TopkState* __restrict__ st,
+                                                                 Cand* __restrict__ cand, unsigned cap, int k, int P,
+                                                                 int64_t col_stride, const int64_t* __restrict__ excl,
+                                                                 int32_t* __restrict__ ids_out,
+                                                                 double* __restrict__ vals_out) {
     extern __shared__ unsigned long long sm_hi[];
-    st += blockIdx.x;
-    cand += (size_t)blockIdx.x * cap;
-    ids_out += (size_t)blockIdx.x * k;
-    vals_out += (size_t)blockIdx.x * k;
+    __shared__ unsigned hist[256];
+    __shared__ Prefix pre;
+    __shared__ unsigned found;
     unsigned* sm_lo = (unsigned*)(sm_hi + P);
-    unsigned cnt = st->count;
-    if (cnt > (unsigned)k) cnt = (unsigned)k;  // cannot happen for unique keys; guards the buffer
-    for (int i = threadIdx.x; i < P; i += blockDim.x) {
-        const bool real = i < (int)cnt;
-        sm_hi[i] = real ? cand[i].hi : 0ull;  // (0, 0) is below every real key (ids < 2^31)
-        sm_lo[i] = real ? cand[i].lo : 0u;
+    scores += (int64_t)blockIdx.y * col_stride;
+    st += blockIdx.y;
+    cand += (size_t)blockIdx.y * kCandMax;
+    ids_out += (size_t)blockIdx.y * k;
+    vals_out += (size_t)blockIdx.y * k;
+    if (excl) exclude = excl[blockIdx.y];
+    const unsigned long long bh = st->bound_hi;
+    const unsigned bl = st->bound_lo;
+    const int lane = threadIdx.x & 31;
+    const int64_t stride = (int64_t)gridDim.x * kTopkThreads;
+    const int64_t tid = (int64_t)blockIdx.x * kTopkThreads + threadIdx.x;
+    constexpr int kU = 4;
+    for (int64_t i0 = tid - lane; i0 < n; i0 += stride * kU) {  // warp-uniform
+        double v[kU];
+#pragma unroll
+        for (int u = 0; u < kU; ++u)
+            if (i0 + lane + u * stride < n) v[u] = scores[i0 + lane + u * stride];
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+            const int64_t i = i0 + lane + u * stride;
+            unsigned long long h = 0;
+            const unsigned l = ~(unsigned)i;
+            bool take = i < n && i != exclude;
+            if (take) {
+                h = ordered_bits(v[u]);
+                take = h > bh || (h == bh && l >= bl);
+            }
+            const unsigned mask = __ballot_sync(0xffffffffu, take);
+            if (!mask) continue;
+            unsigned slot = 0;
+            if (lane == 0) slot = atomicAdd(&st->count, (unsigned)__popc(mask));
+            slot = __shfl_sync(0xffffffffu, slot, 0) + (unsigned)__popc(mask & ((1u << lane) - 1u));
+            if (take && slot < cap) cand[slot] = Cand{h, l, 0u};
+        }
     }
+    if (!last_block(&st->ticket[1])) return;
+    unsigned cnt = *(volatile unsigned*)&st->count;
+    if (cnt <= cap) {
+        for (int i = threadIdx.x; i < (int)cnt; i += kTopkThreads) {
+            sm_hi[i] = __ldcg(&cand[i].hi);
+            sm_lo[i] = __ldcg(&cand[i].lo);
+        }
+    } else {
+        radix_select<0>(n, (unsigned)k, 0u, pre, hist, [&](int64_t i, unsigned long long& h, unsigned& l) {
+            h = ordered_bits(scores[i]);
+            l = ~(unsigned)i;
+            return i != exclude;
+        });
+        if (threadIdx.x == 0) found = 0u;
+        __syncthreads();
+        const Prefix s = pre;
+        for (int64_t i = threadIdx.x; i < n; i += kTopkThreads) {
+            if (i == exclude) continue;
+            const unsigned long long h = ordered_bits(scores[i]);
+            const unsigned l = ~(unsigned)i;
+            if (cmp_prefix(h, l, s, s.depth) < 0) continue;
+            const unsigned slot = atomicAdd(&found, 1u);
+            if (slot < (unsigned)P) {  // k keys, or all of them where there are fewer
+                sm_hi[slot] = h;
+                sm_lo[slot] = l;
+            }
+        }
+        __syncthreads();
+        cnt = found < (unsigned)P ? found : (unsigned)P;
+    }
+    int Q = 1;
+    while (Q < (int)cnt) Q <<= 1;
+    for (int i = threadIdx.x; i < Q; i += kTopkThreads)
+        if (i >= (int)cnt) {
+            sm_hi[i] = 0ull;  // (0, 0) is below every real key (ids < 2^31)
+            sm_lo[i] = 0u;
+        }
     __syncthreads();
-    for (int size = 2; size <= P; size <<= 1) {
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-            for (int i = threadIdx.x; i < P; i += blockDim.x) {
-                const int j = i ^ stride;
-                if (j > i) {
-                    const unsigned long long ah = sm_hi[i], bh = sm_hi[j];
-                    const unsigned al = sm_lo[i], bl = sm_lo[j];
-                    const bool a_less = ah < bh || (ah == bh && al < bl);
-                    const bool desc = (i & size) == 0;  // overall order: descending
-                    if (desc ? a_less : !a_less) {
-                        sm_hi[i] = bh;
-                        sm_hi[j] = ah;
-                        sm_lo[i] = bl;
-                        sm_lo[j] = al;
-                    }
+    for (int size = 2; size <= Q; size <<= 1) {
+        for (int half = size >> 1; half > 0; half >>= 1) {
+            for (int p = threadIdx.x; p < Q / 2; p += kTopkThreads) {
+                const int i = 2 * p - (p & (half - 1)), j = i + half;
+                const unsigned long long ah = sm_hi[i], bh2 = sm_hi[j];
+                const unsigned al = sm_lo[i], bl2 = sm_lo[j];
+                const bool a_less = ah < bh2 || (ah == bh2 && al < bl2);
+                const bool desc = (i & size) == 0;  // overall order: descending
+                if (desc ? a_less : !a_less) {
+                    sm_hi[i] = bh2;
+                    sm_hi[j] = ah;
+                    sm_lo[i] = bl2;
+                    sm_lo[j] = al;
                 }
             }
             __syncthreads();
         }
     }
-    for (int i = threadIdx.x; i < k; i += blockDim.x) {
+    for (int i = threadIdx.x; i < k; i += kTopkThreads) {
         if (i < (int)cnt) {
             ids_out[i] = (int32_t)(~sm_lo[i]);
             vals_out[i] = from_ordered(sm_hi[i]);
@@ -209,64 +356,63 @@ __global__ void __launch_bounds__(1024) topk_sort_kernel(const TopkState* __rest
     }
 }
 
+// Workspace of B columns: states, maxima (hi, lo), candidates.
+constexpr size_t kStateBytes(size_t B) { return (sizeof(TopkState) * B + 255) / 256 * 256; }
+constexpr size_t kColumnBytes = (size_t)kMaxSlices * 12 + sizeof(Cand) * (size_t)kCandMax;
+
+// B selections; column q of scores starts at scores + q * stride, and excl[q] (or exclude
+// where excl is NULL, -1 for none) is left out of it.
+cudaError_t topk_select(cudaStream_t stream, int sms, int64_t n, int32_t B, const double* scores, int64_t col_stride,
+                        int64_t exclude, const int64_t* excl, int32_t k, int32_t* ids_out, double* vals_out, void* ws) {
+    TopkState* st = (TopkState*)ws;
+    unsigned long long* max_hi = (unsigned long long*)((char*)ws + kStateBytes((size_t)B));
+    unsigned* max_lo = (unsigned*)(max_hi + (size_t)B * kMaxSlices);
+    Cand* cand = (Cand*)(max_lo + (size_t)B * kMaxSlices);
+    // one element per thread until the chip is full (two blocks per SM over all columns)
+    int64_t blocks = (n + kTopkThreads - 1) / kTopkThreads;
+    const int64_t most = ((int64_t)sms * 2 + B - 1) / B;
+    if (blocks > most) blocks = most;
+    // (two blocks per SM keep 64 warps loading; with one element per thread and no slices of
+    // several warps a block would select from 16 keys a thread)
+    // slices: enough of them that their k-th maximum is a tight bound (with 4 k of them about
+    // 1.15 k keys reach it), few enough for one block to select from
+    const int64_t threads = blocks * kTopkThreads;
+    const int64_t want = 4 * (int64_t)k < 2048 ? 2048 : (4 * (int64_t)k > 8192 ? 8192 : 4 * (int64_t)k);
+    int G = 1;
+    while (G < kTopkThreads && threads / (2 * G) >= want) G <<= 1;
+    const unsigned cap = (unsigned)(2 * k + 1024 < kCandMax ? 2 * k + 1024 : kCandMax);
+    int P = 1;
+    while (P < (int)cap) P <<= 1;
+    const size_t smem = (size_t)P * 12;
+    cudaError_t e = cudaMemsetAsync(st, 0, sizeof(TopkState) * (size_t)B, stream);
+    if (e != cudaSuccess) return e;
+    if (smem > 48 * 1024 - 2048 &&
+        (e = cudaFuncSetAttribute(topk_pick_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
+            cudaSuccess)
+        return e;
+    const dim3 grid((unsigned)blocks, (unsigned)B);
+    topk_bound_kernel<<<grid, kTopkThreads, 0, stream>>>(n, scores, exclude, st, max_hi, max_lo, G, (unsigned)k,
+                                                         col_stride, excl);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    topk_pick_kernel<<<grid, kTopkThreads, smem, stream>>>(n, scores, exclude, st, cand, cap, k, P, col_stride, excl,
+                                                           ids_out, vals_out);
+    return cudaGetLastError();
+}
+
 }  // namespace
 
-size_t topk_workspace_bytes(int64_t /*n*/) { return sizeof(TopkState) + sizeof(Cand) * (size_t)kTopkMax + 256; }
+size_t topk_batch_workspace_bytes(int32_t B) { return kStateBytes((size_t)B) + kColumnBytes * (size_t)B + 256; }
+
+size_t topk_workspace_bytes(int64_t /*n*/) { return topk_batch_workspace_bytes(1); }
 
 cudaError_t launch_topk(const Graph& g, const double* scores, int64_t exclude, int32_t k, int32_t* ids_out,
                         double* vals_out, void* ws) {
-    TopkState* st = (TopkState*)ws;
-    Cand* cand = (Cand*)((char*)ws + ((sizeof(TopkState) + 255) / 256) * 256);
-    topk_init_kernel<<<1, 256, 0, g.stream>>>(st, (unsigned)k);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    int64_t blocks = (g.n + kBlock - 1) / kBlock;
-    if (blocks > (int64_t)g.sm_count * 4) blocks = (int64_t)g.sm_count * 4;
-    if (blocks < 1) blocks = 1;
-    for (int d = 0; d < 12; ++d) {
-        topk_hist_kernel<<<(unsigned)blocks, kBlock, 0, g.stream>>>(g.n, scores, exclude, st, d, 0, nullptr);
-        topk_select_kernel<<<1, 32, 0, g.stream>>>(st, d);
-    }
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    topk_gather_kernel<<<(unsigned)blocks, kBlock, 0, g.stream>>>(g.n, scores, exclude, st, cand, (unsigned)kTopkMax, 0,
-                                                                  nullptr);
-    int P = 1;
-    while (P < k) P <<= 1;
-    topk_sort_kernel<<<1, 1024, (size_t)P * 12, g.stream>>>(st, cand, k, P, ids_out, vals_out, (unsigned)kTopkMax);
-    return cudaGetLastError();
+    return topk_select(g.stream, g.sm_count, g.n, 1, scores, 0, exclude, nullptr, k, ids_out, vals_out, ws);
 }
 
-size_t topk_batch_workspace_bytes(int32_t B) {
-    return ((sizeof(TopkState) * (size_t)B + 255) / 256) * 256 + sizeof(Cand) * (size_t)kTopkMax * (size_t)B;
-}
-
-// B independent selections: column q of scores starts at scores + q * n; exclude[q]
-// (device, may be NULL for none) is left out of column q.
 cudaError_t launch_topk_batch(const Graph& g, int32_t B, const double* scores, const int64_t* exclude, int32_t k,
                               int32_t* ids_out, double* vals_out, void* ws) {
-    TopkState* st = (TopkState*)ws;
-    Cand* cand = (Cand*)((char*)ws + ((sizeof(TopkState) * (size_t)B + 255) / 256) * 256);
-    topk_init_kernel<<<(unsigned)B, 256, 0, g.stream>>>(st, (unsigned)k);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    int64_t blocks = (g.n + kBlock - 1) / kBlock;
-    int64_t cap = ((int64_t)g.sm_count * 4 + B - 1) / B;
-    if (blocks > cap) blocks = cap;
-    if (blocks < 1) blocks = 1;
-    const dim3 grid((unsigned)blocks, (unsigned)B);
-    for (int d = 0; d < 12; ++d) {
-        topk_hist_kernel<<<grid, kBlock, 0, g.stream>>>(g.n, scores, -1, st, d, g.n, exclude);
-        topk_select_kernel<<<(unsigned)B, 32, 0, g.stream>>>(st, d);
-    }
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    topk_gather_kernel<<<grid, kBlock, 0, g.stream>>>(g.n, scores, -1, st, cand, (unsigned)kTopkMax, g.n, exclude);
-    int P = 1;
-    while (P < k) P <<= 1;
-    topk_sort_kernel<<<(unsigned)B, 1024, (size_t)P * 12, g.stream>>>(st, cand, k, P, ids_out, vals_out,
-                                                                     (unsigned)kTopkMax);
-    return cudaGetLastError();
+    return topk_select(g.stream, g.sm_count, g.n, B, scores, g.n, -1, exclude, k, ids_out, vals_out, ws);
 }
 
 }  // namespace esim
@@ -290,15 +436,14 @@ cudaError_t launch_topk_batch(const Graph& g, int32_t B, const double* scores, c
 // the kernels.  The address is remembered together with the unique id of the CUDA
 // context it was taken in: after a device reset the device has a new context (and
 // the array a new address), so the next call takes the address again.  All calls
-// share the array and it keeps the last call's contents; topk_init_kernel clears
-// the state every call.  Calls whose work overlaps on the GPU (different streams,
+// share the array and it keeps the last call's contents; the state is cleared every
+// call.  Calls whose work overlaps on the GPU (different streams,
 // or several host threads) race on the array.
 // ---------------------------------------------------------------------------
 
 namespace {
 
-constexpr size_t kStaticTopkStateBytes = ((sizeof(esim::TopkState) + 255) / 256) * 256;
-constexpr size_t kStaticTopkScratchBytes = kStaticTopkStateBytes + sizeof(esim::Cand) * (size_t)esim::kTopkMax;
+constexpr size_t kStaticTopkScratchBytes = esim::kStateBytes(1) + esim::kColumnBytes;
 
 static __device__ __align__(256) unsigned char g_topk_static_scratch[kStaticTopkScratchBytes];
 
@@ -389,23 +534,7 @@ extern "C" __attribute__((visibility("default"))) esim_status esim_select_topk_s
     e = static_scratch(dev, &ws, &sms);
     if (e != cudaSuccess)
         return static_fail(ESIM_ECUDA, std::string("static scratch set-up: ") + cudaGetErrorString(e));
-    cudaStream_t st = (cudaStream_t)stream;
-    TopkState* state = (TopkState*)ws;
-    Cand* cand = (Cand*)((char*)ws + kStaticTopkStateBytes);
-    topk_init_kernel<<<1, 256, 0, st>>>(state, (unsigned)k);
-    int64_t blocks = (n + kBlock - 1) / kBlock;
-    if (blocks > (int64_t)sms * 4) blocks = (int64_t)sms * 4;
-    if (blocks < 1) blocks = 1;
-    for (int d = 0; d < 12; ++d) {
-        topk_hist_kernel<<<(unsigned)blocks, kBlock, 0, st>>>(n, scores, exclude, state, d, 0, nullptr);
-        topk_select_kernel<<<1, 32, 0, st>>>(state, d);
-    }
-    topk_gather_kernel<<<(unsigned)blocks, kBlock, 0, st>>>(n, scores, exclude, state, cand, (unsigned)kTopkMax, 0,
-                                                              nullptr);
-    int P = 1;
-    while (P < k) P <<= 1;
-    topk_sort_kernel<<<1, 1024, (size_t)P * 12, st>>>(state, cand, k, P, ids_out, vals_out, (unsigned)kTopkMax);
-    e = cudaGetLastError();
+    e = topk_select((cudaStream_t)stream, sms, n, 1, scores, 0, exclude, nullptr, k, ids_out, vals_out, ws);
     if (e != cudaSuccess) return static_fail(ESIM_ECUDA, std::string("static top-k launch: ") + cudaGetErrorString(e));
     return ESIM_OK;
 }
