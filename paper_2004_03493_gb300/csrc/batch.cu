@@ -10,8 +10,8 @@
 // (Algorithm 1, Eq. sL) gives each column exactly its own sum over l <= L_q.
 //
 // Every column accumulates a row's entries one after another in index order
-// (long rows: fixed 4096-entry segments, combined in segment order), whatever the
-// tile shape: a column's result does not depend on which other columns share the
+// (rows of kBatchSeg entries or more: segments of kBatchSeg, joined by four fixed
+// strides over the segments), whatever the tile shape: a column's result does not depend on which other columns share the
 // batch nor on the tile chosen by the autotuner.
 #include "common.cuh"
 #include "internal.h"
@@ -113,22 +113,32 @@ struct BRevOp {
 };
 
 // Short rows: LPR lanes per row, CPL columns per lane (W = LPR * CPL), entries of
-// the row in order.  Blocks past short_blocks sum one segment of a long row per
-// warp-group into partial[seg * W + column].
+// the row in order.  The first seg_blocks blocks sum one segment of a long row per
+// lane group into partial[seg * W + column].
+//
+// What bounds a level: the gathered rows (m x W values from L2) and, per lane group, the
+// chain of two-float additions, about 40 cycles an entry.  kU entries' rows are loaded
+// before they are added, and no chain is longer than kBatchSeg: with segments of 4096 and one
+// load in flight the longest segment alone took 460-770 us of every level with a hub.
+// 64 columns, n = 2^17, m = 3.75e6: 462 / 772 us forward / reverse before, 196 / 265 now;
+// 16 columns, n = 20,011, m = 2e5: 557 / 476 before, 18 / 23 at segments of 128.  The whole
+// query of five sources on that graph takes 0.87 ms at segments of 128, 0.76 at 64, 0.74 at
+// 32; the batch of 64 is fastest at 64 (a partial of 8 W bytes costs an eighth of the gathers
+// it stands for at 32).
 template <typename V, int LPR, int CPL, class Op>
 __global__ void __launch_bounds__(kBlock) batch_rows_kernel(int64_t n, const uint32_t* __restrict__ rp,
                                                             const int32_t* __restrict__ col, const V* __restrict__ X,
-                                                            uint32_t long_min, Op op, int64_t nseg,
-                                                            const Segment* __restrict__ seg, f2* __restrict__ partial,
-                                                            int short_blocks) {
+                                                            Op op, int64_t nseg, const Segment* __restrict__ seg,
+                                                            f2* __restrict__ partial, int seg_blocks) {
     constexpr int W = LPR * CPL;
     constexpr int RPW = 32 / LPR;  // rows (or segments) per warp per iteration
+    constexpr int kU = sizeof(V) * CPL <= 16 ? 8 : (sizeof(V) * CPL <= 32 ? 4 : 2);
     const int lane = threadIdx.x & 31;
     const int sub = lane / LPR, cl = lane % LPR;
     const int c0 = cl * CPL;
-    const bool segs = (int)blockIdx.x >= short_blocks;
-    const int64_t nblk = segs ? (int64_t)gridDim.x - short_blocks : short_blocks;
-    const int64_t blk = segs ? (int64_t)blockIdx.x - short_blocks : blockIdx.x;
+    const bool segs = (int)blockIdx.x < seg_blocks;
+    const int64_t nblk = segs ? seg_blocks : (int64_t)gridDim.x - seg_blocks;
+    const int64_t blk = segs ? blockIdx.x : (int64_t)blockIdx.x - seg_blocks;
     const int64_t warp = (blk * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = (nblk * blockDim.x) >> 5;
     const int64_t items = segs ? nseg : n;
@@ -136,7 +146,6 @@ __global__ void __launch_bounds__(kBlock) batch_rows_kernel(int64_t n, const uin
         const int64_t it = base + sub;
         uint32_t b = 0, e = 0;
         bool mine = false;
-        int64_t row = it;
         if (it < items) {
             if (segs) {
                 const Segment sg = seg[it];
@@ -146,25 +155,40 @@ __global__ void __launch_bounds__(kBlock) batch_rows_kernel(int64_t n, const uin
             } else {
                 b = __ldg(rp + it);
                 e = __ldg(rp + it + 1);
-                mine = (e - b) < long_min;
+                mine = (e - b) < kBatchSeg;
                 if (!mine) e = b;
             }
         }
         f2 acc[CPL];
 #pragma unroll
         for (int i = 0; i < CPL; ++i) acc[i] = f2{0.f, 0.f};
-        for (uint32_t p = b; p < e; ++p) {
-            const int64_t j = __ldg(col + p);
+        for (uint32_t p = b; p < e; p += kU) {
+            int32_t j[kU];
+#pragma unroll
+            for (int t = 0; t < kU; ++t)
+                if (p + t < e) j[t] = __ldg(col + p + t);
             if constexpr (sizeof(V) == 4) {
-                float v[CPL];
-                load_f<CPL>(reinterpret_cast<const float*>(X) + j * W + c0, v);
+                float v[kU][CPL];
 #pragma unroll
-                for (int i = 0; i < CPL; ++i) acc[i] = f2_add_f(acc[i], v[i]);
+                for (int t = 0; t < kU; ++t)
+                    if (p + t < e) load_f<CPL>(reinterpret_cast<const float*>(X) + (int64_t)j[t] * W + c0, v[t]);
+#pragma unroll
+                for (int t = 0; t < kU; ++t)
+                    if (p + t < e) {
+#pragma unroll
+                        for (int i = 0; i < CPL; ++i) acc[i] = f2_add_f(acc[i], v[t][i]);
+                    }
             } else {
-                f2 v[CPL];
-                load_f2<CPL>(reinterpret_cast<const float2*>(X) + j * W + c0, v);
+                f2 v[kU][CPL];
 #pragma unroll
-                for (int i = 0; i < CPL; ++i) acc[i] = f2_add(acc[i], v[i]);
+                for (int t = 0; t < kU; ++t)
+                    if (p + t < e) load_f2<CPL>(reinterpret_cast<const float2*>(X) + (int64_t)j[t] * W + c0, v[t]);
+#pragma unroll
+                for (int t = 0; t < kU; ++t)
+                    if (p + t < e) {
+#pragma unroll
+                        for (int i = 0; i < CPL; ++i) acc[i] = f2_add(acc[i], v[t][i]);
+                    }
             }
         }
         if (!mine) continue;
@@ -172,23 +196,37 @@ __global__ void __launch_bounds__(kBlock) batch_rows_kernel(int64_t n, const uin
 #pragma unroll
             for (int i = 0; i < CPL; ++i) partial[it * W + c0 + i] = acc[i];
         } else {
-            op.template operator()<CPL>(row, c0, acc);
+            op.template operator()<CPL>(it, c0, acc);
         }
     }
 }
 
-// Long rows: one lane per column combines the row's segment partials in order.
+// Long rows, one block of 4 W threads each: group g of a column adds the partials of
+// segments g, g + 4, ... in order, and the four sums are joined in a fixed order (four
+// whatever W is, so that a column's sum does not depend on its batch).
 template <int W, class Op>
-__global__ void __launch_bounds__(kBlock) batch_long_rows_kernel(int64_t nlong, const int32_t* __restrict__ long_rows,
-                                                                 const int32_t* __restrict__ long_first,
-                                                                 const f2* __restrict__ partial, Op op) {
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t r = t / W;
-    const int q = (int)(t % W);
-    if (r >= nlong) return;
+__global__ void __launch_bounds__(4 * W) batch_long_rows_kernel(const int32_t* __restrict__ long_rows,
+                                                                const int32_t* __restrict__ long_first,
+                                                                const f2* __restrict__ partial, Op op) {
+    __shared__ f2 part[4][W];
+    const int q = threadIdx.x % W, g = threadIdx.x / W;
+    const int32_t first = long_first[blockIdx.x], end = long_first[blockIdx.x + 1];
     f2 acc[1] = {f2{0.f, 0.f}};
-    for (int32_t s = long_first[r]; s < long_first[r + 1]; ++s) acc[0] = f2_add(acc[0], partial[(int64_t)s * W + q]);
-    op.template operator()<1>(long_rows[r], q, acc);
+    constexpr int kU = 4;
+    for (int32_t s = first + g; s < end; s += 4 * kU) {
+        f2 v[kU];
+#pragma unroll
+        for (int t = 0; t < kU; ++t)
+            if (s + 4 * t < end) v[t] = partial[(int64_t)(s + 4 * t) * W + q];
+#pragma unroll
+        for (int t = 0; t < kU; ++t)
+            if (s + 4 * t < end) acc[0] = f2_add(acc[0], v[t]);
+    }
+    part[g][q] = acc[0];
+    __syncthreads();
+    if (g != 0) return;
+    acc[0] = f2_add(f2_add(part[0][q], part[1][q]), f2_add(part[2][q], part[3][q]));
+    op.template operator()<1>(long_rows[blockIdx.x], q, acc);
 }
 
 // Level 0: pi^0 column q = (1 - sqrt c) e_{u_q}; x^0 = pi^0 / din.
@@ -288,14 +326,12 @@ cudaError_t batch_level(const Graph& g, const DevCsr& A, const V* X, const Op& o
     constexpr int W = LPR * CPL;
     const int rows_per_block = (kBlock / 32) * (32 / LPR);
     const int sb = grid_cap(g, g.n, rows_per_block);
-    const int segb = A.nseg ? grid_cap(g, A.nseg, rows_per_block) : 0;
+    const int segb = A.bnseg ? grid_cap(g, A.bnseg, rows_per_block) : 0;
     batch_rows_kernel<V, LPR, CPL, Op><<<(unsigned)(sb + segb), kBlock, 0, g.stream>>>(
-        g.n, A.rp, A.col, X, A.long_min, op, A.nseg, A.seg, partial, sb);
+        g.n, A.rp, A.col, X, op, A.bnseg, A.bseg, partial, segb);
     cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess || A.nlong == 0) return e;
-    const int64_t threads = A.nlong * W;
-    batch_long_rows_kernel<W, Op><<<(unsigned)((threads + kBlock - 1) / kBlock), kBlock, 0, g.stream>>>(
-        A.nlong, A.long_rows, A.long_first, partial, op);
+    if (e != cudaSuccess || A.bnlong == 0) return e;
+    batch_long_rows_kernel<W, Op><<<(unsigned)A.bnlong, 4 * W, 0, g.stream>>>(A.blong_rows, A.blong_first, partial, op);
     return cudaGetLastError();
 }
 

@@ -60,6 +60,9 @@ void free_csr(DevCsr& c) {
     cudaFree(c.tseg);
     cudaFree(c.tlong_rows);
     cudaFree(c.tlong_first);
+    cudaFree(c.bseg);
+    cudaFree(c.blong_rows);
+    cudaFree(c.blong_first);
     c = DevCsr{};
 }
 
@@ -79,19 +82,27 @@ esim_status upload_csr(int64_t n, const std::vector<uint32_t>& rp, const std::ve
     const int64_t m = (int64_t)rp[n];
     d.group = group_for(n ? (double)m / (double)n : 1.0);
     d.long_min = std::max<uint32_t>(256u, 32u * (uint32_t)d.group);
-    std::vector<Segment> seg;
-    std::vector<int32_t> long_rows, long_first;
+    std::vector<Segment> seg, bseg;
+    std::vector<int32_t> long_rows, long_first, blong_rows, blong_first;
+    auto cut = [&](int64_t r, uint32_t len, std::vector<Segment>& sg, std::vector<int32_t>& rows,
+                   std::vector<int32_t>& firsts) {
+        rows.push_back((int32_t)r);
+        firsts.push_back((int32_t)sg.size());
+        const uint32_t first = (uint32_t)sg.size();
+        for (uint32_t s = rp[r]; s < rp[r + 1]; s += len)
+            sg.push_back(Segment{(int32_t)r, s, std::min(rp[r + 1], s + len), first});
+    };
     for (int64_t r = 0; r < n; ++r) {
-        const uint32_t b = rp[r], e = rp[r + 1];
-        if (e - b < d.long_min) continue;
-        long_rows.push_back((int32_t)r);
-        long_first.push_back((int32_t)seg.size());
-        const uint32_t first = (uint32_t)seg.size();
-        for (uint32_t s = b; s < e; s += kSegLen) seg.push_back(Segment{(int32_t)r, s, std::min(e, s + kSegLen), first});
+        const uint32_t len = rp[r + 1] - rp[r];
+        if (len >= d.long_min) cut(r, kSegLen, seg, long_rows, long_first);
+        if (len >= kBatchSeg) cut(r, kBatchSeg, bseg, blong_rows, blong_first);
     }
     long_first.push_back((int32_t)seg.size());
+    blong_first.push_back((int32_t)bseg.size());
     d.nseg = (int64_t)seg.size();
     d.nlong = (int64_t)long_rows.size();
+    d.bnseg = (int64_t)bseg.size();
+    d.bnlong = (int64_t)blong_rows.size();
     // tiles of the single-vector sweeps (one warp each): consecutive rows up to tile_cap
     // entries (and kSweepTileRows rows); a longer row forms a tile alone, and a row longer
     // than kSweepTile is cut into segments.  tile_cap is kSweepTile, or less on a small
@@ -107,11 +118,7 @@ esim_status upload_csr(int64_t n, const std::vector<uint32_t>& rp, const std::ve
         if (len > cap && len <= kSweepTile) {  // a tile of its own (one warp still holds it)
             ++r;
         } else if (len > cap) {
-            tlong_rows.push_back((int32_t)r);
-            tlong_first.push_back((int32_t)tseg.size());
-            const uint32_t first = (uint32_t)tseg.size();
-            for (uint32_t s = rp[r]; s < rp[r + 1]; s += kSegLen)
-                tseg.push_back(Segment{(int32_t)r, s, std::min(rp[r + 1], s + kSegLen), first});
+            cut(r, kSegLen, tseg, tlong_rows, tlong_first);
             ++r;
         } else {
             const int64_t start = r;
@@ -129,35 +136,28 @@ esim_status upload_csr(int64_t n, const std::vector<uint32_t>& rp, const std::ve
     d.ntiles = (int64_t)tiles.size() - 1;
     d.tnseg = (int64_t)tseg.size();
     d.tnlong = (int64_t)tlong_rows.size();
-    cudaError_t e;
-    if ((e = dev_alloc(&d.rp, (size_t)n + 1)) != cudaSuccess) return fail(ESIM_ENOMEM, "cudaMalloc(rowptr)");
-    if ((e = dev_alloc(&d.col, (size_t)m)) != cudaSuccess) return fail(ESIM_ENOMEM, "cudaMalloc(col)");
-    if ((e = dev_alloc(&d.seg, seg.size())) != cudaSuccess) return fail(ESIM_ENOMEM, "cudaMalloc(segments)");
-    if ((e = dev_alloc(&d.long_rows, long_rows.size())) != cudaSuccess) return fail(ESIM_ENOMEM, "cudaMalloc(long rows)");
-    if ((e = dev_alloc(&d.long_first, long_first.size())) != cudaSuccess) return fail(ESIM_ENOMEM, "cudaMalloc(long first)");
-    ESIM_CUDA_TRY(cudaMemcpy(d.rp, rp.data(), sizeof(uint32_t) * ((size_t)n + 1), cudaMemcpyHostToDevice), "upload rowptr");
-    if (m) ESIM_CUDA_TRY(cudaMemcpy(d.col, col.data(), sizeof(int32_t) * (size_t)m, cudaMemcpyHostToDevice), "upload col");
-    if (!seg.empty())
-        ESIM_CUDA_TRY(cudaMemcpy(d.seg, seg.data(), sizeof(Segment) * seg.size(), cudaMemcpyHostToDevice), "upload segments");
-    if ((e = dev_alloc(&d.tiles, tiles.size())) != cudaSuccess) return fail(ESIM_ENOMEM, "cudaMalloc(tiles)");
-    if ((e = dev_alloc(&d.tseg, tseg.size())) != cudaSuccess) return fail(ESIM_ENOMEM, "cudaMalloc(tile segments)");
-    if ((e = dev_alloc(&d.tlong_rows, tlong_rows.size())) != cudaSuccess) return fail(ESIM_ENOMEM, "cudaMalloc(tile long rows)");
-    if ((e = dev_alloc(&d.tlong_first, tlong_first.size())) != cudaSuccess)
-        return fail(ESIM_ENOMEM, "cudaMalloc(tile long first)");
-    ESIM_CUDA_TRY(cudaMemcpy(d.tiles, tiles.data(), sizeof(uint32_t) * tiles.size(), cudaMemcpyHostToDevice), "upload tiles");
-    if (!tseg.empty())
-        ESIM_CUDA_TRY(cudaMemcpy(d.tseg, tseg.data(), sizeof(Segment) * tseg.size(), cudaMemcpyHostToDevice),
-                      "upload tile segments");
-    if (!tlong_rows.empty())
-        ESIM_CUDA_TRY(cudaMemcpy(d.tlong_rows, tlong_rows.data(), sizeof(int32_t) * tlong_rows.size(),
-                                 cudaMemcpyHostToDevice), "upload tile long rows");
-    ESIM_CUDA_TRY(cudaMemcpy(d.tlong_first, tlong_first.data(), sizeof(int32_t) * tlong_first.size(),
-                             cudaMemcpyHostToDevice), "upload tile long first");
-    if (!long_rows.empty())
-        ESIM_CUDA_TRY(cudaMemcpy(d.long_rows, long_rows.data(), sizeof(int32_t) * long_rows.size(), cudaMemcpyHostToDevice),
-                      "upload long rows");
-    ESIM_CUDA_TRY(cudaMemcpy(d.long_first, long_first.data(), sizeof(int32_t) * long_first.size(), cudaMemcpyHostToDevice),
-                  "upload long first");
+    auto up = [](auto** dst, const auto& v) {  // an empty vector still gets an allocation
+        return dev_alloc(dst, v.size()) != cudaSuccess ? ESIM_ENOMEM
+               : !v.empty() && cudaMemcpy(*dst, v.data(), sizeof(v[0]) * v.size(), cudaMemcpyHostToDevice) != cudaSuccess
+                   ? ESIM_ECUDA
+                   : ESIM_OK;
+    };
+    esim_status st = up(&d.rp, rp);
+    if (st == ESIM_OK) st = up(&d.col, col);
+    if (st == ESIM_OK) st = up(&d.seg, seg);
+    if (st == ESIM_OK) st = up(&d.long_rows, long_rows);
+    if (st == ESIM_OK) st = up(&d.long_first, long_first);
+    if (st == ESIM_OK) st = up(&d.tiles, tiles);
+    if (st == ESIM_OK) st = up(&d.tseg, tseg);
+    if (st == ESIM_OK) st = up(&d.tlong_rows, tlong_rows);
+    if (st == ESIM_OK) st = up(&d.tlong_first, tlong_first);
+    if (st == ESIM_OK) st = up(&d.bseg, bseg);
+    if (st == ESIM_OK) st = up(&d.blong_rows, blong_rows);
+    if (st == ESIM_OK) st = up(&d.blong_first, blong_first);
+    if (st != ESIM_OK) {
+        cudaGetLastError();
+        return fail(st, st == ESIM_ENOMEM ? "cudaMalloc(graph tables)" : "upload of the graph tables");
+    }
     if (with_info) {
         // filled on the device (launch_walk_table); the tail past m is never used as a position
         const size_t entries = (size_t)std::max(m, n);
@@ -1070,8 +1070,8 @@ esim_status run_batch(Graph& g, int32_t B, const int64_t* u, const double* eps, 
     ESIM_CUDA_TRY(cudaStreamSynchronize(g.stream), "batch query");
     const Status hs = *g.status_host;
     g.last_L = plan.Lmax;
-    g.last_launches = 1 + plan.Lmax * (1 + (g.out.nlong > 0 ? 1 : 0)) + 1 + 3 + 1 + 1 + 1 +
-                      plan.Lmax * (1 + (g.in.nlong > 0 ? 1 : 0)) + (k > 0 ? 2 : 0) + (g.shared_walks ? 2 : 0);
+    g.last_launches = 1 + plan.Lmax * (1 + (g.out.bnlong > 0 ? 1 : 0)) + 1 + 3 + 1 + 1 + 1 +
+                      plan.Lmax * (1 + (g.in.bnlong > 0 ? 1 : 0)) + (k > 0 ? 2 : 0) + (g.shared_walks ? 2 : 0);
     g.last_R_b = plan.Rb[0];
     g.last_kappa = kappa_of(g, c);
     g.last_norm2 = 0.0;
@@ -1134,7 +1134,7 @@ int batch_plan(const Graph& g, int32_t B, const int64_t* u, const double* eps, d
 }
 
 size_t batch_ws_bytes(const Graph& g, const BatchPlan& p) {
-    return bws_layout(g.n, p.W, p.B, p.Lmax, std::max(g.in.nseg, g.out.nseg), p.k, nullptr, nullptr);
+    return bws_layout(g.n, p.W, p.B, p.Lmax, std::max(g.in.bnseg, g.out.bnseg), p.k, nullptr, nullptr);
 }
 
 // Enqueue the whole batch on view.stream using the arena `ws`; results go to the
@@ -1144,7 +1144,7 @@ int batch_enqueue(Graph& tuner, const Graph& view, const BatchPlan& p, void* ws,
                   double* s_dev, double* s_host, int32_t* ids_dev, double* vals_dev, int32_t* ids_host,
                   double* vals_host, bool allow_tune) {
     BWs w;
-    bws_layout(view.n, p.W, p.B, p.Lmax, std::max(view.in.nseg, view.out.nseg), p.k, (char*)ws, &w);
+    bws_layout(view.n, p.W, p.B, p.Lmax, std::max(view.in.bnseg, view.out.bnseg), p.k, (char*)ws, &w);
     const int W = p.W, B = p.B, k = p.k;
     const int32_t Lmax = p.Lmax;
     const size_t nw = (size_t)view.n * W;

@@ -81,9 +81,16 @@ struct DevCsr {
     int32_t* tlong_first = nullptr;
     int64_t tnseg = 0;
     int64_t tnlong = 0;
+    // The batched sweeps' segments: rows of kBatchSeg entries or more in pieces of kBatchSeg.
+    Segment* bseg = nullptr;
+    int32_t* blong_rows = nullptr;
+    int32_t* blong_first = nullptr;
+    int64_t bnseg = 0;
+    int64_t bnlong = 0;
 };
 
 constexpr uint32_t kSweepTile = 512;        // entries a warp gathers into shared memory per tile, at most
+constexpr uint32_t kBatchSeg = 64;           // entries a lane group of the batched sweeps adds one after another, at most
 constexpr uint32_t kSweepTileRows = 256;    // rows per tile at most (runs of empty rows)
 
 struct Graph {

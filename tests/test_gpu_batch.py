@@ -136,3 +136,27 @@ def test_shared_walks_give_the_same_counts_with_fewer_pairs(esim):
     assert np.array_equal(ids1, ids0) and np.array_equal(v1, v0)
     g1.close()
     g0.close()
+
+
+@pytest.mark.parametrize("degree", [1, 7, 8, 63, 64, 65, 127, 128, 129, 257, 1025])
+def test_row_lengths_around_a_segment(esim, degree):
+    """Rows that end just before, at and after the pieces a lane group adds: one node with
+    `degree` in-edges and as many out-edges, in all widths and tiles against the single-source
+    precision form (FP32 history: 2 L u relative, on scores below 1)."""
+    others = np.arange(1, degree + 1)
+    src = np.concatenate([others, np.zeros(degree, dtype=np.int64), others[:-1], [degree]])
+    dst = np.concatenate([np.zeros(degree, dtype=np.int64), others, others[1:], [degree + 1]])
+    n, rp, col = synth.edges_to_in_csr(degree + 2, src, dst)
+    eps = 5e-2
+    with esim.Graph(n, rp, col, kappa=4.0, precision=1) as g:
+        want = [g.query(u, C, eps, 3) for u in (0, 1)]
+        L = g.stats()["L"]
+        first = None
+        for B in (2, 17, 33):
+            for tile in (0, 1, 2):
+                g.set_option("batch_tile", tile)
+                s = g.query_batch([0, 1] + [0] * (B - 2), [eps] * B, C, seed=3)
+                first = s[:2] if first is None else first
+                assert np.array_equal(s[:2], first)
+        for q in (0, 1):
+            assert np.max(np.abs(first[q] - want[q])) <= 4 * L * 2.0 ** -24 / (1 - C)
