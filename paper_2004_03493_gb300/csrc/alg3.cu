@@ -4,8 +4,8 @@
 // tail walk pairs.
 //
 // Notation: h_l = (P^T)^l(k, .), the distribution of a non-stop walk from k after l
-// steps (FP64 storage; pull sweeps over the out-edge CSR with no decay, on the warp-tile
-// kernel with two-float sums); Zv_l the vector Z_l(k, .) of Lemma 5; P~ the transition
+// steps (FP64 storage; pull sweeps over the out-edge CSR with no decay and two-float
+// sums); Zv_l the vector Z_l(k, .) of Lemma 5; P~ the transition
 // matrix with squared entries.
 // Lemma 5 reads, for each target level j,
 //   Zv_j = c^j h_j^2 - c P~ Zv_{j-1} - sum_{l'=2}^{j-1} c^{l'} sum_{q'} Zv_{j-l'}(q') ((P^T)^{l'}(q', .))^2
@@ -1100,12 +1100,11 @@ cudaError_t alg3_first_meeting(const Graph& g, int64_t k, int depth, double c, v
     A3Ws ws;
     a3_layout(g.n, g.m, g.out.nseg, wsp, &ws);
     const size_t n = (size_t)g.n;
-    const int per_sweep = 1 + (g.out.tnlong > 0 ? 1 : 0);  // tile kernel, long rows
     const int eb = eblocks(g, g.n);
     int count = 0;
     cudaError_t e = launch_walk_distributions(g, k, depth, ws.H, ws.xa, ws.xb);
     if (e != cudaSuccess) return e;
-    count += 1 + depth * per_sweep;
+    count += 1 + depth;
     long long* const zlo_base = ws.Zfx + (size_t)(kAlg3MaxDepth + 1) * n;
     if ((e = cudaMemsetAsync(ws.Zfx, 0, sizeof(long long) * n * (size_t)(depth + 1), g.stream)) != cudaSuccess ||
         (e = cudaMemsetAsync(zlo_base, 0, sizeof(long long) * n * (size_t)(depth + 1), g.stream)) != cudaSuccess)
@@ -1123,7 +1122,7 @@ cudaError_t alg3_first_meeting(const Graph& g, int64_t k, int depth, double c, v
             sq_scale_kernel<<<eb, kBlock, 0, g.stream>>>(g.n, ws.Zv + (size_t)(j - 1) * n, g.inv_din, x2);
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
             if ((e = launch_pull_sum(g, x2, ws.T)) != cudaSuccess) return e;
-            count += 1 + per_sweep;
+            count += 2;
             T = ws.T;
         }
         zv_finalize_kernel<<<eb, kBlock, 0, g.stream>>>(g.n, cpow[(size_t)j], c, ws.H + (size_t)j * n, T,

@@ -56,33 +56,25 @@ void free_csr(DevCsr& c) {
     cudaFree(c.seg);
     cudaFree(c.long_rows);
     cudaFree(c.long_first);
-    cudaFree(c.tiles);
-    cudaFree(c.tseg);
-    cudaFree(c.tlong_rows);
-    cudaFree(c.tlong_first);
+    free_sell(c.sell);
     cudaFree(c.bseg);
     cudaFree(c.blong_rows);
     cudaFree(c.blong_first);
     c = DevCsr{};
 }
 
-int group_for(double avg_degree) {
-    if (avg_degree <= 3.0) return 2;
-    if (avg_degree <= 6.0) return 4;
-    if (avg_degree <= 12.0) return 8;
-    if (avg_degree <= 24.0) return 16;
-    return 32;
-}
-
 constexpr uint32_t kSegLen = 4096;
+constexpr int64_t kLongRowsFrom = 4000000;  // from this many edges on a level is no longer one row's latency
 
 // Upload a host CSR and build its row-split table.
 esim_status upload_csr(int64_t n, const std::vector<uint32_t>& rp, const std::vector<int32_t>& col, DevCsr& d,
-                       bool with_info, int sm_count) {
+                       bool with_info, cudaStream_t stream) {
     const int64_t m = (int64_t)rp[n];
-    d.group = group_for(n ? (double)m / (double)n : 1.0);
-    d.long_min = std::max<uint32_t>(256u, 32u * (uint32_t)d.group);
-    std::vector<Segment> seg, bseg;
+    const double avg = (double)m / (double)n;
+    d.long_min = avg > 12.0 ? (avg > 24.0 ? 1024u : 512u) : 256u;
+    d.sell.row_cap = m >= kLongRowsFrom ? 64u : 32u;
+    std::vector<Segment> seg, bseg, pieces;
+    std::vector<int32_t> piece_rows, piece_first;  // not kept: a piece names its row and its row's first piece
     std::vector<int32_t> long_rows, long_first, blong_rows, blong_first;
     auto cut = [&](int64_t r, uint32_t len, std::vector<Segment>& sg, std::vector<int32_t>& rows,
                    std::vector<int32_t>& firsts) {
@@ -96,6 +88,7 @@ esim_status upload_csr(int64_t n, const std::vector<uint32_t>& rp, const std::ve
         const uint32_t len = rp[r + 1] - rp[r];
         if (len >= d.long_min) cut(r, kSegLen, seg, long_rows, long_first);
         if (len >= kBatchSeg) cut(r, kBatchSeg, bseg, blong_rows, blong_first);
+        if (len > d.sell.row_cap) cut(r, 32 * d.sell.row_cap, pieces, piece_rows, piece_first);
     }
     long_first.push_back((int32_t)seg.size());
     blong_first.push_back((int32_t)bseg.size());
@@ -103,39 +96,6 @@ esim_status upload_csr(int64_t n, const std::vector<uint32_t>& rp, const std::ve
     d.nlong = (int64_t)long_rows.size();
     d.bnseg = (int64_t)bseg.size();
     d.bnlong = (int64_t)blong_rows.size();
-    // tiles of the single-vector sweeps (one warp each): consecutive rows up to tile_cap
-    // entries (and kSweepTileRows rows); a longer row forms a tile alone, and a row longer
-    // than kSweepTile is cut into segments.  tile_cap is kSweepTile, or less on a small
-    // graph so that its tiles still number about 256 per SM (a power of two, at least 64)
-    d.tile_cap = kSweepTile;
-    while (d.tile_cap > 64u && (int64_t)d.tile_cap * 256 * (int64_t)std::max(sm_count, 1) > m) d.tile_cap >>= 1;
-    const uint32_t cap = d.tile_cap;
-    std::vector<uint32_t> tiles{0};
-    std::vector<Segment> tseg;
-    std::vector<int32_t> tlong_rows, tlong_first;
-    for (int64_t r = 0; r < n;) {
-        const uint32_t len = rp[r + 1] - rp[r];
-        if (len > cap && len <= kSweepTile) {  // a tile of its own (one warp still holds it)
-            ++r;
-        } else if (len > cap) {
-            cut(r, kSegLen, tseg, tlong_rows, tlong_first);
-            ++r;
-        } else {
-            const int64_t start = r;
-            uint32_t cnt = 0;
-            while (r < n && r - start < (int64_t)kSweepTileRows) {
-                const uint32_t l = rp[r + 1] - rp[r];
-                if (l > cap || cnt + l > cap) break;
-                cnt += l;
-                ++r;
-            }
-        }
-        tiles.push_back((uint32_t)r);
-    }
-    tlong_first.push_back((int32_t)tseg.size());
-    d.ntiles = (int64_t)tiles.size() - 1;
-    d.tnseg = (int64_t)tseg.size();
-    d.tnlong = (int64_t)tlong_rows.size();
     auto up = [](auto** dst, const auto& v) {  // an empty vector still gets an allocation
         return dev_alloc(dst, v.size()) != cudaSuccess ? ESIM_ENOMEM
                : !v.empty() && cudaMemcpy(*dst, v.data(), sizeof(v[0]) * v.size(), cudaMemcpyHostToDevice) != cudaSuccess
@@ -147,16 +107,18 @@ esim_status upload_csr(int64_t n, const std::vector<uint32_t>& rp, const std::ve
     if (st == ESIM_OK) st = up(&d.seg, seg);
     if (st == ESIM_OK) st = up(&d.long_rows, long_rows);
     if (st == ESIM_OK) st = up(&d.long_first, long_first);
-    if (st == ESIM_OK) st = up(&d.tiles, tiles);
-    if (st == ESIM_OK) st = up(&d.tseg, tseg);
-    if (st == ESIM_OK) st = up(&d.tlong_rows, tlong_rows);
-    if (st == ESIM_OK) st = up(&d.tlong_first, tlong_first);
     if (st == ESIM_OK) st = up(&d.bseg, bseg);
     if (st == ESIM_OK) st = up(&d.blong_rows, blong_rows);
     if (st == ESIM_OK) st = up(&d.blong_first, blong_first);
     if (st != ESIM_OK) {
         cudaGetLastError();
         return fail(st, st == ESIM_ENOMEM ? "cudaMalloc(graph tables)" : "upload of the graph tables");
+    }
+    const cudaError_t se = build_sell(n, d, pieces, stream, d.sell);
+    if (se != cudaSuccess) {
+        cudaGetLastError();
+        return fail(se == cudaErrorMemoryAllocation ? ESIM_ENOMEM : ESIM_ECUDA,
+                    std::string("sliced rows: ") + cudaGetErrorString(se));
     }
     if (with_info) {
         // filled on the device (launch_walk_table); the tail past m is never used as a position
@@ -169,8 +131,11 @@ esim_status upload_csr(int64_t n, const std::vector<uint32_t>& rp, const std::ve
     return ESIM_OK;
 }
 
-size_t partial_count(const Graph& g) {
-    return (size_t)std::max<int64_t>(1, std::max(std::max(g.in.nseg, g.out.nseg), std::max(g.in.tnseg, g.out.tnseg)));
+// The sweeps' scratch, its counts at zero.
+bool alloc_sweep_scratch(const Graph& g, void** p) {
+    const size_t bytes = sweep_scratch_bytes(g);
+    return cudaMalloc(p, bytes) == cudaSuccess && cudaMemsetAsync(*p, 0, bytes, cudaStreamPerThread) == cudaSuccess &&
+           cudaStreamSynchronize(cudaStreamPerThread) == cudaSuccess;
 }
 
 void free_a3workers(Graph& g) {
@@ -197,7 +162,7 @@ int ensure_a3workers(Graph& g, int extra) {
     while ((int)g.a3workers.size() < extra) {
         Graph::A3Worker wk;
         const bool ok = cudaStreamCreateWithFlags(&wk.stream, cudaStreamNonBlocking) == cudaSuccess &&
-                        cudaMalloc(&wk.ws, need) == cudaSuccess && dev_alloc(&wk.partial, partial_count(g)) == cudaSuccess &&
+                        cudaMalloc(&wk.ws, need) == cudaSuccess && alloc_sweep_scratch(g, &wk.partial) &&
                         dev_alloc(&wk.scan_part, (size_t)nb) == cudaSuccess &&
                         dev_alloc(&wk.norm_part, 2 * (size_t)nb) == cudaSuccess;
         if (!ok) {
@@ -796,7 +761,7 @@ esim_status run_query(Graph& g, int64_t u, double c, double eps, uint64_t seed, 
         ESIM_CUDA_TRY(cudaStreamSynchronize(g.stream), "forward sweeps (counting pass)");
         const uint64_t kept = g.status_host->hist_count;
         cap = std::max<uint64_t>(1, std::min<uint64_t>(kept, sparse_capacity(g.n, L, theta)));
-        count_launches = 2 + L * (2 + (g.out.nlong > 0 ? 1 : 0));
+        count_launches = 2 + L * 2;
     }
     esim_status st = ensure_ws(g, L, g.precision, w, cap);
     if (st != ESIM_OK) return st;
@@ -899,13 +864,9 @@ esim_status run_query(Graph& g, int64_t u, double c, double eps, uint64_t seed, 
     ESIM_CUDA_TRY(cudaStreamSynchronize(g.stream), "query");
     const Status hs = *g.status_host;
     g.last_L = L;
-    // kernels launched: forward init + per level (rows [+ long rows]), 3 allocation
+    // kernels launched: forward init + per level, 3 allocation
     // kernels, the sampler, D^, reverse init + per level, and 2 for top-k
-    // the sparse history's sweeps sum in FP64 on the row kernel (long-row table nlong), the
-    // others on the tile kernel (tnlong)
-    const int fwd_per = 1 + (sparse ? (g.out.nlong > 0) : (g.out.tnlong > 0));
-    const int rev_per = 1 + (sparse ? (g.in.nlong > 0) : (g.in.tnlong > 0));
-    g.last_launches = (1 + L * fwd_per) + 3 + 1 + 1 + (1 + L * rev_per) + (k > 0 ? 2 : 0) + extra_launches;
+    g.last_launches = (1 + L) + 3 + 1 + 1 + (1 + L) + (k > 0 ? 2 : 0) + extra_launches;
     if (sparse) g.last_launches += 2 * (L + 1) + count_launches;  // compactions, scatters, counting pass
     g.last_hist_entries = sparse ? std::min<uint64_t>(hs.hist_count, cap) : (uint64_t)(L + 1) * (uint64_t)g.n;
     g.last_R_b = R_b;
@@ -1320,17 +1281,16 @@ esim_status esim_load_graph(int64_t n, const int64_t* in_rowptr, const int32_t* 
             return fail(ESIM_ENOMEM, "device allocation for 1/din");
         }
     }
-    esim_status st = upload_csr(n, in_rp, in_c, g.in, true, g.sm_count);
-    if (st == ESIM_OK) st = upload_csr(n, out_rp, out_c, g.out, false, g.sm_count);
+    esim_status st = upload_csr(n, in_rp, in_c, g.in, true, cudaStreamPerThread);
+    if (st == ESIM_OK) st = upload_csr(n, out_rp, out_c, g.out, false, cudaStreamPerThread);
     if (st != ESIM_OK) {
         release(g);
         delete h;
         return st;
     }
     const int64_t nb = allocate_blocks(n);
-    const size_t npart = partial_count(g);
     bool ok = dev_alloc(&g.status, 1) == cudaSuccess && cudaMallocHost((void**)&g.status_host, sizeof(Status)) == cudaSuccess &&
-              dev_alloc(&g.partial, npart) == cudaSuccess && dev_alloc(&g.scan_part, (size_t)nb) == cudaSuccess &&
+              alloc_sweep_scratch(g, &g.partial) && dev_alloc(&g.scan_part, (size_t)nb) == cudaSuccess &&
               dev_alloc(&g.norm_part, 2 * (size_t)nb) == cudaSuccess &&
               cudaMalloc(&g.topk_ws, topk_stage_offset(n) + (sizeof(double) + sizeof(int32_t)) * kTopkMax) == cudaSuccess &&
               cudaStreamCreateWithFlags(&g.own_stream, cudaStreamNonBlocking) == cudaSuccess &&
@@ -1345,7 +1305,7 @@ esim_status esim_load_graph(int64_t n, const int64_t* in_rowptr, const int32_t* 
     }
     g.scan_blocks = nb;
     g.stream = g.own_stream;
-    cudaError_t we = cudaMemset(g.status, 0, sizeof(Status));
+    cudaError_t we = cudaMemsetAsync(g.status, 0, sizeof(Status), g.stream);
     if (we == cudaSuccess) we = launch_walk_table(g);
     if (we == cudaSuccess) we = cudaStreamSynchronize(g.stream);
     if (we != cudaSuccess) {

@@ -56,8 +56,25 @@ struct Segment {
     uint32_t first;  // index of the row's first segment (rows own consecutive segments)
 };
 
-// A CSR resident on the device, with the row-split table for rows whose length
-// is at least `long_min`.  Long rows are cut into segments of `seg_len` entries.
+// The sliced copy of a CSR for the single-vector sweeps (built by sell.cu).  A slice is 32
+// rows of nearly equal length, one per lane; its steps [off[s], off[s+1]) hold the rows'
+// entries side by side: entry t of lane l's row is col[(off[s] + t) * 32 + l].  A row longer
+// than row_cap is cut into pieces of 32 row_cap entries, and slice s < npieces is piece s:
+// the same layout with the piece's entries t * 32 + l.
+struct SellRows {
+    uint32_t* off = nullptr;    // nslices + 1
+    int2* rows = nullptr;       // 32 per slice: (row, or -1; this lane's entries)
+    int32_t* col = nullptr;     // 32 per step; 0 past a row's end
+    Segment* piece = nullptr;   // npieces: (row, entries, number of the row's first piece)
+    int64_t nslices = 0;
+    int64_t npieces = 0;
+    uint32_t row_cap = 64;
+};
+
+constexpr int kSellWindow = 1024;           // rows sorted by length together
+
+// A CSR resident on the device, with the row-split table of the probe sweeps for rows whose
+// length is at least `long_min`.  Long rows are cut into segments of `seg_len` entries.
 struct DevCsr {
     uint32_t* rp = nullptr;      // n+1
     int32_t* col = nullptr;      // m
@@ -69,18 +86,7 @@ struct DevCsr {
     int64_t nseg = 0;
     int64_t nlong = 0;
     uint32_t long_min = 0;
-    int group = 8;               // threads per short row
-    // The single-vector sweeps' tiles: tile t covers rows [tiles[t], tiles[t+1]) with at
-    // most tile_cap entries in all, or one row longer than that; rows longer than
-    // kSweepTile are cut into segments of their own table (tseg, tlong_rows, tlong_first).
-    uint32_t* tiles = nullptr;   // ntiles + 1
-    int64_t ntiles = 0;
-    uint32_t tile_cap = 0;       // entries per tile, <= kSweepTile (smaller on small graphs)
-    Segment* tseg = nullptr;
-    int32_t* tlong_rows = nullptr;
-    int32_t* tlong_first = nullptr;
-    int64_t tnseg = 0;
-    int64_t tnlong = 0;
+    SellRows sell;
     // The batched sweeps' segments: rows of kBatchSeg entries or more in pieces of kBatchSeg.
     Segment* bseg = nullptr;
     int32_t* blong_rows = nullptr;
@@ -89,9 +95,7 @@ struct DevCsr {
     int64_t bnlong = 0;
 };
 
-constexpr uint32_t kSweepTile = 512;        // entries a warp gathers into shared memory per tile, at most
-constexpr uint32_t kBatchSeg = 64;           // entries a lane group of the batched sweeps adds one after another, at most
-constexpr uint32_t kSweepTileRows = 256;    // rows per tile at most (runs of empty rows)
+constexpr uint32_t kBatchSeg = 64;          // entries a lane group of the batched sweeps adds one after another, at most
 
 struct Graph {
     int device = 0;
@@ -142,7 +146,7 @@ struct Graph {
     struct A3Worker {
         cudaStream_t stream = nullptr;
         void* ws = nullptr;
-        double* partial = nullptr;
+        void* partial = nullptr;
         unsigned long long* scan_part = nullptr;
         double* norm_part = nullptr;
     };
@@ -168,7 +172,7 @@ struct Graph {
     Status* status_host = nullptr; // pinned host copy
     void* ws = nullptr;
     size_t ws_bytes = 0;
-    double* partial = nullptr;    // long-row partial sums (max nseg of in/out)
+    void* partial = nullptr;      // the sweeps' piece sums and arrival counts (sweep_scratch_bytes)
     unsigned long long* scan_part = nullptr;  // scan partials
     double* norm_part = nullptr;
     int64_t scan_blocks = 0;
@@ -185,7 +189,15 @@ struct Graph {
     unsigned long long last_steps_side = 0;
 };
 
+// sell.cu
+cudaError_t build_sell(int64_t n, const DevCsr& csr, const std::vector<Segment>& pieces, cudaStream_t stream,
+                       SellRows& out);
+void free_sell(SellRows& s);
+
 // sweep.cu
+// Bytes of the scratch that sweeps on one stream share: 8 bytes per piece, then a count per
+// piece.  The counts start at zero and every sweep leaves them so.
+size_t sweep_scratch_bytes(const Graph& g);
 cudaError_t launch_forward(const Graph& g, int64_t u, double c, int32_t L, double* hist, double* xa, double* xb);
 cudaError_t launch_reverse(const Graph& g, const double* hist, int32_t L, double c, const double* dhat, double* s_out,
                            double* sa, double* sb);

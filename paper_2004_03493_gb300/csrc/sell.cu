@@ -1,0 +1,139 @@
+// The sliced layout of a CSR that the single-vector sweeps read (internal.h, SellRows):
+// built on the device when a graph is loaded.
+//
+// Rows are sorted by length, longest first, within windows of kSellWindow consecutive
+// rows, so the 32 rows of a slice have nearly the same length and stay close together in
+// every vector that is indexed by row.  The entries of a slice are stored step by step:
+// the 32 rows' t-th entries side by side, so a warp reads them with one coalesced load.
+// Rows of more than row_cap entries take slices of their own, before all others, the lanes
+// side by side along the row.
+#include "common.cuh"
+#include "internal.h"
+
+#include <vector>
+
+namespace esim {
+
+namespace {
+
+// One window per block: sorts its rows by (length descending, row ascending) and writes
+// their (row, length) and, per slice, its longest row.  Cut rows get no place.
+__global__ void __launch_bounds__(kSellWindow) sell_sort_kernel(int64_t n, const uint32_t* __restrict__ rp,
+                                                               uint32_t row_cap, int2* __restrict__ rows,
+                                                               uint32_t* __restrict__ steps) {
+    __shared__ uint32_t key[kSellWindow];
+    const int t = threadIdx.x;
+    const int64_t base = (int64_t)blockIdx.x * kSellWindow;
+    uint32_t mine = 0;  // no row here
+    if (base + t < n) {
+        const uint32_t len = rp[base + t + 1] - rp[base + t];
+        if (len <= row_cap) mine = ((len + 1) << 10) | (uint32_t)(kSellWindow - 1 - t);
+    }
+    key[t] = mine;
+    __syncthreads();
+    for (int size = 2; size <= kSellWindow; size <<= 1)
+        for (int half = size >> 1; half > 0; half >>= 1) {
+            const int j = t ^ half;
+            if (j > t) {
+                const uint32_t a = key[t], b = key[j];
+                if ((t & size) == 0 ? a < b : a > b) {
+                    key[t] = b;
+                    key[j] = a;
+                }
+            }
+            __syncthreads();
+        }
+    const uint32_t k = key[t];
+    const int64_t at = base + t;
+    rows[at] = k ? make_int2((int)(base + kSellWindow - 1 - (int64_t)(k & (kSellWindow - 1))), (int)(k >> 10) - 1)
+                 : make_int2(-1, 0);
+    if ((t & 31) == 0) steps[at >> 5] = k ? (k >> 10) - 1 : 0u;
+}
+
+// One slice per piece of a long row.
+__global__ void sell_pieces_kernel(int64_t npieces, const Segment* __restrict__ piece, int2* __restrict__ rows,
+                                   uint32_t* __restrict__ steps) {
+    const uint32_t lane = threadIdx.x & 31;
+    for (int64_t s = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; s < npieces;
+         s += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+        const uint32_t len = piece[s].end - piece[s].beg;
+        rows[s * 32 + lane] = make_int2(piece[s].row, (int)(len > lane ? (len - lane + 31) / 32 : 0u));
+        if (lane == 0) steps[s] = (len + 31) / 32;
+    }
+}
+
+// The entries, slice by slice: one warp per slice.
+__global__ void __launch_bounds__(kBlock) sell_fill_kernel(int64_t nslices, int64_t npieces,
+                                                          const uint32_t* __restrict__ off,
+                                                          const int2* __restrict__ rows,
+                                                          const Segment* __restrict__ piece,
+                                                          const uint32_t* __restrict__ rp,
+                                                          const int32_t* __restrict__ col, int32_t* __restrict__ out) {
+    const int lane = threadIdx.x & 31;
+    for (int64_t s = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; s < nslices;
+         s += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+        const int2 r = rows[s * 32 + lane];
+        const uint32_t o0 = off[s], o1 = off[s + 1];
+        const bool wide = s < npieces;
+        const uint32_t beg = wide ? piece[s].beg + lane : (r.x < 0 ? 0u : rp[r.x]);
+        for (uint32_t t = 0; t < o1 - o0; ++t)
+            out[((size_t)o0 + t) * 32 + lane] = t < (uint32_t)r.y ? col[beg + (wide ? 32 * t : t)] : 0;
+    }
+}
+
+}  // namespace
+
+cudaError_t build_sell(int64_t n, const DevCsr& csr, const std::vector<Segment>& pieces, cudaStream_t stream,
+                       SellRows& out) {
+    cudaError_t e = cudaSuccess;
+    out.npieces = (int64_t)pieces.size();
+    const int64_t windows = (n + kSellWindow - 1) / kSellWindow;
+    out.nslices = out.npieces + windows * (kSellWindow / 32);
+    std::vector<uint32_t> steps((size_t)out.nslices + 1);
+    if ((e = cudaMalloc((void**)&out.off, sizeof(uint32_t) * ((size_t)out.nslices + 1))) != cudaSuccess ||
+        (e = cudaMalloc((void**)&out.rows, sizeof(int2) * (size_t)out.nslices * 32)) != cudaSuccess ||
+        (e = cudaMalloc((void**)&out.piece, sizeof(Segment) * (size_t)(out.npieces ? out.npieces : 1))) != cudaSuccess)
+        return e;
+    if (out.npieces) {
+        if ((e = cudaMemcpyAsync(out.piece, pieces.data(), sizeof(Segment) * pieces.size(), cudaMemcpyHostToDevice,
+                                 stream)) != cudaSuccess)
+            return e;
+        sell_pieces_kernel<<<(unsigned)((out.npieces * 32 + kBlock - 1) / kBlock), kBlock, 0, stream>>>(
+            out.npieces, out.piece, out.rows, out.off);
+    }
+    sell_sort_kernel<<<(unsigned)windows, kSellWindow, 0, stream>>>(
+        n, csr.rp, out.row_cap, out.rows + out.npieces * 32, out.off + out.npieces);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    // offsets in steps of 32 entries: the prefix sum of the slices' lengths, on the host
+    if ((e = cudaMemcpyAsync(steps.data(), out.off, sizeof(uint32_t) * (size_t)out.nslices, cudaMemcpyDeviceToHost,
+                             stream)) != cudaSuccess ||
+        (e = cudaStreamSynchronize(stream)) != cudaSuccess)
+        return e;
+    uint64_t total = 0;  // below 2^32: a step holds at least one entry, and m < 2^32
+    for (int64_t s = 0; s < out.nslices; ++s) {
+        const uint32_t len = steps[(size_t)s];
+        steps[(size_t)s] = (uint32_t)total;
+        total += len;
+    }
+    steps[(size_t)out.nslices] = (uint32_t)total;
+    if ((e = cudaMemcpyAsync(out.off, steps.data(), sizeof(uint32_t) * steps.size(), cudaMemcpyHostToDevice, stream)) !=
+        cudaSuccess)
+        return e;
+    if ((e = cudaMalloc((void**)&out.col, sizeof(int32_t) * 32 * (size_t)(total ? total : 1))) != cudaSuccess) return e;
+    int64_t blocks = (out.nslices * 32 + kBlock - 1) / kBlock;
+    if (blocks > 65536) blocks = 65536;
+    sell_fill_kernel<<<(unsigned)blocks, kBlock, 0, stream>>>(out.nslices, out.npieces, out.off, out.rows,
+                                                             out.piece, csr.rp, csr.col, out.col);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    return cudaStreamSynchronize(stream);  // pieces and steps are the caller's and this call's
+}
+
+void free_sell(SellRows& s) {
+    cudaFree(s.off);
+    cudaFree(s.rows);
+    cudaFree(s.piece);
+    cudaFree(s.col);
+    s = SellRows{};
+}
+
+}  // namespace esim

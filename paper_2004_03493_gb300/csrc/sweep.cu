@@ -11,8 +11,8 @@
 // forward product pulls along out-edges with the 1/din factor folded into the
 // gathered vector x; (P^T s)(j) = (1/din(j)) sum_{i in I(j)} s(i) pulls along
 // in-edges.  Both are atomic-free and deterministic: each row's sum is formed in
-// a fixed order by one thread group (short rows) or by fixed segments plus an
-// in-order combine (long rows).
+// a fixed order by one lane (short rows) or by fixed pieces, joined by one warp in a
+// fixed order (long rows).
 //
 // Two arithmetic forms share the kernels through a value/accumulator policy:
 //   FP64  -- the plain method: the history pi^l and the result s in FP64.  GB300's
@@ -34,8 +34,6 @@
 #include "internal.h"
 #include "twofloat.cuh"
 
-#include <type_traits>
-
 namespace esim {
 
 // ---------------------------------------------------------------- policies
@@ -47,6 +45,7 @@ struct Pol64 {  // FP64 values, FP64 sums
     static __device__ __forceinline__ A add(A a, V v) { return a + v; }
     static __device__ __forceinline__ A combine(A a, A b) { return a + b; }
     static __device__ __forceinline__ A shfl(A a, int o, int w) { return __shfl_down_sync(0xffffffffu, a, o, w); }
+    static __device__ __forceinline__ A fresh(const A* p) { return __ldcg(p); }
 };
 
 struct Pol32c {  // FP32 values, two-float sums
@@ -56,6 +55,10 @@ struct Pol32c {  // FP32 values, two-float sums
     static __device__ __forceinline__ A add(A a, V v) { return f2_add_f(a, v); }
     static __device__ __forceinline__ A combine(A a, A b) { return f2_add(a, b); }
     static __device__ __forceinline__ A shfl(A a, int o, int w) { return f2_shfl_down(a, o, w); }
+    static __device__ __forceinline__ A fresh(const A* p) {  // past the L1: other SMs wrote it in this launch
+        const float2 v = __ldcg(reinterpret_cast<const float2*>(p));
+        return f2{v.x, v.y};
+    }
 };
 
 struct Pol2f {  // two-float values (float2: hi, lo), two-float sums
@@ -65,25 +68,17 @@ struct Pol2f {  // two-float values (float2: hi, lo), two-float sums
     static __device__ __forceinline__ A add(A a, V v) { return f2_add(a, f2{v.x, v.y}); }
     static __device__ __forceinline__ A combine(A a, A b) { return f2_add(a, b); }
     static __device__ __forceinline__ A shfl(A a, int o, int w) { return f2_shfl_down(a, o, w); }
+    static __device__ __forceinline__ A fresh(const A* p) {  // past the L1: other SMs wrote it in this launch
+        const float2 v = __ldcg(reinterpret_cast<const float2*>(p));
+        return f2{v.x, v.y};
+    }
 };
 
 template <class Pol>
-__device__ __forceinline__ typename Pol::A block_combine(typename Pol::A v, typename Pol::A* smem) {
-    using A = typename Pol::A;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int nw = (blockDim.x + 31) >> 5;
+__device__ __forceinline__ typename Pol::A warp_combine(typename Pol::A v) {  // lane 0 has the result
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v = Pol::combine(v, Pol::shfl(v, o, 32));
-    if (lane == 0) smem[wid] = v;
-    __syncthreads();
-    A r = Pol::zero();
-    if (wid == 0) {
-        r = lane < nw ? smem[lane] : Pol::zero();
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) r = Pol::combine(r, Pol::shfl(r, o, 32));
-    }
-    __syncthreads();
-    return r;
+    return v;
 }
 
 // ---------------------------------------------------------------- row epilogues
@@ -196,165 +191,79 @@ struct ReverseOpD {
     }
 };
 
-// ---------------------------------------------------------------- row kernels
+// ---------------------------------------------------------------- row kernel
 //
 // A sweep level is gather-bound: each entry reads one value x[col[p]] from a vector
 // that sits in L2, and a random 4- or 8-byte gather costs a 32-byte sector whatever its
-// width.  The tile kernel keeps every lane gathering and no warp waiting on another:
-// each warp takes a tile of consecutive rows holding at most tile_cap (<= kSweepTile)
-// entries, gathers all of its entries (coalesced column loads, eight gathers in
-// flight per lane) into its own slice of shared memory, and then sums the rows from
-// there -- rows of up to 32 entries one lane each (two chains, even and odd entries),
-// longer rows by the whole warp (lanes stride the row, a fixed shuffle tree joins
-// them).  Rows longer than a tile are cut into segments: the blocks past tile_blocks
-// sum one segment each into partial[], and long_rows_kernel adds a row's partials in
-// order.  Every row's sum has a fixed order, so the sweeps are deterministic.
-
+// width.  One warp takes one slice (32 rows of nearly equal length, one per lane; sell.cu):
+// every lane adds its own row's entries one after another in two chains (even and odd
+// ones), eight gathers in flight, the next eight column numbers loaded before the gathers
+// are waited for.  No shared memory is used, so the L1 keeps the values of the nodes with
+// many edges; an entry costs about 16 instructions instead of 54.
+// Rows longer than row_cap (32 below four million edges, 64 from there on: a lane's chain is
+// most of a small level's time) are summed by a warp each, lanes side by side along the row,
+// first in the grid; a row longer than 32 row_cap entries is cut into pieces, and the warp
+// that counts in the last of them adds their sums.  Both joins are fixed shuffle trees.
+// Every row's sum has a fixed order, so the sweeps are deterministic.
+//
+// BEFOREAFTER
 template <class Pol, class Op>
-__global__ void __launch_bounds__(kBlock) tile_rows_kernel(const uint32_t* __restrict__ rp,
-                                                           const int32_t* __restrict__ col,
-                                                           const typename Pol::V* __restrict__ x,
-                                                           const uint32_t* __restrict__ tiles, int64_t ntiles,
-                                                           uint32_t tile_cap, Op op, int64_t nseg,
-                                                           const Segment* __restrict__ seg,
-                                                           typename Pol::A* __restrict__ partial, int tile_blocks) {
-    using A = typename Pol::A;
+__global__ void __launch_bounds__(kBlock) sell_rows_kernel(const SellRows A, const uint32_t* __restrict__ rp,
+                                                          const typename Pol::V* __restrict__ x, Op op,
+                                                          typename Pol::A* __restrict__ partial,
+                                                          unsigned* __restrict__ arrived) {
+    using Acc = typename Pol::A;
     using V = typename Pol::V;
-    constexpr int kWarps = kBlock / 32;
     constexpr int kU = 8;  // gathers in flight per lane
-    __shared__ V vals[kWarps][kSweepTile];
-    __shared__ A red[kWarps];
-    if ((int)blockIdx.x >= tile_blocks) {
-        const int64_t nsb = (int64_t)gridDim.x - tile_blocks;
-        for (int64_t s = (int64_t)blockIdx.x - tile_blocks; s < nseg; s += nsb) {
-            const Segment sg = seg[s];
-            A acc = Pol::zero();
-            for (uint32_t p = sg.beg + threadIdx.x; p < sg.end; p += blockDim.x) acc = Pol::add(acc, x[__ldg(col + p)]);
-            acc = block_combine<Pol>(acc, red);
-            if (threadIdx.x == 0) partial[s] = acc;
+    const int lane = threadIdx.x & 31;
+    const int64_t s = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (s >= A.nslices) return;
+    const uint32_t o0 = __ldg(A.off + s), steps = __ldg(A.off + s + 1) - o0;
+    const int2 r = __ldg(A.rows + s * 32 + lane);
+    const uint32_t len = (uint32_t)r.y;
+    const int32_t* __restrict__ c = A.col + (size_t)o0 * 32 + lane;
+    int32_t j[kU];
+#pragma unroll
+    for (int u = 0; u < kU; ++u)
+        if ((uint32_t)u < steps) j[u] = __ldg(c + u * 32);
+    Acc acc0 = Pol::zero(), acc1 = Pol::zero();
+    for (uint32_t t = 0; t < steps; t += kU) {
+        V g[kU];
+#pragma unroll
+        for (int u = 0; u < kU; ++u)
+            if (t + u < len) g[u] = x[j[u]];
+        c += kU * 32;
+#pragma unroll
+        for (int u = 0; u < kU; ++u)
+            if (t + kU + u < steps) j[u] = __ldg(c + u * 32);
+#pragma unroll
+        for (int u = 0; u < kU; u += 2) {
+            if (t + u < len) acc0 = Pol::add(acc0, g[u]);
+            if (t + u + 1 < len) acc1 = Pol::add(acc1, g[u + 1]);
         }
+    }
+    const Acc acc = Pol::combine(acc0, acc1);
+    if (s >= A.npieces) {
+        if (r.x >= 0) op((int64_t)r.x, acc);
         return;
     }
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    V* my = vals[wid];
-    const int64_t nwarps = (int64_t)tile_blocks * kWarps;
-    for (int64_t t = (int64_t)blockIdx.x * kWarps + wid; t < ntiles; t += nwarps) {
-        const uint32_t r0 = __ldg(tiles + t), r1 = __ldg(tiles + t + 1);
-        const uint32_t b = __ldg(rp + r0), e = __ldg(rp + r1);
-        if (e - b > kSweepTile) continue;  // one long row: the segment blocks sum it (warp-uniform)
-        for (uint32_t p = b + lane; p < e; p += 32 * kU) {
-            V g[kU];
-#pragma unroll
-            for (int u = 0; u < kU; ++u) {
-                const uint32_t q = p + (uint32_t)(32 * u);
-                if (q < e) g[u] = x[__ldg(col + q)];
-            }
-#pragma unroll
-            for (int u = 0; u < kU; ++u) {
-                const uint32_t q = p + (uint32_t)(32 * u);
-                if (q < e) my[q - b] = g[u];
-            }
+    Acc sum = warp_combine<Pol>(acc);
+    const uint32_t deg = __ldg(rp + r.x + 1) - __ldg(rp + r.x), piece = 32 * A.row_cap;
+    if (deg > piece) {
+        const uint32_t first = A.piece[s].first, count = (deg + piece - 1) / piece;
+        unsigned last = 0;
+        if (lane == 0) {
+            partial[s] = sum;
+            __threadfence();
+            last = atomicInc(arrived + first, count - 1) == count - 1;  // wraps to 0 for the next sweep
+            __threadfence();
         }
-        __syncwarp();
-        for (uint32_t base = r0; base < r1; base += 32) {
-            const uint32_t r = base + (uint32_t)lane;
-            uint32_t rb = 0, re = 0;
-            if (r < r1) {
-                rb = __ldg(rp + r);
-                re = __ldg(rp + r + 1);
-            }
-            const bool big = re - rb > 32u;
-            if (r < r1 && !big) {
-                A acc0 = Pol::zero(), acc1 = Pol::zero();
-                uint32_t q = rb;
-                for (; q + 1 < re; q += 2) {
-                    acc0 = Pol::add(acc0, my[q - b]);
-                    acc1 = Pol::add(acc1, my[q + 1 - b]);
-                }
-                if (q < re) acc0 = Pol::add(acc0, my[q - b]);
-                op((int64_t)r, Pol::combine(acc0, acc1));
-            }
-            unsigned mask = __ballot_sync(0xffffffffu, big);
-            while (mask) {
-                const int src = __ffs(mask) - 1;
-                mask &= mask - 1u;
-                const uint32_t wb = __shfl_sync(0xffffffffu, rb, src), we = __shfl_sync(0xffffffffu, re, src);
-                A acc = Pol::zero();
-                for (uint32_t q = wb + (uint32_t)lane; q < we; q += 32) acc = Pol::add(acc, my[q - b]);
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) acc = Pol::combine(acc, Pol::shfl(acc, o, 32));
-                if (lane == 0) op((int64_t)(base + (uint32_t)src), acc);
-            }
-        }
-        __syncwarp();
+        if (!__shfl_sync(0xffffffffu, last, 0)) return;
+        sum = Pol::zero();
+        for (uint32_t i = (uint32_t)lane; i < count; i += 32) sum = Pol::combine(sum, Pol::fresh(partial + first + i));
+        sum = warp_combine<Pol>(sum);
     }
-}
-
-// FP64 sums (Pol64: Algorithm 3's Lemma 5 sweeps and the sparse history) use a row
-// kernel with G lanes per row instead: its short dependency chains suit the slow FP64
-// unit on the small graphs those sweeps run on.
-// Blocks [0, short_blocks) sweep the short rows, G lanes per row; the remaining
-// blocks each combine one segment of a long row into partial[].
-template <class Pol, int G, class Op>
-__global__ void __launch_bounds__(kBlock) rows_kernel(int64_t n, const uint32_t* __restrict__ rp,
-                                                      const int32_t* __restrict__ col,
-                                                      const typename Pol::V* __restrict__ x, uint32_t long_min, Op op,
-                                                      int64_t nseg, const Segment* __restrict__ seg,
-                                                      typename Pol::A* __restrict__ partial, int short_blocks) {
-    using A = typename Pol::A;
-    __shared__ A red[kBlock / 32];
-    if ((int)blockIdx.x >= short_blocks) {
-        const int64_t nsb = (int64_t)gridDim.x - short_blocks;
-        for (int64_t s = (int64_t)blockIdx.x - short_blocks; s < nseg; s += nsb) {
-            const Segment sg = seg[s];
-            A acc = Pol::zero();
-            for (uint32_t p = sg.beg + threadIdx.x; p < sg.end; p += blockDim.x) acc = Pol::add(acc, x[__ldg(col + p)]);
-            acc = block_combine<Pol>(acc, red);
-            if (threadIdx.x == 0) partial[s] = acc;
-        }
-        return;
-    }
-    constexpr int RPW = 32 / G;  // rows per warp per iteration
-    const int lane = threadIdx.x & 31;
-    const int sub = lane / G, gl = lane % G;
-    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)short_blocks * blockDim.x) >> 5;
-    for (int64_t base = warp * RPW; base < n; base += nwarps * RPW) {
-        const int64_t row = base + sub;
-        uint32_t b = 0, e = 0;
-        bool mine = false;
-        if (row < n) {
-            b = __ldg(rp + row);
-            e = __ldg(rp + row + 1);
-            mine = (e - b) < long_min;
-            if (!mine) e = b;
-        }
-        A acc0 = Pol::zero(), acc1 = Pol::zero();
-        uint32_t p = b + gl;
-        for (; p + G < e; p += 2 * G) {
-            const int32_t c0 = __ldg(col + p), c1 = __ldg(col + p + G);
-            acc0 = Pol::add(acc0, x[c0]);
-            acc1 = Pol::add(acc1, x[c1]);
-        }
-        if (p < e) acc0 = Pol::add(acc0, x[__ldg(col + p)]);
-        A acc = Pol::combine(acc0, acc1);
-#pragma unroll
-        for (int o = G / 2; o > 0; o >>= 1) acc = Pol::combine(acc, Pol::shfl(acc, o, G));
-        if (gl == 0 && mine) op(row, acc);
-    }
-}
-
-// One warp per long row: combine the row's segment partials in order.
-template <class Pol, class Op>
-__global__ void __launch_bounds__(kBlock) long_rows_kernel(int64_t nlong, const int32_t* __restrict__ long_rows,
-                                                           const int32_t* __restrict__ long_first,
-                                                           const typename Pol::A* __restrict__ partial, Op op) {
-    const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (w >= nlong || lane != 0) return;
-    typename Pol::A acc = Pol::zero();
-    for (int32_t s = long_first[w]; s < long_first[w + 1]; ++s) acc = Pol::combine(acc, partial[s]);
-    op(long_rows[w], acc);
+    if (lane == 0) op((int64_t)r.x, sum);
 }
 
 // ---------------------------------------------------------------- level 0
@@ -488,6 +397,11 @@ __global__ void __launch_bounds__(kBlock) scatter_level_kernel(const uint64_t* _
     }
 }
 
+size_t scratch_pieces(const Graph& g) {
+    const int64_t p = g.in.sell.npieces > g.out.sell.npieces ? g.in.sell.npieces : g.out.sell.npieces;
+    return (size_t)(p ? p : 1);
+}
+
 int elementwise_blocks(const Graph& g, int64_t n) {
     int64_t b = (n + kBlock - 1) / kBlock;
     int64_t cap = (int64_t)g.sm_count * 8;
@@ -495,65 +409,15 @@ int elementwise_blocks(const Graph& g, int64_t n) {
     return (int)(b < 1 ? 1 : b);
 }
 
-template <class Pol, int G, class Op>
-cudaError_t sweep_level_g(const Graph& g, const DevCsr& A, const typename Pol::V* x, const Op& op) {
-    using Acc = typename Pol::A;
-    Acc* partial = reinterpret_cast<Acc*>(g.partial);
-    int64_t rows_per_block = kBlock / G;
-    int64_t sb = (g.n + rows_per_block - 1) / rows_per_block;
-    int64_t cap = (int64_t)g.sm_count * 16;
-    if (sb > cap) sb = cap;
-    if (sb < 1) sb = 1;
-    int64_t segb = A.nseg;
-    if (segb > (int64_t)g.sm_count * 16) segb = (int64_t)g.sm_count * 16;
-    rows_kernel<Pol, G, Op><<<(unsigned)(sb + segb), kBlock, 0, g.stream>>>(g.n, A.rp, A.col, x, A.long_min, op, A.nseg,
-                                                                            A.seg, partial, (int)sb);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    if (A.nlong > 0) {
-        int64_t blocks = (A.nlong * 32 + kBlock - 1) / kBlock;
-        long_rows_kernel<Pol, Op><<<(unsigned)blocks, kBlock, 0, g.stream>>>(A.nlong, A.long_rows, A.long_first,
-                                                                             partial, op);
-        e = cudaGetLastError();
-    }
-    return e;
-}
-
-template <class Pol, class Op>
-cudaError_t sweep_level_rows(const Graph& g, const DevCsr& A, const typename Pol::V* x, const Op& op) {
-    switch (A.group) {
-        case 2: return sweep_level_g<Pol, 2>(g, A, x, op);
-        case 4: return sweep_level_g<Pol, 4>(g, A, x, op);
-        case 8: return sweep_level_g<Pol, 8>(g, A, x, op);
-        case 16: return sweep_level_g<Pol, 16>(g, A, x, op);
-        default: return sweep_level_g<Pol, 32>(g, A, x, op);
-    }
-}
-
 template <class Pol, class Op>
 cudaError_t sweep_level(const Graph& g, const DevCsr& A, const typename Pol::V* x, const Op& op) {
-    if constexpr (std::is_same<Pol, Pol64>::value) return sweep_level_rows<Pol>(g, A, x, op);
     using Acc = typename Pol::A;
+    static_assert(sizeof(Acc) == 8, "piece sums are 8 bytes");
     Acc* partial = reinterpret_cast<Acc*>(g.partial);
-    // one block per eight tiles (the hardware balances the blocks over the SMs), then the
-    // segment blocks
-    const int64_t warps = kBlock / 32;
-    int64_t tb = (A.ntiles + warps - 1) / warps;
-    if (tb < 1) tb = 1;
-    const int64_t cap = (int64_t)g.sm_count * 8;
-    int64_t segb = A.tnseg;
-    if (segb > cap) segb = cap;
-    tile_rows_kernel<Pol, Op><<<(unsigned)(tb + segb), kBlock, 0, g.stream>>>(
-        A.rp, A.col, x, A.tiles, A.ntiles, A.tile_cap, op, A.tnseg, A.tseg, partial, (int)tb);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    if (A.tnlong > 0) {
-        int64_t blocks = (A.tnlong * 32 + kBlock - 1) / kBlock;
-        long_rows_kernel<Pol, Op><<<(unsigned)blocks, kBlock, 0, g.stream>>>(A.tnlong, A.tlong_rows, A.tlong_first,
-                                                                             partial, op);
-        e = cudaGetLastError();
-    }
-    return e;
+    unsigned* arrived = reinterpret_cast<unsigned*>(partial + scratch_pieces(g));
+    const int64_t blocks = (A.sell.nslices * 32 + kBlock - 1) / kBlock;
+    sell_rows_kernel<Pol, Op><<<(unsigned)blocks, kBlock, 0, g.stream>>>(A.sell, A.rp, x, op, partial, arrived);
+    return cudaGetLastError();
 }
 
 f2 host_f2(double v) {
@@ -562,6 +426,8 @@ f2 host_f2(double v) {
 }
 
 }  // namespace
+
+size_t sweep_scratch_bytes(const Graph& g) { return scratch_pieces(g) * (8 + sizeof(unsigned)); }
 
 cudaError_t launch_forward(const Graph& g, int64_t u, double c, int32_t L, double* hist, double* xa, double* xb) {
     const double sc = sqrt(c);
