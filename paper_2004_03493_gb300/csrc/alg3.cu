@@ -118,11 +118,11 @@ __global__ void scatter_ids_kernel(int64_t n, const uint64_t* __restrict__ flag,
 
 // x = v / din^2 as a two-float: the input of the squared-transition sweep P~ v
 __global__ void sq_scale_kernel(int64_t n, const double* __restrict__ v, const double* __restrict__ inv_din,
-                                float2* __restrict__ x) {
+                                const uint32_t* __restrict__ pos, float2* __restrict__ x) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const double w = inv_din[i];
         const f2 t = double_to_f2_bits(v[i] * (w * w));
-        x[i] = make_float2(t.hi, t.lo);
+        x[at_pos(pos, i)] = make_float2(t.hi, t.lo);
     }
 }
 
@@ -1119,7 +1119,7 @@ cudaError_t alg3_first_meeting(const Graph& g, int64_t k, int depth, double c, v
         const double* T = nullptr;
         if (j >= 2) {  // T = P~ Zv_{j-1}
             float2* x2 = reinterpret_cast<float2*>(ws.x);  // n 8-byte entries
-            sq_scale_kernel<<<eb, kBlock, 0, g.stream>>>(g.n, ws.Zv + (size_t)(j - 1) * n, g.inv_din, x2);
+            sq_scale_kernel<<<eb, kBlock, 0, g.stream>>>(g.n, ws.Zv + (size_t)(j - 1) * n, g.inv_din, g.out.sell.pos, x2);
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
             if ((e = launch_pull_sum(g, x2, ws.T)) != cudaSuccess) return e;
             count += 2;

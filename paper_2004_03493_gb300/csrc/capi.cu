@@ -68,7 +68,7 @@ constexpr int64_t kLongRowsFrom = 4000000;  // from this many edges on a level i
 
 // Upload a host CSR and build its row-split table.
 esim_status upload_csr(int64_t n, const std::vector<uint32_t>& rp, const std::vector<int32_t>& col, DevCsr& d,
-                       bool with_info, cudaStream_t stream) {
+                       bool with_info, const std::vector<uint32_t>& uses_rp, cudaStream_t stream) {
     const int64_t m = (int64_t)rp[n];
     const double avg = (double)m / (double)n;
     d.long_min = avg > 12.0 ? (avg > 24.0 ? 1024u : 512u) : 256u;
@@ -114,7 +114,7 @@ esim_status upload_csr(int64_t n, const std::vector<uint32_t>& rp, const std::ve
         cudaGetLastError();
         return fail(st, st == ESIM_ENOMEM ? "cudaMalloc(graph tables)" : "upload of the graph tables");
     }
-    const cudaError_t se = build_sell(n, d, pieces, stream, d.sell);
+    const cudaError_t se = build_sell(n, d, pieces, uses_rp, stream, d.sell);
     if (se != cudaSuccess) {
         cudaGetLastError();
         return fail(se == cudaErrorMemoryAllocation ? ESIM_ENOMEM : ESIM_ECUDA,
@@ -1281,8 +1281,8 @@ esim_status esim_load_graph(int64_t n, const int64_t* in_rowptr, const int32_t* 
             return fail(ESIM_ENOMEM, "device allocation for 1/din");
         }
     }
-    esim_status st = upload_csr(n, in_rp, in_c, g.in, true, cudaStreamPerThread);
-    if (st == ESIM_OK) st = upload_csr(n, out_rp, out_c, g.out, false, cudaStreamPerThread);
+    esim_status st = upload_csr(n, in_rp, in_c, g.in, true, out_rp, cudaStreamPerThread);
+    if (st == ESIM_OK) st = upload_csr(n, out_rp, out_c, g.out, false, in_rp, cudaStreamPerThread);
     if (st != ESIM_OK) {
         release(g);
         delete h;

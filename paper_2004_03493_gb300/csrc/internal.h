@@ -61,6 +61,9 @@ struct Segment {
 // entries side by side: entry t of lane l's row is col[(off[s] + t) * 32 + l].  A row longer
 // than row_cap is cut into pieces of 32 row_cap entries, and slice s < npieces is piece s:
 // the same layout with the piece's entries t * 32 + l.
+// The gathered vector keeps the nodes that most entries name (its hubs) together: node i's
+// value is at pos[i], hubs first, every other node in order after them (pos NULL: at i).
+// col holds positions.
 struct SellRows {
     uint32_t* off = nullptr;    // nslices + 1
     int2* rows = nullptr;       // 32 per slice: (row, or -1; this lane's entries)
@@ -69,7 +72,11 @@ struct SellRows {
     int64_t nslices = 0;
     int64_t npieces = 0;
     uint32_t row_cap = 64;
+    uint32_t* pos = nullptr;    // n, or NULL
+    uint32_t hubs = 0;
 };
+
+__host__ __device__ inline int64_t at_pos(const uint32_t* pos, int64_t i) { return pos ? (int64_t)pos[i] : i; }
 
 constexpr int kSellWindow = 1024;           // rows sorted by length together
 
@@ -190,8 +197,8 @@ struct Graph {
 };
 
 // sell.cu
-cudaError_t build_sell(int64_t n, const DevCsr& csr, const std::vector<Segment>& pieces, cudaStream_t stream,
-                       SellRows& out);
+cudaError_t build_sell(int64_t n, const DevCsr& csr, const std::vector<Segment>& pieces,
+                       const std::vector<uint32_t>& uses_rp, cudaStream_t stream, SellRows& out);
 void free_sell(SellRows& s);
 
 // sweep.cu

@@ -10,11 +10,19 @@
 #include "common.cuh"
 #include "internal.h"
 
+#include <algorithm>
 #include <vector>
 
 namespace esim {
 
 namespace {
+
+// Hubs.  A gathered value occupies a whole 128-byte line of the L1, about 1800 lines; side by
+// side the hubs share lines of 16 (FP32c: 32) values.  n = 1e6, m = 1.75e7, L = 33, forward and
+// reverse, FP64 / FP32c: 4.75 / 4.36 ms without, 4.61 / 4.07 with 8192 hubs, 4.67 / 4.10 with
+// 16384, 4.76 / 4.19 with 32768.  Loads that keep the hubs and pass the others by the L1 are
+// two instructions a gather and lose (4.87 / 4.19).
+constexpr uint32_t kSellHubs = 8192;
 
 // One window per block: sorts its rows by (length descending, row ascending) and writes
 // their (row, length) and, per slice, its longest row.  Cut rows get no place.
@@ -68,7 +76,8 @@ __global__ void __launch_bounds__(kBlock) sell_fill_kernel(int64_t nslices, int6
                                                           const int2* __restrict__ rows,
                                                           const Segment* __restrict__ piece,
                                                           const uint32_t* __restrict__ rp,
-                                                          const int32_t* __restrict__ col, int32_t* __restrict__ out) {
+                                                          const int32_t* __restrict__ col,
+                                                          const uint32_t* __restrict__ pos, int32_t* __restrict__ out) {
     const int lane = threadIdx.x & 31;
     for (int64_t s = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; s < nslices;
          s += ((int64_t)gridDim.x * blockDim.x) >> 5) {
@@ -77,15 +86,43 @@ __global__ void __launch_bounds__(kBlock) sell_fill_kernel(int64_t nslices, int6
         const bool wide = s < npieces;
         const uint32_t beg = wide ? piece[s].beg + lane : (r.x < 0 ? 0u : rp[r.x]);
         for (uint32_t t = 0; t < o1 - o0; ++t)
-            out[((size_t)o0 + t) * 32 + lane] = t < (uint32_t)r.y ? col[beg + (wide ? 32 * t : t)] : 0;
+            out[((size_t)o0 + t) * 32 + lane] = t < (uint32_t)r.y ? (int32_t)at_pos(pos, col[beg + (wide ? 32 * t : t)]) : 0;
     }
 }
 
 }  // namespace
 
-cudaError_t build_sell(int64_t n, const DevCsr& csr, const std::vector<Segment>& pieces, cudaStream_t stream,
-                       SellRows& out) {
+// Positions of the gathered vector: the at most kSellHubs nodes with the most uses (node i has
+// uses_rp[i+1] - uses_rp[i] of them, the row lengths of the transpose) first.  Empty where
+// that would gain nothing: every node is one, or they have no more than twice their share.
+std::vector<uint32_t> hub_positions(int64_t n, const std::vector<uint32_t>& uses_rp, uint32_t* hubs) {
+    *hubs = 0;
+    if (n <= (int64_t)kSellHubs) return {};
+    constexpr uint32_t kTop = 1u << 16;  // uses above this are alike
+    std::vector<uint32_t> count(kTop + 1, 0);
+    auto uses = [&](int64_t i) { return std::min(uses_rp[(size_t)i + 1] - uses_rp[(size_t)i], kTop); };
+    for (int64_t i = 0; i < n; ++i) ++count[uses(i)];
+    uint32_t least = kTop + 1, h = 0;  // hubs: the nodes with at least this many uses
+    while (least > 1 && h + count[least - 1] <= kSellHubs) h += count[--least];
+    uint64_t share = 0;
+    for (int64_t i = 0; i < n; ++i)
+        if (uses(i) >= least) share += uses_rp[(size_t)i + 1] - uses_rp[(size_t)i];
+    if (h == 0 || (double)share * (double)n < 2.0 * (double)h * (double)uses_rp[(size_t)n]) return {};
+    std::vector<uint32_t> pos((size_t)n);
+    uint32_t hub = 0, other = h;
+    for (int64_t i = 0; i < n; ++i) pos[(size_t)i] = uses(i) >= least ? hub++ : other++;
+    *hubs = h;
+    return pos;
+}
+
+cudaError_t build_sell(int64_t n, const DevCsr& csr, const std::vector<Segment>& pieces,
+                       const std::vector<uint32_t>& uses_rp, cudaStream_t stream, SellRows& out) {
     cudaError_t e = cudaSuccess;
+    const std::vector<uint32_t> pos = hub_positions(n, uses_rp, &out.hubs);
+    if (!pos.empty() && ((e = cudaMalloc((void**)&out.pos, sizeof(uint32_t) * pos.size())) != cudaSuccess ||
+                         (e = cudaMemcpyAsync(out.pos, pos.data(), sizeof(uint32_t) * pos.size(),
+                                              cudaMemcpyHostToDevice, stream)) != cudaSuccess))
+        return e;
     out.npieces = (int64_t)pieces.size();
     const int64_t windows = (n + kSellWindow - 1) / kSellWindow;
     out.nslices = out.npieces + windows * (kSellWindow / 32);
@@ -123,7 +160,7 @@ cudaError_t build_sell(int64_t n, const DevCsr& csr, const std::vector<Segment>&
     int64_t blocks = (out.nslices * 32 + kBlock - 1) / kBlock;
     if (blocks > 65536) blocks = 65536;
     sell_fill_kernel<<<(unsigned)blocks, kBlock, 0, stream>>>(out.nslices, out.npieces, out.off, out.rows,
-                                                             out.piece, csr.rp, csr.col, out.col);
+                                                             out.piece, csr.rp, csr.col, out.pos, out.col);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     return cudaStreamSynchronize(stream);  // pieces and steps are the caller's and this call's
 }
@@ -133,6 +170,7 @@ void free_sell(SellRows& s) {
     cudaFree(s.rows);
     cudaFree(s.piece);
     cudaFree(s.col);
+    cudaFree(s.pos);
     s = SellRows{};
 }
 

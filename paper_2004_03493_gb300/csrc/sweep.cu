@@ -86,45 +86,38 @@ __device__ __forceinline__ typename Pol::A warp_combine(typename Pol::A v) {  //
 struct ForwardOp {  // FP64
     double sc;
     const double* __restrict__ inv_din;
+    const uint32_t* __restrict__ pos;
     double* __restrict__ pi_out;
-    double* __restrict__ x_out;
+    double* __restrict__ x_out;  // by position
     __device__ __forceinline__ void operator()(int64_t row, double acc) const {
         const double p = sc * acc;
         pi_out[row] = p;
-        x_out[row] = p * inv_din[row];
-    }
-};
-
-struct ReverseOp {  // FP64; 1/a is a host constant (an FP64 division per row is costly on GB300)
-    double sc;
-    double inv_a;
-    const double* __restrict__ inv_din;
-    const double* __restrict__ dhat;
-    const double* __restrict__ h;  // pi^{L-l}
-    double* __restrict__ s_out;
-    __device__ __forceinline__ void operator()(int64_t row, double acc) const {
-        s_out[row] = (sc * acc) * inv_din[row] + dhat[row] * h[row] * inv_a;
+        x_out[at_pos(pos, row)] = p * inv_din[row];
     }
 };
 
 struct ReverseSparseOp {  // FP64; the D^ pi^{L-l} / a term is scattered from the sparse history
     double sc;
     const double* __restrict__ inv_din;
+    const uint32_t* __restrict__ pos;  // NULL for the last level, whose result is by node
     double* __restrict__ s_out;
-    __device__ __forceinline__ void operator()(int64_t row, double acc) const { s_out[row] = (sc * acc) * inv_din[row]; }
+    __device__ __forceinline__ void operator()(int64_t row, double acc) const {
+        s_out[at_pos(pos, row)] = (sc * acc) * inv_din[row];
+    }
 };
 
 struct ForwardOp32c {  // FP32 storage, two-float sum
     f2 sc;
     const uint32_t* __restrict__ in_rp;
+    const uint32_t* __restrict__ pos;
     float* __restrict__ pi_out;
-    float* __restrict__ x_out;
+    float* __restrict__ x_out;  // by position
     __device__ __forceinline__ void operator()(int64_t row, f2 acc) const {
         const f2 p = f2_mul(acc, sc);
         const float pf = __fadd_rn(p.hi, p.lo);
         pi_out[row] = pf;
         const uint32_t d = in_rp[row + 1] - in_rp[row];
-        x_out[row] = d ? __fdiv_rn(pf, (float)d) : 0.f;
+        x_out[at_pos(pos, row)] = d ? __fdiv_rn(pf, (float)d) : 0.f;
     }
 };
 
@@ -134,9 +127,10 @@ template <bool kFinal>
 struct ReverseOp2f {
     f2 sc;
     const uint32_t* __restrict__ rp;
+    const uint32_t* __restrict__ pos;
     const float2* __restrict__ w;
     const float* __restrict__ h;
-    float2* __restrict__ s_out;
+    float2* __restrict__ s_out;  // by position
     double* __restrict__ s_final;
     __device__ __forceinline__ void operator()(int64_t row, f2 acc) const {
         const uint32_t d = rp[row + 1] - rp[row];
@@ -145,7 +139,7 @@ struct ReverseOp2f {
         const float2 wv = w[row];
         const f2 s = f2_add(prop, f2_mul_f(f2{wv.x, wv.y}, h[row]));
         if (kFinal) s_final[row] = f2_to_double(s);
-        else s_out[row] = make_float2(s.hi, s.lo);
+        else s_out[at_pos(pos, row)] = make_float2(s.hi, s.lo);
     }
 };
 
@@ -154,14 +148,15 @@ struct ReverseOp2f {
 struct ForwardOpD {
     f2 sc;
     const uint32_t* __restrict__ in_rp;
+    const uint32_t* __restrict__ pos;
     double* __restrict__ pi_out;
-    float2* __restrict__ x_out;
+    float2* __restrict__ x_out;  // by position
     __device__ __forceinline__ void operator()(int64_t row, f2 acc) const {
         const f2 p = f2_mul(acc, sc);
         pi_out[row] = f2_to_double_bits(p);
         const uint32_t d = in_rp[row + 1] - in_rp[row];
         const f2 x = d ? f2_div_f(p, (float)d) : f2{0.f, 0.f};
-        x_out[row] = make_float2(x.hi, x.lo);
+        x_out[at_pos(pos, row)] = make_float2(x.hi, x.lo);
     }
 };
 
@@ -178,16 +173,17 @@ struct ReverseOpD {
     f2 sc;
     f2 a;
     const uint32_t* __restrict__ rp;
+    const uint32_t* __restrict__ pos;
     const double* __restrict__ dhat;
     const double* __restrict__ h;
-    float2* __restrict__ s_out;
+    float2* __restrict__ s_out;  // by position
     double* __restrict__ s_final;
     __device__ __forceinline__ void operator()(int64_t row, f2 acc) const {
         const uint32_t d = rp[row + 1] - rp[row];
         const f2 prop = d ? f2_div_f(f2_mul(acc, sc), (float)d) : f2{0.f, 0.f};
         const f2 s = f2_add(prop, diag_term(dhat[row], h[row], a));
         if (kFinal) s_final[row] = f2_to_double_bits(s);
-        else s_out[row] = make_float2(s.hi, s.lo);
+        else s_out[at_pos(pos, row)] = make_float2(s.hi, s.lo);
     }
 };
 
@@ -206,7 +202,11 @@ struct ReverseOpD {
 // that counts in the last of them adds their sums.  Both joins are fixed shuffle trees.
 // Every row's sum has a fixed order, so the sweeps are deterministic.
 //
-// BEFOREAFTER
+// n = 1e6, m = 1.75e7: 81 / 83 us a forward / reverse level in FP64 storage, against 128 / 137
+// on warp tiles staged in shared memory (54 instructions an entry, 9 % L1 hits); FP64 sums
+// (sparse history) 98 against 316 on eight or sixteen lanes a row.  n = 1e5, m = 1e6: 11-12
+// against 20-23.  What is left is the L2's rate of scattered sectors (tags 63 % busy, L1
+// path 66 %).
 template <class Pol, class Op>
 __global__ void __launch_bounds__(kBlock) sell_rows_kernel(const SellRows A, const uint32_t* __restrict__ rp,
                                                           const typename Pol::V* __restrict__ x, Op op,
@@ -268,57 +268,51 @@ __global__ void __launch_bounds__(kBlock) sell_rows_kernel(const SellRows A, con
 
 // ---------------------------------------------------------------- level 0
 
-__global__ void forward_init_kernel(int64_t n, int64_t u, double a, const double* __restrict__ inv_din,
+__global__ void forward_init_kernel(int64_t n, int64_t u, const uint32_t* __restrict__ pos, double a, const double* __restrict__ inv_din,
                                     double* __restrict__ pi0, double* __restrict__ x0) {
+    const int64_t pu = at_pos(pos, u);
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         pi0[i] = i == u ? a : 0.0;
-        x0[i] = i == u ? a * inv_din[i] : 0.0;
+        x0[i] = i == pu ? a * inv_din[u] : 0.0;
     }
 }
 
 // FP64 form, level 0: pi^0 = a e_u (FP64), x^0 = a / din(u) e_u as a two-float.
-__global__ void forward_init_d_kernel(int64_t n, int64_t u, double a, float xhi, float xlo,
+__global__ void forward_init_d_kernel(int64_t n, int64_t u, const uint32_t* __restrict__ pos, double a,
+                                      float xhi, float xlo,
                                       double* __restrict__ pi0, float2* __restrict__ x0) {
+    const int64_t pu = at_pos(pos, u);
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         pi0[i] = i == u ? a : 0.0;
-        x0[i] = i == u ? make_float2(xhi, xlo) : make_float2(0.f, 0.f);
+        x0[i] = i == pu ? make_float2(xhi, xlo) : make_float2(0.f, 0.f);
     }
 }
 
 // FP64 form: s^0 = D^ pi^L / a as a two-float (in FP64 when L = 0).
-__global__ void reverse_init_d_kernel(int64_t n, float a_hi, float a_lo, const double* __restrict__ dhat,
+__global__ void reverse_init_d_kernel(int64_t n, const uint32_t* __restrict__ pos, float a_hi, float a_lo,
+                                      const double* __restrict__ dhat,
                                       const double* __restrict__ h, float2* __restrict__ s0,
                                       double* __restrict__ s_final) {
     const f2 a{a_hi, a_lo};
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const f2 s = diag_term(dhat[i], h[i], a);
         if (s_final) s_final[i] = f2_to_double_bits(s);
-        else s0[i] = make_float2(s.hi, s.lo);
+        else s0[at_pos(pos, i)] = make_float2(s.hi, s.lo);
     }
 }
 
-__global__ void forward_init32_kernel(int64_t n, int64_t u, float a, const uint32_t* __restrict__ in_rp,
+__global__ void forward_init32_kernel(int64_t n, int64_t u, const uint32_t* __restrict__ pos, float a, float xv,
                                       float* __restrict__ pi0, float* __restrict__ x0) {
+    const int64_t pu = at_pos(pos, u);
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        float p = 0.f, xv = 0.f;
-        if (i == u) {
-            p = a;
-            const uint32_t d = in_rp[i + 1] - in_rp[i];
-            xv = d ? __fdiv_rn(a, (float)d) : 0.f;
-        }
-        pi0[i] = p;
-        x0[i] = xv;
+        pi0[i] = i == u ? a : 0.f;
+        x0[i] = i == pu ? xv : 0.f;
     }
-}
-
-__global__ void reverse_init_kernel(int64_t n, double inv_a, const double* __restrict__ dhat,
-                                    const double* __restrict__ h, double* __restrict__ s0) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        s0[i] = dhat[i] * h[i] * inv_a;
 }
 
 // w = D^ / a as two-floats, and s^0 = w pi^L (float2, or FP64 when L = 0)
-__global__ void reverse_init2f_kernel(int64_t n, double inv_a, const double* __restrict__ dhat,
+__global__ void reverse_init2f_kernel(int64_t n, const uint32_t* __restrict__ pos, double inv_a,
+                                      const double* __restrict__ dhat,
                                       const float* __restrict__ h, float2* __restrict__ w, float2* __restrict__ s0,
                                       double* __restrict__ s_final) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
@@ -326,7 +320,7 @@ __global__ void reverse_init2f_kernel(int64_t n, double inv_a, const double* __r
         w[i] = make_float2(wv.hi, wv.lo);
         const f2 s = f2_mul_f(wv, h[i]);
         if (s_final) s_final[i] = f2_to_double(s);
-        else s0[i] = make_float2(s.hi, s.lo);
+        else s0[at_pos(pos, i)] = make_float2(s.hi, s.lo);
     }
 }
 
@@ -387,13 +381,15 @@ __global__ void __launch_bounds__(kBlock) compact_level_kernel(int64_t n, const 
 __global__ void __launch_bounds__(kBlock) scatter_level_kernel(const uint64_t* __restrict__ lvl, int level,
                                                                const int32_t* __restrict__ idx,
                                                                const double* __restrict__ val,
-                                                               const double* __restrict__ dhat, double inv_a,
+                                                               const double* __restrict__ dhat,
+                                                               const uint32_t* __restrict__ pos, double inv_a,
                                                                double* __restrict__ s) {
     const uint64_t beg = lvl[level], end = lvl[level + 1];
     for (uint64_t p = beg + (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; p < end;
          p += (uint64_t)gridDim.x * blockDim.x) {
         const int32_t k = idx[p];
-        s[k] = s[k] + dhat[k] * val[p] * inv_a;
+        const int64_t q = at_pos(pos, k);
+        s[q] = s[q] + dhat[k] * val[p] * inv_a;
     }
 }
 
@@ -435,12 +431,13 @@ cudaError_t launch_forward(const Graph& g, int64_t u, double c, int32_t L, doubl
     const uint32_t din_u = (*g.din_host)[(size_t)u];
     const f2 x0 = din_u ? host_f2(a / (double)din_u) : f2{0.f, 0.f};
     float2* x[2] = {reinterpret_cast<float2*>(xa), reinterpret_cast<float2*>(xb)};
-    forward_init_d_kernel<<<elementwise_blocks(g, g.n), kBlock, 0, g.stream>>>(g.n, u, a, x0.hi, x0.lo, hist, x[0]);
+    forward_init_d_kernel<<<elementwise_blocks(g, g.n), kBlock, 0, g.stream>>>(g.n, u, g.out.sell.pos, a, x0.hi, x0.lo,
+                                                                               hist, x[0]);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const f2 sc2 = host_f2(sc);
     for (int32_t l = 1; l <= L; ++l) {
-        ForwardOpD op{sc2, g.in.rp, hist + (size_t)l * (size_t)g.n, x[l & 1]};
+        ForwardOpD op{sc2, g.in.rp, g.out.sell.pos, hist + (size_t)l * (size_t)g.n, x[l & 1]};
         e = sweep_level<Pol2f>(g, g.out, x[(l - 1) & 1], op);
         if (e != cudaSuccess) return e;
     }
@@ -458,7 +455,7 @@ cudaError_t launch_reverse(const Graph& g, const double* hist, int32_t L, double
     auto buf = [&](int32_t l) { return ((L - 1 - l) & 1) == 0 ? A : S; };
     const f2 a2 = host_f2(a);
     reverse_init_d_kernel<<<elementwise_blocks(g, g.n), kBlock, 0, g.stream>>>(
-        g.n, a2.hi, a2.lo, dhat, hist + (size_t)L * g.n, L > 0 ? buf(0) : nullptr, L == 0 ? s_out : nullptr);
+        g.n, g.in.sell.pos, a2.hi, a2.lo, dhat, hist + (size_t)L * g.n, L > 0 ? buf(0) : nullptr, L == 0 ? s_out : nullptr);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const f2 sc2 = host_f2(sc);
@@ -466,10 +463,10 @@ cudaError_t launch_reverse(const Graph& g, const double* hist, int32_t L, double
         const float2* sp = buf(l - 1);
         const double* h = hist + (size_t)(L - l) * g.n;
         if (l < L) {
-            ReverseOpD<false> op{sc2, a2, g.in.rp, dhat, h, buf(l), nullptr};
+            ReverseOpD<false> op{sc2, a2, g.in.rp, g.in.sell.pos, dhat, h, buf(l), nullptr};
             e = sweep_level<Pol2f>(g, g.in, sp, op);
         } else {
-            ReverseOpD<true> op{sc2, a2, g.in.rp, dhat, h, nullptr, s_out};
+            ReverseOpD<true> op{sc2, a2, g.in.rp, g.in.sell.pos, dhat, h, nullptr, s_out};
             e = sweep_level<Pol2f>(g, g.in, sp, op);
         }
         if (e != cudaSuccess) return e;
@@ -488,13 +485,13 @@ cudaError_t launch_forward_sparse(const Graph& g, int64_t u, double c, int32_t L
     if (h.lvl && (e = cudaMemsetAsync(h.lvl, 0, sizeof(uint64_t) * (size_t)(L + 2), g.stream)) != cudaSuccess)
         return e;
     const int eb = elementwise_blocks(g, g.n);
-    forward_init_kernel<<<eb, kBlock, 0, g.stream>>>(g.n, u, a, g.inv_din, lev, xa);
+    forward_init_kernel<<<eb, kBlock, 0, g.stream>>>(g.n, u, g.out.sell.pos, a, g.inv_din, lev, xa);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     compact_level_kernel<<<eb, kBlock, 0, g.stream>>>(g.n, lev, pi_run, 1, theta, h, 0, g.status);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     double* x[2] = {xa, xb};
     for (int32_t l = 1; l <= L; ++l) {
-        ForwardOp op{sc, g.inv_din, lev, x[l & 1]};
+        ForwardOp op{sc, g.inv_din, g.out.sell.pos, lev, x[l & 1]};
         if ((e = sweep_level<Pol64>(g, g.out, x[(l - 1) & 1], op)) != cudaSuccess) return e;
         compact_level_kernel<<<eb, kBlock, 0, g.stream>>>(g.n, lev, pi_run, 0, theta, h, l, g.status);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
@@ -512,13 +509,15 @@ cudaError_t launch_reverse_sparse(const Graph& g, const SparseHist& h, int32_t L
     const unsigned sb = (unsigned)g.sm_count * 4;
     cudaError_t e = launch_fill(g, g.n, 0.0, buf[L & 1]);
     if (e != cudaSuccess) return e;
-    scatter_level_kernel<<<sb, kBlock, 0, g.stream>>>(h.lvl, L, h.idx, h.val, dhat, 1.0 / a, buf[L & 1]);
+    scatter_level_kernel<<<sb, kBlock, 0, g.stream>>>(h.lvl, L, h.idx, h.val, dhat, L > 0 ? g.in.sell.pos : nullptr, 1.0 / a,
+                                                 buf[L & 1]);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     for (int32_t l = 1; l <= L; ++l) {
         double* sn = buf[(L - l) & 1];
-        ReverseSparseOp op{sc, g.inv_din, sn};
+        const uint32_t* pos = l < L ? g.in.sell.pos : nullptr;  // the last level's result is by node
+        ReverseSparseOp op{sc, g.inv_din, pos, sn};
         if ((e = sweep_level<Pol64>(g, g.in, buf[(L - l + 1) & 1], op)) != cudaSuccess) return e;
-        scatter_level_kernel<<<sb, kBlock, 0, g.stream>>>(h.lvl, L - l, h.idx, h.val, dhat, 1.0 / a, sn);
+        scatter_level_kernel<<<sb, kBlock, 0, g.stream>>>(h.lvl, L - l, h.idx, h.val, dhat, pos, 1.0 / a, sn);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -532,12 +531,13 @@ cudaError_t launch_walk_distributions(const Graph& g, int64_t u, int steps, doub
     const uint32_t din_u = (*g.din_host)[(size_t)u];
     const f2 x0 = din_u ? host_f2(1.0 / (double)din_u) : f2{0.f, 0.f};
     float2* x[2] = {reinterpret_cast<float2*>(xa), reinterpret_cast<float2*>(xb)};
-    forward_init_d_kernel<<<elementwise_blocks(g, g.n), kBlock, 0, g.stream>>>(g.n, u, 1.0, x0.hi, x0.lo, H, x[0]);
+    forward_init_d_kernel<<<elementwise_blocks(g, g.n), kBlock, 0, g.stream>>>(g.n, u, g.out.sell.pos, 1.0, x0.hi,
+                                                                               x0.lo, H, x[0]);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const f2 one{1.f, 0.f};
     for (int l = 1; l <= steps; ++l) {
-        ForwardOpD op{one, g.in.rp, H + (size_t)l * (size_t)g.n, x[l & 1]};
+        ForwardOpD op{one, g.in.rp, g.out.sell.pos, H + (size_t)l * (size_t)g.n, x[l & 1]};
         e = sweep_level<Pol2f>(g, g.out, x[(l - 1) & 1], op);
         if (e != cudaSuccess) return e;
     }
@@ -549,8 +549,8 @@ struct PlainOpD {
     __device__ __forceinline__ void operator()(int64_t row, f2 acc) const { out[row] = f2_to_double_bits(acc); }
 };
 
-// out(i) = sum_{j in Out(i)} x(j): the pull product over out-edges without weights, x as
-// two-floats, the sums in two-float, out in FP64.
+// out(i) = sum_{j in Out(i)} x(j): the pull product over out-edges without weights, x by
+// position (g.out.sell.pos) as two-floats, the sums in two-float, out in FP64.
 cudaError_t launch_pull_sum(const Graph& g, const float2* x, double* out) {
     return sweep_level<Pol2f>(g, g.out, x, PlainOpD{out});
 }
@@ -558,13 +558,15 @@ cudaError_t launch_pull_sum(const Graph& g, const float2* x, double* out) {
 cudaError_t launch_forward32(const Graph& g, int64_t u, double c, int32_t L, float* hist, float* xa, float* xb) {
     const double sc = sqrt(c);
     const float a = (float)(1.0 - sc);
-    forward_init32_kernel<<<elementwise_blocks(g, g.n), kBlock, 0, g.stream>>>(g.n, u, a, g.in.rp, hist, xa);
+    const uint32_t din_u = (*g.din_host)[(size_t)u];
+    forward_init32_kernel<<<elementwise_blocks(g, g.n), kBlock, 0, g.stream>>>(
+        g.n, u, g.out.sell.pos, a, din_u ? a / (float)din_u : 0.f, hist, xa);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     float* x[2] = {xa, xb};
     const f2 sc2 = host_f2(sc);
     for (int32_t l = 1; l <= L; ++l) {
-        ForwardOp32c op{sc2, g.in.rp, hist + (size_t)l * (size_t)g.n, x[l & 1]};
+        ForwardOp32c op{sc2, g.in.rp, g.out.sell.pos, hist + (size_t)l * (size_t)g.n, x[l & 1]};
         e = sweep_level<Pol32c>(g, g.out, x[(l - 1) & 1], op);
         if (e != cudaSuccess) return e;
     }
@@ -577,7 +579,7 @@ cudaError_t launch_reverse32(const Graph& g, const float* hist, int32_t L, doubl
     const double a = 1.0 - sc;
     float2* buf[2] = {sa, sb};
     reverse_init2f_kernel<<<elementwise_blocks(g, g.n), kBlock, 0, g.stream>>>(
-        g.n, 1.0 / a, dhat, hist + (size_t)L * g.n, w, buf[0], L == 0 ? s_out : nullptr);
+        g.n, g.in.sell.pos, 1.0 / a, dhat, hist + (size_t)L * g.n, w, buf[0], L == 0 ? s_out : nullptr);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const f2 sc2 = host_f2(sc);
@@ -585,10 +587,10 @@ cudaError_t launch_reverse32(const Graph& g, const float* hist, int32_t L, doubl
         const float2* sp = buf[(l - 1) & 1];
         const float* h = hist + (size_t)(L - l) * g.n;
         if (l < L) {
-            ReverseOp2f<false> op{sc2, g.in.rp, w, h, buf[l & 1], nullptr};
+            ReverseOp2f<false> op{sc2, g.in.rp, g.in.sell.pos, w, h, buf[l & 1], nullptr};
             e = sweep_level<Pol2f>(g, g.in, sp, op);
         } else {
-            ReverseOp2f<true> op{sc2, g.in.rp, w, h, nullptr, s_out};
+            ReverseOp2f<true> op{sc2, g.in.rp, g.in.sell.pos, w, h, nullptr, s_out};
             e = sweep_level<Pol2f>(g, g.in, sp, op);
         }
         if (e != cudaSuccess) return e;
