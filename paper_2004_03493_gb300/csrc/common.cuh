@@ -40,4 +40,26 @@ __device__ __forceinline__ T block_sum(T v, T* smem) {
     return r;
 }
 
+// Programmatic dependent launch: a kernel that starts with prior_done() may be launched with
+// launch_after(), which lets it start while the kernel before it in the stream still runs.
+// What it does before prior_done() touches nothing that an earlier kernel of the stream
+// writes.  next_may_start() lets the kernel after it start likewise.
+__device__ __forceinline__ void prior_done() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void next_may_start() { asm volatile("griddepcontrol.launch_dependents;"); }
+
+template <class... Params, class... Args>
+cudaError_t launch_after(cudaStream_t stream, unsigned blocks, unsigned threads, void (*kernel)(Params...),
+                         Args&&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(threads);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, Params(args)...);
+}
+
 }  // namespace esim

@@ -217,6 +217,7 @@ __global__ void __launch_bounds__(kBlock) sell_rows_kernel(const SellRows A, con
     constexpr int kU = 8;  // gathers in flight per lane
     const int lane = threadIdx.x & 31;
     const int64_t s = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    next_may_start();
     if (s >= A.nslices) return;
     const uint32_t o0 = __ldg(A.off + s), steps = __ldg(A.off + s + 1) - o0;
     const int2 r = __ldg(A.rows + s * 32 + lane);
@@ -226,6 +227,7 @@ __global__ void __launch_bounds__(kBlock) sell_rows_kernel(const SellRows A, con
 #pragma unroll
     for (int u = 0; u < kU; ++u)
         if ((uint32_t)u < steps) j[u] = __ldg(c + u * 32);
+    prior_done();  // until here only the graph is read; the level before wrote x
     Acc acc0 = Pol::zero(), acc1 = Pol::zero();
     for (uint32_t t = 0; t < steps; t += kU) {
         V g[kU];
@@ -412,8 +414,8 @@ cudaError_t sweep_level(const Graph& g, const DevCsr& A, const typename Pol::V* 
     Acc* partial = reinterpret_cast<Acc*>(g.partial);
     unsigned* arrived = reinterpret_cast<unsigned*>(partial + scratch_pieces(g));
     const int64_t blocks = (A.sell.nslices * 32 + kBlock - 1) / kBlock;
-    sell_rows_kernel<Pol, Op><<<(unsigned)blocks, kBlock, 0, g.stream>>>(A.sell, A.rp, x, op, partial, arrived);
-    return cudaGetLastError();
+    return launch_after(g.stream, (unsigned)blocks, kBlock, sell_rows_kernel<Pol, Op>, A.sell, A.rp, x, op, partial,
+                        arrived);
 }
 
 f2 host_f2(double v) {
