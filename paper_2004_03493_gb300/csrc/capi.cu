@@ -138,6 +138,14 @@ bool alloc_sweep_scratch(const Graph& g, void** p) {
            cudaStreamSynchronize(cudaStreamPerThread) == cudaSuccess;
 }
 
+// The allocation's and the scans' tile sums, their ticket at zero.
+bool alloc_scan_scratch(int64_t n, unsigned long long** part, double** norm) {
+    const size_t nb = (size_t)allocate_blocks(n);
+    return dev_alloc(part, nb + 1) == cudaSuccess && dev_alloc(norm, 2 * nb) == cudaSuccess &&
+           cudaMemsetAsync(*part + nb, 0, sizeof(**part), cudaStreamPerThread) == cudaSuccess &&
+           cudaStreamSynchronize(cudaStreamPerThread) == cudaSuccess;
+}
+
 void free_a3workers(Graph& g) {
     for (auto& wk : g.a3workers) {
         if (wk.stream) {
@@ -158,13 +166,11 @@ void free_a3workers(Graph& g) {
 int ensure_a3workers(Graph& g, int extra) {
     const size_t need = alg3_workspace_bytes(g);
     if (g.a3worker_ws_bytes < need) free_a3workers(g);
-    const int64_t nb = allocate_blocks(g.n);
     while ((int)g.a3workers.size() < extra) {
         Graph::A3Worker wk;
         const bool ok = cudaStreamCreateWithFlags(&wk.stream, cudaStreamNonBlocking) == cudaSuccess &&
                         cudaMalloc(&wk.ws, need) == cudaSuccess && alloc_sweep_scratch(g, &wk.partial) &&
-                        dev_alloc(&wk.scan_part, (size_t)nb) == cudaSuccess &&
-                        dev_alloc(&wk.norm_part, 2 * (size_t)nb) == cudaSuccess;
+                        alloc_scan_scratch(g.n, &wk.scan_part, &wk.norm_part);
         if (!ok) {
             cudaGetLastError();
             if (wk.stream) cudaStreamDestroy(wk.stream);
@@ -451,10 +457,10 @@ esim_status launch_side_walks(Graph& g, const Ws& w, const uint64_t* off, double
 esim_status start_side_walks(Graph& g, const Ws& w, double c, uint64_t seed, int* launches) {
     ESIM_CUDA_TRY(launch_mask_R(g, w.R, w.cand, (1u << 0) | (1u << 2), w.R2), "side nodes' R");
     const int64_t nb = allocate_blocks(g.n);
-    ESIM_CUDA_TRY(launch_scan_R(g, g.n, w.R2, w.off2, g.scan_part, nullptr, g.norm_part + nb, false), "side nodes' scan");
+    ESIM_CUDA_TRY(launch_scan_R(g, g.n, w.R2, w.off2, g.scan_part, g.norm_part + nb, false), "side nodes' scan");
     esim_status st = launch_side_walks(g, w, w.off2, c, seed, w.depth);
     if (st != ESIM_OK) return st;
-    *launches += 5;
+    *launches += 4;
     return ESIM_OK;
 }
 
@@ -723,8 +729,8 @@ esim_status plan_alg3(Graph& g, const Ws& w, double c, double R_b, int* launches
     if (zs != ESIM_OK) return zs;
     g.last_alg3_nodes = used;
     const int64_t nb = allocate_blocks(g.n);
-    ESIM_CUDA_TRY(launch_scan_R(g, g.n, w.R, w.off, g.scan_part, nullptr, g.norm_part + nb), "Algorithm 3 rescan");
-    *launches += 3;
+    ESIM_CUDA_TRY(launch_scan_R(g, g.n, w.R, w.off, g.scan_part, g.norm_part + nb), "Algorithm 3 rescan");
+    *launches += 2;
     return ESIM_OK;
 }
 
@@ -777,7 +783,7 @@ esim_status run_query(Graph& g, int64_t u, double c, double eps, uint64_t seed, 
     else if (g.precision == 0) ESIM_CUDA_TRY(launch_forward(g, u, c, L, w.hist, w.xa, w.xb), "forward sweeps");
     else ESIM_CUDA_TRY(launch_forward32(g, u, c, L, w.hist32, w.xa32, w.xb32), "forward sweeps (FP32c)");
     if (g.timing) cudaEventRecord(g.ev[1], g.stream);
-    // kernels of the allocation, sampling and D^ phases (the default counts 3 + 1 + 1)
+    // kernels of the allocation, sampling and D^ phases (the default counts 2 + 1 + 1)
     int extra_launches = 0;
     bool side_used = false;
     g.last_alg3_nodes = 0;
@@ -790,7 +796,7 @@ esim_status run_query(Graph& g, int64_t u, double c, double eps, uint64_t seed, 
             cudaEventRecord(g.ev[3], g.stream);
         }
         ESIM_CUDA_TRY(launch_fill(g, g.n, 1.0 - c, w.dhat), "dhat (ParSim)");
-        extra_launches -= 4;
+        extra_launches -= 3;
     } else {
         if (sparse)  // pi was summed level by level during the forward sweeps
             ESIM_CUDA_TRY(launch_allocate(g, w.pirun, 0, R_b, g.alloc_mode, w.pi, w.R, w.off), "allocation");
@@ -811,7 +817,7 @@ esim_status run_query(Graph& g, int64_t u, double c, double eps, uint64_t seed, 
         if (side) {
             // the remaining candidates' walks here; the side stream's counts for the rest
             ESIM_CUDA_TRY(launch_mask_R(g, w.R, w.cand, 1u << 1, w.R2), "candidates' R");
-            ESIM_CUDA_TRY(launch_scan_R(g, g.n, w.R2, w.offc, g.scan_part, nullptr, g.norm_part + allocate_blocks(g.n),
+            ESIM_CUDA_TRY(launch_scan_R(g, g.n, w.R2, w.offc, g.scan_part, g.norm_part + allocate_blocks(g.n),
                                         false),
                           "candidates' scan");
             if (g.timing) cudaEventRecord(g.ev[6], g.stream);
@@ -819,7 +825,7 @@ esim_status run_query(Graph& g, int64_t u, double c, double eps, uint64_t seed, 
             if (g.timing) cudaEventRecord(g.ev[7], g.stream);
             ESIM_CUDA_TRY(cudaStreamWaitEvent(g.stream, g.side_ev[1], 0), "wait for the side walks");
             ESIM_CUDA_TRY(launch_merge_counts(g, w.cand, w.nm2, w.nonmeet), "merge counts");
-            extra_launches += 5;
+            extra_launches += 4;
         } else {
             if (g.timing) cudaEventRecord(g.ev[6], g.stream);
             ESIM_CUDA_TRY(launch_sample(g, w.off, c, seed, w.nonmeet, nullptr, g.alg3 ? w.depth : nullptr),
@@ -864,9 +870,9 @@ esim_status run_query(Graph& g, int64_t u, double c, double eps, uint64_t seed, 
     ESIM_CUDA_TRY(cudaStreamSynchronize(g.stream), "query");
     const Status hs = *g.status_host;
     g.last_L = L;
-    // kernels launched: forward init + per level, 3 allocation
+    // kernels launched: forward init + per level, 2 allocation
     // kernels, the sampler, D^, reverse init + per level, and 2 for top-k
-    g.last_launches = (1 + L) + 3 + 1 + 1 + (1 + L) + (k > 0 ? 2 : 0) + extra_launches;
+    g.last_launches = (1 + L) + 2 + 1 + 1 + (1 + L) + (k > 0 ? 2 : 0) + extra_launches;
     if (sparse) g.last_launches += 2 * (L + 1) + count_launches;  // compactions, scatters, counting pass
     g.last_hist_entries = sparse ? std::min<uint64_t>(hs.hist_count, cap) : (uint64_t)(L + 1) * (uint64_t)g.n;
     g.last_R_b = R_b;
@@ -914,7 +920,6 @@ struct BWs {
     int32_t* L;       // W
     double* Rb;       // W
     unsigned long long* part_R;  // tiles of B n
-    double* part_norm;
     double* part_Rd;
     void* topk;       // batched top-k state
     int32_t* ids;     // B k (staging)
@@ -948,8 +953,7 @@ size_t bws_layout(int64_t n_, int W, int B, int32_t Lmax, int64_t nseg_max, int 
     t.L = (int32_t*)take(4 * W);
     t.Rb = (double*)take(8 * W);
     const size_t nb = (size_t)allocate_blocks((int64_t)bn);
-    t.part_R = (unsigned long long*)take(8 * nb);
-    t.part_norm = (double*)take(8 * nb);
+    t.part_R = (unsigned long long*)take(8 * (nb + 1));
     t.part_Rd = (double*)take(8 * nb);
     t.topk = take(topk_batch_workspace_bytes(B));
     t.ids = (int32_t*)take(4 * (size_t)B * (size_t)std::max(k, 1));
@@ -1031,7 +1035,7 @@ esim_status run_batch(Graph& g, int32_t B, const int64_t* u, const double* eps, 
     ESIM_CUDA_TRY(cudaStreamSynchronize(g.stream), "batch query");
     const Status hs = *g.status_host;
     g.last_L = plan.Lmax;
-    g.last_launches = 1 + plan.Lmax * (1 + (g.out.bnlong > 0 ? 1 : 0)) + 1 + 3 + 1 + 1 + 1 +
+    g.last_launches = 1 + plan.Lmax * (1 + (g.out.bnlong > 0 ? 1 : 0)) + 1 + 2 + 1 + 1 + 1 +
                       plan.Lmax * (1 + (g.in.bnlong > 0 ? 1 : 0)) + (k > 0 ? 2 : 0) + (g.shared_walks ? 2 : 0);
     g.last_R_b = plan.Rb[0];
     g.last_kappa = kappa_of(g, c);
@@ -1116,6 +1120,7 @@ int batch_enqueue(Graph& tuner, const Graph& view, const BatchPlan& p, void* ws,
     ESIM_CUDA_TRY(cudaMemcpyAsync(w.u, p.u, sizeof(int64_t) * W, cudaMemcpyHostToDevice, stream), "upload sources");
     ESIM_CUDA_TRY(cudaMemcpyAsync(w.L, p.Lq, sizeof(int32_t) * W, cudaMemcpyHostToDevice, stream), "upload depths");
     ESIM_CUDA_TRY(cudaMemcpyAsync(w.Rb, p.Rb, sizeof(double) * W, cudaMemcpyHostToDevice, stream), "upload R_b");
+    ESIM_CUDA_TRY(cudaMemsetAsync(w.part_R + allocate_blocks(N), 0, sizeof(*w.part_R), stream), "reset scan ticket");
     if (timing) cudaEventRecord(view.ev[0], stream);
     ESIM_CUDA_TRY(launch_batch_forward_init(view, W, B, w.u, c, w.hist, w.xa), "batch forward init");
     const int wi = batch_wi(W);
@@ -1135,7 +1140,7 @@ int batch_enqueue(Graph& tuner, const Graph& view, const BatchPlan& p, void* ws,
     if (view.shared_walks) {
         // one walk set per node: intervals between the distinct R_q(k), sampled once
         ESIM_CUDA_TRY(launch_shared_plan(view, B, w.R, w.scount, w.rbase), "shared walk plan");
-        ESIM_CUDA_TRY(launch_scan_R(view, N, w.scount, w.off, w.part_R, w.part_norm, w.part_Rd), "shared walk scan");
+        ESIM_CUDA_TRY(launch_scan_R(view, N, w.scount, w.off, w.part_R, w.part_Rd), "shared walk scan");
         if (timing) cudaEventRecord(view.ev[2], stream);
         ESIM_CUDA_TRY(launch_sample_segments(view, N, w.off, c, seed, w.scount, nullptr, nullptr, B, w.rbase),
                       "batch walk pairs (shared)");
@@ -1143,7 +1148,7 @@ int batch_enqueue(Graph& tuner, const Graph& view, const BatchPlan& p, void* ws,
         ESIM_CUDA_TRY(launch_shared_columns(view, B, w.R, w.rbase, w.off, w.scount, w.nonmeet), "shared walk counts");
         ESIM_CUDA_TRY(launch_dhat_from_R(view, N, w.nonmeet, w.R, w.dhat), "batch dhat");
     } else {
-        ESIM_CUDA_TRY(launch_scan_R(view, N, w.R, w.off, w.part_R, w.part_norm, w.part_Rd), "batch scan");
+        ESIM_CUDA_TRY(launch_scan_R(view, N, w.R, w.off, w.part_R, w.part_Rd), "batch scan");
         if (timing) cudaEventRecord(view.ev[2], stream);
         ESIM_CUDA_TRY(launch_sample_segments(view, N, w.off, c, seed, w.nonmeet, nullptr), "batch walk pairs");
         if (timing) cudaEventRecord(view.ev[3], stream);
@@ -1288,10 +1293,8 @@ esim_status esim_load_graph(int64_t n, const int64_t* in_rowptr, const int32_t* 
         delete h;
         return st;
     }
-    const int64_t nb = allocate_blocks(n);
     bool ok = dev_alloc(&g.status, 1) == cudaSuccess && cudaMallocHost((void**)&g.status_host, sizeof(Status)) == cudaSuccess &&
-              alloc_sweep_scratch(g, &g.partial) && dev_alloc(&g.scan_part, (size_t)nb) == cudaSuccess &&
-              dev_alloc(&g.norm_part, 2 * (size_t)nb) == cudaSuccess &&
+              alloc_sweep_scratch(g, &g.partial) && alloc_scan_scratch(n, &g.scan_part, &g.norm_part) &&
               cudaMalloc(&g.topk_ws, topk_stage_offset(n) + (sizeof(double) + sizeof(int32_t)) * kTopkMax) == cudaSuccess &&
               cudaStreamCreateWithFlags(&g.own_stream, cudaStreamNonBlocking) == cudaSuccess &&
               cudaStreamCreateWithFlags(&g.side_stream, cudaStreamNonBlocking) == cudaSuccess &&
@@ -1303,9 +1306,9 @@ esim_status esim_load_graph(int64_t n, const int64_t* in_rowptr, const int32_t* 
         delete h;
         return fail(ESIM_ENOMEM, "device allocation for graph workspace");
     }
-    g.scan_blocks = nb;
     g.stream = g.own_stream;
     cudaError_t we = cudaMemsetAsync(g.status, 0, sizeof(Status), g.stream);
+    if (we == cudaSuccess) we = cudaMemsetAsync(g.topk_ws, 0, topk_stage_offset(n), g.stream);  // its tickets
     if (we == cudaSuccess) we = launch_walk_table(g);
     if (we == cudaSuccess) we = cudaStreamSynchronize(g.stream);
     if (we != cudaSuccess) {

@@ -48,11 +48,12 @@ __device__ __forceinline__ void prior_done() { asm volatile("griddepcontrol.wait
 __device__ __forceinline__ void next_may_start() { asm volatile("griddepcontrol.launch_dependents;"); }
 
 template <class... Params, class... Args>
-cudaError_t launch_after(cudaStream_t stream, unsigned blocks, unsigned threads, void (*kernel)(Params...),
+cudaError_t launch_after(cudaStream_t stream, dim3 blocks, unsigned threads, size_t smem, void (*kernel)(Params...),
                          Args&&... args) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(blocks);
+    cfg.gridDim = blocks;
     cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;

@@ -180,9 +180,8 @@ struct Graph {
     void* ws = nullptr;
     size_t ws_bytes = 0;
     void* partial = nullptr;      // the sweeps' piece sums and arrival counts (sweep_scratch_bytes)
-    unsigned long long* scan_part = nullptr;  // scan partials
-    double* norm_part = nullptr;
-    int64_t scan_blocks = 0;
+    unsigned long long* scan_part = nullptr;  // allocate_blocks(n) tile sums and a ticket
+    double* norm_part = nullptr;              // 2 allocate_blocks(n)
     void* topk_ws = nullptr;
     // timing events
     cudaEvent_t ev[8] = {};
@@ -254,9 +253,11 @@ cudaError_t launch_plan_scatter(const Graph& g, const PlanEntry* plan, int count
                                 uint8_t* cand);
 cudaError_t launch_dhat_segments(const Graph& g, int64_t nseg, const uint64_t* nonmeet, const uint64_t* off,
                                  double* dhat);
-// record = false: an auxiliary scan that leaves the status block (sum of R, budget) alone
+// record = false: an auxiliary scan that leaves the status block (sum of R, budget) alone.
+// part_R: allocate_blocks(N) + 1 entries, the last one (a ticket) zero before and after;
+// part_Rd: allocate_blocks(N)
 cudaError_t launch_scan_R(const Graph& g, int64_t N, const uint64_t* R, uint64_t* off, unsigned long long* part_R,
-                          double* part_norm, double* part_Rd, bool record = true);
+                          double* part_Rd, bool record = true);
 uint32_t walk_threshold(double c);
 
 // capi.cu: record a message for esim_last_error() and return `status` (as an esim_status int)

@@ -24,12 +24,18 @@
 
 namespace esim {
 
-constexpr int kAllocItems = 8;
-constexpr int64_t kAllocTile = (int64_t)kBlock * kAllocItems;
-constexpr int kScanThreads = 1024;
+// Nodes per thread of the allocation's and the scans' tiles: one where the nodes then fill the
+// chip anyway and a thread's chain of loads is what the kernel takes, eight from there on, so
+// that the tile sums stay few enough for one block to scan.
+constexpr int kScanItems = 8;
+constexpr int64_t kOneItemUpTo = 1 << 18;
+static int scan_items(int64_t n) { return n <= kOneItemUpTo ? 1 : kScanItems; }
 constexpr uint32_t kWalkMaxSteps = 65536;
 
-int64_t allocate_blocks(int64_t n) { return (n + kAllocTile - 1) / kAllocTile; }
+int64_t allocate_blocks(int64_t n) {
+    const int64_t tile = (int64_t)kBlock * scan_items(n);
+    return (n + tile - 1) / tile;
+}
 
 uint32_t walk_threshold(double c) {
     double v = floor(sqrt(c) * 4294967296.0);
@@ -68,36 +74,103 @@ __device__ __forceinline__ unsigned long long block_exclusive_scan(unsigned long
 }
 
 // pi(k) = sum over levels of hist, in level order: FP64 sums for an FP64 history,
-// two-float sums (rounded to FP64) for an FP32 history.
+// two-float sums (rounded to FP64) for an FP32 history.  kU levels are loaded at a time: they
+// are n apart, and one after another their latencies would add up to most of a small query.
+template <typename H, class Add>
+__device__ __forceinline__ void each_level(const H* __restrict__ hist, int64_t n, int64_t k, int32_t L, const Add& add) {
+    constexpr int kU = 8;
+    for (int32_t l0 = 0; l0 <= L; l0 += kU) {
+        H v[kU];
+#pragma unroll
+        for (int u = 0; u < kU; ++u)
+            if (l0 + u <= L) v[u] = hist[(size_t)(l0 + u) * (size_t)n + (size_t)k];
+#pragma unroll
+        for (int u = 0; u < kU; ++u)
+            if (l0 + u <= L) add(v[u]);
+    }
+}
+
 __device__ __forceinline__ double level_sum(const double* __restrict__ hist, int64_t n, int64_t k, int32_t L) {
     double p = 0.0;
-    for (int32_t l = 0; l <= L; ++l) p += hist[(size_t)l * (size_t)n + (size_t)k];
+    each_level(hist, n, k, L, [&](double v) { p += v; });
     return p;
 }
 
 __device__ __forceinline__ double level_sum(const float* __restrict__ hist, int64_t n, int64_t k, int32_t L) {
     f2 p = f2{0.f, 0.f};
-    for (int32_t l = 0; l <= L; ++l) p = f2_add_f(p, hist[(size_t)l * (size_t)n + (size_t)k]);
+    each_level(hist, n, k, L, [&](float v) { p = f2_add_f(p, v); });
     return f2_to_double(p);
 }
 
-// pi(k), R(k) per node; per-tile sums of R (exact and in double) and of pi^2.
-template <typename H>
+// The last block of a grid to get here: exclusive scan of the tile sums (in place), the total
+// into off[n] and the status block, the budget check.  The ticket wraps to zero.
+struct TileSums {
+    unsigned long long* R;   // gridDim.x, and the ticket behind them (zero before the launch)
+    double* Rd;              // gridDim.x: the same in double
+    double* norm;            // gridDim.x sums of pi^2, or NULL
+};
+
+__device__ __forceinline__ void finish_tiles(const TileSums& t, double budget, uint64_t* __restrict__ off_n,
+                                             Status* __restrict__ st) {
+    __shared__ bool last;
+    __shared__ unsigned long long su[32];
+    __shared__ double sd[32];
+    if (threadIdx.x == 0) {  // it wrote this block's sums
+        __threadfence();
+        last = atomicInc(reinterpret_cast<unsigned*>(t.R + gridDim.x), gridDim.x - 1) == gridDim.x - 1;
+        __threadfence();
+    }
+    __syncthreads();
+    if (!last) return;
+    const int64_t nblocks = gridDim.x;
+    const int64_t per = (nblocks + blockDim.x - 1) / blockDim.x;
+    const int64_t b0 = (int64_t)threadIdx.x * per;
+    const int64_t b1 = b0 + per < nblocks ? b0 + per : nblocks;
+    unsigned long long local = 0;
+    double nrm = 0.0, rd = 0.0;
+    for (int64_t b = b0; b < b1; ++b) {
+        local += __ldcg(t.R + b);
+        if (t.norm) nrm += __ldcg(t.norm + b);
+        rd += __ldcg(t.Rd + b);
+    }
+    unsigned long long total;
+    unsigned long long run = block_exclusive_scan(local, su, &total);
+    for (int64_t b = b0; b < b1; ++b) {
+        const unsigned long long v = __ldcg(t.R + b);
+        t.R[b] = run;
+        run += v;
+    }
+    nrm = block_sum(nrm, sd);
+    rd = block_sum(rd, sd);
+    if (threadIdx.x == 0) {
+        *off_n = total;
+        if (st) {  // NULL: an auxiliary scan that records nothing
+            st->sum_R = total;
+            if (t.norm) st->pi_norm2 = nrm;
+            if (rd > budget || rd >= 1.8e19) atomicOr(&st->err, kErrBudget);
+        }
+    }
+}
+
+// pi(k), R(k) per node; per-tile sums of R (exact and in double) and of pi^2, and their scan.
+// Bound by the history's bytes on large graphs (n = 1e6, L = 33, FP64: 272 MB), by the chain
+// of loads on small ones (n = 2000, L = 11: 29 us with eight nodes a thread and one load at a
+// time and the tile sums' scan in a launch of its own, 10 now with that scan in its last block).
+template <typename H, int kItems>
 __global__ void __launch_bounds__(kBlock) alloc_reduce_kernel(int64_t n, const H* __restrict__ hist, int32_t L,
                                                               double R_b, int mode, const uint32_t* __restrict__ exact_din,
                                                               double* __restrict__ pi_out,
-                                                              uint64_t* __restrict__ R_out,
-                                                              unsigned long long* __restrict__ part_R,
-                                                              double* __restrict__ part_norm,
-                                                              double* __restrict__ part_Rd, Status* __restrict__ st) {
+                                                              uint64_t* __restrict__ R_out, const TileSums tiles,
+                                                              double budget, uint64_t* __restrict__ off_n,
+                                                              Status* __restrict__ st) {
     __shared__ unsigned long long red_u[kBlock / 32];
     __shared__ double red_d[kBlock / 32];
-    const int64_t base = (int64_t)blockIdx.x * kAllocTile;
+    const int64_t base = (int64_t)blockIdx.x * kBlock * kItems;
     unsigned long long sum_r = 0;
     double norm = 0.0, sum_rd = 0.0;
     bool overflow = false;
 #pragma unroll 1
-    for (int i = 0; i < kAllocItems; ++i) {
+    for (int i = 0; i < kItems; ++i) {
         const int64_t k = base + (int64_t)i * kBlock + threadIdx.x;
         if (k >= n) break;
         const double p = level_sum(hist, n, k, L);
@@ -122,60 +195,25 @@ __global__ void __launch_bounds__(kBlock) alloc_reduce_kernel(int64_t n, const H
     norm = block_sum(norm, red_d);
     sum_rd = block_sum(sum_rd, red_d);
     if (threadIdx.x == 0) {
-        part_R[blockIdx.x] = sum_r;
-        part_norm[blockIdx.x] = norm;
-        part_Rd[blockIdx.x] = sum_rd;
+        tiles.R[blockIdx.x] = sum_r;
+        tiles.norm[blockIdx.x] = norm;
+        tiles.Rd[blockIdx.x] = sum_rd;
     }
-}
-
-// One block: exclusive scan of the tile sums (in place), totals into the status
-// block and off[n]; the budget check.
-__global__ void __launch_bounds__(kScanThreads) alloc_partials_kernel(int64_t nblocks, unsigned long long* part_R,
-                                                                      const double* __restrict__ part_norm,
-                                                                      const double* __restrict__ part_Rd,
-                                                                      double budget, uint64_t* __restrict__ off_n,
-                                                                      Status* __restrict__ st) {
-    __shared__ unsigned long long su[32];
-    __shared__ double sd[32];
-    const int64_t per = (nblocks + kScanThreads - 1) / kScanThreads;
-    const int64_t b0 = (int64_t)threadIdx.x * per;
-    const int64_t b1 = b0 + per < nblocks ? b0 + per : nblocks;
-    unsigned long long local = 0;
-    double nrm = 0.0, rd = 0.0;
-    for (int64_t b = b0; b < b1; ++b) {
-        local += part_R[b];
-        if (part_norm) nrm += part_norm[b];
-        rd += part_Rd[b];
-    }
-    unsigned long long total;
-    unsigned long long run = block_exclusive_scan(local, su, &total);
-    for (int64_t b = b0; b < b1; ++b) {
-        const unsigned long long v = part_R[b];
-        part_R[b] = run;
-        run += v;
-    }
-    nrm = block_sum(nrm, sd);
-    rd = block_sum(rd, sd);
-    if (threadIdx.x == 0) {
-        *off_n = total;
-        if (st) {  // NULL: an auxiliary scan that records nothing
-            st->sum_R = total;
-            if (part_norm) st->pi_norm2 = nrm;
-            if (rd > budget || rd >= 1.8e19) atomicOr(&st->err, kErrBudget);
-        }
-    }
+    finish_tiles(tiles, budget, off_n, st);
 }
 
 // off[k] = tile offset + exclusive prefix of R within the tile.
+template <int kItems>
 __global__ void __launch_bounds__(kBlock) alloc_scan_kernel(int64_t n, const uint64_t* __restrict__ R,
                                                             const unsigned long long* __restrict__ tile_off,
                                                             uint64_t* __restrict__ off) {
     __shared__ unsigned long long su[32];
-    const int64_t base = (int64_t)blockIdx.x * kAllocTile + (int64_t)threadIdx.x * kAllocItems;
-    unsigned long long v[kAllocItems];
+    const int64_t base = ((int64_t)blockIdx.x * kBlock + threadIdx.x) * kItems;
+    prior_done();
+    unsigned long long v[kItems];
     unsigned long long local = 0;
 #pragma unroll
-    for (int i = 0; i < kAllocItems; ++i) {
+    for (int i = 0; i < kItems; ++i) {
         const int64_t k = base + i;
         v[i] = k < n ? R[k] : 0ull;
         local += v[i];
@@ -183,31 +221,32 @@ __global__ void __launch_bounds__(kBlock) alloc_scan_kernel(int64_t n, const uin
     unsigned long long total;
     unsigned long long run = tile_off[blockIdx.x] + block_exclusive_scan(local, su, &total);
 #pragma unroll
-    for (int i = 0; i < kAllocItems; ++i) {
+    for (int i = 0; i < kItems; ++i) {
         const int64_t k = base + i;
         if (k < n) off[k] = run;
         run += v[i];
     }
 }
 
+static cudaError_t scan_offsets(const Graph& g, int64_t N, const uint64_t* R, const unsigned long long* tile_off,
+                                uint64_t* off) {
+    const unsigned nb = (unsigned)allocate_blocks(N);
+    return scan_items(N) == 1
+               ? launch_after(g.stream, dim3(nb), kBlock, 0, alloc_scan_kernel<1>, N, R, tile_off, off)
+               : launch_after(g.stream, dim3(nb), kBlock, 0, alloc_scan_kernel<kScanItems>, N, R, tile_off, off);
+}
+
 template <typename H>
 cudaError_t launch_allocate_t(const Graph& g, const H* hist, int32_t L, double R_b, int mode, double* pi_out,
                               uint64_t* R_out, uint64_t* off) {
     const int64_t nb = allocate_blocks(g.n);
-    unsigned long long* part_R = g.scan_part;
-    double* part_norm = g.norm_part;
-    double* part_Rd = g.norm_part + nb;
-    alloc_reduce_kernel<H><<<(unsigned)nb, kBlock, 0, g.stream>>>(g.n, hist, L, R_b, mode,
-                                                                  g.alg3 ? g.in.rp : nullptr, pi_out, R_out, part_R,
-                                                                  part_norm, part_Rd, g.status);
-    cudaError_t e = cudaGetLastError();
+    const TileSums tiles{g.scan_part, g.norm_part + nb, g.norm_part};
+    auto* kernel = scan_items(g.n) == 1 ? alloc_reduce_kernel<H, 1> : alloc_reduce_kernel<H, kScanItems>;
+    kernel<<<(unsigned)nb, kBlock, 0, g.stream>>>(g.n, hist, L, R_b, mode, g.alg3 ? g.in.rp : nullptr, pi_out, R_out,
+                                                  tiles, g.pair_budget, off + g.n, g.status);
+    const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    alloc_partials_kernel<<<1, kScanThreads, 0, g.stream>>>(nb, part_R, part_norm, part_Rd, g.pair_budget,
-                                                            off + g.n, g.status);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    alloc_scan_kernel<<<(unsigned)nb, kBlock, 0, g.stream>>>(g.n, R_out, part_R, off);
-    return cudaGetLastError();
+    return scan_offsets(g, g.n, R_out, g.scan_part, off);
 }
 
 cudaError_t launch_allocate(const Graph& g, const double* hist, int32_t L, double R_b, int mode, double* pi_out,
@@ -605,6 +644,7 @@ __global__ void __launch_bounds__(kBlock, 6) sample_pairs_kernel(const __grid_co
 
 __global__ void dhat_kernel(int64_t n, const uint64_t* __restrict__ nonmeet, const uint64_t* __restrict__ off,
                             double* __restrict__ dhat) {
+    prior_done();
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
         const uint64_t R = off[k + 1] - off[k];
         dhat[k] = R ? (double)nonmeet[k] / (double)R : 0.0;
@@ -748,20 +788,20 @@ cudaError_t launch_dhat_segments(const Graph& g, int64_t nseg, const uint64_t* n
                                  double* dhat) {
     int64_t b = (nseg + kBlock - 1) / kBlock;
     if (b > (int64_t)g.sm_count * 8) b = (int64_t)g.sm_count * 8;
-    dhat_kernel<<<(unsigned)(b < 1 ? 1 : b), kBlock, 0, g.stream>>>(nseg, nonmeet, off, dhat);
-    return cudaGetLastError();
+    return launch_after(g.stream, dim3((unsigned)(b < 1 ? 1 : b)), kBlock, 0, dhat_kernel, nseg, nonmeet, off, dhat);
 }
 
-// Scan of a ready R array of N segments (batches): tile sums, tile offsets, off[].
+// Scan of a ready R array of N segments (batches): tile sums and their scan, then off[].
+template <int kItems>
 __global__ void __launch_bounds__(kBlock) tile_sums_kernel(int64_t N, const uint64_t* __restrict__ R,
-                                                           unsigned long long* __restrict__ part_R,
-                                                           double* __restrict__ part_Rd) {
+                                                           const TileSums tiles, double budget,
+                                                           uint64_t* __restrict__ off_n, Status* __restrict__ st) {
     __shared__ unsigned long long red_u[kBlock / 32];
     __shared__ double red_d[kBlock / 32];
-    const int64_t base = (int64_t)blockIdx.x * kAllocTile;
+    const int64_t base = (int64_t)blockIdx.x * kBlock * kItems;
     unsigned long long su = 0;
     double sd = 0.0;
-    for (int i = 0; i < kAllocItems; ++i) {
+    for (int i = 0; i < kItems; ++i) {
         const int64_t k = base + (int64_t)i * kBlock + threadIdx.x;
         if (k < N) {
             su += R[k];
@@ -771,24 +811,21 @@ __global__ void __launch_bounds__(kBlock) tile_sums_kernel(int64_t N, const uint
     su = block_sum(su, red_u);
     sd = block_sum(sd, red_d);
     if (threadIdx.x == 0) {
-        part_R[blockIdx.x] = su;
-        part_Rd[blockIdx.x] = sd;
+        tiles.R[blockIdx.x] = su;
+        tiles.Rd[blockIdx.x] = sd;
     }
+    finish_tiles(tiles, budget, off_n, st);
 }
 
 cudaError_t launch_scan_R(const Graph& g, int64_t N, const uint64_t* R, uint64_t* off, unsigned long long* part_R,
-                          double* part_norm, double* part_Rd, bool record) {
+                          double* part_Rd, bool record) {
     const int64_t nb = allocate_blocks(N);
-    (void)part_norm;  // the scan of a ready R leaves the recorded ||pi||^2 as it is
-    tile_sums_kernel<<<(unsigned)nb, kBlock, 0, g.stream>>>(N, R, part_R, part_Rd);
-    cudaError_t e = cudaGetLastError();
+    const TileSums tiles{part_R, part_Rd, nullptr};  // the scan of a ready R leaves the recorded ||pi||^2 as it is
+    auto* kernel = scan_items(N) == 1 ? tile_sums_kernel<1> : tile_sums_kernel<kScanItems>;
+    kernel<<<(unsigned)nb, kBlock, 0, g.stream>>>(N, R, tiles, g.pair_budget, off + N, record ? g.status : nullptr);
+    const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    alloc_partials_kernel<<<1, kScanThreads, 0, g.stream>>>(nb, part_R, nullptr, part_Rd, g.pair_budget, off + N,
-                                                            record ? g.status : nullptr);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    alloc_scan_kernel<<<(unsigned)nb, kBlock, 0, g.stream>>>(N, R, part_R, off);
-    return cudaGetLastError();
+    return scan_offsets(g, N, R, part_R, off);
 }
 
 }  // namespace esim

@@ -283,6 +283,7 @@ __global__ void forward_init_kernel(int64_t n, int64_t u, const uint32_t* __rest
 __global__ void forward_init_d_kernel(int64_t n, int64_t u, const uint32_t* __restrict__ pos, double a,
                                       float xhi, float xlo,
                                       double* __restrict__ pi0, float2* __restrict__ x0) {
+    prior_done();
     const int64_t pu = at_pos(pos, u);
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         pi0[i] = i == u ? a : 0.0;
@@ -295,6 +296,7 @@ __global__ void reverse_init_d_kernel(int64_t n, const uint32_t* __restrict__ po
                                       const double* __restrict__ dhat,
                                       const double* __restrict__ h, float2* __restrict__ s0,
                                       double* __restrict__ s_final) {
+    prior_done();
     const f2 a{a_hi, a_lo};
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const f2 s = diag_term(dhat[i], h[i], a);
@@ -305,6 +307,7 @@ __global__ void reverse_init_d_kernel(int64_t n, const uint32_t* __restrict__ po
 
 __global__ void forward_init32_kernel(int64_t n, int64_t u, const uint32_t* __restrict__ pos, float a, float xv,
                                       float* __restrict__ pi0, float* __restrict__ x0) {
+    prior_done();
     const int64_t pu = at_pos(pos, u);
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         pi0[i] = i == u ? a : 0.f;
@@ -317,6 +320,7 @@ __global__ void reverse_init2f_kernel(int64_t n, const uint32_t* __restrict__ po
                                       const double* __restrict__ dhat,
                                       const float* __restrict__ h, float2* __restrict__ w, float2* __restrict__ s0,
                                       double* __restrict__ s_final) {
+    prior_done();
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const f2 wv = f2_from_double(dhat[i] * inv_a);
         w[i] = make_float2(wv.hi, wv.lo);
@@ -407,6 +411,12 @@ int elementwise_blocks(const Graph& g, int64_t n) {
     return (int)(b < 1 ? 1 : b);
 }
 
+// A kernel over all nodes: kernel(n, args...)
+template <class... Params, class... Args>
+cudaError_t each_node(const Graph& g, void (*kernel)(int64_t, Params...), Args&&... args) {
+    return launch_after(g.stream, dim3((unsigned)elementwise_blocks(g, g.n)), kBlock, 0, kernel, g.n, args...);
+}
+
 template <class Pol, class Op>
 cudaError_t sweep_level(const Graph& g, const DevCsr& A, const typename Pol::V* x, const Op& op) {
     using Acc = typename Pol::A;
@@ -414,8 +424,8 @@ cudaError_t sweep_level(const Graph& g, const DevCsr& A, const typename Pol::V* 
     Acc* partial = reinterpret_cast<Acc*>(g.partial);
     unsigned* arrived = reinterpret_cast<unsigned*>(partial + scratch_pieces(g));
     const int64_t blocks = (A.sell.nslices * 32 + kBlock - 1) / kBlock;
-    return launch_after(g.stream, (unsigned)blocks, kBlock, sell_rows_kernel<Pol, Op>, A.sell, A.rp, x, op, partial,
-                        arrived);
+    return launch_after(g.stream, dim3((unsigned)blocks), kBlock, 0, sell_rows_kernel<Pol, Op>, A.sell, A.rp, x, op,
+                        partial, arrived);
 }
 
 f2 host_f2(double v) {
@@ -433,9 +443,7 @@ cudaError_t launch_forward(const Graph& g, int64_t u, double c, int32_t L, doubl
     const uint32_t din_u = (*g.din_host)[(size_t)u];
     const f2 x0 = din_u ? host_f2(a / (double)din_u) : f2{0.f, 0.f};
     float2* x[2] = {reinterpret_cast<float2*>(xa), reinterpret_cast<float2*>(xb)};
-    forward_init_d_kernel<<<elementwise_blocks(g, g.n), kBlock, 0, g.stream>>>(g.n, u, g.out.sell.pos, a, x0.hi, x0.lo,
-                                                                               hist, x[0]);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = each_node(g, forward_init_d_kernel, u, g.out.sell.pos, a, x0.hi, x0.lo, hist, x[0]);
     if (e != cudaSuccess) return e;
     const f2 sc2 = host_f2(sc);
     for (int32_t l = 1; l <= L; ++l) {
@@ -456,9 +464,8 @@ cudaError_t launch_reverse(const Graph& g, const double* hist, int32_t L, double
     float2* S = reinterpret_cast<float2*>(s_out);
     auto buf = [&](int32_t l) { return ((L - 1 - l) & 1) == 0 ? A : S; };
     const f2 a2 = host_f2(a);
-    reverse_init_d_kernel<<<elementwise_blocks(g, g.n), kBlock, 0, g.stream>>>(
-        g.n, g.in.sell.pos, a2.hi, a2.lo, dhat, hist + (size_t)L * g.n, L > 0 ? buf(0) : nullptr, L == 0 ? s_out : nullptr);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = each_node(g, reverse_init_d_kernel, g.in.sell.pos, a2.hi, a2.lo, dhat, hist + (size_t)L * g.n,
+                              L > 0 ? buf(0) : nullptr, L == 0 ? s_out : nullptr);
     if (e != cudaSuccess) return e;
     const f2 sc2 = host_f2(sc);
     for (int32_t l = 1; l <= L; ++l) {
@@ -533,9 +540,7 @@ cudaError_t launch_walk_distributions(const Graph& g, int64_t u, int steps, doub
     const uint32_t din_u = (*g.din_host)[(size_t)u];
     const f2 x0 = din_u ? host_f2(1.0 / (double)din_u) : f2{0.f, 0.f};
     float2* x[2] = {reinterpret_cast<float2*>(xa), reinterpret_cast<float2*>(xb)};
-    forward_init_d_kernel<<<elementwise_blocks(g, g.n), kBlock, 0, g.stream>>>(g.n, u, g.out.sell.pos, 1.0, x0.hi,
-                                                                               x0.lo, H, x[0]);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = each_node(g, forward_init_d_kernel, u, g.out.sell.pos, 1.0, x0.hi, x0.lo, H, x[0]);
     if (e != cudaSuccess) return e;
     const f2 one{1.f, 0.f};
     for (int l = 1; l <= steps; ++l) {
@@ -561,9 +566,7 @@ cudaError_t launch_forward32(const Graph& g, int64_t u, double c, int32_t L, flo
     const double sc = sqrt(c);
     const float a = (float)(1.0 - sc);
     const uint32_t din_u = (*g.din_host)[(size_t)u];
-    forward_init32_kernel<<<elementwise_blocks(g, g.n), kBlock, 0, g.stream>>>(
-        g.n, u, g.out.sell.pos, a, din_u ? a / (float)din_u : 0.f, hist, xa);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = each_node(g, forward_init32_kernel, u, g.out.sell.pos, a, din_u ? a / (float)din_u : 0.f, hist, xa);
     if (e != cudaSuccess) return e;
     float* x[2] = {xa, xb};
     const f2 sc2 = host_f2(sc);
@@ -580,9 +583,8 @@ cudaError_t launch_reverse32(const Graph& g, const float* hist, int32_t L, doubl
     const double sc = sqrt(c);
     const double a = 1.0 - sc;
     float2* buf[2] = {sa, sb};
-    reverse_init2f_kernel<<<elementwise_blocks(g, g.n), kBlock, 0, g.stream>>>(
-        g.n, g.in.sell.pos, 1.0 / a, dhat, hist + (size_t)L * g.n, w, buf[0], L == 0 ? s_out : nullptr);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = each_node(g, reverse_init2f_kernel, g.in.sell.pos, 1.0 / a, dhat, hist + (size_t)L * g.n, w,
+                              buf[0], L == 0 ? s_out : nullptr);
     if (e != cudaSuccess) return e;
     const f2 sc2 = host_f2(sc);
     for (int32_t l = 1; l <= L; ++l) {

@@ -37,7 +37,7 @@ struct TopkState {
     unsigned long long bound_hi;
     unsigned int bound_lo;
     unsigned int count;       // keys collected
-    unsigned int ticket[2];   // blocks of the two launches that have finished
+    unsigned int ticket[2];   // blocks of the two launches that have finished; each wraps to zero
     unsigned int pad[2];
 };
 
@@ -159,7 +159,7 @@ __device__ __forceinline__ bool last_block(unsigned* ticket) {
     __shared__ bool last;
     __threadfence();
     __syncthreads();
-    if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    if (threadIdx.x == 0) last = atomicInc(ticket, gridDim.x - 1) == gridDim.x - 1;
     __syncthreads();
     if (last) __threadfence();
     return last;
@@ -184,6 +184,7 @@ __global__ void __launch_bounds__(kTopkThreads) topk_bound_kernel(int64_t n, con
     unsigned long long hi = 0;
     unsigned lo = 0;  // 0: no element yet (~i is never 0)
     constexpr int kU = 4;  // loads in flight
+    prior_done();
     for (int64_t i0 = tid; i0 < n; i0 += stride * kU) {
         double v[kU];
 #pragma unroll
@@ -237,6 +238,7 @@ __global__ void __launch_bounds__(kTopkThreads) topk_bound_kernel(int64_t n, con
     if (threadIdx.x == 0) {
         st->bound_hi = pre.hi;
         st->bound_lo = pre.lo;
+        st->count = 0u;
     }
 }
 
@@ -259,6 +261,7 @@ __global__ void __launch_bounds__(kTopkThreads) topk_pick_kernel(int64_t n, cons
     cand += (size_t)blockIdx.y * kCandMax;
     ids_out += (size_t)blockIdx.y * k;
     vals_out += (size_t)blockIdx.y * k;
+    prior_done();
     if (excl) exclude = excl[blockIdx.y];
     const unsigned long long bh = st->bound_hi;
     const unsigned bl = st->bound_lo;
@@ -361,9 +364,11 @@ constexpr size_t kStateBytes(size_t B) { return (sizeof(TopkState) * B + 255) / 
 constexpr size_t kColumnBytes = (size_t)kMaxSlices * 12 + sizeof(Cand) * (size_t)kCandMax;
 
 // B selections; column q of scores starts at scores + q * stride, and excl[q] (or exclude
-// where excl is NULL, -1 for none) is left out of it.
+// where excl is NULL, -1 for none) is left out of it.  The tickets in ws are zero before and
+// after; clear: they may not be (a workspace used before, or by calls that raced).
 cudaError_t topk_select(cudaStream_t stream, int sms, int64_t n, int32_t B, const double* scores, int64_t col_stride,
-                        int64_t exclude, const int64_t* excl, int32_t k, int32_t* ids_out, double* vals_out, void* ws) {
+                        int64_t exclude, const int64_t* excl, int32_t k, int32_t* ids_out, double* vals_out, void* ws,
+                        bool clear) {
     TopkState* st = (TopkState*)ws;
     unsigned long long* max_hi = (unsigned long long*)((char*)ws + kStateBytes((size_t)B));
     unsigned* max_lo = (unsigned*)(max_hi + (size_t)B * kMaxSlices);
@@ -384,19 +389,18 @@ cudaError_t topk_select(cudaStream_t stream, int sms, int64_t n, int32_t B, cons
     int P = 1;
     while (P < (int)cap) P <<= 1;
     const size_t smem = (size_t)P * 12;
-    cudaError_t e = cudaMemsetAsync(st, 0, sizeof(TopkState) * (size_t)B, stream);
-    if (e != cudaSuccess) return e;
+    cudaError_t e = cudaSuccess;
+    if (clear && (e = cudaMemsetAsync(st, 0, sizeof(TopkState) * (size_t)B, stream)) != cudaSuccess) return e;
     if (smem > 48 * 1024 - 2048 &&
         (e = cudaFuncSetAttribute(topk_pick_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
             cudaSuccess)
         return e;
     const dim3 grid((unsigned)blocks, (unsigned)B);
-    topk_bound_kernel<<<grid, kTopkThreads, 0, stream>>>(n, scores, exclude, st, max_hi, max_lo, G, (unsigned)k,
-                                                         col_stride, excl);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    topk_pick_kernel<<<grid, kTopkThreads, smem, stream>>>(n, scores, exclude, st, cand, cap, k, P, col_stride, excl,
-                                                           ids_out, vals_out);
-    return cudaGetLastError();
+    e = launch_after(stream, grid, kTopkThreads, 0, topk_bound_kernel, n, scores, exclude, st, max_hi, max_lo, G,
+                     (unsigned)k, col_stride, excl);
+    if (e != cudaSuccess) return e;
+    return launch_after(stream, grid, kTopkThreads, smem, topk_pick_kernel, n, scores, exclude, st, cand, cap, k, P,
+                        col_stride, excl, ids_out, vals_out);
 }
 
 }  // namespace
@@ -407,12 +411,12 @@ size_t topk_workspace_bytes(int64_t /*n*/) { return topk_batch_workspace_bytes(1
 
 cudaError_t launch_topk(const Graph& g, const double* scores, int64_t exclude, int32_t k, int32_t* ids_out,
                         double* vals_out, void* ws) {
-    return topk_select(g.stream, g.sm_count, g.n, 1, scores, 0, exclude, nullptr, k, ids_out, vals_out, ws);
+    return topk_select(g.stream, g.sm_count, g.n, 1, scores, 0, exclude, nullptr, k, ids_out, vals_out, ws, false);
 }
 
 cudaError_t launch_topk_batch(const Graph& g, int32_t B, const double* scores, const int64_t* exclude, int32_t k,
                               int32_t* ids_out, double* vals_out, void* ws) {
-    return topk_select(g.stream, g.sm_count, g.n, B, scores, g.n, -1, exclude, k, ids_out, vals_out, ws);
+    return topk_select(g.stream, g.sm_count, g.n, B, scores, g.n, -1, exclude, k, ids_out, vals_out, ws, true);
 }
 
 }  // namespace esim
@@ -436,8 +440,7 @@ cudaError_t launch_topk_batch(const Graph& g, int32_t B, const double* scores, c
 // the kernels.  The address is remembered together with the unique id of the CUDA
 // context it was taken in: after a device reset the device has a new context (and
 // the array a new address), so the next call takes the address again.  All calls
-// share the array and it keeps the last call's contents; the state is cleared every
-// call.  Calls whose work overlaps on the GPU (different streams,
+// share the array and it keeps the last call's contents; the state is cleared every call.  Calls whose work overlaps on the GPU (different streams,
 // or several host threads) race on the array.
 // ---------------------------------------------------------------------------
 
@@ -534,7 +537,7 @@ extern "C" __attribute__((visibility("default"))) esim_status esim_select_topk_s
     e = static_scratch(dev, &ws, &sms);
     if (e != cudaSuccess)
         return static_fail(ESIM_ECUDA, std::string("static scratch set-up: ") + cudaGetErrorString(e));
-    e = topk_select((cudaStream_t)stream, sms, n, 1, scores, 0, exclude, nullptr, k, ids_out, vals_out, ws);
+    e = topk_select((cudaStream_t)stream, sms, n, 1, scores, 0, exclude, nullptr, k, ids_out, vals_out, ws, true);
     if (e != cudaSuccess) return static_fail(ESIM_ECUDA, std::string("static top-k launch: ") + cudaGetErrorString(e));
     return ESIM_OK;
 }
