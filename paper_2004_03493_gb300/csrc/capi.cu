@@ -51,15 +51,7 @@ cudaError_t dev_alloc(T** p, size_t count) {
 void free_csr(DevCsr& c) {
     cudaFree(c.rp);
     cudaFree(c.col);
-    cudaFree(c.info);
-    cudaFree(c.walk);
-    cudaFree(c.seg);
-    cudaFree(c.long_rows);
-    cudaFree(c.long_first);
-    free_sell(c.sell);
-    cudaFree(c.bseg);
-    cudaFree(c.blong_rows);
-    cudaFree(c.blong_first);
+    cudaFree(c.tables);
     c = DevCsr{};
 }
 
@@ -67,7 +59,7 @@ constexpr uint32_t kSegLen = 4096;
 constexpr int64_t kLongRowsFrom = 4000000;  // from this many edges on a level is no longer one row's latency
 
 // Upload a host CSR and build its row-split table.
-esim_status upload_csr(int64_t n, const std::vector<uint32_t>& rp, const std::vector<int32_t>& col, DevCsr& d,
+esim_status upload_csr(int64_t n, const std::vector<uint32_t>& rp, const int32_t* col, DevCsr& d,
                        bool with_info, const std::vector<uint32_t>& uses_rp, cudaStream_t stream) {
     const int64_t m = (int64_t)rp[n];
     const double avg = (double)m / (double)n;
@@ -96,38 +88,58 @@ esim_status upload_csr(int64_t n, const std::vector<uint32_t>& rp, const std::ve
     d.nlong = (int64_t)long_rows.size();
     d.bnseg = (int64_t)bseg.size();
     d.bnlong = (int64_t)blong_rows.size();
-    auto up = [](auto** dst, const auto& v) {  // an empty vector still gets an allocation
-        return dev_alloc(dst, v.size()) != cudaSuccess ? ESIM_ENOMEM
-               : !v.empty() && cudaMemcpy(*dst, v.data(), sizeof(v[0]) * v.size(), cudaMemcpyHostToDevice) != cudaSuccess
-                   ? ESIM_ECUDA
-                   : ESIM_OK;
+    std::vector<uint32_t> off, pos;
+    plan_sell(n, rp, pieces, uses_rp, d.sell, off, pos);
+    // One allocation and one copy for the tables, and the space the device fills behind them:
+    // a load makes few calls of a size-independent cost.
+    size_t bytes = 0;
+    auto place = [&bytes](size_t b) {
+        const size_t at = bytes;
+        bytes += (b + 255) / 256 * 256;
+        return at;
     };
-    esim_status st = up(&d.rp, rp);
-    if (st == ESIM_OK) st = up(&d.col, col);
-    if (st == ESIM_OK) st = up(&d.seg, seg);
-    if (st == ESIM_OK) st = up(&d.long_rows, long_rows);
-    if (st == ESIM_OK) st = up(&d.long_first, long_first);
-    if (st == ESIM_OK) st = up(&d.bseg, bseg);
-    if (st == ESIM_OK) st = up(&d.blong_rows, blong_rows);
-    if (st == ESIM_OK) st = up(&d.blong_first, blong_first);
-    if (st != ESIM_OK) {
+    std::vector<char> stage;
+    auto put = [&](const auto& v) {
+        const size_t b = v.size() * sizeof(v[0]), at = place(b);
+        stage.resize(bytes);
+        if (b) memcpy(stage.data() + at, v.data(), b);
+        return at;
+    };
+    const size_t o_seg = put(seg), o_lr = put(long_rows), o_lf = put(long_first), o_bseg = put(bseg),
+                 o_br = put(blong_rows), o_bf = put(blong_first), o_off = put(off), o_piece = put(pieces), o_pos = put(pos);
+    const size_t entries = with_info ? (size_t)std::max(m, n) : 0;
+    const size_t o_rows = place(sizeof(int2) * 32 * (size_t)d.sell.nslices),
+                 o_col = place(sizeof(int32_t) * 32 * (size_t)off.back()),
+                 o_info = place(with_info ? sizeof(uint2) * (size_t)n : 0), o_walk = place(sizeof(uint2) * entries);
+    if (dev_alloc(&d.rp, (size_t)n + 1) != cudaSuccess || dev_alloc(&d.col, (size_t)m) != cudaSuccess ||
+        dev_alloc(&d.tables, bytes) != cudaSuccess) {
         cudaGetLastError();
-        return fail(st, st == ESIM_ENOMEM ? "cudaMalloc(graph tables)" : "upload of the graph tables");
+        return fail(ESIM_ENOMEM, "cudaMalloc(graph tables)");
     }
-    const cudaError_t se = build_sell(n, d, pieces, uses_rp, stream, d.sell);
-    if (se != cudaSuccess) {
-        cudaGetLastError();
-        return fail(se == cudaErrorMemoryAllocation ? ESIM_ENOMEM : ESIM_ECUDA,
-                    std::string("sliced rows: ") + cudaGetErrorString(se));
+    d.seg = (Segment*)(d.tables + o_seg);
+    d.long_rows = (int32_t*)(d.tables + o_lr);
+    d.long_first = (int32_t*)(d.tables + o_lf);
+    d.bseg = (Segment*)(d.tables + o_bseg);
+    d.blong_rows = (int32_t*)(d.tables + o_br);
+    d.blong_first = (int32_t*)(d.tables + o_bf);
+    d.sell.off = (uint32_t*)(d.tables + o_off);
+    d.sell.piece = (Segment*)(d.tables + o_piece);
+    d.sell.pos = pos.empty() ? nullptr : (uint32_t*)(d.tables + o_pos);
+    d.sell.rows = (int2*)(d.tables + o_rows);
+    d.sell.col = (int32_t*)(d.tables + o_col);
+    if (with_info) {  // filled on the device (launch_walk_table); the tail past m is never a position
+        d.info = (uint2*)(d.tables + o_info);
+        d.walk = (uint2*)(d.tables + o_walk);
     }
-    if (with_info) {
-        // filled on the device (launch_walk_table); the tail past m is never used as a position
-        const size_t entries = (size_t)std::max(m, n);
-        if (dev_alloc(&d.info, (size_t)n) != cudaSuccess) return fail(ESIM_ENOMEM, "cudaMalloc(row info)");
-        if (dev_alloc(&d.walk, entries) != cudaSuccess) return fail(ESIM_ENOMEM, "cudaMalloc(walk table)");
-        if ((int64_t)entries > m)
-            ESIM_CUDA_TRY(cudaMemset(d.walk + m, 0, sizeof(uint2) * (entries - (size_t)m)), "clear walk table tail");
-    }
+    ESIM_CUDA_TRY(cudaMemcpyAsync(d.rp, rp.data(), sizeof(uint32_t) * ((size_t)n + 1), cudaMemcpyHostToDevice, stream),
+                  "upload rowptr");
+    if (m)
+        ESIM_CUDA_TRY(cudaMemcpyAsync(d.col, col, sizeof(int32_t) * (size_t)m, cudaMemcpyHostToDevice, stream),
+                      "upload col");
+    ESIM_CUDA_TRY(cudaMemcpyAsync(d.tables, stage.data(), stage.size(), cudaMemcpyHostToDevice, stream),
+                  "upload graph tables");
+    ESIM_CUDA_TRY(fill_sell(n, d, stream), "sliced rows");
+    ESIM_CUDA_TRY(cudaStreamSynchronize(stream), "graph tables");  // the host vectors are this call's
     return ESIM_OK;
 }
 
@@ -1241,7 +1253,7 @@ esim_status esim_load_graph(int64_t n, const int64_t* in_rowptr, const int32_t* 
     // out-CSR list targets j in increasing order)
     std::vector<uint32_t> in_rp((size_t)n + 1), out_rp((size_t)n + 1, 0);
     for (int64_t j = 0; j <= n; ++j) in_rp[j] = (uint32_t)in_rowptr[j];
-    std::vector<int32_t> in_c(in_col, in_col + m), out_c((size_t)m);
+    std::vector<int32_t> out_c((size_t)m);
     for (int64_t p = 0; p < m; ++p) out_rp[(size_t)in_col[p] + 1]++;
     for (int64_t i = 0; i < n; ++i) out_rp[i + 1] += out_rp[i];
     {
@@ -1251,17 +1263,17 @@ esim_status esim_load_graph(int64_t n, const int64_t* in_rowptr, const int32_t* 
     }
     {
         // repeated in-edges (Algorithm 3 needs a simple graph) and the host in-degrees
-        std::vector<int64_t> mark((size_t)n, -1);
+        std::vector<int32_t> mark((size_t)n, -1);
         auto din = std::make_shared<std::vector<uint32_t>>((size_t)n);
         for (int64_t j = 0; j < n && !g.has_duplicates; ++j)
             for (int64_t p = in_rowptr[j]; p < in_rowptr[j + 1]; ++p) {
-                if (mark[in_col[p]] == j) {
+                if (mark[in_col[p]] == (int32_t)j) {
                     g.has_duplicates = true;
                     break;
                 }
-                mark[in_col[p]] = j;
+                mark[in_col[p]] = (int32_t)j;
             }
-        for (int64_t j = 0; j < n; ++j) (*din)[j] = (uint32_t)(in_rowptr[j + 1] - in_rowptr[j]);
+        for (int64_t j = 0; j < n; ++j) (*din)[j] = in_rp[j + 1] - in_rp[j];
         g.din_host = din;
     }
     {
@@ -1286,8 +1298,8 @@ esim_status esim_load_graph(int64_t n, const int64_t* in_rowptr, const int32_t* 
             return fail(ESIM_ENOMEM, "device allocation for 1/din");
         }
     }
-    esim_status st = upload_csr(n, in_rp, in_c, g.in, true, out_rp, cudaStreamPerThread);
-    if (st == ESIM_OK) st = upload_csr(n, out_rp, out_c, g.out, false, in_rp, cudaStreamPerThread);
+    esim_status st = upload_csr(n, in_rp, in_col, g.in, true, out_rp, cudaStreamPerThread);
+    if (st == ESIM_OK) st = upload_csr(n, out_rp, out_c.data(), g.out, false, in_rp, cudaStreamPerThread);
     if (st != ESIM_OK) {
         release(g);
         delete h;

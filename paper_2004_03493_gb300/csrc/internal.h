@@ -73,7 +73,6 @@ struct SellRows {
     int64_t npieces = 0;
     uint32_t row_cap = 64;
     uint32_t* pos = nullptr;    // n, or NULL
-    uint32_t hubs = 0;
 };
 
 __host__ __device__ inline int64_t at_pos(const uint32_t* pos, int64_t i) { return pos ? (int64_t)pos[i] : i; }
@@ -100,6 +99,7 @@ struct DevCsr {
     int32_t* blong_first = nullptr;
     int64_t bnseg = 0;
     int64_t bnlong = 0;
+    char* tables = nullptr;  // one allocation: every table above but rp and col
 };
 
 constexpr uint32_t kBatchSeg = 64;          // entries a lane group of the batched sweeps adds one after another, at most
@@ -196,9 +196,12 @@ struct Graph {
 };
 
 // sell.cu
-cudaError_t build_sell(int64_t n, const DevCsr& csr, const std::vector<Segment>& pieces,
-                       const std::vector<uint32_t>& uses_rp, cudaStream_t stream, SellRows& out);
-void free_sell(SellRows& s);
+// Slices of a CSR whose row_cap is set: counts, offsets (nslices + 1) and positions (n, or empty).
+void plan_sell(int64_t n, const std::vector<uint32_t>& rp, const std::vector<Segment>& pieces,
+               const std::vector<uint32_t>& uses_rp, SellRows& out, std::vector<uint32_t>& off,
+               std::vector<uint32_t>& pos);
+// Fills csr.sell.rows and .col from the uploaded CSR, offsets, pieces and positions.
+cudaError_t fill_sell(int64_t n, const DevCsr& csr, cudaStream_t stream);
 
 // sweep.cu
 // Bytes of the scratch that sweeps on one stream share: 8 bytes per piece, then a count per

@@ -1,5 +1,5 @@
 // The sliced layout of a CSR that the single-vector sweeps read (internal.h, SellRows):
-// built on the device when a graph is loaded.
+// planned on the host and filled on the device when a graph is loaded.
 //
 // Rows are sorted by length, longest first, within windows of kSellWindow consecutive
 // rows, so the 32 rows of a slice have nearly the same length and stay close together in
@@ -25,10 +25,9 @@ namespace {
 constexpr uint32_t kSellHubs = 8192;
 
 // One window per block: sorts its rows by (length descending, row ascending) and writes
-// their (row, length) and, per slice, its longest row.  Cut rows get no place.
+// their (row, length).  Cut rows get no place.
 __global__ void __launch_bounds__(kSellWindow) sell_sort_kernel(int64_t n, const uint32_t* __restrict__ rp,
-                                                               uint32_t row_cap, int2* __restrict__ rows,
-                                                               uint32_t* __restrict__ steps) {
+                                                               uint32_t row_cap, int2* __restrict__ rows) {
     __shared__ uint32_t key[kSellWindow];
     const int t = threadIdx.x;
     const int64_t base = (int64_t)blockIdx.x * kSellWindow;
@@ -52,21 +51,17 @@ __global__ void __launch_bounds__(kSellWindow) sell_sort_kernel(int64_t n, const
             __syncthreads();
         }
     const uint32_t k = key[t];
-    const int64_t at = base + t;
-    rows[at] = k ? make_int2((int)(base + kSellWindow - 1 - (int64_t)(k & (kSellWindow - 1))), (int)(k >> 10) - 1)
+    rows[base + t] = k ? make_int2((int)(base + kSellWindow - 1 - (int64_t)(k & (kSellWindow - 1))), (int)(k >> 10) - 1)
                  : make_int2(-1, 0);
-    if ((t & 31) == 0) steps[at >> 5] = k ? (k >> 10) - 1 : 0u;
 }
 
 // One slice per piece of a long row.
-__global__ void sell_pieces_kernel(int64_t npieces, const Segment* __restrict__ piece, int2* __restrict__ rows,
-                                   uint32_t* __restrict__ steps) {
+__global__ void sell_pieces_kernel(int64_t npieces, const Segment* __restrict__ piece, int2* __restrict__ rows) {
     const uint32_t lane = threadIdx.x & 31;
     for (int64_t s = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; s < npieces;
          s += ((int64_t)gridDim.x * blockDim.x) >> 5) {
         const uint32_t len = piece[s].end - piece[s].beg;
         rows[s * 32 + lane] = make_int2(piece[s].row, (int)(len > lane ? (len - lane + 31) / 32 : 0u));
-        if (lane == 0) steps[s] = (len + 31) / 32;
     }
 }
 
@@ -90,88 +85,77 @@ __global__ void __launch_bounds__(kBlock) sell_fill_kernel(int64_t nslices, int6
     }
 }
 
-}  // namespace
-
 // Positions of the gathered vector: the at most kSellHubs nodes with the most uses (node i has
 // uses_rp[i+1] - uses_rp[i] of them, the row lengths of the transpose) first.  Empty where
 // that would gain nothing: every node is one, or they have no more than twice their share.
-std::vector<uint32_t> hub_positions(int64_t n, const std::vector<uint32_t>& uses_rp, uint32_t* hubs) {
-    *hubs = 0;
+std::vector<uint32_t> hub_positions(int64_t n, const std::vector<uint32_t>& uses_rp) {
     if (n <= (int64_t)kSellHubs) return {};
     constexpr uint32_t kTop = 1u << 16;  // uses above this are alike
-    std::vector<uint32_t> count(kTop + 1, 0);
     auto uses = [&](int64_t i) { return std::min(uses_rp[(size_t)i + 1] - uses_rp[(size_t)i], kTop); };
+    uint32_t most = 0;
+    for (int64_t i = 0; i < n; ++i) most = std::max(most, uses(i));
+    std::vector<uint32_t> count((size_t)most + 1, 0);
     for (int64_t i = 0; i < n; ++i) ++count[uses(i)];
-    uint32_t least = kTop + 1, h = 0;  // hubs: the nodes with at least this many uses
-    while (least > 1 && h + count[least - 1] <= kSellHubs) h += count[--least];
+    uint32_t least = most + 1, h = 0;  // hubs: the nodes with at least this many uses
     uint64_t share = 0;
-    for (int64_t i = 0; i < n; ++i)
-        if (uses(i) >= least) share += uses_rp[(size_t)i + 1] - uses_rp[(size_t)i];
+    while (least > 1 && h + count[least - 1] <= kSellHubs) {
+        h += count[--least];
+        share += (uint64_t)count[least] * least;
+    }
     if (h == 0 || (double)share * (double)n < 2.0 * (double)h * (double)uses_rp[(size_t)n]) return {};
     std::vector<uint32_t> pos((size_t)n);
     uint32_t hub = 0, other = h;
     for (int64_t i = 0; i < n; ++i) pos[(size_t)i] = uses(i) >= least ? hub++ : other++;
-    *hubs = h;
     return pos;
 }
 
-cudaError_t build_sell(int64_t n, const DevCsr& csr, const std::vector<Segment>& pieces,
-                       const std::vector<uint32_t>& uses_rp, cudaStream_t stream, SellRows& out) {
-    cudaError_t e = cudaSuccess;
-    const std::vector<uint32_t> pos = hub_positions(n, uses_rp, &out.hubs);
-    if (!pos.empty() && ((e = cudaMalloc((void**)&out.pos, sizeof(uint32_t) * pos.size())) != cudaSuccess ||
-                         (e = cudaMemcpyAsync(out.pos, pos.data(), sizeof(uint32_t) * pos.size(),
-                                              cudaMemcpyHostToDevice, stream)) != cudaSuccess))
-        return e;
+}  // namespace
+
+void plan_sell(int64_t n, const std::vector<uint32_t>& rp, const std::vector<Segment>& pieces,
+               const std::vector<uint32_t>& uses_rp, SellRows& out, std::vector<uint32_t>& off,
+               std::vector<uint32_t>& pos) {
+    pos = hub_positions(n, uses_rp);
     out.npieces = (int64_t)pieces.size();
     const int64_t windows = (n + kSellWindow - 1) / kSellWindow;
     out.nslices = out.npieces + windows * (kSellWindow / 32);
-    std::vector<uint32_t> steps((size_t)out.nslices + 1);
-    if ((e = cudaMalloc((void**)&out.off, sizeof(uint32_t) * ((size_t)out.nslices + 1))) != cudaSuccess ||
-        (e = cudaMalloc((void**)&out.rows, sizeof(int2) * (size_t)out.nslices * 32)) != cudaSuccess ||
-        (e = cudaMalloc((void**)&out.piece, sizeof(Segment) * (size_t)(out.npieces ? out.npieces : 1))) != cudaSuccess)
-        return e;
-    if (out.npieces) {
-        if ((e = cudaMemcpyAsync(out.piece, pieces.data(), sizeof(Segment) * pieces.size(), cudaMemcpyHostToDevice,
-                                 stream)) != cudaSuccess)
-            return e;
-        sell_pieces_kernel<<<(unsigned)((out.npieces * 32 + kBlock - 1) / kBlock), kBlock, 0, stream>>>(
-            out.npieces, out.piece, out.rows, out.off);
-    }
-    sell_sort_kernel<<<(unsigned)windows, kSellWindow, 0, stream>>>(
-        n, csr.rp, out.row_cap, out.rows + out.npieces * 32, out.off + out.npieces);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    // offsets in steps of 32 entries: the prefix sum of the slices' lengths, on the host
-    if ((e = cudaMemcpyAsync(steps.data(), out.off, sizeof(uint32_t) * (size_t)out.nslices, cudaMemcpyDeviceToHost,
-                             stream)) != cudaSuccess ||
-        (e = cudaStreamSynchronize(stream)) != cudaSuccess)
-        return e;
+    off.clear();
+    off.reserve((size_t)out.nslices + 1);
     uint64_t total = 0;  // below 2^32: a step holds at least one entry, and m < 2^32
-    for (int64_t s = 0; s < out.nslices; ++s) {
-        const uint32_t len = steps[(size_t)s];
-        steps[(size_t)s] = (uint32_t)total;
-        total += len;
+    auto slice = [&](uint32_t steps) {
+        off.push_back((uint32_t)total);
+        total += steps;
+    };
+    for (const Segment& p : pieces) slice((p.end - p.beg + 31) / 32);
+    std::vector<uint32_t> count((size_t)out.row_cap + 1);
+    for (int64_t w = 0; w < windows; ++w) {  // a slice's steps: the longest of its 32 rows, the first in sorted order
+        std::fill(count.begin(), count.end(), 0u);
+        const int64_t end = std::min(n, (w + 1) * kSellWindow);
+        for (int64_t r = w * kSellWindow; r < end; ++r) {
+            const uint32_t len = rp[(size_t)r + 1] - rp[(size_t)r];
+            if (len <= out.row_cap) ++count[len];
+        }
+        uint32_t rows = 0, next = 0;
+        for (int64_t len = out.row_cap; len >= 0; --len) {
+            rows += count[(size_t)len];
+            for (; next < rows; next += 32) slice((uint32_t)len);
+        }
+        for (; next < (uint32_t)kSellWindow; next += 32) slice(0);
     }
-    steps[(size_t)out.nslices] = (uint32_t)total;
-    if ((e = cudaMemcpyAsync(out.off, steps.data(), sizeof(uint32_t) * steps.size(), cudaMemcpyHostToDevice, stream)) !=
-        cudaSuccess)
-        return e;
-    if ((e = cudaMalloc((void**)&out.col, sizeof(int32_t) * 32 * (size_t)(total ? total : 1))) != cudaSuccess) return e;
+    off.push_back((uint32_t)total);
+}
+
+cudaError_t fill_sell(int64_t n, const DevCsr& csr, cudaStream_t stream) {
+    const SellRows& out = csr.sell;
+    if (out.npieces)
+        sell_pieces_kernel<<<(unsigned)((out.npieces * 32 + kBlock - 1) / kBlock), kBlock, 0, stream>>>(
+            out.npieces, out.piece, out.rows);
+    sell_sort_kernel<<<(unsigned)((n + kSellWindow - 1) / kSellWindow), kSellWindow, 0, stream>>>(
+        n, csr.rp, out.row_cap, out.rows + out.npieces * 32);
     int64_t blocks = (out.nslices * 32 + kBlock - 1) / kBlock;
     if (blocks > 65536) blocks = 65536;
     sell_fill_kernel<<<(unsigned)blocks, kBlock, 0, stream>>>(out.nslices, out.npieces, out.off, out.rows,
                                                              out.piece, csr.rp, csr.col, out.pos, out.col);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    return cudaStreamSynchronize(stream);  // pieces and steps are the caller's and this call's
-}
-
-void free_sell(SellRows& s) {
-    cudaFree(s.off);
-    cudaFree(s.rows);
-    cudaFree(s.piece);
-    cudaFree(s.col);
-    cudaFree(s.pos);
-    s = SellRows{};
+    return cudaGetLastError();
 }
 
 }  // namespace esim
