@@ -36,94 +36,20 @@ namespace esim {
 
 namespace {
 
-constexpr int kDotBlocks = 1024;
+constexpr int kSumBlocks = 1024;   // of zv_finalize_kernel, at most
 constexpr int kProbeW = 32;      // probe columns per block (one warp lane each)
 constexpr int kGroupMax = 8;     // probe blocks per launch
 constexpr int kPushChunk = 64;   // in-edges per push work item
 constexpr size_t kProbeBudget = (size_t)2 << 30;  // device bytes for the probe groups
 
-// ---------------------------------------------------------------- dense FP64 helpers
-
-// partial[block] of sum_i a(i)^2 (kind 0) or sum_i a(i) (kind 2)
-__global__ void __launch_bounds__(kBlock) wsum_kernel(int64_t n, const double* __restrict__ a, int kind,
-                                                      double* __restrict__ partial) {
-    __shared__ double red[kBlock / 32];
-    double acc = 0.0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const double v = a[i];
-        acc += kind == 2 ? v : v * v;
-    }
-    acc = block_sum(acc, red);
-    if (threadIdx.x == 0) partial[blockIdx.x] = acc;
-}
-
-__global__ void sum_partials_kernel(int count, const double* __restrict__ partial, double* __restrict__ out) {
-    __shared__ double red[32];
-    double acc = 0.0;
-    const int per = (count + blockDim.x - 1) / blockDim.x;
-    for (int i = threadIdx.x * per; i < (int)((threadIdx.x + 1) * per) && i < count; ++i) acc += partial[i];
-    acc = block_sum(acc, red);
-    if (threadIdx.x == 0) *out = acc;
-}
+// ---------------------------------------------------------------- supports, finalised levels
 
 // Supports of the walk distributions of up to 32 nodes at once, as bit sets: bit c
-// of B_l(i) says (P^T)^l(k_c, i) != 0.  B_{l+1}(i) = OR over j in Out(i) of B_l(j)
-// (a pull over the out-edge CSR, one warp per row), and lane c of each warp counts
-// the rows with bit c set; one integer atomic per column and block gives
-// |supp h_l| for each of the 32 nodes.
-__global__ void reach_init_kernel(const int32_t* __restrict__ ks, int count, uint32_t* __restrict__ Bm) {
-    if ((int)threadIdx.x < count) atomicOr(Bm + ks[threadIdx.x], 1u << threadIdx.x);
-}
-
-__global__ void __launch_bounds__(kBlock) reach_step_kernel(int64_t n, const uint32_t* __restrict__ rp,
-                                                            const int32_t* __restrict__ col,
-                                                            const uint32_t* __restrict__ Bcur,
-                                                            uint32_t* __restrict__ Bnext,
-                                                            unsigned long long* __restrict__ counts) {
-    constexpr int kWarps = kBlock / 32;
-    __shared__ unsigned long long red[kWarps][32];
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    const int64_t nw = (int64_t)gridDim.x * kWarps;
-    unsigned long long cnt = 0ull;
-    for (int64_t row = (int64_t)blockIdx.x * kWarps + wib; row < n; row += nw) {
-        const uint32_t b = __ldg(rp + row), e = __ldg(rp + row + 1);
-        uint32_t acc = 0u;
-        for (uint32_t p = b + lane; p < e; p += 32) acc |= Bcur[__ldg(col + p)];
-        acc = __reduce_or_sync(0xffffffffu, acc);
-        if (lane == 0) Bnext[row] = acc;
-        cnt += (acc >> lane) & 1u;
-    }
-    red[wib][lane] = cnt;
-    __syncthreads();
-    if (wib == 0) {
-        unsigned long long t = 0ull;
-#pragma unroll
-        for (int w = 0; w < kWarps; ++w) t += red[w][lane];
-        if (t) atomicAdd(counts + lane, t);
-    }
-}
-
-// flag(i) = h(i) != 0, as the uint64 counts of the offset scan
-__global__ void flag_kernel(int64_t n, const double* __restrict__ h, uint64_t* __restrict__ flag) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        flag[i] = h[i] != 0.0 ? 1ull : 0ull;
-}
-
-// ids[off(i)] = i for the flagged i: the support in ascending order
-__global__ void scatter_ids_kernel(int64_t n, const uint64_t* __restrict__ flag, const uint64_t* __restrict__ off,
-                                   int32_t* __restrict__ ids) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        if (flag[i]) ids[off[i]] = (int32_t)i;
-}
-
-// x = v / din^2 as a two-float: the input of the squared-transition sweep P~ v
-__global__ void sq_scale_kernel(int64_t n, const double* __restrict__ v, const double* __restrict__ inv_din,
-                                const uint32_t* __restrict__ pos, float2* __restrict__ x) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const double w = inv_din[i];
-        const f2 t = double_to_f2_bits(v[i] * (w * w));
-        x[at_pos(pos, i)] = make_float2(t.hi, t.lo);
-    }
+// of B_l(i) says (P^T)^l(k_c, i) != 0, kept at i's position in the vectors the forward
+// sweeps gather; launch_reach takes a step and counts |supp h_l| for each of the nodes.
+__global__ void reach_init_kernel(const int32_t* __restrict__ ks, int count, const uint32_t* __restrict__ pos,
+                                  uint32_t* __restrict__ Bm) {
+    if ((int)threadIdx.x < count) atomicOr(Bm + at_pos(pos, ks[threadIdx.x]), 1u << threadIdx.x);
 }
 
 // Probe terms of the levels below d are summed in signed two-word fixed point (integer
@@ -142,16 +68,48 @@ __device__ __forceinline__ void zacc_split(double t, long long& hi, long long& l
     lo = __double2ll_rn((s - (double)hi) * kZLo);  // s - hi is exact (|s - hi| <= 1/2)
 }
 
-// Zv_j = c^j h_j^2 - c T + (probe terms), T = P~ Zv_{j-1} (T = NULL at j = 1)
-__global__ void zv_finalize_kernel(int64_t n, double cj, double c, const double* __restrict__ h,
-                                   const double* __restrict__ T, const long long* __restrict__ zhi,
-                                   const long long* __restrict__ zlo, double* __restrict__ zv) {
+// Zv_j = c^j h_j^2 - c T + (probe terms), T = P~ Zv_{j-1} (T = NULL at j = 1); x = Zv_j / din^2
+// as a two-float, by position (x = NULL at the last level): the input of the next level's
+// squared-transition sweep; *sum = the sum of Zv_j: block sums in a fixed order by the last
+// block (the ticket wraps to zero).
+__global__ void __launch_bounds__(kBlock) zv_finalize_kernel(int64_t n, double cj, double c, const double* __restrict__ h,
+                                                             const double* __restrict__ T,
+                                                             const long long* __restrict__ zhi,
+                                                             const long long* __restrict__ zlo, double* __restrict__ zv,
+                                                             const double* __restrict__ inv_din,
+                                                             const uint32_t* __restrict__ pos, float2* __restrict__ x,
+                                                             double* __restrict__ partial, unsigned* __restrict__ ticket,
+                                                             double* __restrict__ sum) {
+    __shared__ double red[kBlock / 32];
+    __shared__ bool last;
+    prior_done();
+    double acc = 0.0;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const double hv = h[i];
         double z = cj * (hv * hv);
         if (T) z -= c * T[i];
-        zv[i] = z + ((double)zhi[i] * (1.0 / kZOne) + (double)zlo[i] * (1.0 / (kZOne * kZLo)));
+        z += (double)zhi[i] * (1.0 / kZOne) + (double)zlo[i] * (1.0 / (kZOne * kZLo));
+        zv[i] = z;
+        acc += z;
+        if (x) {
+            const double w = inv_din[i];
+            const f2 t = double_to_f2_bits(z * (w * w));
+            x[at_pos(pos, i)] = make_float2(t.hi, t.lo);
+        }
     }
+    acc = block_sum(acc, red);
+    if (threadIdx.x == 0) {
+        partial[blockIdx.x] = acc;
+        __threadfence();
+        last = atomicInc(ticket, gridDim.x - 1) == gridDim.x - 1;
+        __threadfence();
+    }
+    __syncthreads();
+    if (!last) return;
+    acc = 0.0;
+    for (unsigned i = threadIdx.x; i < gridDim.x; i += blockDim.x) acc += __ldcg(partial + i);
+    acc = block_sum(acc, red);
+    if (threadIdx.x == 0) *sum = acc;
 }
 
 // ---------------------------------------------------------------- probes
@@ -176,13 +134,16 @@ constexpr double kInvOne = 1.0 / 9223372036854775808.0;  // 2^-63
 // exceed (m + n) / alg3_push_div (default 4) the step and all later ones of the block
 // run the dense pull.
 // Both forms give the same integers, so the switch changes no bit of the result.
+// x is not kept zero outside the frontier: a push reads the frontier's rows only, all of
+// them written by the step before, and the first dense step tells them by their marks, which
+// the step before leaves set (later dense steps find every row written).
 // The frontier, its in-edge count and the work list of 64-entry chunks live on the
 // device; the kernels of a step read the same counters, so all agree on the form
 // without a host round trip.
 struct ProbeStepCnt {
-    unsigned int fcount;      // rows in F_s
-    unsigned int wcount;      // push work items of F_s (64-entry chunks of in-rows)
-    unsigned long long push;  // in-edges of F_s
+    unsigned long long front;  // rows in F_s (high word) and their in-edges (low word): one atomic adds both
+    unsigned int wcount;       // push work items of F_s (64-entry chunks of in-rows)
+    unsigned int pad;
 };
 
 struct ProbeCtl {
@@ -193,14 +154,14 @@ struct ProbeCtl {
 
 __device__ __forceinline__ bool probe_dense_at(const ProbeCtl* ctl, int s, unsigned long long thr) {
     const int d = *(volatile const int*)&ctl->dense_plus1;
-    return (d != 0 && d - 1 <= s) || ctl->st[s].push > thr;
+    return (d != 0 && d - 1 <= s) || (ctl->st[s].front & 0xffffffffull) > thr;
 }
 
 // The buffers of a probe group: block b (blockIdx.y) owns slice b of each.
 struct ProbeGroup {
     unsigned long long* X[2];   // x ping-pong, 32 n each
     unsigned long long* Hn;     // push accumulator, 32 n (zero between steps)
-    uint32_t* mark;             // n (zero between steps)
+    uint32_t* mark;             // n (zero between steps; the frontier's set before the first dense step)
     int32_t* F[2];              // frontiers, n each
     int2* W[2];                 // push work items, nw each
     unsigned long long* ppart;  // dense long-row partials, 32 nseg
@@ -272,7 +233,7 @@ __device__ __forceinline__ void probe_flush_colsum(unsigned long long v, unsigne
 // Group start (one warp per block): x_0 = e_{q'} / din(q') per column, F_0 = the
 // sources, their work items, fresh counters and column sums.
 __global__ void probe_init_kernel(ProbeGroup G, const int32_t* __restrict__ ids, int count,
-                                  const uint32_t* __restrict__ in_rp) {
+                                  const uint32_t* __restrict__ in_rp, unsigned long long thr) {
     const int b = blockIdx.y, lane = threadIdx.x;
     ProbeCtl* ctl = G.ctl + b;
     uint32_t* z = (uint32_t*)ctl;
@@ -285,8 +246,12 @@ __global__ void probe_init_kernel(ProbeGroup G, const int32_t* __restrict__ ids,
     if (lane < cnt) {
         q = ids[b * kProbeW + lane];
         d = in_rp[q + 1] - in_rp[q];
-        G.X[0][(size_t)b * G.nx + (size_t)q * kProbeW + lane] = d ? kOne / d : 0ull;
         G.F[0][(size_t)b * G.n + lane] = q;
+    }
+    const unsigned long long x0 = d ? kOne / d : 0ull;
+    for (int t = 0; t < cnt; ++t) {  // source t's row: its own column, zero in the others
+        const int32_t row = __shfl_sync(0xffffffffu, q, t);
+        G.X[0][(size_t)b * G.nx + (size_t)row * kProbeW + lane] = lane == t ? x0 : 0ull;
     }
     const unsigned int nch = (d + kPushChunk - 1) / kPushChunk;
     unsigned int incl = nch;
@@ -301,11 +266,11 @@ __global__ void probe_init_kernel(ProbeGroup G, const int32_t* __restrict__ ids,
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) dsum += __shfl_xor_sync(0xffffffffu, dsum, o);
     const unsigned int total = __shfl_sync(0xffffffffu, incl, 31);
+    if (dsum > thr && q >= 0) G.mark[(size_t)b * G.n + q] = 1u;  // step 0 is dense already
     __syncwarp();
     if (lane == 0) {
-        ctl->st[0].fcount = (unsigned int)cnt;
+        ctl->st[0].front = (unsigned long long)cnt << 32 | dsum;
         ctl->st[0].wcount = total;
-        ctl->st[0].push = dsum;
     }
     G.colsum[(size_t)b * kProbeW + lane] = 0ull;
 }
@@ -344,21 +309,18 @@ __global__ void __launch_bounds__(kBlock) probe_push_kernel(ProbeGroup G, ProbeS
             const uint32_t p = p0 + lane;
             const int32_t mine = p < end ? __ldg(a.in_col + p) : -1;
             bool fresh = false;
-            unsigned long long din_new = 0;
+            unsigned int din_new = 0;
             if (mine >= 0) {
                 fresh = atomicExch(mark + mine, 1u) == 0u;
                 if (fresh) din_new = __ldg(a.in_rp + mine + 1) - __ldg(a.in_rp + mine);
             }
             const unsigned fm = __ballot_sync(0xffffffffu, fresh);
             if (fm) {
-                unsigned long long dsum = din_new;
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) dsum += __shfl_xor_sync(0xffffffffu, dsum, o);
+                const unsigned int dsum = __reduce_add_sync(0xffffffffu, din_new);  // distinct rows: below m < 2^32
                 unsigned int base = 0;
-                if (lane == 0) {
-                    base = atomicAdd(&ctl->st[a.s + 1].fcount, (unsigned int)__popc(fm));
-                    atomicAdd(&ctl->st[a.s + 1].push, dsum);
-                }
+                if (lane == 0)
+                    base = (unsigned int)(atomicAdd(&ctl->st[a.s + 1].front,
+                                                    (unsigned long long)__popc(fm) << 32 | dsum) >> 32);
                 base = __shfl_sync(0xffffffffu, base, 0);
                 if (fresh) Fnext[base + __popc(fm & ((1u << lane) - 1u))] = mine;
             }
@@ -371,52 +333,91 @@ __global__ void __launch_bounds__(kBlock) probe_push_kernel(ProbeGroup G, ProbeS
     }
 }
 
-// Sparse epilogue: the rows of F_{s+1} (h_{s+1} from the accumulator, which is
-// cleared), the next step's work items; then x_s is cleared on F_s.
+// Sparse epilogue: the rows of F_{s+1} (h_{s+1} from the accumulator, which is cleared) and
+// the next step's work items, if that step pushes.  A warp takes up to 32 rows at a time and
+// reserves their items with one atomic: with one atomic a row on the block's one counter, and
+// items listed for dense steps too, this kernel took up to 0.55 ms and was the largest of the
+// probes.
 __global__ void __launch_bounds__(kBlock) probe_sparse_epi_kernel(ProbeGroup G, ProbeStepArgs a) {
     const int b = blockIdx.y;
     ProbeCtl* ctl = G.ctl + b;
     if (probe_dense_at(ctl, a.s, a.thr)) return;
+    const bool push_next = !a.last && !probe_dense_at(ctl, a.s + 1, a.thr);
+    const bool keep_marks = !a.last && !push_next;  // for the first dense step
     const int lane = threadIdx.x & 31;
     unsigned long long* Hn = G.Hn + (size_t)b * G.nx;
     uint32_t* mark = G.mark + (size_t)b * G.n;
     const int32_t* Fnext = G.F[(a.s + 1) & 1] + (size_t)b * G.n;
-    const int32_t* Fcur = G.F[a.s & 1] + (size_t)b * G.n;
-    unsigned long long* Xcur = G.X[a.src] + (size_t)b * G.nx;
     unsigned long long* Xnext = G.X[a.src ^ 1] + (size_t)b * G.nx;
     int2* Wnext = G.W[(a.s + 1) & 1] + (size_t)b * G.nw;
     const double* coef = G.coef + (size_t)b * kProbeW;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const unsigned int nf = ctl->st[a.s + 1].fcount;
+    const unsigned int nwarps = (gridDim.x * blockDim.x) >> 5;
+    const unsigned int w0 = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const unsigned int nf = (unsigned int)(ctl->st[a.s + 1].front >> 32);
+    unsigned int rows = (nf + nwarps - 1) / nwarps;  // per warp and turn
+    rows = rows < 1 ? 1 : (rows > 32 ? 32 : rows);
     unsigned long long nacc = 0ull;
-    for (int64_t r = w0; r < (int64_t)nf; r += nwarps) {
-        const int32_t i = Fnext[r];
-        const size_t at = (size_t)i * kProbeW + lane;
-        const unsigned long long H = Hn[at];
-        Hn[at] = 0ull;
-        if (lane == 0) {
-            mark[i] = 0u;
-            const uint32_t d = __ldg(a.in_rp + i + 1) - __ldg(a.in_rp + i);
-            if (!a.last && d) {
-                const unsigned int nch = (d + kPushChunk - 1) / kPushChunk;
-                const unsigned int base = atomicAdd(&ctl->st[a.s + 1].wcount, nch);
-                for (unsigned int ch = 0; ch < nch; ++ch) Wnext[base + ch] = make_int2(i, (int)ch);
-            }
+    for (unsigned long long r0 = (unsigned long long)w0 * rows; r0 < nf; r0 += (unsigned long long)nwarps * rows) {
+        const int cnt = (int)(nf - r0 < rows ? nf - r0 : rows);  // warp-uniform
+        int32_t mine = 0;
+        unsigned int nch = 0;
+        if (lane < cnt) {
+            mine = Fnext[r0 + lane];
+            if (!keep_marks) mark[mine] = 0u;
+            if (push_next) nch = (__ldg(a.in_rp + mine + 1) - __ldg(a.in_rp + mine) + kPushChunk - 1) / kPushChunk;
         }
-        nacc += probe_row_out(i, H, lane, a, Xnext, coef);
+        if (push_next) {
+            unsigned int incl = nch;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned int v = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += v;
+            }
+            unsigned int base = 0;
+            if (lane == 31 && incl) base = atomicAdd(&ctl->st[a.s + 1].wcount, incl);
+            base = __shfl_sync(0xffffffffu, base, 31) + incl - nch;
+            for (unsigned int ch = 0; ch < nch; ++ch) Wnext[base + ch] = make_int2(mine, (int)ch);
+        }
+        constexpr int kU = 4;  // rows in flight
+        for (int t0 = 0; t0 < cnt; t0 += kU) {
+            unsigned long long H[kU];
+            int32_t i[kU];
+#pragma unroll
+            for (int u = 0; u < kU; ++u) {
+                i[u] = __shfl_sync(0xffffffffu, mine, (t0 + u) & 31);
+                if (t0 + u < cnt) H[u] = Hn[(size_t)i[u] * kProbeW + lane];
+            }
+#pragma unroll
+            for (int u = 0; u < kU; ++u)
+                if (t0 + u < cnt) {
+                    Hn[(size_t)i[u] * kProbeW + lane] = 0ull;
+                    nacc += probe_row_out(i[u], H[u], lane, a, Xnext, coef);
+                }
+        }
     }
-    const unsigned int nc = ctl->st[a.s].fcount;
-    for (int64_t r = w0; r < (int64_t)nc; r += nwarps) Xcur[(size_t)Fcur[r] * kProbeW + lane] = 0ull;
     if (a.mode == 2) probe_flush_colsum(nacc, G.colsum + (size_t)b * kProbeW);
 }
 
-// Sum of X(col[p], lane) over entries [b, e), eight gathers in flight (integer adds).
+// Sum of X(col[p], lane) over entries [b, e), eight gathers in flight (integer adds).  marked
+// (the first dense step): only the rows with a mark hold values.
 __device__ __forceinline__ unsigned long long probe_range(const int32_t* __restrict__ col,
-                                                          const unsigned long long* __restrict__ X, uint32_t b,
-                                                          uint32_t e, int lane) {
+                                                          const unsigned long long* __restrict__ X,
+                                                          const uint32_t* __restrict__ marked, uint32_t b, uint32_t e,
+                                                          int lane) {
     unsigned long long acc = 0ull;
     uint32_t p = b;
+    if (marked) {
+        for (; p < e; p += 32) {  // the lanes look up 32 marks; the frontier's rows follow one by one
+            const int32_t mine = p + lane < e ? __ldg(col + p + lane) : 0;
+            unsigned set = __ballot_sync(0xffffffffu, p + lane < e && marked[mine] != 0u);
+            while (set) {
+                const int t = __ffs(set) - 1;
+                set &= set - 1u;
+                acc += X[(size_t)__shfl_sync(0xffffffffu, mine, t) * kProbeW + lane];
+            }
+        }
+        return acc;
+    }
     for (; p + 8 <= e; p += 8) {
         int32_t j[8];
         unsigned long long v[8];
@@ -448,6 +449,8 @@ __global__ void __launch_bounds__(kBlock) probe_rows_kernel(ProbeGroup G, ProbeS
     const int lane = threadIdx.x & 31;
     const int wib = threadIdx.x >> 5;
     const unsigned long long* X = G.X[a.src] + (size_t)b * G.nx;
+    const int went = *(volatile const int*)&ctl->dense_plus1;
+    const uint32_t* marked = went == 0 || went == a.s + 1 ? G.mark + (size_t)b * G.n : nullptr;
     if ((int)blockIdx.x >= short_blocks) {
         __shared__ unsigned long long red[kWarps][kProbeW];
         unsigned long long* partial = G.ppart + (size_t)b * G.np;
@@ -458,7 +461,7 @@ __global__ void __launch_bounds__(kBlock) probe_rows_kernel(ProbeGroup G, ProbeS
             uint32_t bb = sg.beg + (uint32_t)wib * per;
             if (bb > sg.end) bb = sg.end;
             const uint32_t e = bb + per < sg.end ? bb + per : sg.end;
-            red[wib][lane] = probe_range(col, X, bb, e, lane);
+            red[wib][lane] = probe_range(col, X, marked, bb, e, lane);
             __syncthreads();
             if (wib == 0) {
                 unsigned long long t = 0ull;
@@ -477,7 +480,7 @@ __global__ void __launch_bounds__(kBlock) probe_rows_kernel(ProbeGroup G, ProbeS
     for (int64_t row = (int64_t)blockIdx.x * kWarps + wib; row < G.n; row += nw) {
         const uint32_t rb = __ldg(rp + row), re = __ldg(rp + row + 1);
         if (re - rb >= long_min) continue;  // warp-uniform: a long row
-        nacc += probe_row_out(row, probe_range(col, X, rb, re, lane), lane, a, Xnext, coef);
+        nacc += probe_row_out(row, probe_range(col, X, marked, rb, re, lane), lane, a, Xnext, coef);
     }
     if (a.mode == 2) probe_flush_colsum(nacc, G.colsum + (size_t)b * kProbeW);
 }
@@ -502,7 +505,7 @@ __global__ void __launch_bounds__(kBlock) probe_long_rows_kernel(ProbeGroup G, P
 }
 
 // Group end: zlast += the sum over blocks and columns, in order, of
-// c^{steps} Zv_i(q'_col) colsum(b, col); blocks that went dense clear both x buffers.
+// c^{steps} Zv_i(q'_col) colsum(b, col); blocks that went dense clear their marks.
 __global__ void probe_end_kernel(ProbeGroup G, const int32_t* __restrict__ ids, int count,
                                  const double* __restrict__ zv_src, double cl, double* __restrict__ zlast,
                                  const int32_t* __restrict__ pos, unsigned long long* __restrict__ colsum_out) {
@@ -517,12 +520,9 @@ __global__ void probe_end_kernel(ProbeGroup G, const int32_t* __restrict__ ids, 
     }
     const int b = blockIdx.y;
     if (G.ctl[b].dense_plus1 == 0) return;
-    unsigned long long* xa = G.X[0] + (size_t)b * G.nx;
-    unsigned long long* xb = G.X[1] + (size_t)b * G.nx;
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < G.nx; i += (size_t)gridDim.x * blockDim.x) {
-        xa[i] = 0ull;
-        xb[i] = 0ull;
-    }
+    uint32_t* mark = G.mark + (size_t)b * G.n;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < G.n; i += (int64_t)gridDim.x * blockDim.x)
+        mark[i] = 0u;
 }
 
 // The last probe level (probes of length 2 from the support of h_{d-2}) needs of each
@@ -941,14 +941,13 @@ struct A3Ws {
     double* x;        // n: sweep input
     double* xa;       // n
     double* xb;       // n
-    uint64_t* flag;   // n
-    uint64_t* off;    // n + 1
-    int32_t* ids;     // n
+    uint64_t* nsup;   // 1: support size
+    int32_t* ids;     // n: the support
     uint32_t* Ba;     // reach bit sets (32 nodes per word)
     uint32_t* Bb;
     unsigned long long* rcounts;  // (D + 1) x 32 support sizes
-    double* partial;  // kDotBlocks (dot products)
-    double* sums;     // 64: [j] = sum_q Zv_j(q); [63] = the last level's probe terms
+    double* partial;  // kSumBlocks block sums
+    double* sums;     // 64: [j] = sum_q Zv_j(q); [62] a ticket; [63] = the last level's probe terms
     unsigned long long* g2;  // n: column sums g_2 of the last probe level, by support position
     int32_t* big_ids;        // n: support nodes too large for the two-hop table
     int32_t* big_pos;        // n: their support positions
@@ -976,13 +975,12 @@ size_t a3_layout(int64_t n_, int64_t m_, int64_t nseg, void* base, A3Ws* out) {
     w.x = (double*)take(8 * n);
     w.xa = (double*)take(8 * n);
     w.xb = (double*)take(8 * n);
-    w.flag = (uint64_t*)take(8 * n);
-    w.off = (uint64_t*)take(8 * (n + 1));
+    w.nsup = (uint64_t*)take(8);
     w.ids = (int32_t*)take(4 * n);
     w.Ba = (uint32_t*)take(4 * n);
     w.Bb = (uint32_t*)take(4 * n);
     w.rcounts = (unsigned long long*)take(8 * 32 * (D + 1));
-    w.partial = (double*)take(8 * kDotBlocks);
+    w.partial = (double*)take(8 * kSumBlocks);
     w.sums = (double*)take(8 * 64);
     w.g2 = (unsigned long long*)take(8 * n);
     w.big_ids = (int32_t*)take(4 * n);
@@ -1012,13 +1010,6 @@ size_t a3_layout(int64_t n_, int64_t m_, int64_t nseg, void* base, A3Ws* out) {
     P.colsum = (unsigned long long*)take(8 * kProbeW * gz);
     if (out) *out = w;
     return o;
-}
-
-cudaError_t dsum(const Graph& g, const double* a, int kind, const A3Ws& ws, double* out_dev, int* count) {
-    wsum_kernel<<<kDotBlocks, kBlock, 0, g.stream>>>(g.n, a, kind, ws.partial);
-    sum_partials_kernel<<<1, 1024, 0, g.stream>>>(kDotBlocks, ws.partial, out_dev);
-    *count += 2;
-    return cudaGetLastError();
 }
 
 // One probe step for a group of nb blocks: push, dense pull (whichever the counters
@@ -1071,16 +1062,12 @@ cudaError_t alg3_supports(const Graph& g, const int32_t* ks_host, int count, int
             (e = cudaMemcpyAsync(ws.ids, ks_host + c0, sizeof(int32_t) * (size_t)cnt, cudaMemcpyHostToDevice,
                                  g.stream)) != cudaSuccess)
             return e;
-        reach_init_kernel<<<1, 32, 0, g.stream>>>(ws.ids, cnt, ws.Ba);
+        reach_init_kernel<<<1, 32, 0, g.stream>>>(ws.ids, cnt, g.out.sell.pos, ws.Ba);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         ++nl;
         uint32_t* B[2] = {ws.Ba, ws.Bb};
-        int64_t blocks = (g.n + kBlock / 32 - 1) / (kBlock / 32);
-        if (blocks > (int64_t)g.sm_count * 16) blocks = (int64_t)g.sm_count * 16;
         for (int l = 1; l <= levels; ++l) {
-            reach_step_kernel<<<(unsigned)blocks, kBlock, 0, g.stream>>>(g.n, g.out.rp, g.out.col, B[(l - 1) & 1],
-                                                                         B[l & 1], ws.rcounts + (size_t)l * 32);
-            if ((e = cudaGetLastError()) != cudaSuccess) return e;
+            if ((e = launch_reach(g, B[(l - 1) & 1], B[l & 1], ws.rcounts + (size_t)l * 32)) != cudaSuccess) return e;
             ++nl;
         }
         std::vector<unsigned long long> host((size_t)32 * (kAlg3MaxDepth + 1));
@@ -1096,11 +1083,12 @@ cudaError_t alg3_supports(const Graph& g, const int32_t* ks_host, int count, int
     return cudaSuccess;
 }
 
-cudaError_t alg3_first_meeting(const Graph& g, int64_t k, int depth, double c, void* wsp, double* z_out, int* launches) {
+static cudaError_t first_meeting(const Graph& g, int64_t k, int depth, double c, void* wsp, int* clean, double* z_out,
+                                 int* launches) {
     A3Ws ws;
     a3_layout(g.n, g.m, g.out.nseg, wsp, &ws);
     const size_t n = (size_t)g.n;
-    const int eb = eblocks(g, g.n);
+    const int eb = std::min(eblocks(g, g.n), kSumBlocks);
     int count = 0;
     cudaError_t e = launch_walk_distributions(g, k, depth, ws.H, ws.xa, ws.xb);
     if (e != cudaSuccess) return e;
@@ -1110,7 +1098,6 @@ cudaError_t alg3_first_meeting(const Graph& g, int64_t k, int depth, double c, v
         (e = cudaMemsetAsync(zlo_base, 0, sizeof(long long) * n * (size_t)(depth + 1), g.stream)) != cudaSuccess)
         return e;
     if ((e = cudaMemsetAsync(ws.sums, 0, sizeof(double) * 64, g.stream)) != cudaSuccess) return e;
-    int cleared = 0;  // probe blocks made zero so far (each group leaves its blocks zero)
     std::vector<double> cpow((size_t)depth + 1, 1.0);
     for (int j = 1; j <= depth; ++j) cpow[(size_t)j] = cpow[(size_t)j - 1] * c;
     const unsigned long long thr = (unsigned long long)(g.m + g.n) / (unsigned long long)std::max(1, g.alg3_push_div);
@@ -1118,29 +1105,21 @@ cudaError_t alg3_first_meeting(const Graph& g, int64_t k, int depth, double c, v
         double* zv = ws.Zv + (size_t)j * n;
         const double* T = nullptr;
         if (j >= 2) {  // T = P~ Zv_{j-1}
-            float2* x2 = reinterpret_cast<float2*>(ws.x);  // n 8-byte entries
-            sq_scale_kernel<<<eb, kBlock, 0, g.stream>>>(g.n, ws.Zv + (size_t)(j - 1) * n, g.inv_din, g.out.sell.pos, x2);
-            if ((e = cudaGetLastError()) != cudaSuccess) return e;
-            if ((e = launch_pull_sum(g, x2, ws.T)) != cudaSuccess) return e;
-            count += 2;
+            if ((e = launch_pull_sum(g, reinterpret_cast<float2*>(ws.x), ws.T)) != cudaSuccess) return e;
+            ++count;
             T = ws.T;
         }
-        zv_finalize_kernel<<<eb, kBlock, 0, g.stream>>>(g.n, cpow[(size_t)j], c, ws.H + (size_t)j * n, T,
-                                                        ws.Zfx + (size_t)j * n, zlo_base + (size_t)j * n, zv);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        e = launch_after(g.stream, dim3((unsigned)eb), kBlock, 0, zv_finalize_kernel, g.n, cpow[(size_t)j], c,
+                         ws.H + (size_t)j * n, T, ws.Zfx + (size_t)j * n, zlo_base + (size_t)j * n, zv, g.inv_din,
+                         g.out.sell.pos, j < depth ? reinterpret_cast<float2*>(ws.x) : nullptr, ws.partial,
+                         reinterpret_cast<unsigned*>(ws.sums + 62), ws.sums + j);
+        if (e != cudaSuccess) return e;
         ++count;
-        if ((e = dsum(g, zv, 2, ws, ws.sums + j, &count)) != cudaSuccess) return e;
         // probes from the support of h_j feed the levels j+2 .. depth: the row terms of a
         // level below depth, only the column sums for the last level
         if (j > depth - 2) continue;
-        flag_kernel<<<eb, kBlock, 0, g.stream>>>(g.n, ws.H + (size_t)j * n, ws.flag);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        if ((e = launch_scan_R(g, g.n, ws.flag, ws.off, g.scan_part, g.norm_part + allocate_blocks(g.n),
-                               false)) != cudaSuccess)
-            return e;
-        scatter_ids_kernel<<<eb, kBlock, 0, g.stream>>>(g.n, ws.flag, ws.off, ws.ids);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        count += 4;
+        if ((e = launch_support(g, ws.H + (size_t)j * n, ws.ids, ws.nsup)) != cudaSuccess) return e;
+        count += 2;
         const int steps = depth - j;
         // the last two probe levels run one warp per node where its neighbourhood fits the
         // tables: g_2 for the last, the row terms and g_3 for the one below it
@@ -1149,13 +1128,13 @@ cudaError_t alg3_first_meeting(const Graph& g, int64_t k, int depth, double c, v
             if ((e = cudaMemsetAsync(ws.nbig, 0, 2 * sizeof(unsigned int), g.stream)) != cudaSuccess) return e;
             if (steps == 2) {
                 probe_g2_kernel<<<(unsigned)(g.sm_count * 5), kG2Warps * 32, 0, g.stream>>>(
-                    ws.off + n, ws.ids, g.in.rp, g.in.col, g.din_magic, ws.g2, ws.big_ids, ws.big_pos, ws.nbig);
+                    ws.nsup, ws.ids, g.in.rp, g.in.col, g.din_magic, ws.g2, ws.big_ids, ws.big_pos, ws.nbig);
             } else {
                 if ((e = cudaFuncSetAttribute(probe_g3_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               (int)kG3Smem)) != cudaSuccess)
                     return e;
                 probe_g3_kernel<<<(unsigned)(g.sm_count * 2), kG3Warps * 32, kG3Smem, g.stream>>>(
-                    ws.off + n, ws.ids, g.in.rp, g.in.col, g.din_magic, zv, cpow[2], ws.Zfx + (size_t)(j + 2) * n,
+                    ws.nsup, ws.ids, g.in.rp, g.in.col, g.din_magic, zv, cpow[2], ws.Zfx + (size_t)(j + 2) * n,
                     zlo_base + (size_t)(j + 2) * n, ws.g2, ws.big_ids, ws.big_pos, ws.nbig);
             }
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
@@ -1181,7 +1160,7 @@ cudaError_t alg3_first_meeting(const Graph& g, int64_t k, int depth, double c, v
         }
         uint64_t nsup = 0;
         unsigned int nbig = 0;
-        if ((e = cudaMemcpyAsync(&nsup, ws.off + n, sizeof(uint64_t), cudaMemcpyDeviceToHost, g.stream)) != cudaSuccess)
+        if ((e = cudaMemcpyAsync(&nsup, ws.nsup, sizeof(uint64_t), cudaMemcpyDeviceToHost, g.stream)) != cudaSuccess)
             return e;
         if (hashed && (e = cudaMemcpyAsync(&nbig, ws.nbig + 1, sizeof(unsigned int), cudaMemcpyDeviceToHost,
                                            g.stream)) != cudaSuccess)
@@ -1192,20 +1171,18 @@ cudaError_t alg3_first_meeting(const Graph& g, int64_t k, int depth, double c, v
         const int32_t* probe_ids = hashed ? ws.big2_ids : ws.ids;
         const uint64_t per_group = (uint64_t)kProbeW * (uint64_t)ws.group;
         const int need_blocks = (int)std::min<uint64_t>((uint64_t)ws.group, (nprobe + kProbeW - 1) / kProbeW);
-        if (need_blocks > cleared) {  // blocks [cleared, need_blocks) of each buffer
-            const size_t b0 = (size_t)cleared, nbk = (size_t)(need_blocks - cleared);
-            if ((e = cudaMemsetAsync(ws.G.X[0] + b0 * ws.G.nx, 0, 8 * ws.G.nx * nbk, g.stream)) != cudaSuccess ||
-                (e = cudaMemsetAsync(ws.G.X[1] + b0 * ws.G.nx, 0, 8 * ws.G.nx * nbk, g.stream)) != cudaSuccess ||
-                (e = cudaMemsetAsync(ws.G.Hn + b0 * ws.G.nx, 0, 8 * ws.G.nx * nbk, g.stream)) != cudaSuccess ||
+        if (need_blocks > *clean) {  // accumulators and marks of blocks [*clean, need_blocks): every group leaves them zero
+            const size_t b0 = (size_t)*clean, nbk = (size_t)(need_blocks - *clean);
+            if ((e = cudaMemsetAsync(ws.G.Hn + b0 * ws.G.nx, 0, 8 * ws.G.nx * nbk, g.stream)) != cudaSuccess ||
                 (e = cudaMemsetAsync(ws.G.mark + b0 * n, 0, 4 * n * nbk, g.stream)) != cudaSuccess)
                 return e;
-            cleared = need_blocks;
+            *clean = need_blocks;
         }
         for (uint64_t g0 = 0; g0 < nprobe; g0 += per_group) {
             const int cnt = (int)std::min<uint64_t>(per_group, nprobe - g0);
             const int nb = (cnt + kProbeW - 1) / kProbeW;
             const int32_t* ids = probe_ids + g0;
-            probe_init_kernel<<<dim3(1, (unsigned)nb), kProbeW, 0, g.stream>>>(ws.G, ids, cnt, g.in.rp);
+            probe_init_kernel<<<dim3(1, (unsigned)nb), kProbeW, 0, g.stream>>>(ws.G, ids, cnt, g.in.rp, thr);
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
             ++count;
             for (int lp = 1; lp <= steps; ++lp) {
@@ -1229,7 +1206,7 @@ cudaError_t alg3_first_meeting(const Graph& g, int64_t k, int depth, double c, v
             ++count;
         }
         if (hashed && nsup > 0) {
-            probe_g2_total_kernel<<<1, 1024, 0, g.stream>>>(ws.off + n, ws.ids, zv, cpow[(size_t)steps], ws.g2,
+            probe_g2_total_kernel<<<1, 1024, 0, g.stream>>>(ws.nsup, ws.ids, zv, cpow[(size_t)steps], ws.g2,
                                                             ws.sums + 63);
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
             ++count;
@@ -1242,6 +1219,13 @@ cudaError_t alg3_first_meeting(const Graph& g, int64_t k, int depth, double c, v
     z_out[depth - 1] -= sums[63];  // the last level's probe terms, kept as column sums
     if (launches) *launches += count;
     return cudaSuccess;
+}
+
+cudaError_t alg3_first_meeting(const Graph& g, int64_t k, int depth, double c, void* wsp, int* clean, double* z_out,
+                               int* launches) {
+    const cudaError_t e = first_meeting(g, k, depth, c, wsp, clean, z_out, launches);
+    if (e != cudaSuccess) *clean = 0;  // a probe group may have been left halfway
+    return e;
 }
 
 cudaError_t launch_dhat_alg3(const Graph& g, const uint64_t* counts, const uint64_t* off, const uint8_t* depth,

@@ -371,6 +371,7 @@ esim_status ensure_a3ws(Graph& g) {
     cudaFree(g.a3ws);
     g.a3ws = nullptr;
     g.a3ws_bytes = 0;
+    g.a3ws_clean = 0;
     if (cudaMalloc(&g.a3ws, need) != cudaSuccess) {
         cudaGetLastError();
         return fail(ESIM_ENOMEM, "cudaMalloc(Algorithm 3 workspace of " + std::to_string(need) + " bytes)");
@@ -552,21 +553,24 @@ esim_status alg3_zsums_of(Graph& g, const uint8_t* depth_dev, const std::vector<
         auto run = [&](int wi) {
             Graph view = g;
             void* ws = g.a3ws;
+            int* clean = &g.a3ws_clean;
             if (wi > 0) {
-                const Graph::A3Worker& wk = g.a3workers[(size_t)wi - 1];
+                Graph::A3Worker& wk = g.a3workers[(size_t)wi - 1];
                 if ((errs[(size_t)wi] = cudaSetDevice(g.device)) != cudaSuccess) return;
                 view.stream = wk.stream;
                 view.partial = wk.partial;
                 view.scan_part = wk.scan_part;
                 view.norm_part = wk.norm_part;
                 ws = wk.ws;
+                clean = &wk.clean;
             }
             for (;;) {
                 const size_t i = next.fetch_add(1);
                 if (i >= deep.size()) return;
                 const int d = deep[i].second;
                 double z[kAlg3MaxDepth] = {};
-                const cudaError_t e = alg3_first_meeting(view, deep[i].first, d, c, ws, z, &counts[(size_t)wi]);
+                const cudaError_t e = alg3_first_meeting(view, deep[i].first, d, c, ws, clean, z,
+                                                         &counts[(size_t)wi]);
                 if (e != cudaSuccess) {
                     errs[(size_t)wi] = e;
                     next.store(deep.size());  // the others stop after their current node
@@ -1685,7 +1689,7 @@ esim_status esim_alg3_first_meeting(esim_graph* h, int64_t k, int32_t depth, dou
     ESIM_CUDA_TRY(cudaSetDevice(g.device), "cudaSetDevice");
     esim_status a3 = ensure_a3ws(g);
     if (a3 != ESIM_OK) return a3;
-    ESIM_CUDA_TRY(alg3_first_meeting(g, k, depth, c, g.a3ws, z_out, nullptr), "Algorithm 3 first meetings");
+    ESIM_CUDA_TRY(alg3_first_meeting(g, k, depth, c, g.a3ws, &g.a3ws_clean, z_out, nullptr), "Algorithm 3 first meetings");
     return ESIM_OK;
 }
 

@@ -146,6 +146,7 @@ struct Graph {
     std::shared_ptr<std::vector<uint32_t>> din_host;  // in-degrees, for the exploitation plan
     void* a3ws = nullptr;         // Algorithm 3 scratch (FP64 vectors, dot partials)
     size_t a3ws_bytes = 0;
+    int a3ws_clean = 0;           // its probe blocks known to be zero
     void* a3pws = nullptr;        // the paper's depth rule: support bit sets and edge tables
     size_t a3pws_bytes = 0;
     // Algorithm 3: extra workers for the one-node Lemma 5 computations, each with its own
@@ -153,6 +154,7 @@ struct Graph {
     struct A3Worker {
         cudaStream_t stream = nullptr;
         void* ws = nullptr;
+        int clean = 0;            // probe blocks of ws known to be zero
         void* partial = nullptr;
         unsigned long long* scan_part = nullptr;
         double* norm_part = nullptr;
@@ -213,6 +215,9 @@ cudaError_t launch_reverse(const Graph& g, const double* hist, int32_t L, double
 cudaError_t launch_forward32(const Graph& g, int64_t u, double c, int32_t L, float* hist, float* xa, float* xb);
 cudaError_t launch_walk_distributions(const Graph& g, int64_t u, int steps, double* H, double* xa, double* xb);
 cudaError_t launch_pull_sum(const Graph& g, const float2* x, double* out);
+// one step of 32 supports: bit c of next(i) = OR over j in Out(i) of bit c of cur(j), both by
+// position (g.out.sell.pos); counts[c] += the nodes with bit c
+cudaError_t launch_reach(const Graph& g, const uint32_t* cur, uint32_t* next, unsigned long long* counts);
 cudaError_t launch_reverse32(const Graph& g, const float* hist, int32_t L, double c, const double* dhat,
                              double* s_out, float2* w, float2* sa, float2* sb);
 cudaError_t launch_forward_sparse(const Graph& g, int64_t u, double c, int32_t L, double theta, const SparseHist& h,
@@ -261,6 +266,8 @@ cudaError_t launch_dhat_segments(const Graph& g, int64_t nseg, const uint64_t* n
 // part_Rd: allocate_blocks(N)
 cudaError_t launch_scan_R(const Graph& g, int64_t N, const uint64_t* R, uint64_t* off, unsigned long long* part_R,
                           double* part_Rd, bool record = true);
+// the nodes with h != 0, ascending, and their number (device), with g's scan scratch
+cudaError_t launch_support(const Graph& g, const double* h, int32_t* ids, uint64_t* count);
 uint32_t walk_threshold(double c);
 
 // capi.cu: record a message for esim_last_error() and return `status` (as an esim_status int)
@@ -293,7 +300,8 @@ size_t alg3_workspace_bytes(const Graph& g);
 cudaError_t alg3_supports(const Graph& g, const int32_t* ks, int count, int levels, void* ws, uint64_t* supp_out,
                           int* launches);
 // Z_1..Z_depth of node k (Lemma 5) into z_out (host), depth <= kAlg3MaxDepth; synchronises g.stream.
-cudaError_t alg3_first_meeting(const Graph& g, int64_t k, int depth, double c, void* ws, double* z_out,
+// *clean: probe blocks of ws whose accumulators and marks are zero (0 for a new workspace); kept.
+cudaError_t alg3_first_meeting(const Graph& g, int64_t k, int depth, double c, void* ws, int* clean, double* z_out,
                                int* launches);
 cudaError_t launch_dhat_alg3(const Graph& g, const uint64_t* counts, const uint64_t* off, const uint8_t* depth,
                              const double* zsum, double c, double* dhat);

@@ -106,7 +106,7 @@ __device__ __forceinline__ double level_sum(const float* __restrict__ hist, int6
 // into off[n] and the status block, the budget check.  The ticket wraps to zero.
 struct TileSums {
     unsigned long long* R;   // gridDim.x, and the ticket behind them (zero before the launch)
-    double* Rd;              // gridDim.x: the same in double
+    double* Rd;              // gridDim.x: the same in double, or NULL
     double* norm;            // gridDim.x sums of pi^2, or NULL
 };
 
@@ -131,7 +131,7 @@ __device__ __forceinline__ void finish_tiles(const TileSums& t, double budget, u
     for (int64_t b = b0; b < b1; ++b) {
         local += __ldcg(t.R + b);
         if (t.norm) nrm += __ldcg(t.norm + b);
-        rd += __ldcg(t.Rd + b);
+        if (t.Rd) rd += __ldcg(t.Rd + b);
     }
     unsigned long long total;
     unsigned long long run = block_exclusive_scan(local, su, &total);
@@ -826,6 +826,51 @@ cudaError_t launch_scan_R(const Graph& g, int64_t N, const uint64_t* R, uint64_t
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     return scan_offsets(g, N, R, part_R, off);
+}
+
+// The nodes with h != 0, ascending, into ids, and their number: tile counts and their scan,
+// then the ids.
+template <int kItems>
+__global__ void __launch_bounds__(kBlock) support_tiles_kernel(int64_t n, const double* __restrict__ h,
+                                                               const TileSums tiles, uint64_t* __restrict__ count) {
+    __shared__ unsigned long long red[kBlock / 32];
+    prior_done();
+    const int64_t base = ((int64_t)blockIdx.x * kBlock + threadIdx.x) * kItems;
+    unsigned long long c = 0;
+#pragma unroll
+    for (int i = 0; i < kItems; ++i) c += base + i < n && h[base + i] != 0.0;
+    c = block_sum(c, red);
+    if (threadIdx.x == 0) tiles.R[blockIdx.x] = c;
+    finish_tiles(tiles, 0.0, count, nullptr);
+}
+
+template <int kItems>
+__global__ void __launch_bounds__(kBlock) support_ids_kernel(int64_t n, const double* __restrict__ h,
+                                                             const unsigned long long* __restrict__ tile_off,
+                                                             int32_t* __restrict__ ids) {
+    __shared__ unsigned long long su[32];
+    prior_done();
+    const int64_t base = ((int64_t)blockIdx.x * kBlock + threadIdx.x) * kItems;
+    unsigned set = 0;
+#pragma unroll
+    for (int i = 0; i < kItems; ++i) set |= base + i < n && h[base + i] != 0.0 ? 1u << i : 0u;
+    unsigned long long total;
+    unsigned long long at = tile_off[blockIdx.x] + block_exclusive_scan((unsigned long long)__popc(set), su, &total);
+#pragma unroll
+    for (int i = 0; i < kItems; ++i)
+        if (set >> i & 1u) ids[at++] = (int32_t)(base + i);
+}
+
+cudaError_t launch_support(const Graph& g, const double* h, int32_t* ids, uint64_t* count) {
+    const unsigned nb = (unsigned)allocate_blocks(g.n);
+    const TileSums tiles{g.scan_part, nullptr, nullptr};
+    const bool one = scan_items(g.n) == 1;
+    const cudaError_t e = one ? launch_after(g.stream, dim3(nb), kBlock, 0, support_tiles_kernel<1>, g.n, h, tiles, count)
+                              : launch_after(g.stream, dim3(nb), kBlock, 0, support_tiles_kernel<kScanItems>, g.n, h,
+                                             tiles, count);
+    if (e != cudaSuccess) return e;
+    return one ? launch_after(g.stream, dim3(nb), kBlock, 0, support_ids_kernel<1>, g.n, h, g.scan_part, ids)
+               : launch_after(g.stream, dim3(nb), kBlock, 0, support_ids_kernel<kScanItems>, g.n, h, g.scan_part, ids);
 }
 
 }  // namespace esim
