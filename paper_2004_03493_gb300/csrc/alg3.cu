@@ -338,7 +338,7 @@ __global__ void __launch_bounds__(kBlock) probe_push_kernel(ProbeGroup G, ProbeS
 // reserves their items with one atomic: with one atomic a row on the block's one counter, and
 // items listed for dense steps too, this kernel took up to 0.55 ms and was the largest of the
 // probes.
-__global__ void __launch_bounds__(kBlock) probe_sparse_epi_kernel(ProbeGroup G, ProbeStepArgs a) {
+__global__ void __launch_bounds__(kBlock, 5) probe_sparse_epi_kernel(ProbeGroup G, ProbeStepArgs a) {
     const int b = blockIdx.y;
     ProbeCtl* ctl = G.ctl + b;
     if (probe_dense_at(ctl, a.s, a.thr)) return;
@@ -870,24 +870,37 @@ __global__ void __launch_bounds__(kCtaThreads) probe_g3_cta_kernel(const unsigne
     }
 }
 
-// *zlast += sum_i (cl Zv(ids[i])) (colsum[i] 2^-63), i < count, in a fixed order: thread t
-// takes i = t, t + 1024, ... and a fixed tree adds the threads' partials.
-__global__ void __launch_bounds__(1024) probe_g2_total_kernel(const uint64_t* __restrict__ count_dev,
-                                                              const int32_t* __restrict__ ids,
-                                                              const double* __restrict__ zv_src, double cl,
-                                                              const unsigned long long* __restrict__ colsum,
-                                                              double* __restrict__ zlast) {
-    __shared__ double red[1024];
+// *zlast += sum_i (cl Zv(ids[i])) (colsum[i] 2^-63), i < count, in a fixed order: every thread
+// strides over the support, fixed trees add a block's threads, and the last block adds the
+// blocks' sums (the ticket wraps to zero).  Blocks of 256 threads, as all kernels that run beside
+// the side sampler: one block of 1024 threads had to wait for its end.
+__global__ void __launch_bounds__(kBlock) probe_g2_total_kernel(const uint64_t* __restrict__ count_dev,
+                                                                const int32_t* __restrict__ ids,
+                                                                const double* __restrict__ zv_src, double cl,
+                                                                const unsigned long long* __restrict__ colsum,
+                                                                double* __restrict__ partial,
+                                                                unsigned* __restrict__ ticket,
+                                                                double* __restrict__ zlast) {
+    __shared__ double red[kBlock / 32];
+    __shared__ bool last;
+    prior_done();
     const int64_t count = (int64_t)*count_dev;
     double t = 0.0;
-    for (int64_t i = threadIdx.x; i < count; i += 1024) t += (cl * zv_src[ids[i]]) * ((double)colsum[i] * kInvOne);
-    red[threadIdx.x] = t;
-    __syncthreads();
-    for (int w = 512; w > 0; w >>= 1) {
-        if ((int)threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-        __syncthreads();
+    for (int64_t i = (int64_t)blockIdx.x * kBlock + threadIdx.x; i < count; i += (int64_t)gridDim.x * kBlock)
+        t += (cl * zv_src[ids[i]]) * ((double)colsum[i] * kInvOne);
+    t = block_sum(t, red);
+    if (threadIdx.x == 0) {
+        partial[blockIdx.x] = t;
+        __threadfence();
+        last = atomicInc(ticket, gridDim.x - 1) == gridDim.x - 1;
+        __threadfence();
     }
-    if (threadIdx.x == 0) *zlast += red[0];
+    __syncthreads();
+    if (!last) return;
+    t = 0.0;
+    for (unsigned i = threadIdx.x; i < gridDim.x; i += kBlock) t += __ldcg(partial + i);
+    t = block_sum(t, red);
+    if (threadIdx.x == 0) *zlast += t;
 }
 
 // D^ of Algorithm 3 for exploited nodes (depth > 0), of Algorithm 2 for the others,
@@ -1206,9 +1219,11 @@ static cudaError_t first_meeting(const Graph& g, int64_t k, int depth, double c,
             ++count;
         }
         if (hashed && nsup > 0) {
-            probe_g2_total_kernel<<<1, 1024, 0, g.stream>>>(ws.nsup, ws.ids, zv, cpow[(size_t)steps], ws.g2,
-                                                            ws.sums + 63);
-            if ((e = cudaGetLastError()) != cudaSuccess) return e;
+            const unsigned blocks = (unsigned)std::min<uint64_t>((nsup + kBlock - 1) / kBlock, (uint64_t)g.sm_count);
+            e = launch_after(g.stream, dim3(blocks), kBlock, 0, probe_g2_total_kernel, ws.nsup, ws.ids, zv,
+                             cpow[(size_t)steps], ws.g2, ws.partial, reinterpret_cast<unsigned*>(ws.sums + 62),
+                             ws.sums + 63);
+            if (e != cudaSuccess) return e;
             ++count;
         }
     }

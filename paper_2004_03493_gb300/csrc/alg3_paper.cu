@@ -15,9 +15,9 @@
 // The supports are bit sets, one row of ceil(n/32) words per node: S_0 is the
 // identity and S_(j+1)(q) = OR over x in I(q) of S_j(x), a pull over the in-edge CSR.
 // A first pass over the levels gives the table e_j(q); a second pass rebuilds S_j and
-// adds each still undecided node's terms.  All counts are integers, so the depths
-// are exact.  The bit sets take 2 n ceil(n/32) words: the rule is offered for graphs
-// whose bit sets fit kPaperBitsBudget.
+// adds each still undecided node's terms (first for levels up to 4, then 8, then 16).
+// All counts are integers, so the depths are exact.  The bit sets take 2 n ceil(n/32)
+// words: the rule is offered for graphs whose bit sets fit kPaperBitsBudget.
 #include "common.cuh"
 #include "internal.h"
 #include "twohop.cuh"
@@ -59,7 +59,25 @@ __global__ void __launch_bounds__(kBlock) bits_step_kernel(int64_t n, int64_t wo
     }
 }
 
-// e(q) = sum of din(x) over the bits x of row q; one warp per row.
+// For every non-zero word of a bit row (words 32-bit words): f(word number, word), the whole warp
+// together.  The words are read 32 at a time, one per lane.
+template <class F>
+__device__ __forceinline__ void each_word(const uint32_t* __restrict__ row, int64_t words, const F& f) {
+    const int lane = threadIdx.x & 31;
+    for (int64_t w0 = 0; w0 < words; w0 += 32) {
+        const uint32_t mine = w0 + lane < words ? row[w0 + lane] : 0u;
+        unsigned some = __ballot_sync(0xffffffffu, mine != 0u);
+        while (some) {
+            const int t = __ffs(some) - 1;
+            some &= some - 1u;
+            f(w0 + t, __shfl_sync(0xffffffffu, mine, t));
+        }
+    }
+}
+
+// e(q) = sum of din(x) over the bits x of row q; one warp per row, lane b of a word's turn adds
+// bit b's node: the 32 in-degrees are one coalesced load.  With each lane walking the bits of its
+// own words, one dependent load a bit, this took 56 us a level at n = 3001 (WEIGHTUS now).
 __global__ void __launch_bounds__(kBlock) bits_weight_kernel(int64_t n, int64_t words, const uint32_t* __restrict__ B,
                                                             const uint32_t* __restrict__ rp,
                                                             unsigned long long* __restrict__ e) {
@@ -67,14 +85,10 @@ __global__ void __launch_bounds__(kBlock) bits_weight_kernel(int64_t n, int64_t 
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
     for (int64_t q = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); q < n; q += warps) {
         unsigned long long sum = 0;
-        for (int64_t w = lane; w < words; w += 32) {
-            uint32_t bits = B[q * words + w];
-            while (bits) {
-                const int64_t x = w * 32 + (__ffs(bits) - 1);
-                sum += rp[x + 1] - rp[x];
-                bits &= bits - 1;
-            }
-        }
+        each_word(B + q * words, words, [&](int64_t w, uint32_t bits) {
+            const int64_t x = w * 32 + lane;
+            if (bits >> lane & 1u) sum += rp[x + 1] - rp[x];
+        });
         sum = warp_sum_u64(sum);
         if (lane == 0) e[q] = sum;
     }
@@ -103,13 +117,9 @@ __global__ void __launch_bounds__(kBlock) paper_level_kernel(int count, const in
         const int t = (int)(it % terms);
         const unsigned long long* et = etab + (int64_t)t * n;
         unsigned long long sum = 0;
-        for (int64_t w = lane; w < words; w += 32) {
-            uint32_t bits = B[k * words + w];
-            while (bits) {
-                sum += et[w * 32 + (__ffs(bits) - 1)];
-                bits &= bits - 1;
-            }
-        }
+        each_word(B + k * words, words, [&](int64_t w, uint32_t bits) {
+            if (bits >> lane & 1u) sum += et[w * 32 + lane];
+        });
         sum = warp_sum_u64(sum);
         if (lane == 0) W[(int64_t)(j + t) * n + k] += sum;
     }
@@ -249,48 +259,71 @@ cudaError_t alg3_paper_depths(const Graph& g, const uint64_t* R, double c, int m
     const int ib = (int)std::max<int64_t>(1, std::min<int64_t>((n * words + kBlock - 1) / kBlock,
                                                                 (int64_t)g.sm_count * 16));
     const int rb = grid_for(g, n);
-    // pass 1: e_j(q) for j = 0..D
-    bits_identity_kernel<<<ib, kBlock, 0, st>>>(n, words, B0);
-    bits_weight_kernel<<<rb, kBlock, 0, st>>>(n, words, B0, g.in.rp, etab);
-    nl += 2;
-    uint32_t* cur = B0;
-    uint32_t* nxt = B1;
-    for (int j = 1; j <= D; ++j) {
-        bits_step_kernel<<<rb, kBlock, 0, st>>>(n, words, g.in.rp, g.in.col, cur, nxt);
-        bits_weight_kernel<<<rb, kBlock, 0, st>>>(n, words, nxt, g.in.rp, etab + (size_t)j * n);
-        std::swap(cur, nxt);
-        nl += 2;
-    }
-    // pass 2: the levels again, the undecided nodes' counts and decisions
-    cudaError_t e = cudaMemsetAsync(W, 0, (size_t)(D + 1) * n * 8, st);
+    // pass 2's undecided nodes
+    cudaError_t e = cudaMemsetAsync(C, 0, (size_t)n * 8, st);
     if (e != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(C, 0, (size_t)n * 8, st)) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(counts, 0, 256, st)) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(depth, 0, (size_t)n, st)) != cudaSuccess) return e;
     paper_alive_kernel<<<rb, kBlock, 0, st>>>(n, R, alive[0], counts);
-    bits_identity_kernel<<<ib, kBlock, 0, st>>>(n, words, B0);
-    nl += 2;
-    cur = B0;
-    nxt = B1;
+    ++nl;
     unsigned count = 0;
-    if ((e = cudaMemcpyAsync(&count, counts, sizeof(unsigned), cudaMemcpyDeviceToHost, st)) != cudaSuccess) return e;
-    if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;
-    for (int j = 0; j <= D && count > 0; ++j) {
-        if (j > 0) {
-            bits_step_kernel<<<rb, kBlock, 0, st>>>(n, words, g.in.rp, g.in.col, cur, nxt);
-            std::swap(cur, nxt);
+    // A decision at level l needs the tables e_0 .. e_l only, and most nodes stop within a few
+    // levels: the tables are made up to level 4, then 8, then 16, and the nodes still undecided
+    // after them start again (their counts with them).
+    uint32_t* cur = B0;
+    uint32_t* nxt = B1;
+    int have = -1;  // tables e_0 .. e_have
+    for (int upto = std::min(D, 4); ; upto = std::min(D, 2 * upto)) {
+        // pass 1: e_j(q) for j = 0..upto
+        bits_identity_kernel<<<ib, kBlock, 0, st>>>(n, words, B0);
+        ++nl;
+        cur = B0;
+        nxt = B1;
+        for (int j = 0; j <= upto; ++j) {
+            if (j > 0) {
+                bits_step_kernel<<<rb, kBlock, 0, st>>>(n, words, g.in.rp, g.in.col, cur, nxt);
+                std::swap(cur, nxt);
+                ++nl;
+            }
+            if (j <= have) continue;
+            bits_weight_kernel<<<rb, kBlock, 0, st>>>(n, words, cur, g.in.rp, etab + (size_t)j * n);
             ++nl;
         }
-        const int a = j & 1;
-        paper_level_kernel<<<grid_for(g, (int64_t)count * (D - j + 1)), kBlock, 0, st>>>(
-            (int)count, alive[a], n, words, cur, etab, j, D, W);
-        paper_decide_kernel<<<(count + kBlock - 1) / kBlock, kBlock, 0, st>>>(
-            (int)count, alive[a], n, j, D, sqrt(c), R, W, C, depth, alive[a ^ 1], counts + (j + 1));
-        nl += 2;
-        if ((e = cudaMemcpyAsync(&count, counts + (j + 1), sizeof(unsigned), cudaMemcpyDeviceToHost, st)) !=
+        have = upto;
+        // pass 2: the levels again, the undecided nodes' counts and decisions
+        if ((e = cudaMemsetAsync(W, 0, (size_t)(upto + 1) * n * 8, st)) != cudaSuccess) return e;
+        if ((e = cudaMemsetAsync(C, 0, (size_t)n * 8, st)) != cudaSuccess) return e;
+        if ((e = cudaMemsetAsync(counts + 1, 0, 256 - sizeof(unsigned), st)) != cudaSuccess) return e;
+        bits_identity_kernel<<<ib, kBlock, 0, st>>>(n, words, B0);
+        ++nl;
+        cur = B0;
+        nxt = B1;
+        if ((e = cudaMemcpyAsync(&count, counts, sizeof(unsigned), cudaMemcpyDeviceToHost, st)) != cudaSuccess) return e;
+        if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;
+        int in = 0;
+        for (int j = 0; j <= upto && count > 0; ++j) {
+            if (j > 0) {
+                bits_step_kernel<<<rb, kBlock, 0, st>>>(n, words, g.in.rp, g.in.col, cur, nxt);
+                std::swap(cur, nxt);
+                ++nl;
+            }
+            paper_level_kernel<<<grid_for(g, (int64_t)count * (upto - j + 1)), kBlock, 0, st>>>(
+                (int)count, alive[in], n, words, cur, etab, j, upto, W);
+            paper_decide_kernel<<<(count + kBlock - 1) / kBlock, kBlock, 0, st>>>(
+                (int)count, alive[in], n, j, D, sqrt(c), R, W, C, depth, alive[in ^ 1], counts + (j + 1));
+            in ^= 1;
+            nl += 2;
+            if ((e = cudaMemcpyAsync(&count, counts + (j + 1), sizeof(unsigned), cudaMemcpyDeviceToHost, st)) !=
+                cudaSuccess)
+                return e;
+            if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;
+        }
+        if (count == 0 || upto == D) break;
+        // the undecided ones are the next round's start
+        if (in != 0) std::swap(alive[0], alive[1]);
+        if ((e = cudaMemcpyAsync(counts, counts + (upto + 1), sizeof(unsigned), cudaMemcpyDeviceToDevice, st)) !=
             cudaSuccess)
             return e;
-        if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;
     }
     if (launches) *launches += nl;
     return cudaGetLastError();

@@ -323,8 +323,10 @@ __device__ __forceinline__ uint32_t segment_node(unsigned long long seg, unsigne
 // stream per thread over a (rowptr, col) CSR, which this replaces, took 130 instructions and
 // two dependent loads per walk and step, and a fixed share of the pairs per thread: 11.8 ms
 // there, and 207 against 122 ms on a batch of 64 sources.
-// Six blocks of 256 threads per SM measured as 5 (8.4 against 8.5 ms) and leave the side
-// launch's register share as it was.
+// Eight blocks of 192 threads fill an SM as six of 256 do (8.32 and 8.36 ms).  The smaller ones
+// leave the planning room beside four or five of them: with five, the n = 1e5 top-50 query
+// takes 39.0 against 43.4 ms, with four 38.5 against 39.0.
+constexpr int kWalkBlock = 192;
 constexpr uint32_t kRunMin = 128;        // shortest run of one segment that gets a loop of its own
 constexpr uint32_t kChunkMin = 256;      // pairs per chunk where there are many
 constexpr uint32_t kChunkMax = 16384;    // few enough that the warps finish together
@@ -429,7 +431,7 @@ __device__ __forceinline__ uint32_t run_one(const WalkArgs& a, uint32_t k, uint2
     // While 32 more pairs are left every lane has one, and before iteration 65535 no pair is
     // that long: neither is tested here.
     uint32_t it = 0;
-    for (; next + 32 <= len && it < kWalkMaxSteps - 1; ++it) {
+    auto step = [&]() {
         const uint4 w = words();
         const bool cont = walk_move<kNarrow>(w, kForced && t < d, a.T, A, B, rlo, rhi, k, t, a.walk, K);
         const bool go = cont & !same_node<kNarrow>(A, B);
@@ -439,7 +441,13 @@ __device__ __forceinline__ uint32_t run_one(const WalkArgs& a, uint32_t k, uint2
         ++t;
         if (!go) restart(next + __popc(done & lanes_below()));
         next += __popc(done);
-    }
+    };
+    if (!kForced)  // two steps a turn: 1.5 % less (forced pairs are slower for it)
+        for (; next + 64 <= len && it < kWalkMaxSteps - 2; it += 2) {
+            step();
+            step();
+        }
+    for (; next + 32 <= len && it < kWalkMaxSteps - 1; ++it) step();
     steps += it;
     bool active = rlo - rlo0 < len;
     while (__any_sync(0xffffffffu, active)) {
@@ -575,19 +583,24 @@ __device__ __forceinline__ unsigned long long run_many(const WalkArgs& a, unsign
 
 // Persistent walk-pair sampler (see above).  work: the chunk counter, zero before and
 // after the launch (the last block to finish clears it); ticket likewise.
-template <bool kNarrow>
-__global__ void __launch_bounds__(kBlock, 6) sample_pairs_kernel(const __grid_constant__ WalkArgs a, const __grid_constant__ PhiloxKeys K,
+// kSide: the launch beside the planning's kernels, a function of its own for its carve-out.  An SM
+// divides its L1 and shared memory when a block comes to it idle, and a block that needs more
+// shared memory than the division gives waits until the SM is idle again.  The sampler uses
+// next to none and stays for the whole launch, so with the division left to it every planning
+// kernel with tables in shared memory waited for its end and nothing overlapped.
+template <bool kNarrow, bool kSide>
+__global__ void __launch_bounds__(kWalkBlock, 8) sample_pairs_kernel(const __grid_constant__ WalkArgs a, const __grid_constant__ PhiloxKeys K,
                                                                  double budget,
                                                                  unsigned long long* __restrict__ steps_out,
                                                                  Status* __restrict__ st, SampleWork* __restrict__ work) {
-    __shared__ unsigned long long wsteps[kBlock / 32];
+    __shared__ unsigned long long wsteps[kWalkBlock / 32];
     unsigned long long total = __ldg(a.off + a.nseg);
     if ((double)total > budget || (st->err & kErrBudget)) {
         if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&st->err, kErrBudget);
         total = 0ull;  // no walks; the block still counts itself in the ticket below
     }
     const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const unsigned long long nwarps = (unsigned long long)gridDim.x * (kBlock / 32);
+    const unsigned long long nwarps = (unsigned long long)gridDim.x * (kWalkBlock / 32);
     // A few pairs are spread over all warps, 32 or more each: the launch then lasts as long as
     // its longest pair (18,000 pairs: the query takes 329 us, 370 with chunks of 256).  Many go
     // in chunks of at least kChunkMin, which pay for the search for their segment, about
@@ -636,7 +649,7 @@ __global__ void __launch_bounds__(kBlock, 6) sample_pairs_kernel(const __grid_co
     __syncthreads();
     if (threadIdx.x == 0) {
         unsigned long long s = 0;
-        for (int w = 0; w < kBlock / 32; ++w) s += wsteps[w];
+        for (int w = 0; w < kWalkBlock / 32; ++w) s += wsteps[w];
         if (s) atomicAdd(steps_out, s);
         if (atomicInc(&work->done, gridDim.x - 1) == gridDim.x - 1) work->next = 0ull;  // every chunk was taken
     }
@@ -757,7 +770,7 @@ cudaError_t launch_sample_segments(const Graph& g, int64_t nseg, const uint64_t*
     }
     if (g_sample_blocks_per_sm == 0) {
         int b = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, sample_pairs_kernel<true>, kBlock, 0);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, (sample_pairs_kernel<true, false>), kWalkBlock, 0);
         if (e != cudaSuccess) return e;
         g_sample_blocks_per_sm = b > 0 ? b : 1;
     }
@@ -766,10 +779,14 @@ cudaError_t launch_sample_segments(const Graph& g, int64_t nseg, const uint64_t*
     const unsigned blocks = (unsigned)(g.sm_count * per_sm);
     const WalkArgs a{g.in.info, g.in.walk, off, depth, (unsigned long long*)nonmeet, (uint64_t)nseg, (uint64_t)g.n,
                      SharedSegs{rbase ? shared_B : 0, rbase}, walk_threshold(c)};
-    // the side launch may run beside a launch on the query's own stream: each has its counter
-    SampleWork* work = &g.status->work[steps == &g.status->pair_steps_side ? 1 : 0];
-    auto* kernel = walk_narrow(g) ? sample_pairs_kernel<true> : sample_pairs_kernel<false>;
-    kernel<<<blocks, kBlock, 0, g.stream>>>(a, philox_keys(seed), g.pair_budget, steps, g.status, work);
+    const bool side = steps == &g.status->pair_steps_side;  // it may run beside a launch on the query's own stream
+    SampleWork* work = &g.status->work[side ? 1 : 0];
+    auto* kernel = walk_narrow(g) ? (side ? sample_pairs_kernel<true, true> : sample_pairs_kernel<true, false>)
+                                  : (side ? sample_pairs_kernel<false, true> : sample_pairs_kernel<false, false>);
+    if (side && (e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                          cudaSharedmemCarveoutMaxShared)) != cudaSuccess)
+        return e;
+    kernel<<<blocks, kWalkBlock, 0, g.stream>>>(a, philox_keys(seed), g.pair_budget, steps, g.status, work);
     return cudaGetLastError();
 }
 
