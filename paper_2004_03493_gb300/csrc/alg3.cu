@@ -234,6 +234,7 @@ __device__ __forceinline__ void probe_flush_colsum(unsigned long long v, unsigne
 // sources, their work items, fresh counters and column sums.
 __global__ void probe_init_kernel(ProbeGroup G, const int32_t* __restrict__ ids, int count,
                                   const uint32_t* __restrict__ in_rp, unsigned long long thr) {
+    prior_done();
     const int b = blockIdx.y, lane = threadIdx.x;
     ProbeCtl* ctl = G.ctl + b;
     uint32_t* z = (uint32_t*)ctl;
@@ -278,6 +279,7 @@ __global__ void probe_init_kernel(ProbeGroup G, const int32_t* __restrict__ ids,
 // coef(b, col) = c^{l'} Zv_i(q'_col); 0 for unused columns
 __global__ void probe_coef_kernel(ProbeGroup G, const int32_t* __restrict__ ids, int count,
                                   const double* __restrict__ zv_src, double cl) {
+    prior_done();
     const int i = blockIdx.y * kProbeW + threadIdx.x;
     G.coef[i] = i < count ? cl * zv_src[ids[i]] : 0.0;
 }
@@ -286,6 +288,7 @@ __global__ void probe_coef_kernel(ProbeGroup G, const int32_t* __restrict__ ids,
 // all 32 columns; each lane marks one entry's row and the new rows are appended to
 // F_{s+1} with one atomic per warp.
 __global__ void __launch_bounds__(kBlock) probe_push_kernel(ProbeGroup G, ProbeStepArgs a) {
+    prior_done();
     const int b = blockIdx.y;
     ProbeCtl* ctl = G.ctl + b;
     if (probe_dense_at(ctl, a.s, a.thr)) return;
@@ -339,6 +342,7 @@ __global__ void __launch_bounds__(kBlock) probe_push_kernel(ProbeGroup G, ProbeS
 // items listed for dense steps too, this kernel took up to 0.55 ms and was the largest of the
 // probes.
 __global__ void __launch_bounds__(kBlock, 5) probe_sparse_epi_kernel(ProbeGroup G, ProbeStepArgs a) {
+    prior_done();
     const int b = blockIdx.y;
     ProbeCtl* ctl = G.ctl + b;
     if (probe_dense_at(ctl, a.s, a.thr)) return;
@@ -433,14 +437,15 @@ __device__ __forceinline__ unsigned long long probe_range(const int32_t* __restr
 }
 
 // Dense step: h(i, col) = sum_{j in Out(i)} x_s(j, col), a pull over the out-edge CSR
-// for 32 columns at once.  Short rows: one warp per row, lane = column.  Long rows:
-// one block per 4096-entry segment, each warp adding a contiguous eighth of it into
-// the segment's partial; probe_long_rows_kernel adds a row's partials.
+// for 32 columns at once.  Short rows: one warp per row, lane = column.  Rows of long_min
+// entries or more: one block per segment, each warp adding a contiguous eighth of it; a row of
+// one segment is finished there, probe_long_rows_kernel adds the partials of the others.
 __global__ void __launch_bounds__(kBlock) probe_rows_kernel(ProbeGroup G, ProbeStepArgs a,
                                                             const uint32_t* __restrict__ rp,
                                                             const int32_t* __restrict__ col, uint32_t long_min,
                                                             int64_t nseg, const Segment* __restrict__ seg,
                                                             int short_blocks) {
+    prior_done();
     constexpr int kWarps = kBlock / 32;
     const int b = blockIdx.y;
     ProbeCtl* ctl = G.ctl + b;
@@ -454,6 +459,8 @@ __global__ void __launch_bounds__(kBlock) probe_rows_kernel(ProbeGroup G, ProbeS
     if ((int)blockIdx.x >= short_blocks) {
         __shared__ unsigned long long red[kWarps][kProbeW];
         unsigned long long* partial = G.ppart + (size_t)b * G.np;
+        unsigned long long* Xnext = G.X[a.src ^ 1] + (size_t)b * G.nx;
+        unsigned long long nacc = 0ull;
         const int64_t nsb = (int64_t)gridDim.x - short_blocks;
         for (int64_t s = (int64_t)blockIdx.x - short_blocks; s < nseg; s += nsb) {  // uniform per block
             const Segment sg = seg[s];
@@ -467,10 +474,13 @@ __global__ void __launch_bounds__(kBlock) probe_rows_kernel(ProbeGroup G, ProbeS
                 unsigned long long t = 0ull;
 #pragma unroll
                 for (int w = 0; w < kWarps; ++w) t += red[w][lane];
-                partial[(size_t)s * kProbeW + lane] = t;
+                if (sg.end - sg.beg == __ldg(rp + sg.row + 1) - __ldg(rp + sg.row))
+                    nacc += probe_row_out(sg.row, t, lane, a, Xnext, G.coef + (size_t)b * kProbeW);
+                else partial[(size_t)s * kProbeW + lane] = t;
             }
             __syncthreads();
         }
+        if (a.mode == 2) probe_flush_colsum(nacc, G.colsum + (size_t)b * kProbeW);
         return;
     }
     unsigned long long* Xnext = G.X[a.src ^ 1] + (size_t)b * G.nx;
@@ -487,7 +497,9 @@ __global__ void __launch_bounds__(kBlock) probe_rows_kernel(ProbeGroup G, ProbeS
 
 __global__ void __launch_bounds__(kBlock) probe_long_rows_kernel(ProbeGroup G, ProbeStepArgs a, int64_t nlong,
                                                                  const int32_t* __restrict__ long_rows,
-                                                                 const int32_t* __restrict__ long_first) {
+                                                                 const int32_t* __restrict__ long_first,
+                                                                 const uint32_t* __restrict__ rp, uint32_t seg_len) {
+    prior_done();
     const int b = blockIdx.y;
     if (!probe_dense_at(G.ctl + b, a.s, a.thr)) return;
     const int lane = threadIdx.x & 31;
@@ -498,8 +510,10 @@ __global__ void __launch_bounds__(kBlock) probe_long_rows_kernel(ProbeGroup G, P
     unsigned long long nacc = 0ull;
     if (w < nlong) {  // warp-uniform
         unsigned long long acc = 0ull;
-        for (int32_t s = long_first[w]; s < long_first[w + 1]; ++s) acc += partial[(size_t)s * kProbeW + lane];
-        nacc = probe_row_out(long_rows[w], acc, lane, a, Xnext, coef);
+        const int32_t row = long_rows[w], first = long_first[w];
+        const int32_t count = (int32_t)((rp[row + 1] - rp[row] + seg_len - 1) / seg_len);
+        for (int32_t s = first; s < first + count; ++s) acc += partial[(size_t)s * kProbeW + lane];
+        nacc = probe_row_out(row, acc, lane, a, Xnext, coef);
     }
     if (a.mode == 2) probe_flush_colsum(nacc, G.colsum + (size_t)b * kProbeW);
 }
@@ -509,6 +523,7 @@ __global__ void __launch_bounds__(kBlock) probe_long_rows_kernel(ProbeGroup G, P
 __global__ void probe_end_kernel(ProbeGroup G, const int32_t* __restrict__ ids, int count,
                                  const double* __restrict__ zv_src, double cl, double* __restrict__ zlast,
                                  const int32_t* __restrict__ pos, unsigned long long* __restrict__ colsum_out) {
+    prior_done();
     if (blockIdx.x == 0 && blockIdx.y == 0) {
         if (colsum_out) {  // the caller sums the terms: hand over the column sums
             for (int i = threadIdx.x; i < count; i += blockDim.x) colsum_out[pos[i]] = G.colsum[i];
@@ -1030,29 +1045,27 @@ size_t a3_layout(int64_t n_, int64_t m_, int64_t nseg, void* base, A3Ws* out) {
 cudaError_t probe_step(const Graph& g, const A3Ws& ws, const ProbeStepArgs& a, int nb, int* count) {
     const DevCsr& A = g.out;
     const unsigned sparse_blocks = (unsigned)std::max(1, g.sm_count * 4 / nb);
-    probe_push_kernel<<<dim3(sparse_blocks, (unsigned)nb), kBlock, 0, g.stream>>>(ws.G, a);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_after(g.stream, dim3(sparse_blocks, (unsigned)nb), kBlock, 0, probe_push_kernel, ws.G, a);
     if (e != cudaSuccess) return e;
-    const int wpb = kBlock / 32;
-    int64_t sb = (g.n + wpb - 1) / wpb;
-    if (sb > (int64_t)g.sm_count * 16) sb = (int64_t)g.sm_count * 16;
-    if (sb < 1) sb = 1;
-    int64_t segb = A.nseg;  // one block per segment
-    if (segb > (int64_t)g.sm_count * 8) segb = (int64_t)g.sm_count * 8;
-    probe_rows_kernel<<<dim3((unsigned)(sb + segb), (unsigned)nb), kBlock, 0, g.stream>>>(
-        ws.G, a, A.rp, A.col, A.long_min, A.nseg, A.seg, (int)sb);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    // The chip's worth of blocks over all nb of them, not per probe block: most launches find
+    // their blocks on the other form, and 30,000 blocks took 15 us just to leave (mean of all
+    // launches of an n = 1e5 query: 26.6 us with 16 blocks per SM and probe block, 12.9 now).
+    int64_t sb = std::max(1, g.sm_count * 8 / nb);
+    sb = std::min<int64_t>(sb, (g.n + kBlock / 32 - 1) / (kBlock / 32));
+    const int64_t segb = std::min<int64_t>(A.nseg, std::max(1, g.sm_count * 4 / nb));
+    e = launch_after(g.stream, dim3((unsigned)(sb + segb), (unsigned)nb), kBlock, 0, probe_rows_kernel, ws.G, a, A.rp,
+                     A.col, A.long_min, A.nseg, A.seg, (int)sb);
+    if (e != cudaSuccess) return e;
     *count += 2;
     if (A.nlong > 0) {
         const int64_t blocks = (A.nlong * 32 + kBlock - 1) / kBlock;
-        probe_long_rows_kernel<<<dim3((unsigned)blocks, (unsigned)nb), kBlock, 0, g.stream>>>(ws.G, a, A.nlong,
-                                                                                              A.long_rows, A.long_first);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        e = launch_after(g.stream, dim3((unsigned)blocks, (unsigned)nb), kBlock, 0, probe_long_rows_kernel, ws.G, a,
+                         A.nlong, A.long_rows, A.long_first, A.rp, A.seg_len);
+        if (e != cudaSuccess) return e;
         ++*count;
     }
-    probe_sparse_epi_kernel<<<dim3(sparse_blocks, (unsigned)nb), kBlock, 0, g.stream>>>(ws.G, a);
     ++*count;
-    return cudaGetLastError();
+    return launch_after(g.stream, dim3(sparse_blocks, (unsigned)nb), kBlock, 0, probe_sparse_epi_kernel, ws.G, a);
 }
 
 }  // namespace
@@ -1195,8 +1208,9 @@ static cudaError_t first_meeting(const Graph& g, int64_t k, int depth, double c,
             const int cnt = (int)std::min<uint64_t>(per_group, nprobe - g0);
             const int nb = (cnt + kProbeW - 1) / kProbeW;
             const int32_t* ids = probe_ids + g0;
-            probe_init_kernel<<<dim3(1, (unsigned)nb), kProbeW, 0, g.stream>>>(ws.G, ids, cnt, g.in.rp, thr);
-            if ((e = cudaGetLastError()) != cudaSuccess) return e;
+            if ((e = launch_after(g.stream, dim3(1, (unsigned)nb), kProbeW, 0, probe_init_kernel, ws.G, ids, cnt, g.in.rp,
+                                  thr)) != cudaSuccess)
+                return e;
             ++count;
             for (int lp = 1; lp <= steps; ++lp) {
                 ProbeStepArgs a{g.in.rp, g.in.col, g.din_magic, lp - 1, (lp - 1) & 1, 0, lp == steps ? 1 : 0,
@@ -1204,18 +1218,18 @@ static cudaError_t first_meeting(const Graph& g, int64_t k, int depth, double c,
                 if (lp == steps) {
                     a.mode = 2;
                 } else if (lp >= 2) {
-                    probe_coef_kernel<<<dim3(1, (unsigned)nb), kProbeW, 0, g.stream>>>(ws.G, ids, cnt, zv,
-                                                                                       cpow[(size_t)lp]);
-                    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+                    if ((e = launch_after(g.stream, dim3(1, (unsigned)nb), kProbeW, 0, probe_coef_kernel, ws.G, ids, cnt,
+                                          zv, cpow[(size_t)lp])) != cudaSuccess)
+                        return e;
                     ++count;
                     a.mode = 1;
                 }
                 if ((e = probe_step(g, ws, a, nb, &count)) != cudaSuccess) return e;
             }
-            probe_end_kernel<<<dim3((unsigned)g.sm_count, (unsigned)nb), kBlock, 0, g.stream>>>(
-                ws.G, ids, cnt, zv, cpow[(size_t)steps], ws.sums + 63, hashed ? ws.big2_pos + g0 : nullptr,
-                hashed ? ws.g2 : nullptr);
-            if ((e = cudaGetLastError()) != cudaSuccess) return e;
+            if ((e = launch_after(g.stream, dim3((unsigned)g.sm_count, (unsigned)nb), kBlock, 0, probe_end_kernel, ws.G, ids,
+                                  cnt, zv, cpow[(size_t)steps], ws.sums + 63, hashed ? ws.big2_pos + g0 : nullptr,
+                                  hashed ? ws.g2 : nullptr)) != cudaSuccess)
+                return e;
             ++count;
         }
         if (hashed && nsup > 0) {

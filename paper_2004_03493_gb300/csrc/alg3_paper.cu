@@ -59,20 +59,33 @@ __global__ void __launch_bounds__(kBlock) bits_step_kernel(int64_t n, int64_t wo
     }
 }
 
-// For every non-zero word of a bit row (words 32-bit words): f(word number, word), the whole warp
-// together.  The words are read 32 at a time, one per lane.
+// Sum over the set bits of a bit row (words 32-bit words) of value(bit number), per lane: lane b
+// takes bit b of every word.  The words are read 32 at a time, one per lane, and the values of
+// four non-zero words are in flight together.
 template <class F>
-__device__ __forceinline__ void each_word(const uint32_t* __restrict__ row, int64_t words, const F& f) {
+__device__ __forceinline__ unsigned long long sum_bits(const uint32_t* __restrict__ row, int64_t words, const F& value) {
+    constexpr int kU = 4;
     const int lane = threadIdx.x & 31;
+    unsigned long long sum = 0;
     for (int64_t w0 = 0; w0 < words; w0 += 32) {
         const uint32_t mine = w0 + lane < words ? row[w0 + lane] : 0u;
         unsigned some = __ballot_sync(0xffffffffu, mine != 0u);
         while (some) {
-            const int t = __ffs(some) - 1;
-            some &= some - 1u;
-            f(w0 + t, __shfl_sync(0xffffffffu, mine, t));
+            unsigned long long v[kU];
+#pragma unroll
+            for (int u = 0; u < kU; ++u) {
+                v[u] = 0;
+                if (some) {
+                    const int t = __ffs(some) - 1;
+                    some &= some - 1u;
+                    if (__shfl_sync(0xffffffffu, mine, t) >> lane & 1u) v[u] = value((w0 + t) * 32 + lane);
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < kU; ++u) sum += v[u];
         }
     }
+    return sum;
 }
 
 // e(q) = sum of din(x) over the bits x of row q; one warp per row, lane b of a word's turn adds
@@ -84,12 +97,8 @@ __global__ void __launch_bounds__(kBlock) bits_weight_kernel(int64_t n, int64_t 
     const int lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
     for (int64_t q = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); q < n; q += warps) {
-        unsigned long long sum = 0;
-        each_word(B + q * words, words, [&](int64_t w, uint32_t bits) {
-            const int64_t x = w * 32 + lane;
-            if (bits >> lane & 1u) sum += rp[x + 1] - rp[x];
-        });
-        sum = warp_sum_u64(sum);
+        const unsigned long long sum = warp_sum_u64(
+            sum_bits(B + q * words, words, [&](int64_t x) { return (unsigned long long)(rp[x + 1] - rp[x]); }));
         if (lane == 0) e[q] = sum;
     }
 }
@@ -116,11 +125,7 @@ __global__ void __launch_bounds__(kBlock) paper_level_kernel(int count, const in
         const int64_t k = alive[it / terms];
         const int t = (int)(it % terms);
         const unsigned long long* et = etab + (int64_t)t * n;
-        unsigned long long sum = 0;
-        each_word(B + k * words, words, [&](int64_t w, uint32_t bits) {
-            if (bits >> lane & 1u) sum += et[w * 32 + lane];
-        });
-        sum = warp_sum_u64(sum);
+        const unsigned long long sum = warp_sum_u64(sum_bits(B + k * words, words, [&](int64_t x) { return et[x]; }));
         if (lane == 0) W[(int64_t)(j + t) * n + k] += sum;
     }
 }

@@ -55,15 +55,16 @@ void free_csr(DevCsr& c) {
     c = DevCsr{};
 }
 
-constexpr uint32_t kSegLen = 4096;
+constexpr uint32_t kSegLen = 4096;         // probe sweeps: entries a block adds, an eighth of them each warp
+constexpr uint32_t kProbeLongMin = 512;    // shortest row of a block; 1024/64, 2048/128, 1024/256 measured the same
 constexpr int64_t kLongRowsFrom = 4000000;  // from this many edges on a level is no longer one row's latency
 
 // Upload a host CSR and build its row-split table.
 esim_status upload_csr(int64_t n, const std::vector<uint32_t>& rp, const int32_t* col, DevCsr& d,
                        bool with_info, const std::vector<uint32_t>& uses_rp, cudaStream_t stream) {
     const int64_t m = (int64_t)rp[n];
-    const double avg = (double)m / (double)n;
-    d.long_min = avg > 12.0 ? (avg > 24.0 ? 1024u : 512u) : 256u;
+    d.long_min = kProbeLongMin;
+    d.seg_len = kSegLen;
     d.sell.row_cap = m >= kLongRowsFrom ? 64u : 32u;
     std::vector<Segment> seg, bseg, pieces;
     std::vector<int32_t> piece_rows, piece_first;  // not kept: a piece names its row and its row's first piece
@@ -78,7 +79,8 @@ esim_status upload_csr(int64_t n, const std::vector<uint32_t>& rp, const int32_t
     };
     for (int64_t r = 0; r < n; ++r) {
         const uint32_t len = rp[r + 1] - rp[r];
-        if (len >= d.long_min) cut(r, kSegLen, seg, long_rows, long_first);
+        if (len > kSegLen) cut(r, kSegLen, seg, long_rows, long_first);
+        else if (len >= d.long_min) seg.push_back(Segment{(int32_t)r, rp[r], rp[r + 1], (uint32_t)seg.size()});
         if (len >= kBatchSeg) cut(r, kBatchSeg, bseg, blong_rows, blong_first);
         if (len > d.sell.row_cap) cut(r, 32 * d.sell.row_cap, pieces, piece_rows, piece_first);
     }

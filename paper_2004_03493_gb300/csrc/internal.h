@@ -79,8 +79,8 @@ __host__ __device__ inline int64_t at_pos(const uint32_t* pos, int64_t i) { retu
 
 constexpr int kSellWindow = 1024;           // rows sorted by length together
 
-// A CSR resident on the device, with the row-split table of the probe sweeps for rows whose
-// length is at least `long_min`.  Long rows are cut into segments of `seg_len` entries.
+// A CSR resident on the device, with the segments of the probe sweeps: a row of long_min
+// entries or more is one, a row of more than seg_len several (those rows are in long_rows).
 struct DevCsr {
     uint32_t* rp = nullptr;      // n+1
     int32_t* col = nullptr;      // m
@@ -88,10 +88,11 @@ struct DevCsr {
     uint2* walk = nullptr;       // max(m, n): info of the node behind each in-edge (walks)
     Segment* seg = nullptr;      // nseg
     int32_t* long_rows = nullptr;  // nlong row ids
-    int32_t* long_first = nullptr; // nlong+1: first segment of each long row
+    int32_t* long_first = nullptr; // nlong: first segment of each long row
     int64_t nseg = 0;
     int64_t nlong = 0;
     uint32_t long_min = 0;
+    uint32_t seg_len = 0;
     SellRows sell;
     // The batched sweeps' segments: rows of kBatchSeg entries or more in pieces of kBatchSeg.
     Segment* bseg = nullptr;
