@@ -925,7 +925,7 @@ __global__ void dhat_alg3_kernel(int64_t n, const uint64_t* __restrict__ counts,
                                  const uint32_t* __restrict__ in_rp, double c, double* __restrict__ dhat) {
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
         const uint64_t R = off[k + 1] - off[k];
-        const double ratio = R ? (double)counts[k] / (double)R : 0.0;
+        const double ratio = pair_ratio(counts[k], R);
         double d = ratio;
         const unsigned dk = depth[k];
         if (dk) {

@@ -133,6 +133,7 @@ __global__ void __launch_bounds__(kBlock) batch_rows_kernel(int64_t n, const uin
     constexpr int W = LPR * CPL;
     constexpr int RPW = 32 / LPR;  // rows (or segments) per warp per iteration
     constexpr int kU = sizeof(V) * CPL <= 16 ? 8 : (sizeof(V) * CPL <= 32 ? 4 : 2);
+    prior_done();
     const int lane = threadIdx.x & 31;
     const int sub = lane / LPR, cl = lane % LPR;
     const int c0 = cl * CPL;
@@ -209,10 +210,11 @@ __global__ void __launch_bounds__(4 * W) batch_long_rows_kernel(const int32_t* _
                                                                 const int32_t* __restrict__ long_first,
                                                                 const f2* __restrict__ partial, Op op) {
     __shared__ f2 part[4][W];
+    prior_done();
     const int q = threadIdx.x % W, g = threadIdx.x / W;
     const int32_t first = long_first[blockIdx.x], end = long_first[blockIdx.x + 1];
     f2 acc[1] = {f2{0.f, 0.f}};
-    constexpr int kU = 4;
+    constexpr int kU = 16;  // a hub's partials in flight
     for (int32_t s = first + g; s < end; s += 4 * kU) {
         f2 v[kU];
 #pragma unroll
@@ -233,6 +235,7 @@ __global__ void __launch_bounds__(4 * W) batch_long_rows_kernel(const int32_t* _
 __global__ void batch_forward_init_kernel(int64_t n, int W, int B, const int64_t* __restrict__ u, float a,
                                           const uint32_t* __restrict__ in_rp, float* __restrict__ hist0,
                                           float* __restrict__ x0) {
+    prior_done();
     const int64_t total = n * W;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
         const int64_t row = i / W;
@@ -254,6 +257,7 @@ __global__ void batch_forward_init_kernel(int64_t n, int W, int B, const int64_t
 __global__ void __launch_bounds__(kBlock) batch_alloc_kernel(int64_t n, int W, int B, const float* __restrict__ hist,
                                                              int32_t Lmax, const double* __restrict__ Rb, int mode,
                                                              uint64_t* __restrict__ R, Status* __restrict__ st) {
+    prior_done();
     __shared__ unsigned long long tile[64][33];
     const int64_t k0 = (int64_t)blockIdx.x * 32;
     const size_t level_stride = (size_t)n * W;
@@ -264,7 +268,16 @@ __global__ void __launch_bounds__(kBlock) batch_alloc_kernel(int64_t n, int W, i
         unsigned long long r = 0;
         if (k < n && q < B) {
             f2 p = f2{0.f, 0.f};
-            for (int32_t l = 0; l <= Lmax; ++l) p = f2_add_f(p, hist[(size_t)l * level_stride + (size_t)k * W + q]);
+            constexpr int kU = 8;  // levels loaded together, added in order
+            for (int32_t l0 = 0; l0 <= Lmax; l0 += kU) {
+                float v[kU];
+#pragma unroll
+                for (int u = 0; u < kU; ++u)
+                    if (l0 + u <= Lmax) v[u] = hist[(size_t)(l0 + u) * level_stride + (size_t)k * W + q];
+#pragma unroll
+                for (int u = 0; u < kU; ++u)
+                    if (l0 + u <= Lmax) p = f2_add_f(p, v[u]);
+            }
             const double pd = f2_to_double(p);
             const double v = mode == 0 ? Rb[q] * (pd * pd) : Rb[q] * pd;
             if (v >= 9.2e18 || v != v) {
@@ -291,6 +304,7 @@ __global__ void __launch_bounds__(kBlock) batch_reverse_init_kernel(int64_t n, i
                                                                     const double* __restrict__ dhat, double inv_a,
                                                                     const float* __restrict__ hL, float2* __restrict__ w,
                                                                     float2* __restrict__ s0, double* __restrict__ s_out) {
+    prior_done();
     __shared__ double tile[64][33];
     const int64_t k0 = (int64_t)blockIdx.x * 32;
     for (int idx = threadIdx.x; idx < 32 * B; idx += blockDim.x) {
@@ -327,12 +341,12 @@ cudaError_t batch_level(const Graph& g, const DevCsr& A, const V* X, const Op& o
     const int rows_per_block = (kBlock / 32) * (32 / LPR);
     const int sb = grid_cap(g, g.n, rows_per_block);
     const int segb = A.bnseg ? grid_cap(g, A.bnseg, rows_per_block) : 0;
-    batch_rows_kernel<V, LPR, CPL, Op><<<(unsigned)(sb + segb), kBlock, 0, g.stream>>>(
-        g.n, A.rp, A.col, X, op, A.bnseg, A.bseg, partial, segb);
-    cudaError_t e = cudaGetLastError();
+    const cudaError_t e = launch_after(g.stream, dim3((unsigned)(sb + segb)), kBlock, 0,
+                                       batch_rows_kernel<V, LPR, CPL, Op>, g.n, A.rp, A.col, X, op, A.bnseg, A.bseg,
+                                       partial, segb);
     if (e != cudaSuccess || A.bnlong == 0) return e;
-    batch_long_rows_kernel<W, Op><<<(unsigned)A.bnlong, 4 * W, 0, g.stream>>>(A.blong_rows, A.blong_first, partial, op);
-    return cudaGetLastError();
+    return launch_after(g.stream, dim3((unsigned)A.bnlong), 4 * W, 0, batch_long_rows_kernel<W, Op>, A.blong_rows,
+                        A.blong_first, partial, op);
 }
 
 }  // namespace
@@ -400,6 +414,7 @@ cudaError_t launch_batch_reverse_level(const Graph& g, int W, int B, int tile, b
 // past the node's distinct counts).
 __global__ void shared_plan_kernel(int64_t n, int B, const uint64_t* __restrict__ R, uint64_t* __restrict__ len,
                                    uint64_t* __restrict__ rbase) {
+    prior_done();
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
         uint64_t t[kBatchMax];
         int m = 0;
@@ -431,6 +446,7 @@ __global__ void shared_plan_kernel(int64_t n, int B, const uint64_t* __restrict_
 __global__ void shared_columns_kernel(int64_t n, int B, const uint64_t* __restrict__ R,
                                       const uint64_t* __restrict__ rbase, const uint64_t* __restrict__ soff,
                                       const uint64_t* __restrict__ scount, uint64_t* __restrict__ nonmeet) {
+    prior_done();
     const int64_t N = n * (int64_t)B;
     for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < N; idx += (int64_t)gridDim.x * blockDim.x) {
         const int64_t q = idx / n, k = idx % n;
@@ -449,47 +465,46 @@ __global__ void shared_columns_kernel(int64_t n, int B, const uint64_t* __restri
 
 __global__ void dhat_from_R_kernel(int64_t N, const uint64_t* __restrict__ nonmeet, const uint64_t* __restrict__ R,
                                    double* __restrict__ dhat) {
+    prior_done();
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x)
-        dhat[i] = R[i] ? (double)nonmeet[i] / (double)R[i] : 0.0;
+        dhat[i] = pair_ratio(nonmeet[i], R[i]);
 }
 
 cudaError_t launch_shared_plan(const Graph& g, int B, const uint64_t* R, uint64_t* len, uint64_t* rbase) {
-    shared_plan_kernel<<<grid_cap(g, g.n, kBlock), kBlock, 0, g.stream>>>(g.n, B, R, len, rbase);
-    return cudaGetLastError();
+    return launch_after(g.stream, dim3((unsigned)grid_cap(g, g.n, kBlock)), kBlock, 0, shared_plan_kernel, g.n,
+                        B, R, len, rbase);
 }
 
 cudaError_t launch_shared_columns(const Graph& g, int B, const uint64_t* R, const uint64_t* rbase, const uint64_t* soff,
                                   const uint64_t* scount, uint64_t* nonmeet) {
-    shared_columns_kernel<<<grid_cap(g, g.n * B, kBlock), kBlock, 0, g.stream>>>(g.n, B, R, rbase, soff, scount,
-                                                                                  nonmeet);
-    return cudaGetLastError();
+    return launch_after(g.stream, dim3((unsigned)grid_cap(g, g.n * B, kBlock)), kBlock, 0, shared_columns_kernel,
+                        g.n, B, R, rbase, soff, scount, nonmeet);
 }
 
 cudaError_t launch_dhat_from_R(const Graph& g, int64_t N, const uint64_t* nonmeet, const uint64_t* R, double* dhat) {
-    dhat_from_R_kernel<<<grid_cap(g, N, kBlock), kBlock, 0, g.stream>>>(N, nonmeet, R, dhat);
-    return cudaGetLastError();
+    return launch_after(g.stream, dim3((unsigned)grid_cap(g, N, kBlock)), kBlock, 0, dhat_from_R_kernel, N,
+                        nonmeet, R, dhat);
 }
 
 cudaError_t launch_batch_forward_init(const Graph& g, int W, int B, const int64_t* u, double c, float* hist0,
                                       float* x0) {
     const int blocks = grid_cap(g, g.n * W, kBlock);
-    batch_forward_init_kernel<<<blocks, kBlock, 0, g.stream>>>(g.n, W, B, u, (float)(1.0 - sqrt(c)), g.in.rp, hist0, x0);
-    return cudaGetLastError();
+    return launch_after(g.stream, dim3((unsigned)blocks), kBlock, 0, batch_forward_init_kernel, g.n, W, B, u,
+                        (float)(1.0 - sqrt(c)), g.in.rp, hist0, x0);
 }
 
 cudaError_t launch_batch_alloc(const Graph& g, int W, int B, const float* hist, int32_t Lmax, const double* Rb,
                                int mode, uint64_t* R) {
     const int64_t blocks = (g.n + 31) / 32;
-    batch_alloc_kernel<<<(unsigned)blocks, kBlock, 0, g.stream>>>(g.n, W, B, hist, Lmax, Rb, mode, R, g.status);
-    return cudaGetLastError();
+    return launch_after(g.stream, dim3((unsigned)blocks), kBlock, 0, batch_alloc_kernel, g.n, W, B, hist, Lmax, Rb,
+                        mode, R, g.status);
 }
 
 cudaError_t launch_batch_reverse_init(const Graph& g, int W, int B, const double* dhat, double c, const float* hL,
                                       float2* w, float2* s0, double* s_out_if_final) {
     const int64_t blocks = (g.n + 31) / 32;
-    batch_reverse_init_kernel<<<(unsigned)blocks, kBlock, 0, g.stream>>>(g.n, W, B, dhat, 1.0 / (1.0 - sqrt(c)), hL,
-                                                                          w, s0, s_out_if_final);
-    return cudaGetLastError();
+    return launch_after(g.stream, dim3((unsigned)blocks), kBlock, 0, batch_reverse_init_kernel, g.n, W, B, dhat,
+                        1.0 / (1.0 - sqrt(c)), hL, w, s0, s_out_if_final);
 }
 
 }  // namespace esim

@@ -40,6 +40,13 @@ __device__ __forceinline__ T block_sum(T v, T* smem) {
     return r;
 }
 
+// count / R as a double (0 for R = 0), count <= R.  Many nodes have few pairs that all end alike;
+// 0 and 1 are exact without the division, which is slow here.
+__device__ __forceinline__ double pair_ratio(uint64_t count, uint64_t R) {
+    if (count == 0 || R == 0) return 0.0;
+    return count == R ? 1.0 : (double)count / (double)R;
+}
+
 // Programmatic dependent launch: a kernel that starts with prior_done() may be launched with
 // launch_after(), which lets it start while the kernel before it in the stream still runs.
 // What it does before prior_done() touches nothing that an earlier kernel of the stream

@@ -659,8 +659,7 @@ __global__ void dhat_kernel(int64_t n, const uint64_t* __restrict__ nonmeet, con
                             double* __restrict__ dhat) {
     prior_done();
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
-        const uint64_t R = off[k + 1] - off[k];
-        dhat[k] = R ? (double)nonmeet[k] / (double)R : 0.0;
+        dhat[k] = pair_ratio(nonmeet[k], off[k + 1] - off[k]);
     }
 }
 

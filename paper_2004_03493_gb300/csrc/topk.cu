@@ -178,13 +178,13 @@ __global__ void __launch_bounds__(kTopkThreads) topk_bound_kernel(int64_t n, con
     st += blockIdx.y;
     max_hi += (size_t)blockIdx.y * kMaxSlices;
     max_lo += (size_t)blockIdx.y * kMaxSlices;
-    if (excl) exclude = excl[blockIdx.y];
     const int64_t tid = (int64_t)blockIdx.x * kTopkThreads + threadIdx.x;
     const int64_t stride = (int64_t)gridDim.x * kTopkThreads;
     unsigned long long hi = 0;
     unsigned lo = 0;  // 0: no element yet (~i is never 0)
     constexpr int kU = 4;  // loads in flight
     prior_done();
+    if (excl) exclude = excl[blockIdx.y];
     for (int64_t i0 = tid; i0 < n; i0 += stride * kU) {
         double v[kU];
 #pragma unroll
