@@ -68,8 +68,8 @@ METRIC = "single-source SimRank top-k queries/s (Chung-Lu n=1e5 m=1e6, eps=1e-6,
 # 2 row loads, 2 neighbour loads
 INSTR_PER_PAIR_STEP = 48.0
 # DRAM bytes of one sampler launch of the bench query, one-pass ncu capture of the current
-# kernel (dram__bytes_read.sum + dram__bytes_write.sum; the graph once, it stays in L2)
-SAMPLER_TRAFFIC = 6.09e6
+# kernel (dram__bytes_read.sum + dram__bytes_write.sum; the walk table once, it stays in L2)
+SAMPLER_TRAFFIC = 9.72e6
 # Algorithm 3 options of the timed configuration beyond the cost-model rule and depth 8:
 # the 128 heaviest nodes are candidates, the side sampler takes 5 blocks per SM during
 # the planning (chosen by timing the ten sources on GB300; the library defaults are 64

@@ -65,7 +65,7 @@ esim_status upload_csr(int64_t n, const std::vector<uint32_t>& rp, const int32_t
     const int64_t m = (int64_t)rp[n];
     d.long_min = kProbeLongMin;
     d.seg_len = kSegLen;
-    d.sell.row_cap = m >= kLongRowsFrom ? 64u : 32u;
+    d.sell.row_cap = m >= kLongRowsFrom ? kLargeRowCap : kSmallRowCap;
     std::vector<Segment> seg, bseg, pieces;
     std::vector<int32_t> piece_rows, piece_first;  // not kept: a piece names its row and its row's first piece
     std::vector<int32_t> long_rows, long_first, blong_rows, blong_first;

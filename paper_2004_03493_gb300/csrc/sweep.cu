@@ -34,6 +34,8 @@
 #include "internal.h"
 #include "twofloat.cuh"
 
+#include <type_traits>
+
 namespace esim {
 
 // ---------------------------------------------------------------- policies
@@ -193,7 +195,7 @@ struct ReverseOpD {
 // that sits in L2, and a random 4- or 8-byte gather costs a 32-byte sector whatever its
 // width.  One warp takes one slice (32 rows of nearly equal length, one per lane; sell.cu):
 // every lane adds its own row's entries one after another in two chains (even and odd
-// ones), eight gathers in flight, the next eight column numbers loaded before the gathers
+// ones), kU gathers in flight, the next kU column numbers loaded before the gathers
 // are waited for.  No shared memory is used, so the L1 keeps the values of the nodes with
 // many edges; an entry costs about 16 instructions instead of 54.
 // Rows longer than row_cap (32 below four million edges, 64 from there on: a lane's chain is
@@ -202,19 +204,30 @@ struct ReverseOpD {
 // that counts in the last of them adds their sums.  Both joins are fixed shuffle trees.
 // Every row's sum has a fixed order, so the sweeps are deterministic.
 //
-// n = 1e6, m = 1.75e7: 81 / 83 us a forward / reverse level in FP64 storage, against 128 / 137
-// on warp tiles staged in shared memory (54 instructions an entry, 9 % L1 hits); FP64 sums
+// n = 1e6, m = 1.75e7: 81 / 83 us a forward / reverse level in FP64 storage with eight gathers in
+// flight (about a tenth less with four), against 128 / 137 on warp tiles staged in shared memory (54 instructions an entry, 9 % L1 hits); FP64 sums
 // (sparse history) 98 against 316 on eight or sixteen lanes a row.  n = 1e5, m = 1e6: 11-12
 // against 20-23.  What is left is the L2's rate of scattered sectors (tags 63 % busy, L1
 // path 66 %).
-template <class Pol, class Op>
-__global__ void __launch_bounds__(kBlock) sell_rows_kernel(const SellRows A, const uint32_t* __restrict__ rp,
+// Gathers in flight per lane: eight where a level is one row's latency; four on large graphs, where
+// the warps, not the lanes, have to cover it (half the registers a lane, for two-floats seven
+// blocks an SM).  n = 1e6, m = 1.75e7, L = 33, FP64 / FP32c sweeps: 4.60 / 4.08 ms with eight, 4.12 /
+// 3.85 with four; the FP32c query at n = 1e5 415 us with eight, 447 with four.
+template <class Pol, int kU>
+constexpr int sell_min_blocks() {
+    return kU == 4 && sizeof(typename Pol::V) == 8 && sizeof(typename Pol::A) == sizeof(f2) &&
+                   !std::is_same<typename Pol::V, double>::value
+               ? 7
+               : 1;
+}
+
+template <class Pol, int kU, class Op>
+__global__ void __launch_bounds__(kBlock, (sell_min_blocks<Pol, kU>())) sell_rows_kernel(const SellRows A, const uint32_t* __restrict__ rp,
                                                           const typename Pol::V* __restrict__ x, Op op,
                                                           typename Pol::A* __restrict__ partial,
                                                           unsigned* __restrict__ arrived) {
     using Acc = typename Pol::A;
     using V = typename Pol::V;
-    constexpr int kU = 8;  // gathers in flight per lane
     const int lane = threadIdx.x & 31;
     const int64_t s = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     next_may_start();
@@ -498,8 +511,8 @@ cudaError_t sweep_level(const Graph& g, const DevCsr& A, const typename Pol::V* 
     Acc* partial = reinterpret_cast<Acc*>(g.partial);
     unsigned* arrived = reinterpret_cast<unsigned*>(partial + scratch_pieces(g));
     const int64_t blocks = (A.sell.nslices * 32 + kBlock - 1) / kBlock;
-    return launch_after(g.stream, dim3((unsigned)blocks), kBlock, 0, sell_rows_kernel<Pol, Op>, A.sell, A.rp, x, op,
-                        partial, arrived);
+    auto* kernel = A.sell.row_cap == kLargeRowCap ? sell_rows_kernel<Pol, 4, Op> : sell_rows_kernel<Pol, 8, Op>;
+    return launch_after(g.stream, dim3((unsigned)blocks), kBlock, 0, kernel, A.sell, A.rp, x, op, partial, arrived);
 }
 
 f2 host_f2(double v) {
