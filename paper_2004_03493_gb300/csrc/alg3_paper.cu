@@ -90,7 +90,7 @@ __device__ __forceinline__ unsigned long long sum_bits(const uint32_t* __restric
 
 // e(q) = sum of din(x) over the bits x of row q; one warp per row, lane b of a word's turn adds
 // bit b's node: the 32 in-degrees are one coalesced load.  With each lane walking the bits of its
-// own words, one dependent load a bit, this took 56 us a level at n = 3001 (WEIGHTUS now).
+// own words, one dependent load a bit, this took 56 us a level at n = 3001 (now 23).
 __global__ void __launch_bounds__(kBlock) bits_weight_kernel(int64_t n, int64_t words, const uint32_t* __restrict__ B,
                                                             const uint32_t* __restrict__ rp,
                                                             unsigned long long* __restrict__ e) {

@@ -317,9 +317,9 @@ __device__ __forceinline__ uint32_t segment_node(unsigned long long seg, unsigne
 //
 // What bounds it: the generator.  A Philox block is 20 wide multiplies, 4 cycles each on a
 // scheduler's multiply pipe, and 40 three-input XORs, 2 cycles each on its integer pipe;
-// alone it reaches 426 G blocks/s on this chip.  run_one needs 17 of the multiplies, 103
-// instructions per warp and step in all, and runs at 270 G pair-steps/s (9.5e8 pairs on the
-// n = 2000 graph at the paper's kappa: 8.4 ms; the multiply pipe 75 % busy).  One pair
+// alone it reaches 426 G blocks/s on this chip.  run_one needs 17 of the multiplies, 95
+// instructions per warp and step in all, and runs at 282 G pair-steps/s (9.5e8 pairs on the
+// n = 2000 graph at the paper's kappa: 8.0 ms; the multiply pipe 78 % busy).  One pair
 // stream per thread over a (rowptr, col) CSR, which this replaces, took 130 instructions and
 // two dependent loads per walk and step, and a fixed share of the pairs per thread: 11.8 ms
 // there, and 207 against 122 ms on a batch of 64 sources.

@@ -428,7 +428,7 @@ cudaError_t launch_topk_batch(const Graph& g, int32_t B, const double* scores, c
 // which owns every byte of device memory (a fixed arena or a memory-capped
 // serving process), and latency-critical threads that must not pay the device
 // synchronisation cudaMalloc/cudaFree may cause.  For them the selection's
-// scratch (its radix-select state and the candidate list, about 66 KB) lives in
+// scratch (the slices' maxima and the candidate list, about 328 KB) lives in
 // the file-scope array below instead of a library or caller allocation.  Every
 // GPU that loads the library holds this array until the process exits.
 //
@@ -440,8 +440,9 @@ cudaError_t launch_topk_batch(const Graph& g, int32_t B, const double* scores, c
 // the kernels.  The address is remembered together with the unique id of the CUDA
 // context it was taken in: after a device reset the device has a new context (and
 // the array a new address), so the next call takes the address again.  All calls
-// share the array and it keeps the last call's contents; the state is cleared every call.  Calls whose work overlaps on the GPU (different streams,
-// or several host threads) race on the array.
+// share the array and it keeps the last call's contents; the state is cleared every call.
+// Calls whose work overlaps on the GPU (different streams, or several host threads) race on
+// the array.
 // ---------------------------------------------------------------------------
 
 namespace {
