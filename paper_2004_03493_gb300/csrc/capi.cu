@@ -59,13 +59,34 @@ constexpr uint32_t kSegLen = 4096;         // probe sweeps: entries a block adds
 constexpr uint32_t kProbeLongMin = 512;    // shortest row of a block; 1024/64, 2048/128, 1024/256 measured the same
 constexpr int64_t kLongRowsFrom = 4000000;  // from this many edges on a level is no longer one row's latency
 
+// The longest row that one lane sums (SellRows, internal.h).  A lane's chain of gathers is most of
+// a small level's time and a warp per row shortens it, as long as all warps of the level are on
+// the chip at once: the smallest cap that leaves no more of them than that.  Forward, allocation and
+// reverse at eps = 1e-4 in FP64, with caps of 32 / 16 / 8: random n = 2001, m = 16,009 174 / 160 / 138 us
+// (877 warps at 8), n = 20,001, m = 160,009 209 / 189 / 275 (709 and 8854), m = 400,021
+// 252 / 442 / 484 (16,303); skewed n = 20,001, m = 200,011 302 / 268 / 259 (4577), n = 50,001, m = 500,011
+// 345 / 313 / 423 (5940 and 11,381), n = 100,003, m = 1,000,031 397 / 441 / 627 (11,446).
+uint32_t sell_row_cap(int64_t n, const std::vector<uint32_t>& rp) {
+    constexpr int64_t kResidentWarps = 152 * 40;  // 48 registers a thread
+    if ((int64_t)rp[n] >= kLongRowsFrom) return kLargeRowCap;
+    for (uint32_t cap = kLeastRowCap; cap < kSmallRowCap; cap *= 2) {
+        int64_t warps = (n + kSellWindow - 1) / kSellWindow * (kSellWindow / 32);
+        for (int64_t r = 0; r < n && warps <= kResidentWarps; ++r) {
+            const int64_t len = (int64_t)(rp[r + 1] - rp[r]);
+            if (len > (int64_t)cap) warps += (len + 32 * cap - 1) / (32 * cap);
+        }
+        if (warps <= kResidentWarps) return cap;
+    }
+    return kSmallRowCap;
+}
+
 // Upload a host CSR and build its row-split table.
 esim_status upload_csr(int64_t n, const std::vector<uint32_t>& rp, const int32_t* col, DevCsr& d,
                        bool with_info, const std::vector<uint32_t>& uses_rp, cudaStream_t stream) {
     const int64_t m = (int64_t)rp[n];
     d.long_min = kProbeLongMin;
     d.seg_len = kSegLen;
-    d.sell.row_cap = m >= kLongRowsFrom ? kLargeRowCap : kSmallRowCap;
+    d.sell.row_cap = sell_row_cap(n, rp);
     std::vector<Segment> seg, bseg, pieces;
     std::vector<int32_t> piece_rows, piece_first;  // not kept: a piece names its row and its row's first piece
     std::vector<int32_t> long_rows, long_first, blong_rows, blong_first;

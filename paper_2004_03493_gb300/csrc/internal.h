@@ -78,7 +78,7 @@ struct SellRows {
 __host__ __device__ inline int64_t at_pos(const uint32_t* pos, int64_t i) { return pos ? (int64_t)pos[i] : i; }
 
 constexpr int kSellWindow = 1024;           // rows sorted by length together
-constexpr uint32_t kSmallRowCap = 32, kLargeRowCap = 64;
+constexpr uint32_t kLeastRowCap = 8, kSmallRowCap = 32, kLargeRowCap = 64;
 
 // A CSR resident on the device, with the segments of the probe sweeps: a row of long_min
 // entries or more is one, a row of more than seg_len several (those rows are in long_rows).

@@ -198,8 +198,8 @@ struct ReverseOpD {
 // ones), kU gathers in flight, the next kU column numbers loaded before the gathers
 // are waited for.  No shared memory is used, so the L1 keeps the values of the nodes with
 // many edges; an entry costs about 16 instructions instead of 54.
-// Rows longer than row_cap (32 below four million edges, 64 from there on: a lane's chain is
-// most of a small level's time) are summed by a warp each, lanes side by side along the row,
+// Rows longer than row_cap (8 to 32 below four million edges, 64 from there on: a lane's chain is
+// most of a small level's time; capi.cu) are summed by a warp each, lanes side by side along the row,
 // first in the grid; a row longer than 32 row_cap entries is cut into pieces, and the warp
 // that counts in the last of them adds their sums.  Both joins are fixed shuffle trees.
 // Every row's sum has a fixed order, so the sweeps are deterministic.
