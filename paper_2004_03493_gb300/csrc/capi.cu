@@ -69,14 +69,16 @@ constexpr int64_t kLongRowsFrom = 4000000;  // from this many edges on a level i
 uint32_t sell_row_cap(int64_t n, const std::vector<uint32_t>& rp) {
     constexpr int64_t kResidentWarps = 152 * 40;  // 48 registers a thread
     if ((int64_t)rp[n] >= kLongRowsFrom) return kLargeRowCap;
-    for (uint32_t cap = kLeastRowCap; cap < kSmallRowCap; cap *= 2) {
-        int64_t warps = (n + kSellWindow - 1) / kSellWindow * (kSellWindow / 32);
-        for (int64_t r = 0; r < n && warps <= kResidentWarps; ++r) {
-            const int64_t len = (int64_t)(rp[r + 1] - rp[r]);
-            if (len > (int64_t)cap) warps += (len + 32 * cap - 1) / (32 * cap);
-        }
-        if (warps <= kResidentWarps) return cap;
+    constexpr uint32_t kCaps[2] = {kLeastRowCap, 2 * kLeastRowCap};
+    static_assert(2 * kCaps[1] == kSmallRowCap, "a cap between would be left out");
+    int64_t warps[2];
+    warps[0] = warps[1] = (n + kSellWindow - 1) / kSellWindow * (kSellWindow / 32);
+    for (int64_t r = 0; r < n; ++r) {  // one pass without branches; lengths are below kLongRowsFrom
+        const uint32_t len = rp[r + 1] - rp[r];
+        for (int i = 0; i < 2; ++i) warps[i] += len > kCaps[i] ? (len + 32 * kCaps[i] - 1) / (32 * kCaps[i]) : 0u;
     }
+    for (int i = 0; i < 2; ++i)
+        if (warps[i] <= kResidentWarps) return kCaps[i];
     return kSmallRowCap;
 }
 
