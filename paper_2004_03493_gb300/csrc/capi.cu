@@ -235,6 +235,9 @@ void release(Graph& g) {
     cudaFree(g.inv_din);
     cudaFree(g.din_magic);
     cudaFree(g.status);
+    cudaFree(g.sample_taken);
+    for (auto& ev : g.sample_ev)
+        if (ev) cudaEventDestroy(ev);
     if (g.status_host) cudaFreeHost(g.status_host);
     cudaFree(g.ws);
     cudaFree(g.bws);
@@ -480,7 +483,8 @@ esim_status launch_side_walks(Graph& g, const Ws& w, const uint64_t* off, double
             if (!ev) ESIM_CUDA_TRY(cudaEventCreate(&ev), "cudaEventCreate");
         cudaEventRecord(g.side_tev[0], g.side_stream);
     }
-    ESIM_CUDA_TRY(launch_sample(view, off, c, seed, w.nm2, (uint64_t*)&g.status->pair_steps_side, depth),
+    ESIM_CUDA_TRY(launch_sample(view, off, c, seed, w.nm2, (uint64_t*)&g.status->pair_steps_side, depth,
+                                &g.status->taken[1]),
                   "side walk pairs");
     if (g.timing) cudaEventRecord(g.side_tev[1], g.side_stream);
     ESIM_CUDA_TRY(cudaEventRecord(g.side_ev[1], g.side_stream), "record");
@@ -775,6 +779,26 @@ esim_status plan_alg3(Graph& g, const Ws& w, double c, double R_b, int* launches
     return ESIM_OK;
 }
 
+// The sampler of a step call, with a chunk counter that no other launch in flight uses.  A
+// captured one has none: the graph may be launched on several streams at once.
+esim_status sample_step(Graph& g, const uint64_t* off, double c, uint64_t seed, uint64_t* counts, uint64_t* pair_steps,
+                        const uint8_t* depth) {
+    cudaStreamCaptureStatus capture;
+    ESIM_CUDA_TRY(cudaStreamIsCapturing(g.stream, &capture), "stream capture status");
+    if (capture != cudaStreamCaptureStatusNone) {
+        ESIM_CUDA_TRY(launch_sample(g, off, c, seed, counts, pair_steps, depth, nullptr), "walk pairs");
+        return ESIM_OK;
+    }
+    const unsigned slot = g.sample_slot++ % kSampleSlots;
+    cudaEvent_t& done = g.sample_ev[slot];
+    if (!done) ESIM_CUDA_TRY(cudaEventCreateWithFlags(&done, cudaEventDisableTiming), "cudaEventCreate");
+    ESIM_CUDA_TRY(cudaStreamWaitEvent(g.stream, done, 0), "wait for a chunk counter");
+    ESIM_CUDA_TRY(cudaMemsetAsync(g.sample_taken + slot, 0, sizeof(*g.sample_taken), g.stream), "reset chunk counter");
+    ESIM_CUDA_TRY(launch_sample(g, off, c, seed, counts, pair_steps, depth, g.sample_taken + slot), "walk pairs");
+    ESIM_CUDA_TRY(cudaEventRecord(done, g.stream), "record");
+    return ESIM_OK;
+}
+
 // Runs the whole query; s_dev may be NULL (the workspace holds s); k > 0 adds top-k.
 esim_status run_query(Graph& g, int64_t u, double c, double eps, uint64_t seed, double* s_dev, int32_t k,
                       int32_t* ids_dev, double* vals_dev, double* s_host, int32_t* ids_host, double* vals_host) {
@@ -867,14 +891,16 @@ esim_status run_query(Graph& g, int64_t u, double c, double eps, uint64_t seed, 
                                         false),
                           "candidates' scan");
             if (g.timing) cudaEventRecord(g.ev[6], g.stream);
-            ESIM_CUDA_TRY(launch_sample(g, w.offc, c, seed, w.nonmeet, nullptr, w.depth), "candidates' walk pairs");
+            ESIM_CUDA_TRY(launch_sample(g, w.offc, c, seed, w.nonmeet, nullptr, w.depth, &g.status->taken[0]),
+                          "candidates' walk pairs");
             if (g.timing) cudaEventRecord(g.ev[7], g.stream);
             ESIM_CUDA_TRY(cudaStreamWaitEvent(g.stream, g.side_ev[1], 0), "wait for the side walks");
             ESIM_CUDA_TRY(launch_merge_counts(g, w.cand, w.nm2, w.nonmeet), "merge counts");
             extra_launches += 4;
         } else {
             if (g.timing) cudaEventRecord(g.ev[6], g.stream);
-            ESIM_CUDA_TRY(launch_sample(g, w.off, c, seed, w.nonmeet, nullptr, g.alg3 ? w.depth : nullptr),
+            ESIM_CUDA_TRY(launch_sample(g, w.off, c, seed, w.nonmeet, nullptr, g.alg3 ? w.depth : nullptr,
+                                        &g.status->taken[0]),
                           "walk pairs");
             if (g.timing) cudaEventRecord(g.ev[7], g.stream);
         }
@@ -1188,7 +1214,8 @@ int batch_enqueue(Graph& tuner, const Graph& view, const BatchPlan& p, void* ws,
         ESIM_CUDA_TRY(launch_shared_plan(view, B, w.R, w.scount, w.rbase), "shared walk plan");
         ESIM_CUDA_TRY(launch_scan_R(view, N, w.scount, w.off, w.part_R, w.part_Rd), "shared walk scan");
         if (timing) cudaEventRecord(view.ev[2], stream);
-        ESIM_CUDA_TRY(launch_sample_segments(view, N, w.off, c, seed, w.scount, nullptr, nullptr, B, w.rbase),
+        ESIM_CUDA_TRY(launch_sample_segments(view, N, w.off, c, seed, w.scount, &view.status->taken[0], nullptr, nullptr,
+                                             B, w.rbase),
                       "batch walk pairs (shared)");
         if (timing) cudaEventRecord(view.ev[3], stream);
         ESIM_CUDA_TRY(launch_shared_columns(view, B, w.R, w.rbase, w.off, w.scount, w.nonmeet), "shared walk counts");
@@ -1196,7 +1223,8 @@ int batch_enqueue(Graph& tuner, const Graph& view, const BatchPlan& p, void* ws,
     } else {
         ESIM_CUDA_TRY(launch_scan_R(view, N, w.R, w.off, w.part_R, w.part_Rd), "batch scan");
         if (timing) cudaEventRecord(view.ev[2], stream);
-        ESIM_CUDA_TRY(launch_sample_segments(view, N, w.off, c, seed, w.nonmeet, nullptr), "batch walk pairs");
+        ESIM_CUDA_TRY(launch_sample_segments(view, N, w.off, c, seed, w.nonmeet, &view.status->taken[0], nullptr),
+                      "batch walk pairs");
         if (timing) cudaEventRecord(view.ev[3], stream);
         ESIM_CUDA_TRY(launch_dhat_segments(view, N, w.nonmeet, w.off, w.dhat), "batch dhat");
     }
@@ -1339,7 +1367,8 @@ esim_status esim_load_graph(int64_t n, const int64_t* in_rowptr, const int32_t* 
         delete h;
         return st;
     }
-    bool ok = dev_alloc(&g.status, 1) == cudaSuccess && cudaMallocHost((void**)&g.status_host, sizeof(Status)) == cudaSuccess &&
+    bool ok = dev_alloc(&g.status, 1) == cudaSuccess && dev_alloc(&g.sample_taken, kSampleSlots) == cudaSuccess &&
+              cudaMallocHost((void**)&g.status_host, sizeof(Status)) == cudaSuccess &&
               alloc_sweep_scratch(g, &g.partial) && alloc_scan_scratch(n, &g.scan_part, &g.norm_part) &&
               cudaMalloc(&g.topk_ws, topk_stage_offset(n) + (sizeof(double) + sizeof(int32_t)) * kTopkMax) == cudaSuccess &&
               cudaStreamCreateWithFlags(&g.own_stream, cudaStreamNonBlocking) == cudaSuccess &&
@@ -1595,8 +1624,7 @@ esim_status esim_sample(esim_graph* h, const uint64_t* off, double c, uint64_t s
     if (!off || !nonmeet) return fail(ESIM_EINVAL, "NULL argument");
     if (!(c > 0.0 && c < 1.0)) return fail(ESIM_EINVAL, "need 0 < c < 1");
     ESIM_CUDA_TRY(cudaSetDevice(g.device), "cudaSetDevice");
-    ESIM_CUDA_TRY(launch_sample(g, off, c, seed, nonmeet, pair_steps), "walk pairs");
-    return ESIM_OK;
+    return sample_step(g, off, c, seed, nonmeet, pair_steps, nullptr);
 }
 
 esim_status esim_dhat(esim_graph* h, const uint64_t* nonmeet, const uint64_t* off, double* dhat) {
@@ -1762,8 +1790,7 @@ esim_status esim_sample_depth(esim_graph* h, const uint64_t* off, const uint8_t*
     if (!off || !counts) return fail(ESIM_EINVAL, "NULL argument");
     if (!(c > 0.0 && c < 1.0)) return fail(ESIM_EINVAL, "need 0 < c < 1");
     ESIM_CUDA_TRY(cudaSetDevice(g.device), "cudaSetDevice");
-    ESIM_CUDA_TRY(launch_sample(g, off, c, seed, counts, pair_steps, depth), "walk pairs");
-    return ESIM_OK;
+    return sample_step(g, off, c, seed, counts, pair_steps, depth);
 }
 
 esim_status esim_dhat_alg3(esim_graph* h, const uint64_t* counts, const uint64_t* off, const uint8_t* depth,

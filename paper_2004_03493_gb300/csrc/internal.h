@@ -20,13 +20,6 @@ enum : int {
     kErrCapacity = 4, // the sparse history outgrew its (pigeonhole) capacity
 };
 
-// Chunk counter of one sampler launch: zero before and after it.
-struct SampleWork {
-    unsigned long long next;  // chunks taken beyond every warp's first
-    unsigned int done;        // blocks that have finished
-    unsigned int pad;
-};
-
 // Per-query device status block (one per graph handle).
 struct Status {
     unsigned long long sum_R;
@@ -36,7 +29,7 @@ struct Status {
     unsigned int ticket;             // last-block ticket of the sparse-history compaction
     unsigned long long hist_count;   // sparse history entries so far
     unsigned long long pair_steps_side;  // pair-steps of the side-stream sampler launch
-    SampleWork work[2];              // the sampler on the query's stream, and the side launch
+    unsigned long long taken[2];     // chunk counters of a query's sampler launches: its own stream, the side stream
 };
 
 // Sparse history of one query (sparse linearization): entries [lvl[l], lvl[l+1]) are
@@ -105,6 +98,8 @@ struct DevCsr {
 };
 
 constexpr uint32_t kBatchSeg = 64;          // entries a lane group of the batched sweeps adds one after another, at most
+
+constexpr int kSampleSlots = 16;
 
 struct Graph {
     int device = 0;
@@ -181,6 +176,11 @@ struct Graph {
     // workspace
     Status* status = nullptr;     // device
     Status* status_host = nullptr; // pinned host copy
+    // Chunk counters of the step calls' sampler launches, which may lie on several streams: a launch
+    // takes the next one when the launch that had it before has ended (its event).
+    unsigned long long* sample_taken = nullptr;  // kSampleSlots
+    cudaEvent_t sample_ev[kSampleSlots] = {};
+    unsigned sample_slot = 0;
     void* ws = nullptr;
     size_t ws_bytes = 0;
     void* partial = nullptr;      // the sweeps' piece sums and arrival counts (sweep_scratch_bytes)
@@ -236,7 +236,7 @@ cudaError_t launch_allocate(const Graph& g, const double* hist, int32_t L, doubl
 cudaError_t launch_allocate32(const Graph& g, const float* hist, int32_t L, double R_b, int mode, double* pi_out,
                               uint64_t* R_out, uint64_t* off);
 cudaError_t launch_sample(const Graph& g, const uint64_t* off, double c, uint64_t seed, uint64_t* nonmeet,
-                          uint64_t* pair_steps, const uint8_t* depth = nullptr);
+                          uint64_t* pair_steps, const uint8_t* depth, unsigned long long* taken);
 cudaError_t launch_dhat(const Graph& g, const uint64_t* nonmeet, const uint64_t* off, double* dhat);
 cudaError_t launch_fill(const Graph& g, int64_t n, double value, double* out);
 // R_out(k) = R(k) where bit keep(k) of want_mask is set (keep(k) < 8), else 0
@@ -246,10 +246,11 @@ cudaError_t launch_merge_counts(const Graph& g, const uint8_t* cand, const uint6
 // cand(k) = 1 for the listed nodes
 cudaError_t launch_mark(const Graph& g, const int32_t* ids, int count, uint8_t* mark);
 // batches: nseg = B * n segments, segment q*n + k = node k of column q
+// taken: the launch's chunk counter (sample_pairs_kernel), or NULL
 // shared_B > 0 with rbase: segment s covers pairs [rbase[s], rbase[s] + len) of node s / shared_B
 cudaError_t launch_sample_segments(const Graph& g, int64_t nseg, const uint64_t* off, double c, uint64_t seed,
-                                   uint64_t* nonmeet, uint64_t* pair_steps, const uint8_t* depth = nullptr,
-                                   int shared_B = 0, const uint64_t* rbase = nullptr, bool zero_counts = true);
+                                   uint64_t* nonmeet, unsigned long long* taken, uint64_t* pair_steps,
+                                   const uint8_t* depth = nullptr, int shared_B = 0, const uint64_t* rbase = nullptr, bool zero_counts = true);
 // One planned Algorithm 3 candidate: depth >= 1 sets R(k) and depth(k); early marks
 // cand(k) = 2 (its walks run on the side stream during the rest of the planning)
 struct PlanEntry {

@@ -581,8 +581,10 @@ __device__ __forceinline__ unsigned long long run_many(const WalkArgs& a, unsign
     return g + wend;
 }
 
-// Persistent walk-pair sampler (see above).  work: the chunk counter, zero before and
-// after the launch (the last block to finish clears it); ticket likewise.
+// Persistent walk-pair sampler (see above).  taken: the chunks taken beyond every warp's first,
+// zero before the launch and this launch's alone while it runs; or NULL, and each block takes a
+// fixed share of the chunks, for launches that may run several times at once (a captured
+// graph's).  The fixed shares end unevenly: 64 sources on R-MAT 2^17 115 against 100 ms.
 // kSide: the launch beside the planning's kernels, a function of its own for its carve-out.  An SM
 // divides its L1 and shared memory when a block comes to it idle, and a block that needs more
 // shared memory than the division gives waits until the SM is idle again.  The sampler uses
@@ -592,12 +594,14 @@ template <bool kNarrow, bool kSide>
 __global__ void __launch_bounds__(kWalkBlock, 8) sample_pairs_kernel(const __grid_constant__ WalkArgs a, const __grid_constant__ PhiloxKeys K,
                                                                  double budget,
                                                                  unsigned long long* __restrict__ steps_out,
-                                                                 Status* __restrict__ st, SampleWork* __restrict__ work) {
+                                                                 Status* __restrict__ st,
+                                                                 unsigned long long* __restrict__ taken) {
     __shared__ unsigned long long wsteps[kWalkBlock / 32];
+    __shared__ unsigned long long own;  // taken of this block's chunks (no counter)
     unsigned long long total = __ldg(a.off + a.nseg);
     if ((double)total > budget || (st->err & kErrBudget)) {
         if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&st->err, kErrBudget);
-        total = 0ull;  // no walks; the block still counts itself in the ticket below
+        total = 0ull;  // no walks
     }
     const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const unsigned long long nwarps = (unsigned long long)gridDim.x * (kWalkBlock / 32);
@@ -610,6 +614,8 @@ __global__ void __launch_bounds__(kWalkBlock, 8) sample_pairs_kernel(const __gri
     size = size < 32 ? 32 : (size > kChunkMax ? kChunkMax : size);
     const unsigned long long nchunks = (total + size - 1) / size;
     if (lane == 0) wsteps[wid] = 0ull;
+    if (threadIdx.x == 0) own = kWalkBlock / 32;
+    __syncthreads();
     // consecutive chunks go to different blocks, so that a few chunks use all SMs
     unsigned long long c = (unsigned long long)wid * gridDim.x + blockIdx.x;
     while (c < nchunks) {
@@ -642,7 +648,7 @@ __global__ void __launch_bounds__(kWalkBlock, 8) sample_pairs_kernel(const __gri
         steps = __reduce_add_sync(0xffffffffu, steps);
         if (lane == 0) {
             wsteps[wid] += steps;
-            c = nwarps + atomicAdd(&work->next, 1ull);
+            c = taken ? nwarps + atomicAdd(taken, 1ull) : atomicAdd(&own, 1ull) * gridDim.x + blockIdx.x;
         }
         c = __shfl_sync(0xffffffffu, c, 0);
     }
@@ -651,7 +657,6 @@ __global__ void __launch_bounds__(kWalkBlock, 8) sample_pairs_kernel(const __gri
         unsigned long long s = 0;
         for (int w = 0; w < kWalkBlock / 32; ++w) s += wsteps[w];
         if (s) atomicAdd(steps_out, s);
-        if (atomicInc(&work->done, gridDim.x - 1) == gridDim.x - 1) work->next = 0ull;  // every chunk was taken
     }
 }
 
@@ -752,12 +757,13 @@ cudaError_t launch_mark(const Graph& g, const int32_t* ids, int count, uint8_t* 
 static int g_sample_blocks_per_sm = 0;
 
 cudaError_t launch_sample(const Graph& g, const uint64_t* off, double c, uint64_t seed, uint64_t* nonmeet,
-                          uint64_t* pair_steps, const uint8_t* depth) {
-    return launch_sample_segments(g, g.n, off, c, seed, nonmeet, pair_steps, depth);
+                          uint64_t* pair_steps, const uint8_t* depth, unsigned long long* taken) {
+    return launch_sample_segments(g, g.n, off, c, seed, nonmeet, taken, pair_steps, depth);
 }
 
 cudaError_t launch_sample_segments(const Graph& g, int64_t nseg, const uint64_t* off, double c, uint64_t seed,
-                                   uint64_t* nonmeet, uint64_t* pair_steps, const uint8_t* depth, int shared_B,
+                                   uint64_t* nonmeet, unsigned long long* taken, uint64_t* pair_steps,
+                                   const uint8_t* depth, int shared_B,
                                    const uint64_t* rbase, bool zero_counts) {
     cudaError_t e = cudaSuccess;
     if (zero_counts && (e = cudaMemsetAsync(nonmeet, 0, sizeof(uint64_t) * (size_t)nseg, g.stream)) != cudaSuccess)
@@ -779,13 +785,12 @@ cudaError_t launch_sample_segments(const Graph& g, int64_t nseg, const uint64_t*
     const WalkArgs a{g.in.info, g.in.walk, off, depth, (unsigned long long*)nonmeet, (uint64_t)nseg, (uint64_t)g.n,
                      SharedSegs{rbase ? shared_B : 0, rbase}, walk_threshold(c)};
     const bool side = steps == &g.status->pair_steps_side;  // it may run beside a launch on the query's own stream
-    SampleWork* work = &g.status->work[side ? 1 : 0];
     auto* kernel = walk_narrow(g) ? (side ? sample_pairs_kernel<true, true> : sample_pairs_kernel<true, false>)
                                   : (side ? sample_pairs_kernel<false, true> : sample_pairs_kernel<false, false>);
     if (side && (e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
                                           cudaSharedmemCarveoutMaxShared)) != cudaSuccess)
         return e;
-    kernel<<<blocks, kWalkBlock, 0, g.stream>>>(a, philox_keys(seed), g.pair_budget, steps, g.status, work);
+    kernel<<<blocks, kWalkBlock, 0, g.stream>>>(a, philox_keys(seed), g.pair_budget, steps, g.status, taken);
     return cudaGetLastError();
 }
 

@@ -1,0 +1,75 @@
+"""Calls of one handle that lie on two streams: what each leaves behind does not reach the other."""
+import numpy as np
+import pytest
+
+import synth
+
+pytestmark = pytest.mark.gpu
+
+C = 0.6
+
+
+@pytest.fixture(scope="module")
+def esim():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.fail("CUDA device required for gpu tests")
+    import paper_2004_03493_gb300 as pkg
+    pkg.build()
+    return pkg
+
+
+@pytest.mark.parametrize("sync_between", [False, True])
+def test_samples_on_two_streams(esim, oracle_walks, sync_between):
+    """Two samples with buffers of their own, each of more chunks than the chip holds warps; with
+    sync_between the handle's status block is reset while the first may still run."""
+    import torch
+    n, rp, col = synth.chung_lu(5000, 50000, gamma=2.1, seed=3)
+    rng = np.random.default_rng(4)
+    jobs = []
+    for seed in (7, 8):
+        R = rng.integers(0, 6000, size=n).astype(np.uint64)
+        off = torch.from_numpy(np.concatenate([[0], np.cumsum(R)]).astype(np.uint64)).cuda()
+        jobs.append((seed, off, torch.zeros(n, dtype=torch.uint64, device="cuda"),
+                     torch.zeros(1, dtype=torch.uint64, device="cuda"), oracle_walks.walk_pairs(n, rp, col, R, C, seed)))
+    streams = [torch.cuda.Stream() for _ in jobs]
+    torch.cuda.synchronize()
+    with esim.Graph(n, rp, col) as g:
+        for _ in range(5):
+            for stream, (seed, off, counts, steps, _ref) in zip(streams, jobs):
+                g.set_stream(stream)
+                if sync_between:
+                    g.sync()
+                g.sample(off, C, seed, counts, steps)
+            torch.cuda.synchronize()
+            for _seed, _off, counts, steps, (ref, ref_steps) in jobs:
+                assert np.array_equal(counts.cpu().numpy(), ref)
+                assert int(steps.cpu().numpy()[0]) == ref_steps
+        g.set_stream(None)
+
+
+def test_captured_sample(esim, oracle_walks):
+    """A captured sample has no chunk counter: every block takes a fixed share."""
+    import torch
+    n, rp, col = synth.chung_lu(5000, 50000, gamma=2.1, seed=3)
+    R = np.random.default_rng(6).integers(0, 700, size=n).astype(np.uint64)
+    ref, ref_steps = oracle_walks.walk_pairs(n, rp, col, R, C, 5)
+    off = torch.from_numpy(np.concatenate([[0], np.cumsum(R)]).astype(np.uint64)).cuda()
+    counts = torch.zeros(n, dtype=torch.uint64, device="cuda")
+    steps = torch.zeros(1, dtype=torch.uint64, device="cuda")
+    stream = torch.cuda.Stream()
+    with esim.Graph(n, rp, col) as g:
+        g.set_stream(stream)
+        g.sample(off, C, 4, counts, steps)
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            g.sample(off, C, 5, counts, steps)
+        for _ in range(2):
+            counts.view(torch.int64).fill_(-1)
+            torch.cuda.synchronize()
+            graph.replay()
+            torch.cuda.synchronize()
+            assert np.array_equal(counts.cpu().numpy(), ref)
+            assert int(steps.cpu().numpy()[0]) == ref_steps
+        g.set_stream(None)
