@@ -391,8 +391,9 @@ cudaError_t topk_select(cudaStream_t stream, int sms, int64_t n, int32_t B, cons
     const size_t smem = (size_t)P * 12;
     cudaError_t e = cudaSuccess;
     if (clear && (e = cudaMemsetAsync(st, 0, sizeof(TopkState) * (size_t)B, stream)) != cudaSuccess) return e;
+    // the limit is the process's, for all handles and threads: always the same value, never a lower one
     if (smem > 48 * 1024 - 2048 &&
-        (e = cudaFuncSetAttribute(topk_pick_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
+        (e = cudaFuncSetAttribute(topk_pick_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kCandMax * 12)) !=
             cudaSuccess)
         return e;
     const dim3 grid((unsigned)blocks, (unsigned)B);

@@ -1,4 +1,7 @@
-"""Calls of one handle that lie on two streams: what each leaves behind does not reach the other."""
+"""Calls of one handle that lie on two streams, and of two handles in two threads: what each does
+or leaves behind does not reach the other."""
+import threading
+
 import numpy as np
 import pytest
 
@@ -73,3 +76,32 @@ def test_captured_sample(esim, oracle_walks):
             assert np.array_equal(counts.cpu().numpy(), ref)
             assert int(steps.cpu().numpy()[0]) == ref_steps
         g.set_stream(None)
+
+
+def test_selections_of_different_sizes_in_two_threads(esim):
+    """k = 600 and k = 4096 need different amounts of shared memory for one kernel."""
+    import torch
+    n, rp, col = synth.erdos_renyi(9000, 30000, seed=2)
+    scores = torch.rand(n, dtype=torch.float64, device="cuda")
+    order = torch.sort(scores, descending=True).indices.to(torch.int32)
+    failed = []
+
+    def work(k):
+        try:
+            ids = torch.full((k,), -7, dtype=torch.int32, device="cuda")
+            vals = torch.empty(k, dtype=torch.float64, device="cuda")
+            with esim.Graph(n, rp, col) as g:
+                for _ in range(4000):
+                    g.select_topk(scores, -1, k, ids, vals)
+                g.sync()
+            assert torch.equal(ids, order[:k])
+        except BaseException as e:  # reported by the main thread
+            failed.append((k, e))
+
+    torch.cuda.synchronize()
+    threads = [threading.Thread(target=work, args=(k,)) for k in (600, 4096)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not failed
