@@ -168,19 +168,11 @@ esim_status upload_csr(int64_t n, const std::vector<uint32_t>& rp, const int32_t
     return ESIM_OK;
 }
 
-// The sweeps' scratch, its counts at zero.
-bool alloc_sweep_scratch(const Graph& g, void** p) {
-    const size_t bytes = sweep_scratch_bytes(g);
-    return cudaMalloc(p, bytes) == cudaSuccess && cudaMemsetAsync(*p, 0, bytes, cudaStreamPerThread) == cudaSuccess &&
-           cudaStreamSynchronize(cudaStreamPerThread) == cudaSuccess;
-}
-
-// The allocation's and the scans' tile sums, their ticket at zero.
-bool alloc_scan_scratch(int64_t n, unsigned long long** part, double** norm) {
-    const size_t nb = (size_t)allocate_blocks(n);
-    return dev_alloc(part, nb + 1) == cudaSuccess && dev_alloc(norm, 2 * nb) == cudaSuccess &&
-           cudaMemsetAsync(*part + nb, 0, sizeof(**part), cudaStreamPerThread) == cudaSuccess &&
-           cudaStreamSynchronize(cudaStreamPerThread) == cudaSuccess;
+// The scratch of work on one stream (call_counts), and the allocation's and the scans' tile sums.
+bool alloc_scratch(const Graph& g, void** partial, unsigned long long** part, double** norm) {
+    const size_t nb = (size_t)allocate_blocks(g.n);
+    return cudaMalloc(partial, scratch_bytes(g)) == cudaSuccess && dev_alloc(part, nb) == cudaSuccess &&
+           dev_alloc(norm, 2 * nb) == cudaSuccess;
 }
 
 void free_a3workers(Graph& g) {
@@ -206,8 +198,8 @@ int ensure_a3workers(Graph& g, int extra) {
     while ((int)g.a3workers.size() < extra) {
         Graph::A3Worker wk;
         const bool ok = cudaStreamCreateWithFlags(&wk.stream, cudaStreamNonBlocking) == cudaSuccess &&
-                        cudaMalloc(&wk.ws, need) == cudaSuccess && alloc_sweep_scratch(g, &wk.partial) &&
-                        alloc_scan_scratch(g.n, &wk.scan_part, &wk.norm_part);
+                        cudaMalloc(&wk.ws, need) == cudaSuccess &&
+                        alloc_scratch(g, &wk.partial, &wk.scan_part, &wk.norm_part);
         if (!ok) {
             cudaGetLastError();
             if (wk.stream) cudaStreamDestroy(wk.stream);
@@ -499,7 +491,7 @@ esim_status launch_side_walks(Graph& g, const Ws& w, const uint64_t* off, double
 esim_status start_side_walks(Graph& g, const Ws& w, double c, uint64_t seed, int* launches) {
     ESIM_CUDA_TRY(launch_mask_R(g, w.R, w.cand, (1u << 0) | (1u << 2), w.R2), "side nodes' R");
     const int64_t nb = allocate_blocks(g.n);
-    ESIM_CUDA_TRY(launch_scan_R(g, g.n, w.R2, w.off2, g.scan_part, g.norm_part + nb, false), "side nodes' scan");
+    ESIM_CUDA_TRY(launch_scan_R(g, g.n, w.R2, w.off2, g.scan_part, g.norm_part + nb, scan_ticket(g), false), "side nodes' scan");
     esim_status st = launch_side_walks(g, w, w.off2, c, seed, w.depth);
     if (st != ESIM_OK) return st;
     *launches += 4;
@@ -774,7 +766,7 @@ esim_status plan_alg3(Graph& g, const Ws& w, double c, double R_b, int* launches
     if (zs != ESIM_OK) return zs;
     g.last_alg3_nodes = used;
     const int64_t nb = allocate_blocks(g.n);
-    ESIM_CUDA_TRY(launch_scan_R(g, g.n, w.R, w.off, g.scan_part, g.norm_part + nb), "Algorithm 3 rescan");
+    ESIM_CUDA_TRY(launch_scan_R(g, g.n, w.R, w.off, g.scan_part, g.norm_part + nb, scan_ticket(g)), "Algorithm 3 rescan");
     *launches += 2;
     return ESIM_OK;
 }
@@ -888,7 +880,7 @@ esim_status run_query(Graph& g, int64_t u, double c, double eps, uint64_t seed, 
             // the remaining candidates' walks here; the side stream's counts for the rest
             ESIM_CUDA_TRY(launch_mask_R(g, w.R, w.cand, 1u << 1, w.R2), "candidates' R");
             ESIM_CUDA_TRY(launch_scan_R(g, g.n, w.R2, w.offc, g.scan_part, g.norm_part + allocate_blocks(g.n),
-                                        false),
+                                        scan_ticket(g), false),
                           "candidates' scan");
             if (g.timing) cudaEventRecord(g.ev[6], g.stream);
             ESIM_CUDA_TRY(launch_sample(g, w.offc, c, seed, w.nonmeet, nullptr, w.depth, &g.status->taken[0]),
@@ -992,6 +984,7 @@ struct BWs {
     int32_t* L;       // W
     double* Rb;       // W
     unsigned long long* part_R;  // tiles of B n
+    unsigned* ticket;            // of their scan
     double* part_Rd;
     void* topk;       // batched top-k state
     int32_t* ids;     // B k (staging)
@@ -1025,7 +1018,8 @@ size_t bws_layout(int64_t n_, int W, int B, int32_t Lmax, int64_t nseg_max, int 
     t.L = (int32_t*)take(4 * W);
     t.Rb = (double*)take(8 * W);
     const size_t nb = (size_t)allocate_blocks((int64_t)bn);
-    t.part_R = (unsigned long long*)take(8 * (nb + 1));
+    t.part_R = (unsigned long long*)take(8 * nb);
+    t.ticket = (unsigned*)take(sizeof(unsigned));
     t.part_Rd = (double*)take(8 * nb);
     t.topk = take(topk_batch_workspace_bytes(B));
     t.ids = (int32_t*)take(4 * (size_t)B * (size_t)std::max(k, 1));
@@ -1192,7 +1186,7 @@ int batch_enqueue(Graph& tuner, const Graph& view, const BatchPlan& p, void* ws,
     ESIM_CUDA_TRY(cudaMemcpyAsync(w.u, p.u, sizeof(int64_t) * W, cudaMemcpyHostToDevice, stream), "upload sources");
     ESIM_CUDA_TRY(cudaMemcpyAsync(w.L, p.Lq, sizeof(int32_t) * W, cudaMemcpyHostToDevice, stream), "upload depths");
     ESIM_CUDA_TRY(cudaMemcpyAsync(w.Rb, p.Rb, sizeof(double) * W, cudaMemcpyHostToDevice, stream), "upload R_b");
-    ESIM_CUDA_TRY(cudaMemsetAsync(w.part_R + allocate_blocks(N), 0, sizeof(*w.part_R), stream), "reset scan ticket");
+    ESIM_CUDA_TRY(cudaMemsetAsync(w.ticket, 0, sizeof(*w.ticket), stream), "reset scan ticket");
     if (timing) cudaEventRecord(view.ev[0], stream);
     ESIM_CUDA_TRY(launch_batch_forward_init(view, W, B, w.u, c, w.hist, w.xa), "batch forward init");
     const int wi = batch_wi(W);
@@ -1212,7 +1206,7 @@ int batch_enqueue(Graph& tuner, const Graph& view, const BatchPlan& p, void* ws,
     if (view.shared_walks) {
         // one walk set per node: intervals between the distinct R_q(k), sampled once
         ESIM_CUDA_TRY(launch_shared_plan(view, B, w.R, w.scount, w.rbase), "shared walk plan");
-        ESIM_CUDA_TRY(launch_scan_R(view, N, w.scount, w.off, w.part_R, w.part_Rd), "shared walk scan");
+        ESIM_CUDA_TRY(launch_scan_R(view, N, w.scount, w.off, w.part_R, w.part_Rd, w.ticket), "shared walk scan");
         if (timing) cudaEventRecord(view.ev[2], stream);
         ESIM_CUDA_TRY(launch_sample_segments(view, N, w.off, c, seed, w.scount, &view.status->taken[0], nullptr, nullptr,
                                              B, w.rbase),
@@ -1221,7 +1215,7 @@ int batch_enqueue(Graph& tuner, const Graph& view, const BatchPlan& p, void* ws,
         ESIM_CUDA_TRY(launch_shared_columns(view, B, w.R, w.rbase, w.off, w.scount, w.nonmeet), "shared walk counts");
         ESIM_CUDA_TRY(launch_dhat_from_R(view, N, w.nonmeet, w.R, w.dhat), "batch dhat");
     } else {
-        ESIM_CUDA_TRY(launch_scan_R(view, N, w.R, w.off, w.part_R, w.part_Rd), "batch scan");
+        ESIM_CUDA_TRY(launch_scan_R(view, N, w.R, w.off, w.part_R, w.part_Rd, w.ticket), "batch scan");
         if (timing) cudaEventRecord(view.ev[2], stream);
         ESIM_CUDA_TRY(launch_sample_segments(view, N, w.off, c, seed, w.nonmeet, &view.status->taken[0], nullptr),
                       "batch walk pairs");
@@ -1369,7 +1363,7 @@ esim_status esim_load_graph(int64_t n, const int64_t* in_rowptr, const int32_t* 
     }
     bool ok = dev_alloc(&g.status, 1) == cudaSuccess && dev_alloc(&g.sample_taken, kSampleSlots) == cudaSuccess &&
               cudaMallocHost((void**)&g.status_host, sizeof(Status)) == cudaSuccess &&
-              alloc_sweep_scratch(g, &g.partial) && alloc_scan_scratch(n, &g.scan_part, &g.norm_part) &&
+              alloc_scratch(g, &g.partial, &g.scan_part, &g.norm_part) &&
               cudaMalloc(&g.topk_ws, topk_stage_offset(n) + (sizeof(double) + sizeof(int32_t)) * kTopkMax) == cudaSuccess &&
               cudaStreamCreateWithFlags(&g.own_stream, cudaStreamNonBlocking) == cudaSuccess &&
               cudaStreamCreateWithFlags(&g.side_stream, cudaStreamNonBlocking) == cudaSuccess &&
@@ -1383,7 +1377,6 @@ esim_status esim_load_graph(int64_t n, const int64_t* in_rowptr, const int32_t* 
     }
     g.stream = g.own_stream;
     cudaError_t we = cudaMemsetAsync(g.status, 0, sizeof(Status), g.stream);
-    if (we == cudaSuccess) we = cudaMemsetAsync(g.topk_ws, 0, topk_stage_offset(n), g.stream);  // its tickets
     if (we == cudaSuccess) we = launch_walk_table(g);
     if (we == cudaSuccess) we = cudaStreamSynchronize(g.stream);
     if (we != cudaSuccess) {
@@ -1613,6 +1606,7 @@ esim_status esim_allocate(esim_graph* h, const double* hist, int32_t L, double R
     if (mode != 0 && mode != 1) return fail(ESIM_EINVAL, "mode must be 0 or 1");
     if (!(R_b >= 0.0)) return fail(ESIM_EINVAL, "need R_b >= 0");
     ESIM_CUDA_TRY(cudaSetDevice(g.device), "cudaSetDevice");
+    ESIM_CUDA_TRY(cudaMemsetAsync(scan_ticket(g), 0, sizeof(unsigned), g.stream), "reset ticket");
     ESIM_CUDA_TRY(launch_allocate(g, hist, L, R_b, mode, pi_out, R_out, off), "allocation");
     return ESIM_OK;
 }
@@ -1659,6 +1653,7 @@ esim_status esim_select_topk(esim_graph* h, const double* scores, int64_t exclud
     if (k > kTopkMax) return fail(ESIM_ENOTSUP, "k above 4096");
     if (exclude < -1 || exclude >= g.n) return fail(ESIM_EINVAL, "exclude out of range");
     ESIM_CUDA_TRY(cudaSetDevice(g.device), "cudaSetDevice");
+    ESIM_CUDA_TRY(cudaMemsetAsync(topk_tickets(g), 0, 2 * sizeof(unsigned), g.stream), "reset tickets");
     ESIM_CUDA_TRY(launch_topk(g, scores, exclude, k, ids_out, vals_out, g.topk_ws), "top-k");
     return ESIM_OK;
 }
@@ -1687,6 +1682,7 @@ esim_status esim_allocate_f32(esim_graph* h, const float* hist, int32_t L, doubl
     if (mode != 0 && mode != 1) return fail(ESIM_EINVAL, "mode must be 0 or 1");
     if (!(R_b >= 0.0)) return fail(ESIM_EINVAL, "need R_b >= 0");
     ESIM_CUDA_TRY(cudaSetDevice(g.device), "cudaSetDevice");
+    ESIM_CUDA_TRY(cudaMemsetAsync(scan_ticket(g), 0, sizeof(unsigned), g.stream), "reset ticket");
     ESIM_CUDA_TRY(launch_allocate32(g, hist, L, R_b, mode, pi_out, R_out, off), "allocation (FP32c)");
     return ESIM_OK;
 }

@@ -183,8 +183,8 @@ struct Graph {
     unsigned sample_slot = 0;
     void* ws = nullptr;
     size_t ws_bytes = 0;
-    void* partial = nullptr;      // the sweeps' piece sums and arrival counts (sweep_scratch_bytes)
-    unsigned long long* scan_part = nullptr;  // allocate_blocks(n) tile sums and a ticket
+    void* partial = nullptr;      // the sweeps' piece sums and the counts of arrivals (call_counts)
+    unsigned long long* scan_part = nullptr;  // allocate_blocks(n) tile sums
     double* norm_part = nullptr;              // 2 allocate_blocks(n)
     void* topk_ws = nullptr;
     // timing events
@@ -208,9 +208,24 @@ void plan_sell(int64_t n, const std::vector<uint32_t>& rp, const std::vector<Seg
 cudaError_t fill_sell(int64_t n, const DevCsr& csr, cudaStream_t stream);
 
 // sweep.cu
-// Bytes of the scratch that sweeps on one stream share: 8 bytes per piece, then a count per
-// piece.  The counts start at zero and every sweep leaves them so.
-size_t sweep_scratch_bytes(const Graph& g);
+// The scratch g.partial of work on one stream: 8 bytes per piece, then counts of arrivals: one
+// per piece, the scans' ticket, the top-k's two.  A kernel's last arrival puts its count back to
+// zero for the next kernel, and the first launch of a call clears them all, so that a call which
+// overlapped another on the same scratch spoils nothing after it.
+inline size_t scratch_pieces(const Graph& g) {
+    const int64_t p = g.in.sell.npieces > g.out.sell.npieces ? g.in.sell.npieces : g.out.sell.npieces;
+    return (size_t)(p ? p : 1);
+}
+struct CallCounts {
+    unsigned* p;
+    int64_t n;
+};
+inline CallCounts call_counts(const Graph& g) {
+    return {reinterpret_cast<unsigned*>((char*)g.partial + 8 * scratch_pieces(g)), (int64_t)scratch_pieces(g) + 3};
+}
+inline unsigned* scan_ticket(const Graph& g) { return call_counts(g).p + scratch_pieces(g); }
+inline unsigned* topk_tickets(const Graph& g) { return scan_ticket(g) + 1; }
+inline size_t scratch_bytes(const Graph& g) { return 8 * scratch_pieces(g) + sizeof(unsigned) * (size_t)call_counts(g).n; }
 cudaError_t launch_forward(const Graph& g, int64_t u, double c, int32_t L, double* hist, double* xa, double* xb);
 cudaError_t launch_reverse(const Graph& g, const double* hist, int32_t L, double c, const double* dhat, double* s_out,
                            double* sa, double* sb);
@@ -265,10 +280,9 @@ cudaError_t launch_plan_scatter(const Graph& g, const PlanEntry* plan, int count
 cudaError_t launch_dhat_segments(const Graph& g, int64_t nseg, const uint64_t* nonmeet, const uint64_t* off,
                                  double* dhat);
 // record = false: an auxiliary scan that leaves the status block (sum of R, budget) alone.
-// part_R: allocate_blocks(N) + 1 entries, the last one (a ticket) zero before and after;
-// part_Rd: allocate_blocks(N)
+// part_R, part_Rd: allocate_blocks(N) entries; ticket: zero before and after
 cudaError_t launch_scan_R(const Graph& g, int64_t N, const uint64_t* R, uint64_t* off, unsigned long long* part_R,
-                          double* part_Rd, bool record = true);
+                          double* part_Rd, unsigned* ticket, bool record = true);
 // the nodes with h != 0, ascending, and their number (device), with g's scan scratch
 cudaError_t launch_support(const Graph& g, const double* h, int32_t* ids, uint64_t* count);
 uint32_t walk_threshold(double c);

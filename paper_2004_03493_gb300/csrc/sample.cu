@@ -105,9 +105,10 @@ __device__ __forceinline__ double level_sum(const float* __restrict__ hist, int6
 // The last block of a grid to get here: exclusive scan of the tile sums (in place), the total
 // into off[n] and the status block, the budget check.  The ticket wraps to zero.
 struct TileSums {
-    unsigned long long* R;   // gridDim.x, and the ticket behind them (zero before the launch)
+    unsigned long long* R;   // gridDim.x
     double* Rd;              // gridDim.x: the same in double, or NULL
     double* norm;            // gridDim.x sums of pi^2, or NULL
+    unsigned* ticket;        // zero before the launch
 };
 
 __device__ __forceinline__ void finish_tiles(const TileSums& t, double budget, uint64_t* __restrict__ off_n,
@@ -117,7 +118,7 @@ __device__ __forceinline__ void finish_tiles(const TileSums& t, double budget, u
     __shared__ double sd[32];
     if (threadIdx.x == 0) {  // it wrote this block's sums
         __threadfence();
-        last = atomicInc(reinterpret_cast<unsigned*>(t.R + gridDim.x), gridDim.x - 1) == gridDim.x - 1;
+        last = atomicInc(t.ticket, gridDim.x - 1) == gridDim.x - 1;
         __threadfence();
     }
     __syncthreads();
@@ -240,7 +241,7 @@ template <typename H>
 cudaError_t launch_allocate_t(const Graph& g, const H* hist, int32_t L, double R_b, int mode, double* pi_out,
                               uint64_t* R_out, uint64_t* off) {
     const int64_t nb = allocate_blocks(g.n);
-    const TileSums tiles{g.scan_part, g.norm_part + nb, g.norm_part};
+    const TileSums tiles{g.scan_part, g.norm_part + nb, g.norm_part, scan_ticket(g)};
     auto* kernel = scan_items(g.n) == 1 ? alloc_reduce_kernel<H, 1> : alloc_reduce_kernel<H, kScanItems>;
     kernel<<<(unsigned)nb, kBlock, 0, g.stream>>>(g.n, hist, L, R_b, mode, g.alg3 ? g.in.rp : nullptr, pi_out, R_out,
                                                   tiles, g.pair_budget, off + g.n, g.status);
@@ -839,9 +840,9 @@ __global__ void __launch_bounds__(kBlock) tile_sums_kernel(int64_t N, const uint
 }
 
 cudaError_t launch_scan_R(const Graph& g, int64_t N, const uint64_t* R, uint64_t* off, unsigned long long* part_R,
-                          double* part_Rd, bool record) {
+                          double* part_Rd, unsigned* ticket, bool record) {
     const int64_t nb = allocate_blocks(N);
-    const TileSums tiles{part_R, part_Rd, nullptr};  // the scan of a ready R leaves the recorded ||pi||^2 as it is
+    const TileSums tiles{part_R, part_Rd, nullptr, ticket};  // the scan of a ready R leaves the recorded ||pi||^2 as it is
     auto* kernel = scan_items(N) == 1 ? tile_sums_kernel<1> : tile_sums_kernel<kScanItems>;
     kernel<<<(unsigned)nb, kBlock, 0, g.stream>>>(N, R, tiles, g.pair_budget, off + N, record ? g.status : nullptr);
     const cudaError_t e = cudaGetLastError();
@@ -884,7 +885,7 @@ __global__ void __launch_bounds__(kBlock) support_ids_kernel(int64_t n, const do
 
 cudaError_t launch_support(const Graph& g, const double* h, int32_t* ids, uint64_t* count) {
     const unsigned nb = (unsigned)allocate_blocks(g.n);
-    const TileSums tiles{g.scan_part, nullptr, nullptr};
+    const TileSums tiles{g.scan_part, nullptr, nullptr, scan_ticket(g)};
     const bool one = scan_items(g.n) == 1;
     const cudaError_t e = one ? launch_after(g.stream, dim3(nb), kBlock, 0, support_tiles_kernel<1>, g.n, h, tiles, count)
                               : launch_after(g.stream, dim3(nb), kBlock, 0, support_tiles_kernel<kScanItems>, g.n, h,

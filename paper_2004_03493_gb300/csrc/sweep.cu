@@ -357,8 +357,14 @@ __global__ void __launch_bounds__(kBlock) reach_rows_kernel(const SellRows A, co
 
 // ---------------------------------------------------------------- level 0
 
-__global__ void forward_init_kernel(int64_t n, int64_t u, const uint32_t* __restrict__ pos, double a, const double* __restrict__ inv_din,
+// A call's first launch: no count of arrivals is left from calls before it.
+__device__ __forceinline__ void clear_counts(const CallCounts& c) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < c.n; i += (int64_t)gridDim.x * blockDim.x) c.p[i] = 0u;
+}
+
+__global__ void forward_init_kernel(int64_t n, const CallCounts counts, int64_t u, const uint32_t* __restrict__ pos, double a, const double* __restrict__ inv_din,
                                     double* __restrict__ pi0, double* __restrict__ x0) {
+    clear_counts(counts);
     const int64_t pu = at_pos(pos, u);
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         pi0[i] = i == u ? a : 0.0;
@@ -367,10 +373,11 @@ __global__ void forward_init_kernel(int64_t n, int64_t u, const uint32_t* __rest
 }
 
 // FP64 form, level 0: pi^0 = a e_u (FP64), x^0 = a / din(u) e_u as a two-float.
-__global__ void forward_init_d_kernel(int64_t n, int64_t u, const uint32_t* __restrict__ pos, double a,
+__global__ void forward_init_d_kernel(int64_t n, const CallCounts counts, int64_t u, const uint32_t* __restrict__ pos, double a,
                                       float xhi, float xlo,
                                       double* __restrict__ pi0, float2* __restrict__ x0) {
     prior_done();
+    clear_counts(counts);
     const int64_t pu = at_pos(pos, u);
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         pi0[i] = i == u ? a : 0.0;
@@ -379,11 +386,12 @@ __global__ void forward_init_d_kernel(int64_t n, int64_t u, const uint32_t* __re
 }
 
 // FP64 form: s^0 = D^ pi^L / a as a two-float (in FP64 when L = 0).
-__global__ void reverse_init_d_kernel(int64_t n, const uint32_t* __restrict__ pos, float a_hi, float a_lo,
+__global__ void reverse_init_d_kernel(int64_t n, const CallCounts counts, const uint32_t* __restrict__ pos, float a_hi, float a_lo,
                                       const double* __restrict__ dhat,
                                       const double* __restrict__ h, float2* __restrict__ s0,
                                       double* __restrict__ s_final) {
     prior_done();
+    clear_counts(counts);
     const f2 a{a_hi, a_lo};
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const f2 s = diag_term(dhat[i], h[i], a);
@@ -392,9 +400,10 @@ __global__ void reverse_init_d_kernel(int64_t n, const uint32_t* __restrict__ po
     }
 }
 
-__global__ void forward_init32_kernel(int64_t n, int64_t u, const uint32_t* __restrict__ pos, float a, float xv,
+__global__ void forward_init32_kernel(int64_t n, const CallCounts counts, int64_t u, const uint32_t* __restrict__ pos, float a, float xv,
                                       float* __restrict__ pi0, float* __restrict__ x0) {
     prior_done();
+    clear_counts(counts);
     const int64_t pu = at_pos(pos, u);
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         pi0[i] = i == u ? a : 0.f;
@@ -403,11 +412,12 @@ __global__ void forward_init32_kernel(int64_t n, int64_t u, const uint32_t* __re
 }
 
 // w = D^ / a as two-floats, and s^0 = w pi^L (float2, or FP64 when L = 0)
-__global__ void reverse_init2f_kernel(int64_t n, const uint32_t* __restrict__ pos, double inv_a,
+__global__ void reverse_init2f_kernel(int64_t n, const CallCounts counts, const uint32_t* __restrict__ pos, double inv_a,
                                       const double* __restrict__ dhat,
                                       const float* __restrict__ h, float2* __restrict__ w, float2* __restrict__ s0,
                                       double* __restrict__ s_final) {
     prior_done();
+    clear_counts(counts);
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const f2 wv = f2_from_double(dhat[i] * inv_a);
         w[i] = make_float2(wv.hi, wv.lo);
@@ -486,11 +496,6 @@ __global__ void __launch_bounds__(kBlock) scatter_level_kernel(const uint64_t* _
     }
 }
 
-size_t scratch_pieces(const Graph& g) {
-    const int64_t p = g.in.sell.npieces > g.out.sell.npieces ? g.in.sell.npieces : g.out.sell.npieces;
-    return (size_t)(p ? p : 1);
-}
-
 int elementwise_blocks(const Graph& g, int64_t n) {
     int64_t b = (n + kBlock - 1) / kBlock;
     int64_t cap = (int64_t)g.sm_count * 8;
@@ -498,10 +503,11 @@ int elementwise_blocks(const Graph& g, int64_t n) {
     return (int)(b < 1 ? 1 : b);
 }
 
-// A kernel over all nodes: kernel(n, args...)
+// The first launch of a call, over all nodes: kernel(n, counts, args...)
 template <class... Params, class... Args>
-cudaError_t each_node(const Graph& g, void (*kernel)(int64_t, Params...), Args&&... args) {
-    return launch_after(g.stream, dim3((unsigned)elementwise_blocks(g, g.n)), kBlock, 0, kernel, g.n, args...);
+cudaError_t each_node(const Graph& g, void (*kernel)(int64_t, CallCounts, Params...), Args&&... args) {
+    return launch_after(g.stream, dim3((unsigned)elementwise_blocks(g, g.n)), kBlock, 0, kernel, g.n, call_counts(g),
+                        args...);
 }
 
 template <class Pol, class Op>
@@ -509,7 +515,7 @@ cudaError_t sweep_level(const Graph& g, const DevCsr& A, const typename Pol::V* 
     using Acc = typename Pol::A;
     static_assert(sizeof(Acc) == 8, "piece sums are 8 bytes");
     Acc* partial = reinterpret_cast<Acc*>(g.partial);
-    unsigned* arrived = reinterpret_cast<unsigned*>(partial + scratch_pieces(g));
+    unsigned* arrived = call_counts(g).p;
     const int64_t blocks = (A.sell.nslices * 32 + kBlock - 1) / kBlock;
     auto* kernel = A.sell.row_cap == kLargeRowCap ? sell_rows_kernel<Pol, 4, Op> : sell_rows_kernel<Pol, 8, Op>;
     return launch_after(g.stream, dim3((unsigned)blocks), kBlock, 0, kernel, A.sell, A.rp, x, op, partial, arrived);
@@ -521,8 +527,6 @@ f2 host_f2(double v) {
 }
 
 }  // namespace
-
-size_t sweep_scratch_bytes(const Graph& g) { return scratch_pieces(g) * (8 + sizeof(unsigned)); }
 
 cudaError_t launch_forward(const Graph& g, int64_t u, double c, int32_t L, double* hist, double* xa, double* xb) {
     const double sc = sqrt(c);
@@ -581,7 +585,7 @@ cudaError_t launch_forward_sparse(const Graph& g, int64_t u, double c, int32_t L
     if (h.lvl && (e = cudaMemsetAsync(h.lvl, 0, sizeof(uint64_t) * (size_t)(L + 2), g.stream)) != cudaSuccess)
         return e;
     const int eb = elementwise_blocks(g, g.n);
-    forward_init_kernel<<<eb, kBlock, 0, g.stream>>>(g.n, u, g.out.sell.pos, a, g.inv_din, lev, xa);
+    forward_init_kernel<<<eb, kBlock, 0, g.stream>>>(g.n, call_counts(g), u, g.out.sell.pos, a, g.inv_din, lev, xa);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     compact_level_kernel<<<eb, kBlock, 0, g.stream>>>(g.n, lev, pi_run, 1, theta, h, 0, g.status);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
@@ -651,7 +655,7 @@ cudaError_t launch_pull_sum(const Graph& g, const float2* x, double* out) {
 
 cudaError_t launch_reach(const Graph& g, const uint32_t* cur, uint32_t* next, unsigned long long* counts) {
     unsigned long long* partial = reinterpret_cast<unsigned long long*>(g.partial);
-    unsigned* arrived = reinterpret_cast<unsigned*>(partial + scratch_pieces(g));
+    unsigned* arrived = call_counts(g).p;
     const int64_t blocks = (g.out.sell.nslices * 32 + kBlock - 1) / kBlock;
     return launch_after(g.stream, dim3((unsigned)blocks), kBlock, 0, reach_rows_kernel, g.out.sell, g.out.rp, cur, next,
                         counts, partial, arrived);

@@ -37,8 +37,6 @@ struct TopkState {
     unsigned long long bound_hi;
     unsigned int bound_lo;
     unsigned int count;       // keys collected
-    unsigned int ticket[2];   // blocks of the two launches that have finished; each wraps to zero
-    unsigned int pad[2];
 };
 
 struct Cand {
@@ -169,6 +167,7 @@ __device__ __forceinline__ bool last_block(unsigned* ticket) {
 // block); the last block's bound.  One column per blockIdx.y in both launches.
 __global__ void __launch_bounds__(kTopkThreads) topk_bound_kernel(int64_t n, const double* __restrict__ scores,
                                                                   int64_t exclude, TopkState* __restrict__ st,
+                                                                  unsigned* __restrict__ tickets,
                                                                   unsigned long long* __restrict__ max_hi,
                                                                   unsigned* __restrict__ max_lo, int G, unsigned k,
                                                                   int64_t col_stride, const int64_t* __restrict__ excl) {
@@ -226,7 +225,7 @@ __global__ void __launch_bounds__(kTopkThreads) topk_bound_kernel(int64_t n, con
         max_hi[tid / G] = hi;
         max_lo[tid / G] = lo;
     }
-    if (!last_block(&st->ticket[0])) return;
+    if (!last_block(tickets + 2 * blockIdx.y)) return;
     auto key = [&](int64_t i, unsigned long long& h, unsigned& l) {
         h = __ldcg(max_hi + i);
         l = __ldcg(max_lo + i);
@@ -247,6 +246,7 @@ __global__ void __launch_bounds__(kTopkThreads) topk_bound_kernel(int64_t n, con
 // dynamic shared memory.
 __global__ void __launch_bounds__(kTopkThreads) topk_pick_kernel(int64_t n, const double* __restrict__ scores,
                                                                  int64_t exclude, TopkState* __restrict__ st,
+                                                                 unsigned* __restrict__ tickets,
                                                                  Cand* __restrict__ cand, unsigned cap, int k, int P,
                                                                  int64_t col_stride, const int64_t* __restrict__ excl,
                                                                  int32_t* __restrict__ ids_out,
@@ -292,7 +292,7 @@ __global__ void __launch_bounds__(kTopkThreads) topk_pick_kernel(int64_t n, cons
             if (take && slot < cap) cand[slot] = Cand{h, l, 0u};
         }
     }
-    if (!last_block(&st->ticket[1])) return;
+    if (!last_block(tickets + 2 * blockIdx.y + 1)) return;
     unsigned cnt = *(volatile unsigned*)&st->count;
     if (cnt <= cap) {
         for (int i = threadIdx.x; i < (int)cnt; i += kTopkThreads) {
@@ -359,16 +359,16 @@ __global__ void __launch_bounds__(kTopkThreads) topk_pick_kernel(int64_t n, cons
     }
 }
 
-// Workspace of B columns: states, maxima (hi, lo), candidates.
-constexpr size_t kStateBytes(size_t B) { return (sizeof(TopkState) * B + 255) / 256 * 256; }
+// Workspace of B columns: states, tickets (two each), maxima (hi, lo), candidates.
+constexpr size_t kStateBytes(size_t B) { return ((sizeof(TopkState) + 2 * sizeof(unsigned)) * B + 255) / 256 * 256; }
 constexpr size_t kColumnBytes = (size_t)kMaxSlices * 12 + sizeof(Cand) * (size_t)kCandMax;
 
 // B selections; column q of scores starts at scores + q * stride, and excl[q] (or exclude
-// where excl is NULL, -1 for none) is left out of it.  The tickets in ws are zero before and
-// after; clear: they may not be (a workspace used before, or by calls that raced).
+// where excl is NULL, -1 for none) is left out of it.  tickets: the blocks of the two launches
+// that have finished, two per column, zero before and after; NULL: the workspace's, cleared here.
 cudaError_t topk_select(cudaStream_t stream, int sms, int64_t n, int32_t B, const double* scores, int64_t col_stride,
                         int64_t exclude, const int64_t* excl, int32_t k, int32_t* ids_out, double* vals_out, void* ws,
-                        bool clear) {
+                        unsigned* tickets) {
     TopkState* st = (TopkState*)ws;
     unsigned long long* max_hi = (unsigned long long*)((char*)ws + kStateBytes((size_t)B));
     unsigned* max_lo = (unsigned*)(max_hi + (size_t)B * kMaxSlices);
@@ -390,17 +390,20 @@ cudaError_t topk_select(cudaStream_t stream, int sms, int64_t n, int32_t B, cons
     while (P < (int)cap) P <<= 1;
     const size_t smem = (size_t)P * 12;
     cudaError_t e = cudaSuccess;
-    if (clear && (e = cudaMemsetAsync(st, 0, sizeof(TopkState) * (size_t)B, stream)) != cudaSuccess) return e;
+    if (!tickets) {
+        tickets = (unsigned*)(st + B);
+        if ((e = cudaMemsetAsync(tickets, 0, 2 * sizeof(unsigned) * (size_t)B, stream)) != cudaSuccess) return e;
+    }
     // the limit is the process's, for all handles and threads: always the same value, never a lower one
     if (smem > 48 * 1024 - 2048 &&
         (e = cudaFuncSetAttribute(topk_pick_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kCandMax * 12)) !=
             cudaSuccess)
         return e;
     const dim3 grid((unsigned)blocks, (unsigned)B);
-    e = launch_after(stream, grid, kTopkThreads, 0, topk_bound_kernel, n, scores, exclude, st, max_hi, max_lo, G,
+    e = launch_after(stream, grid, kTopkThreads, 0, topk_bound_kernel, n, scores, exclude, st, tickets, max_hi, max_lo, G,
                      (unsigned)k, col_stride, excl);
     if (e != cudaSuccess) return e;
-    return launch_after(stream, grid, kTopkThreads, smem, topk_pick_kernel, n, scores, exclude, st, cand, cap, k, P,
+    return launch_after(stream, grid, kTopkThreads, smem, topk_pick_kernel, n, scores, exclude, st, tickets, cand, cap, k, P,
                         col_stride, excl, ids_out, vals_out);
 }
 
@@ -412,12 +415,13 @@ size_t topk_workspace_bytes(int64_t /*n*/) { return topk_batch_workspace_bytes(1
 
 cudaError_t launch_topk(const Graph& g, const double* scores, int64_t exclude, int32_t k, int32_t* ids_out,
                         double* vals_out, void* ws) {
-    return topk_select(g.stream, g.sm_count, g.n, 1, scores, 0, exclude, nullptr, k, ids_out, vals_out, ws, false);
+    return topk_select(g.stream, g.sm_count, g.n, 1, scores, 0, exclude, nullptr, k, ids_out, vals_out, ws,
+                       topk_tickets(g));
 }
 
 cudaError_t launch_topk_batch(const Graph& g, int32_t B, const double* scores, const int64_t* exclude, int32_t k,
                               int32_t* ids_out, double* vals_out, void* ws) {
-    return topk_select(g.stream, g.sm_count, g.n, B, scores, g.n, -1, exclude, k, ids_out, vals_out, ws, true);
+    return topk_select(g.stream, g.sm_count, g.n, B, scores, g.n, -1, exclude, k, ids_out, vals_out, ws, nullptr);
 }
 
 }  // namespace esim
@@ -441,7 +445,7 @@ cudaError_t launch_topk_batch(const Graph& g, int32_t B, const double* scores, c
 // the kernels.  The address is remembered together with the unique id of the CUDA
 // context it was taken in: after a device reset the device has a new context (and
 // the array a new address), so the next call takes the address again.  All calls
-// share the array and it keeps the last call's contents; the state is cleared every call.
+// share the array and it keeps the last call's contents; its tickets are cleared every call.
 // Calls whose work overlaps on the GPU (different streams, or several host threads) race on
 // the array.
 // ---------------------------------------------------------------------------
@@ -539,7 +543,7 @@ extern "C" __attribute__((visibility("default"))) esim_status esim_select_topk_s
     e = static_scratch(dev, &ws, &sms);
     if (e != cudaSuccess)
         return static_fail(ESIM_ECUDA, std::string("static scratch set-up: ") + cudaGetErrorString(e));
-    e = topk_select((cudaStream_t)stream, sms, n, 1, scores, 0, exclude, nullptr, k, ids_out, vals_out, ws, true);
+    e = topk_select((cudaStream_t)stream, sms, n, 1, scores, 0, exclude, nullptr, k, ids_out, vals_out, ws, nullptr);
     if (e != cudaSuccess) return static_fail(ESIM_ECUDA, std::string("static top-k launch: ") + cudaGetErrorString(e));
     return ESIM_OK;
 }

@@ -105,3 +105,42 @@ def test_selections_of_different_sizes_in_two_threads(esim):
     for t in threads:
         t.join()
     assert not failed
+
+
+def test_calls_after_an_overlap_are_right(esim):
+    """A forward and a reverse sweep of one handle on two streams share its scratch and may spoil
+    each other (rows cut into pieces, other numbers of them in the two directions); what is called
+    after them, one at a time, gives the same bits as before."""
+    import torch
+    n, rp, col = synth.chung_lu(20000, 400000, gamma=2.1, seed=2)
+    L, k = 12, 700
+    hist, bad = (torch.empty((L + 1) * n, dtype=torch.float64, device="cuda") for _ in range(2))
+    s, bad_s = (torch.empty(n, dtype=torch.float64, device="cuda") for _ in range(2))
+    pi = torch.empty(n, dtype=torch.float64, device="cuda")
+    R = torch.empty(n, dtype=torch.uint64, device="cuda")
+    off = torch.empty(n + 1, dtype=torch.uint64, device="cuda")
+    ids = torch.empty(k, dtype=torch.int32, device="cuda")
+    vals = torch.empty(k, dtype=torch.float64, device="cuda")
+    dhat = torch.from_numpy(synth.uniform_diagonal(n, C)).cuda()
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    torch.cuda.synchronize()
+    with esim.Graph(n, rp, col) as g:
+        def one_by_one():
+            g.set_stream(streams[0])
+            g.forward(3, C, L, hist)
+            g.allocate(hist, L, 1e6, 0, pi, R, off)
+            g.reverse(hist, L, C, dhat, s)
+            g.select_topk(s, 3, k, ids, vals)
+            g.sync()
+            return [t.cpu().numpy().copy() for t in (hist, pi, R, off, s, ids, vals)]
+
+        before = one_by_one()
+        for _ in range(30):
+            g.set_stream(streams[0])
+            g.forward(3, C, L, bad)
+            g.set_stream(streams[1])
+            g.reverse(hist, L, C, dhat, bad_s)
+            torch.cuda.synchronize()
+            for a, b in zip(before, one_by_one()):
+                assert np.array_equal(a, b)
+        g.set_stream(None)
