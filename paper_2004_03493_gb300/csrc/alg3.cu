@@ -72,10 +72,9 @@ __device__ __forceinline__ void zacc_split(double t, long long& hi, long long& l
 // as a two-float, by position (x = NULL at the last level): the input of the next level's
 // squared-transition sweep; *sum = the sum of Zv_j: block sums in a fixed order by the last
 // block (the ticket wraps to zero).
-__global__ void __launch_bounds__(kBlock) zv_finalize_kernel(int64_t n, double cj, double c, const double* __restrict__ h,
-                                                             const double* __restrict__ T,
-                                                             const long long* __restrict__ zhi,
-                                                             const long long* __restrict__ zlo, double* __restrict__ zv,
+__global__ void __launch_bounds__(kBlock) zv_finalize_kernel(int64_t n, double cj, double c, const double* h,
+                                                             const double* T, const long long* zhi, const long long* zlo,
+                                                             double* __restrict__ zv,
                                                              const double* __restrict__ inv_din,
                                                              const uint32_t* __restrict__ pos, float2* __restrict__ x,
                                                              double* __restrict__ partial, unsigned* __restrict__ ticket,
@@ -232,7 +231,7 @@ __device__ __forceinline__ void probe_flush_colsum(unsigned long long v, unsigne
 
 // Group start (one warp per block): x_0 = e_{q'} / din(q') per column, F_0 = the
 // sources, their work items, fresh counters and column sums.
-__global__ void probe_init_kernel(ProbeGroup G, const int32_t* __restrict__ ids, int count,
+__global__ void probe_init_kernel(ProbeGroup G, const int32_t* ids, int count,
                                   const uint32_t* __restrict__ in_rp, unsigned long long thr) {
     prior_done();
     const int b = blockIdx.y, lane = threadIdx.x;
@@ -277,8 +276,8 @@ __global__ void probe_init_kernel(ProbeGroup G, const int32_t* __restrict__ ids,
 }
 
 // coef(b, col) = c^{l'} Zv_i(q'_col); 0 for unused columns
-__global__ void probe_coef_kernel(ProbeGroup G, const int32_t* __restrict__ ids, int count,
-                                  const double* __restrict__ zv_src, double cl) {
+__global__ void probe_coef_kernel(ProbeGroup G, const int32_t* ids, int count,
+                                  const double* zv_src, double cl) {
     prior_done();
     const int i = blockIdx.y * kProbeW + threadIdx.x;
     G.coef[i] = i < count ? cl * zv_src[ids[i]] : 0.0;
@@ -405,8 +404,8 @@ __global__ void __launch_bounds__(kBlock, 5) probe_sparse_epi_kernel(ProbeGroup 
 // Sum of X(col[p], lane) over entries [b, e), eight gathers in flight (integer adds).  marked
 // (the first dense step): only the rows with a mark hold values.
 __device__ __forceinline__ unsigned long long probe_range(const int32_t* __restrict__ col,
-                                                          const unsigned long long* __restrict__ X,
-                                                          const uint32_t* __restrict__ marked, uint32_t b, uint32_t e,
+                                                          const unsigned long long* X,
+                                                          const uint32_t* marked, uint32_t b, uint32_t e,
                                                           int lane) {
     unsigned long long acc = 0ull;
     uint32_t p = b;
@@ -520,9 +519,9 @@ __global__ void __launch_bounds__(kBlock) probe_long_rows_kernel(ProbeGroup G, P
 
 // Group end: zlast += the sum over blocks and columns, in order, of
 // c^{steps} Zv_i(q'_col) colsum(b, col); blocks that went dense clear their marks.
-__global__ void probe_end_kernel(ProbeGroup G, const int32_t* __restrict__ ids, int count,
-                                 const double* __restrict__ zv_src, double cl, double* __restrict__ zlast,
-                                 const int32_t* __restrict__ pos, unsigned long long* __restrict__ colsum_out) {
+__global__ void probe_end_kernel(ProbeGroup G, const int32_t* ids, int count,
+                                 const double* zv_src, double cl, double* __restrict__ zlast,
+                                 const int32_t* pos, unsigned long long* __restrict__ colsum_out) {
     prior_done();
     if (blockIdx.x == 0 && blockIdx.y == 0) {
         if (colsum_out) {  // the caller sums the terms: hand over the column sums
@@ -889,10 +888,10 @@ __global__ void __launch_bounds__(kCtaThreads) probe_g3_cta_kernel(const unsigne
 // strides over the support, fixed trees add a block's threads, and the last block adds the
 // blocks' sums (the ticket wraps to zero).  Blocks of 256 threads, as all kernels that run beside
 // the side sampler: one block of 1024 threads had to wait for its end.
-__global__ void __launch_bounds__(kBlock) probe_g2_total_kernel(const uint64_t* __restrict__ count_dev,
-                                                                const int32_t* __restrict__ ids,
-                                                                const double* __restrict__ zv_src, double cl,
-                                                                const unsigned long long* __restrict__ colsum,
+__global__ void __launch_bounds__(kBlock) probe_g2_total_kernel(const uint64_t* count_dev,
+                                                                const int32_t* ids,
+                                                                const double* zv_src, double cl,
+                                                                const unsigned long long* colsum,
                                                                 double* __restrict__ partial,
                                                                 unsigned* __restrict__ ticket,
                                                                 double* __restrict__ zlast) {

@@ -24,30 +24,30 @@ namespace esim {
 namespace {
 
 template <int CPL>
-__device__ __forceinline__ void load_f(const float* __restrict__ p, float (&v)[CPL]) {
+__device__ __forceinline__ void load_f(const float* p, float (&v)[CPL]) {
     if constexpr (CPL == 1) {
-        v[0] = __ldg(p);
+        v[0] = *p;
     } else if constexpr (CPL == 2) {
-        const float2 a = __ldg(reinterpret_cast<const float2*>(p));
+        const float2 a = *reinterpret_cast<const float2*>(p);
         v[0] = a.x; v[1] = a.y;
     } else {
 #pragma unroll
         for (int i = 0; i < CPL; i += 4) {
-            const float4 a = __ldg(reinterpret_cast<const float4*>(p + i));
+            const float4 a = *reinterpret_cast<const float4*>(p + i);
             v[i] = a.x; v[i + 1] = a.y; v[i + 2] = a.z; v[i + 3] = a.w;
         }
     }
 }
 
 template <int CPL>
-__device__ __forceinline__ void load_f2(const float2* __restrict__ p, f2 (&v)[CPL]) {
+__device__ __forceinline__ void load_f2(const float2* p, f2 (&v)[CPL]) {
     if constexpr (CPL == 1) {
-        const float2 a = __ldg(p);
+        const float2 a = *p;
         v[0] = f2{a.x, a.y};
     } else {
 #pragma unroll
         for (int i = 0; i < CPL; i += 2) {
-            const float4 a = __ldg(reinterpret_cast<const float4*>(p + i));
+            const float4 a = *reinterpret_cast<const float4*>(p + i);
             v[i] = f2{a.x, a.y};
             v[i + 1] = f2{a.z, a.w};
         }
@@ -59,7 +59,7 @@ __device__ __forceinline__ void load_f2(const float2* __restrict__ p, f2 (&v)[CP
 struct BFwdOp {
     f2 sc;
     int level;
-    const int32_t* __restrict__ Lq;  // W
+    const int32_t* Lq;  // W
     const uint32_t* __restrict__ in_rp;
     float* __restrict__ hist_l;  // n x W
     float* __restrict__ x_out;   // n x W
@@ -85,8 +85,8 @@ template <bool kFinal>
 struct BRevOp {
     f2 sc;
     const uint32_t* __restrict__ rp;
-    const float2* __restrict__ w;  // n x W
-    const float* __restrict__ h;   // n x W (history level L_max - l)
+    const float2* w;  // n x W
+    const float* h;   // n x W (history level L_max - l)
     float2* __restrict__ s_next;   // n x W
     double* __restrict__ s_out;    // B x n
     int W;
@@ -127,7 +127,7 @@ struct BRevOp {
 // it stands for at 32).
 template <typename V, int LPR, int CPL, class Op>
 __global__ void __launch_bounds__(kBlock) batch_rows_kernel(int64_t n, const uint32_t* __restrict__ rp,
-                                                            const int32_t* __restrict__ col, const V* __restrict__ X,
+                                                            const int32_t* __restrict__ col, const V* X,
                                                             Op op, int64_t nseg, const Segment* __restrict__ seg,
                                                             f2* __restrict__ partial, int seg_blocks) {
     constexpr int W = LPR * CPL;
@@ -208,7 +208,7 @@ __global__ void __launch_bounds__(kBlock) batch_rows_kernel(int64_t n, const uin
 template <int W, class Op>
 __global__ void __launch_bounds__(4 * W) batch_long_rows_kernel(const int32_t* __restrict__ long_rows,
                                                                 const int32_t* __restrict__ long_first,
-                                                                const f2* __restrict__ partial, Op op) {
+                                                                const f2* partial, Op op) {
     __shared__ f2 part[4][W];
     prior_done();
     const int q = threadIdx.x % W, g = threadIdx.x / W;
@@ -232,7 +232,7 @@ __global__ void __launch_bounds__(4 * W) batch_long_rows_kernel(const int32_t* _
 }
 
 // Level 0: pi^0 column q = (1 - sqrt c) e_{u_q}; x^0 = pi^0 / din.
-__global__ void batch_forward_init_kernel(int64_t n, int W, int B, const int64_t* __restrict__ u, float a,
+__global__ void batch_forward_init_kernel(int64_t n, int W, int B, const int64_t* u, float a,
                                           const uint32_t* __restrict__ in_rp, float* __restrict__ hist0,
                                           float* __restrict__ x0) {
     prior_done();
@@ -254,8 +254,8 @@ __global__ void batch_forward_init_kernel(int64_t n, int W, int B, const int64_t
 // pi_q(k) = sum over levels (two-float), R_q(k) = ceil(R_b,q pi^2) (>= 1 where pi > 0)
 // into the column-major R[q * n + k].  A block takes 32 nodes x W columns; a shared
 // tile turns the node-major reads into column-major writes.
-__global__ void __launch_bounds__(kBlock) batch_alloc_kernel(int64_t n, int W, int B, const float* __restrict__ hist,
-                                                             int32_t Lmax, const double* __restrict__ Rb, int mode,
+__global__ void __launch_bounds__(kBlock) batch_alloc_kernel(int64_t n, int W, int B, const float* hist,
+                                                             int32_t Lmax, const double* Rb, int mode,
                                                              uint64_t* __restrict__ R, Status* __restrict__ st) {
     prior_done();
     __shared__ unsigned long long tile[64][33];
@@ -301,8 +301,8 @@ __global__ void __launch_bounds__(kBlock) batch_alloc_kernel(int64_t n, int W, i
 // w = D^ / (1 - sqrt c) as two-floats, node-major (n x W), from the column-major D^;
 // s^0 = w pi^{L_max} (two-float), or the FP64 output when L_max = 0.
 __global__ void __launch_bounds__(kBlock) batch_reverse_init_kernel(int64_t n, int W, int B,
-                                                                    const double* __restrict__ dhat, double inv_a,
-                                                                    const float* __restrict__ hL, float2* __restrict__ w,
+                                                                    const double* dhat, double inv_a,
+                                                                    const float* hL, float2* __restrict__ w,
                                                                     float2* __restrict__ s0, double* __restrict__ s_out) {
     prior_done();
     __shared__ double tile[64][33];
@@ -412,7 +412,7 @@ cudaError_t launch_batch_reverse_level(const Graph& g, int W, int B, int tile, b
 // the sum of the intervals below R_q(k) -- the same integer as sampling alone.
 // Segments are node-major: segment k*B + i is interval i of node k (zero length
 // past the node's distinct counts).
-__global__ void shared_plan_kernel(int64_t n, int B, const uint64_t* __restrict__ R, uint64_t* __restrict__ len,
+__global__ void shared_plan_kernel(int64_t n, int B, const uint64_t* R, uint64_t* __restrict__ len,
                                    uint64_t* __restrict__ rbase) {
     prior_done();
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
@@ -443,9 +443,9 @@ __global__ void shared_plan_kernel(int64_t n, int B, const uint64_t* __restrict_
 }
 
 // nonmeet(q, k) = the counts of node k's intervals that end at or below R_q(k)
-__global__ void shared_columns_kernel(int64_t n, int B, const uint64_t* __restrict__ R,
-                                      const uint64_t* __restrict__ rbase, const uint64_t* __restrict__ soff,
-                                      const uint64_t* __restrict__ scount, uint64_t* __restrict__ nonmeet) {
+__global__ void shared_columns_kernel(int64_t n, int B, const uint64_t* R,
+                                      const uint64_t* rbase, const uint64_t* soff,
+                                      const uint64_t* scount, uint64_t* __restrict__ nonmeet) {
     prior_done();
     const int64_t N = n * (int64_t)B;
     for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < N; idx += (int64_t)gridDim.x * blockDim.x) {
@@ -463,7 +463,7 @@ __global__ void shared_columns_kernel(int64_t n, int B, const uint64_t* __restri
     }
 }
 
-__global__ void dhat_from_R_kernel(int64_t N, const uint64_t* __restrict__ nonmeet, const uint64_t* __restrict__ R,
+__global__ void dhat_from_R_kernel(int64_t N, const uint64_t* nonmeet, const uint64_t* R,
                                    double* __restrict__ dhat) {
     prior_done();
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x)

@@ -51,6 +51,9 @@ __device__ __forceinline__ double pair_ratio(uint64_t count, uint64_t R) {
 // launch_after(), which lets it start while the kernel before it in the stream still runs.
 // What it does before prior_done() touches nothing that an earlier kernel of the stream
 // writes.  next_may_start() lets the kernel after it start likewise.
+// Such a kernel begins before its inputs are written.  Only the graph's tables are const
+// __restrict__ or read by __ldg in it: the read-only path is for data that does not change while
+// the kernel runs, and the wait does not order its loads.
 __device__ __forceinline__ void prior_done() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void next_may_start() { asm volatile("griddepcontrol.launch_dependents;"); }
 

@@ -205,8 +205,8 @@ __global__ void __launch_bounds__(kBlock) alloc_reduce_kernel(int64_t n, const H
 
 // off[k] = tile offset + exclusive prefix of R within the tile.
 template <int kItems>
-__global__ void __launch_bounds__(kBlock) alloc_scan_kernel(int64_t n, const uint64_t* __restrict__ R,
-                                                            const unsigned long long* __restrict__ tile_off,
+__global__ void __launch_bounds__(kBlock) alloc_scan_kernel(int64_t n, const uint64_t* R,
+                                                            const unsigned long long* tile_off,
                                                             uint64_t* __restrict__ off) {
     __shared__ unsigned long long su[32];
     const int64_t base = ((int64_t)blockIdx.x * kBlock + threadIdx.x) * kItems;
@@ -661,7 +661,7 @@ __global__ void __launch_bounds__(kWalkBlock, 8) sample_pairs_kernel(const __gri
     }
 }
 
-__global__ void dhat_kernel(int64_t n, const uint64_t* __restrict__ nonmeet, const uint64_t* __restrict__ off,
+__global__ void dhat_kernel(int64_t n, const uint64_t* nonmeet, const uint64_t* off,
                             double* __restrict__ dhat) {
     prior_done();
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
@@ -853,7 +853,7 @@ cudaError_t launch_scan_R(const Graph& g, int64_t N, const uint64_t* R, uint64_t
 // The nodes with h != 0, ascending, into ids, and their number: tile counts and their scan,
 // then the ids.
 template <int kItems>
-__global__ void __launch_bounds__(kBlock) support_tiles_kernel(int64_t n, const double* __restrict__ h,
+__global__ void __launch_bounds__(kBlock) support_tiles_kernel(int64_t n, const double* h,
                                                                const TileSums tiles, uint64_t* __restrict__ count) {
     __shared__ unsigned long long red[kBlock / 32];
     prior_done();
@@ -867,8 +867,8 @@ __global__ void __launch_bounds__(kBlock) support_tiles_kernel(int64_t n, const 
 }
 
 template <int kItems>
-__global__ void __launch_bounds__(kBlock) support_ids_kernel(int64_t n, const double* __restrict__ h,
-                                                             const unsigned long long* __restrict__ tile_off,
+__global__ void __launch_bounds__(kBlock) support_ids_kernel(int64_t n, const double* h,
+                                                             const unsigned long long* tile_off,
                                                              int32_t* __restrict__ ids) {
     __shared__ unsigned long long su[32];
     prior_done();

@@ -130,8 +130,8 @@ struct ReverseOp2f {
     f2 sc;
     const uint32_t* __restrict__ rp;
     const uint32_t* __restrict__ pos;
-    const float2* __restrict__ w;
-    const float* __restrict__ h;
+    const float2* w;
+    const float* h;
     float2* __restrict__ s_out;  // by position
     double* __restrict__ s_final;
     __device__ __forceinline__ void operator()(int64_t row, f2 acc) const {
@@ -176,8 +176,8 @@ struct ReverseOpD {
     f2 a;
     const uint32_t* __restrict__ rp;
     const uint32_t* __restrict__ pos;
-    const double* __restrict__ dhat;
-    const double* __restrict__ h;
+    const double* dhat;
+    const double* h;
     float2* __restrict__ s_out;  // by position
     double* __restrict__ s_final;
     __device__ __forceinline__ void operator()(int64_t row, f2 acc) const {
@@ -223,7 +223,7 @@ constexpr int sell_min_blocks() {
 
 template <class Pol, int kU, class Op>
 __global__ void __launch_bounds__(kBlock, (sell_min_blocks<Pol, kU>())) sell_rows_kernel(const SellRows A, const uint32_t* __restrict__ rp,
-                                                          const typename Pol::V* __restrict__ x, Op op,
+                                                          const typename Pol::V* x, Op op,
                                                           typename Pol::A* __restrict__ partial,
                                                           unsigned* __restrict__ arrived) {
     using Acc = typename Pol::A;
@@ -287,7 +287,7 @@ __global__ void __launch_bounds__(kBlock, (sell_min_blocks<Pol, kU>())) sell_row
 // replaces, left a hub's row to one warp: 29 us a level at n = 20,011 and 79 at n = 1e5, now
 // 11.7 and 13.2 (serialised launches).
 __global__ void __launch_bounds__(kBlock) reach_rows_kernel(const SellRows A, const uint32_t* __restrict__ rp,
-                                                           const uint32_t* __restrict__ cur, uint32_t* __restrict__ next,
+                                                           const uint32_t* cur, uint32_t* __restrict__ next,
                                                            unsigned long long* __restrict__ counts,
                                                            unsigned long long* __restrict__ partial,
                                                            unsigned* __restrict__ arrived) {
@@ -387,8 +387,8 @@ __global__ void forward_init_d_kernel(int64_t n, const CallCounts counts, int64_
 
 // FP64 form: s^0 = D^ pi^L / a as a two-float (in FP64 when L = 0).
 __global__ void reverse_init_d_kernel(int64_t n, const CallCounts counts, const uint32_t* __restrict__ pos, float a_hi, float a_lo,
-                                      const double* __restrict__ dhat,
-                                      const double* __restrict__ h, float2* __restrict__ s0,
+                                      const double* dhat,
+                                      const double* h, float2* __restrict__ s0,
                                       double* __restrict__ s_final) {
     prior_done();
     clear_counts(counts);
@@ -413,8 +413,8 @@ __global__ void forward_init32_kernel(int64_t n, const CallCounts counts, int64_
 
 // w = D^ / a as two-floats, and s^0 = w pi^L (float2, or FP64 when L = 0)
 __global__ void reverse_init2f_kernel(int64_t n, const CallCounts counts, const uint32_t* __restrict__ pos, double inv_a,
-                                      const double* __restrict__ dhat,
-                                      const float* __restrict__ h, float2* __restrict__ w, float2* __restrict__ s0,
+                                      const double* dhat,
+                                      const float* h, float2* __restrict__ w, float2* __restrict__ s0,
                                       double* __restrict__ s_final) {
     prior_done();
     clear_counts(counts);

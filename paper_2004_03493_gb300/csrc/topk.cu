@@ -165,12 +165,12 @@ __device__ __forceinline__ bool last_block(unsigned* ticket) {
 
 // Launch 1: the largest key of every slice (the elements of G consecutive threads of a
 // block); the last block's bound.  One column per blockIdx.y in both launches.
-__global__ void __launch_bounds__(kTopkThreads) topk_bound_kernel(int64_t n, const double* __restrict__ scores,
+__global__ void __launch_bounds__(kTopkThreads) topk_bound_kernel(int64_t n, const double* scores,
                                                                   int64_t exclude, TopkState* __restrict__ st,
                                                                   unsigned* __restrict__ tickets,
                                                                   unsigned long long* __restrict__ max_hi,
                                                                   unsigned* __restrict__ max_lo, int G, unsigned k,
-                                                                  int64_t col_stride, const int64_t* __restrict__ excl) {
+                                                                  int64_t col_stride, const int64_t* excl) {
     __shared__ unsigned hist[256];
     __shared__ Prefix pre;
     scores += (int64_t)blockIdx.y * col_stride;
@@ -244,11 +244,11 @@ __global__ void __launch_bounds__(kTopkThreads) topk_bound_kernel(int64_t n, con
 // Launch 2: the keys at or above the bound into cand (cap of them at most); the last block
 // sorts them, descending, and writes the first k.  P, a power of two >= cap, keys fit its
 // dynamic shared memory.
-__global__ void __launch_bounds__(kTopkThreads) topk_pick_kernel(int64_t n, const double* __restrict__ scores,
+__global__ void __launch_bounds__(kTopkThreads) topk_pick_kernel(int64_t n, const double* scores,
                                                                  int64_t exclude, TopkState* __restrict__ st,
                                                                  unsigned* __restrict__ tickets,
                                                                  Cand* __restrict__ cand, unsigned cap, int k, int P,
-                                                                 int64_t col_stride, const int64_t* __restrict__ excl,
+                                                                 int64_t col_stride, const int64_t* excl,
                                                                  int32_t* __restrict__ ids_out,
                                                                  double* __restrict__ vals_out) {
     extern __shared__ unsigned long long sm_hi[];
