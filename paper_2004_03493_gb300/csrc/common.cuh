@@ -70,7 +70,9 @@ cudaError_t launch_after(cudaStream_t stream, dim3 blocks, unsigned threads, siz
     attr.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, Params(args)...);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, Params(args)...);
+    if (e != cudaSuccess) cudaGetLastError();  // returned here, not to the next launch's check as well
+    return e;
 }
 
 }  // namespace esim

@@ -1,5 +1,6 @@
 """Calls of one handle that lie on two streams, and of two handles in two threads: what each does
 or leaves behind does not reach the other."""
+import ctypes
 import threading
 
 import numpy as np
@@ -144,3 +145,32 @@ def test_calls_after_an_overlap_are_right(esim):
             for a, b in zip(before, one_by_one()):
                 assert np.array_equal(a, b)
         g.set_stream(None)
+
+
+def test_a_refused_launch_does_not_fail_the_next_call(esim):
+    """A sweep on a stream whose capture was invalidated is refused; the handle's next call, on a
+    good stream, is not."""
+    import torch
+    n, rp, col = synth.erdos_renyi(300, 1500, seed=2)
+    L = 3
+    hist = torch.empty((L + 1) * n, dtype=torch.float64, device="cuda")
+    off = torch.arange(n + 1, dtype=torch.int64, device="cuda").view(torch.uint64)
+    counts = torch.zeros(n, dtype=torch.uint64, device="cuda")
+    torch.cuda.synchronize()
+    cudart = ctypes.CDLL(f"libcudart.so.{torch.version.cuda.split('.')[0]}")
+    stream = torch.cuda.Stream()
+    handle = ctypes.c_void_p(stream.cuda_stream)
+    with esim.Graph(n, rp, col) as g:
+        g.forward(1, C, L, hist)  # the workspace is there from here on
+        g.sync()
+        assert cudart.cudaStreamBeginCapture(handle, 2) == 0
+        assert cudart.cudaStreamSynchronize(handle) != 0  # not allowed while capturing: the capture is invalid
+        g.set_stream(stream)
+        with pytest.raises(esim.EsimError):
+            g.forward(1, C, L, hist)
+        graph = ctypes.c_void_p()
+        assert cudart.cudaStreamEndCapture(handle, ctypes.byref(graph)) != 0
+        cudart.cudaGetLastError()
+        g.set_stream(None)
+        g.sample(off, C, 3, counts)
+        g.sync()
