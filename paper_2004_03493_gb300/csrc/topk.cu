@@ -4,24 +4,24 @@
 // key is a higher score, and among equal scores a smaller id.  Keys are unique,
 // so the top-k set is unique.
 //
-// Two launches read the scores once each.  The first cuts the nodes into slices (one
-// thread's or a group of lanes' elements, a few thousand in all) and keeps each slice's
-// largest key; its last block to finish finds the k-th largest of those by a radix select
-// over 8-bit digits.  The slices' maxima are k different keys, so the k-th largest of all
-// keys is no smaller: that is a bound below which nothing is selected.  The second launch
-// collects the keys at or above the bound, little more than k of them, and its last block
-// sorts them.  If they are more than its list holds (scores arranged so that a few slices
-// hold most of the large ones), that block selects over all scores by radix itself.
+// Two launches read the scores once each.  The first deals the nodes to slices (a few
+// thousand in all, Deal below) and keeps each slice's largest key; its last block to finish finds
+// the k-th largest of those by a radix select over 8-bit digits.  The slices' maxima are k
+// different keys, so the k-th largest of all keys is no smaller: that is a bound below which
+// nothing is selected.  The second launch collects the keys at or above the bound, little more
+// than k of them, and its last block sorts them.  If they are more than its list holds (large
+// scores in places chosen against the dealing), that block selects over all scores by radix itself.
 //
 // What bounds it: two passes over n scores (8 MB at n = 2^20: 1.2 us each at the HBM rate)
 // and about five dependent small steps.  Histogram and select launches for every digit of
 // the key, most of them with nothing left to do, took 142 us there for k = 100; this takes
-// 30 (and 46 with the maxima read from L2 for every digit instead of once into registers).
+// 26.
 #include "common.cuh"
 #include "internal.h"
 #include "exactsim.h"
 #include <cuda.h>
 
+#include <algorithm>
 #include <mutex>
 #include <string>
 
@@ -82,6 +82,39 @@ __device__ __forceinline__ int cmp_prefix(unsigned long long hi, unsigned lo, co
     return a < b ? -1 : (a > b ? 1 : 0);
 }
 
+// How nodes are dealt to slices.  Scores have order: ids of neighbours, communities or a crawl lie
+// together, and all zeros tie in id order.  A slice of neighbouring ids would hold many of the k
+// best keys, and the bound would let k times its length through (n = 2^20, k = 50: sorted
+// scores took 1255 us, 37 non-zero ones 4612, with slices of 128 neighbours; 29 and 44 now, scores in
+// random order 31).  So groups of 32
+// ids, one coalesced load, are spread over the warps by a multiplication modulo their number, with
+// a factor near the golden ratio of it: group q is dealt to place q * A mod groups, and a
+// run of groups, or every s-th one, falls evenly over the places.  Within its group a lane takes
+// an id rotated by a hash of q, so that one column of a grid of ids does not stay in one lane.
+// A slice is G of the 32 warps of a block, one lane each: the ids of a group are in 32 slices.
+struct Deal {
+    uint32_t groups;   // ceil(n / 32)
+    uint32_t back;     // 1 / A modulo groups: the group at place p is p * back mod groups
+    uint64_t magic;    // floor((2^64 - 1) / groups)
+    // x mod groups, x < 2^58: the quotient's estimate is at most one too small
+    __device__ __forceinline__ uint32_t mod(uint64_t x) const {
+        const uint64_t r = x - __umul64hi(x, magic) * groups;
+        return (uint32_t)(r >= groups ? r - groups : r);
+    }
+};
+
+Deal make_deal(int64_t n) {
+    const int64_t m = (n + 31) / 32;
+    for (int64_t A = (int64_t)((double)m * 0.6180339887498949) + 1;; ++A) {  // the next one with an inverse
+        int64_t r0 = m, r1 = A % m, t0 = 0, t1 = 1;  // r = t A modulo m
+        while (r1) {
+            const int64_t q = r0 / r1, r2 = r0 - q * r1, t2 = t0 - q * t1;
+            r0 = r1, r1 = r2, t0 = t1, t1 = t2;
+        }
+        if (r0 == 1) return Deal{(uint32_t)m, (uint32_t)(t0 < 0 ? t0 + m : t0), ~0ull / (uint64_t)m};
+    }
+}
+
 // One block: fixes digits of `pre` until the keys of the prefix bucket are exactly those
 // still needed, or until at most `slack` more than k keys lie at or above the prefix.
 // key(i, hi, lo) gives key i < count, false where there is none.  Fewer than k keys in
@@ -113,13 +146,21 @@ __device__ void radix_select(int64_t count, unsigned k, unsigned slack, Prefix& 
         };
         if constexpr (kRegs > 0) {
 #pragma unroll
-            for (int u = 0; u < kRegs; ++u) count_key(there[u], rh[u], rl[u]);
+            for (int u = 0; u < kRegs; ++u)
+                if (u * (int64_t)blockDim.x < count) count_key(there[u], rh[u], rl[u]);  // uniform
         } else {
-            for (int64_t base = threadIdx.x & ~31; base < count; base += blockDim.x) {  // warp-uniform
-                unsigned long long hi = 0;
-                unsigned lo = 0;
-                const bool is = base + lane < count && key(base + lane, hi, lo);
-                count_key(is, hi, lo);
+            constexpr int kU = 8;  // keys in flight
+            for (int64_t base = threadIdx.x & ~31; base < count; base += kU * (int64_t)blockDim.x) {  // warp-uniform
+                unsigned long long hi[kU];
+                unsigned lo[kU];
+                bool is[kU];
+#pragma unroll
+                for (int u = 0; u < kU; ++u) {
+                    const int64_t i = base + lane + u * (int64_t)blockDim.x;
+                    is[u] = i < count && key(i, hi[u], lo[u]);
+                }
+#pragma unroll
+                for (int u = 0; u < kU; ++u) count_key(is[u], hi[u], lo[u]);
             }
         }
         __syncthreads();
@@ -163,9 +204,9 @@ __device__ __forceinline__ bool last_block(unsigned* ticket) {
     return last;
 }
 
-// Launch 1: the largest key of every slice (the elements of G consecutive threads of a
-// block); the last block's bound.  One column per blockIdx.y in both launches.
-__global__ void __launch_bounds__(kTopkThreads) topk_bound_kernel(int64_t n, const double* scores,
+// Launch 1: the largest key of every slice; the last block's bound.  One column per blockIdx.y
+// in both launches.
+__global__ void __launch_bounds__(kTopkThreads) topk_bound_kernel(int64_t n, const Deal deal, const double* scores,
                                                                   int64_t exclude, TopkState* __restrict__ st,
                                                                   unsigned* __restrict__ tickets,
                                                                   unsigned long long* __restrict__ max_hi,
@@ -177,50 +218,59 @@ __global__ void __launch_bounds__(kTopkThreads) topk_bound_kernel(int64_t n, con
     st += blockIdx.y;
     max_hi += (size_t)blockIdx.y * kMaxSlices;
     max_lo += (size_t)blockIdx.y * kMaxSlices;
-    const int64_t tid = (int64_t)blockIdx.x * kTopkThreads + threadIdx.x;
-    const int64_t stride = (int64_t)gridDim.x * kTopkThreads;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     unsigned long long hi = 0;
     unsigned lo = 0;  // 0: no element yet (~i is never 0)
-    constexpr int kU = 4;  // loads in flight
-    prior_done();
-    if (excl) exclude = excl[blockIdx.y];
-    for (int64_t i0 = tid; i0 < n; i0 += stride * kU) {
-        double v[kU];
-#pragma unroll
-        for (int u = 0; u < kU; ++u)
-            if (i0 + u * stride < n) v[u] = scores[i0 + u * stride];
-#pragma unroll
-        for (int u = 0; u < kU; ++u) {
-            const int64_t i = i0 + u * stride;
-            if (i >= n || i == exclude) continue;
-            const unsigned long long h = ordered_bits(v[u]);
-            if (lo == 0u || h > hi) {  // ids ascend: among equal scores the first stays
-                hi = h;
-                lo = ~(unsigned)i;
-            }
-        }
-    }
     auto larger = [&](unsigned long long h, unsigned l) {
         if (h > hi || (h == hi && l > lo)) {
             hi = h;
             lo = l;
         }
     };
-    for (int o = 1; o < G && o < 32; o <<= 1) {
-        const unsigned long long h = __shfl_xor_sync(0xffffffffu, hi, o);
-        larger(h, __shfl_xor_sync(0xffffffffu, lo, o));
-    }
-    if (G > 32) {  // slices of several warps
-        __shared__ unsigned long long wh[kTopkThreads / 32];
-        __shared__ unsigned wl[kTopkThreads / 32];
-        if ((threadIdx.x & 31) == 0) {
-            wh[threadIdx.x >> 5] = hi;
-            wl[threadIdx.x >> 5] = lo;
+    prior_done();
+    if (excl) exclude = excl[blockIdx.y];
+    // places of this warp: its number, then every number of warps further
+    const unsigned long long warps = (unsigned long long)gridDim.x * (kTopkThreads / 32);
+    unsigned long long place = (unsigned long long)blockIdx.x * (kTopkThreads / 32) + wid;
+    uint32_t q = deal.mod(place * deal.back);
+    auto node = [&]() {
+        const int64_t i = 32 * (int64_t)q + ((lane + (q * 0x9E3779B9u >> 27)) & 31);
+        return i < n && i != exclude ? i : (int64_t)-1;
+    };
+    if (warps >= deal.groups) {  // one group a warp at most
+        const int64_t i = place < deal.groups ? node() : -1;
+        if (i >= 0) larger(ordered_bits(scores[i]), ~(unsigned)i);
+    } else {
+        const uint32_t step = deal.mod(warps * deal.back);
+        constexpr int kU = 8;  // loads in flight
+        for (; place < deal.groups; place += kU * warps) {
+            double v[kU];
+            int64_t id[kU];
+#pragma unroll
+            for (int u = 0; u < kU; ++u) {
+                id[u] = place + u * warps < deal.groups ? node() : -1;
+                if (id[u] >= 0) v[u] = scores[id[u]];
+                q = q >= deal.groups - step ? q - (deal.groups - step) : q + step;
+            }
+#pragma unroll
+            for (int u = 0; u < kU; ++u)
+                if (id[u] >= 0) larger(ordered_bits(v[u]), ~(unsigned)id[u]);
         }
-        __syncthreads();
-        if ((threadIdx.x & (G - 1)) == 0)
-            for (int w = 1; w < G / 32; ++w) larger(wh[(threadIdx.x >> 5) + w], wl[(threadIdx.x >> 5) + w]);
     }
+    if (G > 1) {  // the maxima of 32 warps' same lane side by side, then of G of them
+        __shared__ unsigned long long wh[32][33];
+        __shared__ unsigned wl[32][33];
+        wh[wid][lane] = hi;
+        wl[wid][lane] = lo;
+        __syncthreads();
+        hi = wh[lane][wid];
+        lo = wl[lane][wid];
+        for (int o = 1; o < G; o <<= 1) {
+            const unsigned long long h = __shfl_xor_sync(0xffffffffu, hi, o);
+            larger(h, __shfl_xor_sync(0xffffffffu, lo, o));
+        }
+    }
+    const int64_t tid = (int64_t)blockIdx.x * kTopkThreads + threadIdx.x;
     if ((threadIdx.x & (G - 1)) == 0) {
         max_hi[tid / G] = hi;
         max_lo[tid / G] = lo;
@@ -231,8 +281,8 @@ __global__ void __launch_bounds__(kTopkThreads) topk_bound_kernel(int64_t n, con
         l = __ldcg(max_lo + i);
         return l != 0u;
     };
-    const int64_t slices = stride / G;
-    if (slices <= 4 * kTopkThreads) radix_select<4>(slices, k, k / 8 + 32, pre, hist, key);
+    const int64_t slices = (int64_t)gridDim.x * kTopkThreads / G;
+    if (slices <= 5 * kTopkThreads) radix_select<5>(slices, k, k / 8 + 32, pre, hist, key);
     else radix_select<0>(slices, k, k / 8 + 32, pre, hist, key);
     if (threadIdx.x == 0) {
         st->bound_hi = pre.hi;
@@ -373,18 +423,18 @@ cudaError_t topk_select(cudaStream_t stream, int sms, int64_t n, int32_t B, cons
     unsigned long long* max_hi = (unsigned long long*)((char*)ws + kStateBytes((size_t)B));
     unsigned* max_lo = (unsigned*)(max_hi + (size_t)B * kMaxSlices);
     Cand* cand = (Cand*)(max_lo + (size_t)B * kMaxSlices);
-    // one element per thread until the chip is full (two blocks per SM over all columns)
-    int64_t blocks = (n + kTopkThreads - 1) / kTopkThreads;
-    const int64_t most = ((int64_t)sms * 2 + B - 1) / B;
-    if (blocks > most) blocks = most;
-    // (two blocks per SM keep 64 warps loading; with one element per thread and no slices of
-    // several warps a block would select from 16 keys a thread)
-    // slices: enough of them that their k-th maximum is a tight bound (with 4 k of them about
-    // 1.15 k keys reach it), few enough for one block to select from
-    const int64_t threads = blocks * kTopkThreads;
+    // Slices: enough of them that their k-th maximum is a tight bound (with 4 k of them about
+    // 1.15 k keys reach it), few enough for one block to select from, five registers a thread.
+    // One element per thread until the chip is full, with one block per SM where its slices (32)
+    // are enough, two otherwise; over all columns together two, and what a column's slices need.
     const int64_t want = 4 * (int64_t)k < 2048 ? 2048 : (4 * (int64_t)k > 8192 ? 8192 : 4 * (int64_t)k);
+    int64_t most = std::max<int64_t>((2 * (int64_t)sms + B - 1) / B, want / kTopkThreads);
+    if (B == 1 && want <= 32 * (int64_t)sms) most = sms;
+    most = std::min<int64_t>(most, kMaxSlices / 32);  // slices of 32 warps always fit
+    const int64_t blocks = std::min<int64_t>((n + kTopkThreads - 1) / kTopkThreads, most);
+    const int64_t threads = blocks * kTopkThreads;
     int G = 1;
-    while (G < kTopkThreads && threads / (2 * G) >= want) G <<= 1;
+    while (G < 32 && threads / (2 * G) >= want) G <<= 1;
     const unsigned cap = (unsigned)(2 * k + 1024 < kCandMax ? 2 * k + 1024 : kCandMax);
     int P = 1;
     while (P < (int)cap) P <<= 1;
@@ -400,7 +450,7 @@ cudaError_t topk_select(cudaStream_t stream, int sms, int64_t n, int32_t B, cons
             cudaSuccess)
         return e;
     const dim3 grid((unsigned)blocks, (unsigned)B);
-    e = launch_after(stream, grid, kTopkThreads, 0, topk_bound_kernel, n, scores, exclude, st, tickets, max_hi, max_lo, G,
+    e = launch_after(stream, grid, kTopkThreads, 0, topk_bound_kernel, n, make_deal(n), scores, exclude, st, tickets, max_hi, max_lo, G,
                      (unsigned)k, col_stride, excl);
     if (e != cudaSuccess) return e;
     return launch_after(stream, grid, kTopkThreads, smem, topk_pick_kernel, n, scores, exclude, st, tickets, cand, cap, k, P,
