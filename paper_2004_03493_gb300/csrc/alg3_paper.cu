@@ -14,10 +14,15 @@
 //
 // The supports are bit sets, one row of ceil(n/32) words per node: S_0 is the
 // identity and S_(j+1)(q) = OR over x in I(q) of S_j(x), a pull over the in-edge CSR.
-// A first pass over the levels gives the table e_j(q); a second pass rebuilds S_j and
-// adds each still undecided node's terms (first for levels up to 4, then 8, then 16).
-// All counts are integers, so the depths are exact.  The bit sets take 2 n ceil(n/32)
-// words: the rule is offered for graphs whose bit sets fit kPaperBitsBudget.
+// Level l needs S_0..S_l and e_0..e_l only: each level's sets and table are made once, kept, and
+// the undecided nodes' W_l follows from them, so the work ends with the deepest node.  All
+// counts are integers, so the depths are exact.  The kept sets take (l + 1) n ceil(n/32) words; what
+// fits kPaperBitsBudget is kept (all 17 levels up to n = 45,000), and deeper nodes of larger
+// graphs make the levels beyond it twice, as two passes over two buffers: first the tables up
+// to the cap, then the sums.  The rule is offered for graphs whose two buffers fit the budget.
+// Levels made anew from the identity in rounds up to 4, 8 and 16 lost on skewed graphs (Chung-Lu
+// n = 20,011, depths up to 10: 1456 ms for the rule, 779 with all tables first, 297 now; n = 2000:
+// 5.1, 2.7 and 1.2; Erdos-Renyi n = 3001, depths up to 5: 0.81, 1.75 and 0.42).
 #include "common.cuh"
 #include "internal.h"
 #include "twohop.cuh"
@@ -29,7 +34,7 @@ namespace esim {
 
 namespace {
 
-constexpr size_t kPaperBitsBudget = (size_t)4 << 30;  // bytes for the two bit-set levels
+constexpr size_t kPaperBitsBudget = (size_t)4 << 30;  // bytes for the levels' bit sets
 
 int64_t words_of(int64_t n) { return (n + 31) / 32; }
 
@@ -110,23 +115,24 @@ __global__ void paper_alive_kernel(int64_t n, const uint64_t* __restrict__ R, in
         if (R[k] > 0) alive[atomicAdd(count, 1u)] = (int32_t)k;
 }
 
-// Level j: W[j+t](k) += sum over q' in S_j(k) of e_t(q'), t = 0..D-j, for the undecided
-// nodes; one warp per (node, t).
-__global__ void __launch_bounds__(kBlock) paper_level_kernel(int count, const int32_t* __restrict__ alive,
-                                                            int64_t n, int64_t words,
-                                                            const uint32_t* __restrict__ B,
-                                                            const unsigned long long* __restrict__ etab, int j,
-                                                            int D, unsigned long long* __restrict__ W) {
+// W[l](k) += sum over q' in S_j(k) of e_(l-j)(q') for the undecided nodes, j = j0..j0+nj-1 and
+// l = l0..l0+nl-1 (j <= l); one warp per (node, j, l).  S: the sets of level j0, `level` words
+// before those of the next one.
+__global__ void __launch_bounds__(kBlock) paper_terms_kernel(int count, const int32_t* __restrict__ alive,
+                                                            int64_t n, int64_t words, const uint32_t* __restrict__ S,
+                                                            int64_t level, int j0, int nj, int l0, int nl,
+                                                            const unsigned long long* __restrict__ etab,
+                                                            unsigned long long* __restrict__ W) {
     const int lane = threadIdx.x & 31;
-    const int terms = D - j + 1;
-    const int64_t items = (int64_t)count * terms;
+    const int64_t items = (int64_t)count * nj * nl;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
     for (int64_t it = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); it < items; it += warps) {
-        const int64_t k = alive[it / terms];
-        const int t = (int)(it % terms);
-        const unsigned long long* et = etab + (int64_t)t * n;
-        const unsigned long long sum = warp_sum_u64(sum_bits(B + k * words, words, [&](int64_t x) { return et[x]; }));
-        if (lane == 0) W[(int64_t)(j + t) * n + k] += sum;
+        const int64_t k = alive[it / (nj * nl)];
+        const int t = (int)(it % (nj * nl)), j = t / nl, l = l0 + t % nl;
+        const unsigned long long* et = etab + (int64_t)(l - j0 - j) * n;
+        const unsigned long long sum =
+            warp_sum_u64(sum_bits(S + j * level + k * words, words, [&](int64_t x) { return et[x]; }));
+        if (lane == 0 && sum) atomicAdd(W + (int64_t)l * n + k, sum);
     }
 }
 
@@ -227,108 +233,101 @@ int grid_for(const Graph& g, int64_t items_per_warp_rows) {
 
 }  // namespace
 
-size_t alg3_paper_bytes(int64_t n, int max_depth) {
-    const size_t words = (size_t)words_of(n);
-    const size_t bits = 2 * (size_t)n * words * 4;
-    const size_t tables = 2 * (size_t)(max_depth + 1) * (size_t)n * 8;  // e table, W table
-    const size_t rest = (size_t)n * 8 + 2 * (size_t)n * 4 + 256;        // C, two alive lists, counters
-    return bits + tables + rest + 8 * 256;
+static size_t aligned(size_t b) { return (b + 255) / 256 * 256; }
+static size_t level_bytes(int64_t n) { return aligned((size_t)n * (size_t)words_of(n) * 4); }
+
+// Tables e and W, C, two alive lists, counters.
+static size_t table_bytes(int64_t n) {
+    return 2 * aligned((size_t)(kAlg3MaxDepth + 1) * (size_t)n * 8) + aligned((size_t)n * 8) + 2 * aligned((size_t)n * 4) + 256;
+}
+
+size_t alg3_paper_bytes(int64_t n, bool least) {
+    const size_t fit = kPaperBitsBudget / level_bytes(n);
+    return table_bytes(n) + level_bytes(n) * (least ? 2 : std::max<size_t>(2, std::min<size_t>(kAlg3MaxDepth + 1, fit)));
 }
 
 bool alg3_paper_fits(int64_t n) { return 2 * (size_t)n * (size_t)words_of(n) * 4 <= kPaperBitsBudget; }
 
-cudaError_t alg3_paper_depths(const Graph& g, const uint64_t* R, double c, int max_depth, void* ws, uint8_t* depth,
-                              int* launches) {
+cudaError_t alg3_paper_depths(const Graph& g, const uint64_t* R, double c, int max_depth, void* ws, size_t ws_bytes,
+                              uint8_t* depth, int* launches) {
     const int64_t n = g.n, words = words_of(n);
     const int D = max_depth;
-    auto align = [](size_t b) { return (b + 255) / 256 * 256; };
     char* p = (char*)ws;
-    uint32_t* B0 = (uint32_t*)p;
-    p += align((size_t)n * words * 4);
-    uint32_t* B1 = (uint32_t*)p;
-    p += align((size_t)n * words * 4);
-    unsigned long long* etab = (unsigned long long*)p;
-    p += align((size_t)(D + 1) * n * 8);
-    unsigned long long* W = (unsigned long long*)p;
-    p += align((size_t)(D + 1) * n * 8);
-    unsigned long long* C = (unsigned long long*)p;
-    p += align((size_t)n * 8);
-    int32_t* alive[2];
-    alive[0] = (int32_t*)p;
-    p += align((size_t)n * 4);
-    alive[1] = (int32_t*)p;
-    p += align((size_t)n * 4);
-    unsigned* counts = (unsigned*)p;  // one counter per level list
+    auto take = [&p](size_t b) {
+        char* at = p;
+        p += aligned(b);
+        return at;
+    };
+    unsigned long long* etab = (unsigned long long*)take((size_t)(kAlg3MaxDepth + 1) * n * 8);
+    unsigned long long* W = (unsigned long long*)take((size_t)(kAlg3MaxDepth + 1) * n * 8);
+    unsigned long long* C = (unsigned long long*)take((size_t)n * 8);
+    int32_t* alive[2] = {(int32_t*)take((size_t)n * 4), (int32_t*)take((size_t)n * 4)};
+    unsigned* counts = (unsigned*)take(256);  // one counter per level list
+    const int buffers = (int)std::min<size_t>(kAlg3MaxDepth + 1, (ws_bytes - table_bytes(n)) / level_bytes(n));
+    const int64_t level = (int64_t)(level_bytes(n) / 4);  // words
+    auto bits = [&](int b) { return (uint32_t*)p + b * level; };
+    // levels 0..kept are kept; two buffers are left for the levels beyond them, if there are any
+    const int kept = buffers > D ? D : buffers - 3;
     cudaStream_t st = g.stream;
     int nl = 0;
     const int ib = (int)std::max<int64_t>(1, std::min<int64_t>((n * words + kBlock - 1) / kBlock,
                                                                 (int64_t)g.sm_count * 16));
     const int rb = grid_for(g, n);
-    // pass 2's undecided nodes
     cudaError_t e = cudaMemsetAsync(C, 0, (size_t)n * 8, st);
     if (e != cudaSuccess) return e;
+    if ((e = cudaMemsetAsync(W, 0, (size_t)(D + 1) * n * 8, st)) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(counts, 0, 256, st)) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(depth, 0, (size_t)n, st)) != cudaSuccess) return e;
     paper_alive_kernel<<<rb, kBlock, 0, st>>>(n, R, alive[0], counts);
     ++nl;
     unsigned count = 0;
-    // A decision at level l needs the tables e_0 .. e_l only, and most nodes stop within a few
-    // levels: the tables are made up to level 4, then 8, then 16, and the nodes still undecided
-    // after them start again (their counts with them).
-    uint32_t* cur = B0;
-    uint32_t* nxt = B1;
-    int have = -1;  // tables e_0 .. e_have
-    for (int upto = std::min(D, 4); ; upto = std::min(D, 2 * upto)) {
-        // pass 1: e_j(q) for j = 0..upto
-        bits_identity_kernel<<<ib, kBlock, 0, st>>>(n, words, B0);
+    if ((e = cudaMemcpyAsync(&count, counts, sizeof(unsigned), cudaMemcpyDeviceToHost, st)) != cudaSuccess) return e;
+    if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;
+    // S_j, from S_(j-1)
+    auto make = [&](int j, const uint32_t* from, uint32_t* to) {
+        if (j == 0) bits_identity_kernel<<<ib, kBlock, 0, st>>>(n, words, to);
+        else bits_step_kernel<<<rb, kBlock, 0, st>>>(n, words, g.in.rp, g.in.col, from, to);
         ++nl;
-        cur = B0;
-        nxt = B1;
-        for (int j = 0; j <= upto; ++j) {
-            if (j > 0) {
-                bits_step_kernel<<<rb, kBlock, 0, st>>>(n, words, g.in.rp, g.in.col, cur, nxt);
-                std::swap(cur, nxt);
-                ++nl;
-            }
-            if (j <= have) continue;
-            bits_weight_kernel<<<rb, kBlock, 0, st>>>(n, words, cur, g.in.rp, etab + (size_t)j * n);
-            ++nl;
-        }
-        have = upto;
-        // pass 2: the levels again, the undecided nodes' counts and decisions
-        if ((e = cudaMemsetAsync(W, 0, (size_t)(upto + 1) * n * 8, st)) != cudaSuccess) return e;
-        if ((e = cudaMemsetAsync(C, 0, (size_t)n * 8, st)) != cudaSuccess) return e;
-        if ((e = cudaMemsetAsync(counts + 1, 0, 256 - sizeof(unsigned), st)) != cudaSuccess) return e;
-        bits_identity_kernel<<<ib, kBlock, 0, st>>>(n, words, B0);
+    };
+    auto weigh = [&](int j, const uint32_t* S) {
+        bits_weight_kernel<<<rb, kBlock, 0, st>>>(n, words, S, g.in.rp, etab + (size_t)j * n);
         ++nl;
-        cur = B0;
-        nxt = B1;
-        if ((e = cudaMemcpyAsync(&count, counts, sizeof(unsigned), cudaMemcpyDeviceToHost, st)) != cudaSuccess) return e;
-        if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;
-        int in = 0;
-        for (int j = 0; j <= upto && count > 0; ++j) {
-            if (j > 0) {
-                bits_step_kernel<<<rb, kBlock, 0, st>>>(n, words, g.in.rp, g.in.col, cur, nxt);
-                std::swap(cur, nxt);
-                ++nl;
-            }
-            paper_level_kernel<<<grid_for(g, (int64_t)count * (upto - j + 1)), kBlock, 0, st>>>(
-                (int)count, alive[in], n, words, cur, etab, j, upto, W);
-            paper_decide_kernel<<<(count + kBlock - 1) / kBlock, kBlock, 0, st>>>(
-                (int)count, alive[in], n, j, D, sqrt(c), R, W, C, depth, alive[in ^ 1], counts + (j + 1));
-            in ^= 1;
-            nl += 2;
-            if ((e = cudaMemcpyAsync(&count, counts + (j + 1), sizeof(unsigned), cudaMemcpyDeviceToHost, st)) !=
-                cudaSuccess)
-                return e;
-            if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;
+    };
+    auto add_terms = [&](const uint32_t* S, int j0, int nj, int l0, int l1) {
+        const int levels = l1 - l0 + 1;
+        paper_terms_kernel<<<grid_for(g, (int64_t)count * nj * levels), kBlock, 0, st>>>(
+            (int)count, alive[l0 & 1], n, words, S, level, j0, nj, l0, levels, etab, W);
+        ++nl;
+    };
+    // after level l: W_l is complete; alive[l & 1] are the undecided nodes, those left go to the other list
+    auto decide = [&](int l) -> cudaError_t {
+        paper_decide_kernel<<<(count + kBlock - 1) / kBlock, kBlock, 0, st>>>(
+            (int)count, alive[l & 1], n, l, D, sqrt(c), R, W, C, depth, alive[(l & 1) ^ 1], counts + (l + 1));
+        ++nl;
+        const cudaError_t ce = cudaMemcpyAsync(&count, counts + (l + 1), sizeof(unsigned), cudaMemcpyDeviceToHost, st);
+        return ce != cudaSuccess ? ce : cudaStreamSynchronize(st);
+    };
+    for (int l = 0; l <= kept && count > 0; ++l) {
+        make(l, l ? bits(l - 1) : nullptr, bits(l));
+        weigh(l, bits(l));
+        add_terms(bits(0), 0, l + 1, l, l);
+        if ((e = decide(l)) != cudaSuccess) return e;
+    }
+    if (count > 0 && kept < D) {
+        uint32_t* pair[2] = {bits(kept + 1), bits(kept + 2)};
+        auto next = [&](int j) {  // S_j in pair[j & 1]
+            make(j, j - 1 == kept ? (kept >= 0 ? bits(kept) : nullptr) : pair[(j - 1) & 1], pair[j & 1]);
+        };
+        for (int j = kept + 1; j <= D; ++j) {
+            next(j);
+            weigh(j, pair[j & 1]);
         }
-        if (count == 0 || upto == D) break;
-        // the undecided ones are the next round's start
-        if (in != 0) std::swap(alive[0], alive[1]);
-        if ((e = cudaMemcpyAsync(counts, counts + (upto + 1), sizeof(unsigned), cudaMemcpyDeviceToDevice, st)) !=
-            cudaSuccess)
-            return e;
+        if (kept >= 0) add_terms(bits(0), 0, kept + 1, kept + 1, D);
+        for (int j = kept + 1; j <= D && count > 0; ++j) {
+            next(j);
+            add_terms(pair[j & 1], j, 1, j, D);
+            if ((e = decide(j)) != cudaSuccess) return e;
+        }
     }
     if (launches) *launches += nl;
     return cudaGetLastError();

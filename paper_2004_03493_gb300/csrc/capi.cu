@@ -503,18 +503,18 @@ esim_status ensure_a3pws(Graph& g) {
         return fail(ESIM_ENOTSUP, "the paper's Algorithm 3 depth rule keeps n x n support bit sets; n = " +
                                       std::to_string(g.n) + " is above its 4 GiB budget (option alg3_rule = 1 "
                                       "chooses depths by the cost model)");
-    const size_t need = alg3_paper_bytes(g.n, kAlg3MaxDepth);
-    if (g.a3pws && g.a3pws_bytes >= need) return ESIM_OK;
-    cudaStreamSynchronize(g.stream);
-    cudaFree(g.a3pws);
-    g.a3pws = nullptr;
-    g.a3pws_bytes = 0;
-    if (cudaMalloc(&g.a3pws, need) != cudaSuccess) {
+    if (g.a3pws) return ESIM_OK;
+    size_t need = 0;
+    for (bool least : {false, true}) {  // the levels that are not kept are made twice
+        need = alg3_paper_bytes(g.n, least);
+        if (cudaMalloc(&g.a3pws, need) == cudaSuccess) {
+            g.a3pws_bytes = need;
+            return ESIM_OK;
+        }
         cudaGetLastError();
-        return fail(ESIM_ENOMEM, "cudaMalloc(Algorithm 3 depth-rule workspace of " + std::to_string(need) + " bytes)");
+        g.a3pws = nullptr;
     }
-    g.a3pws_bytes = need;
-    return ESIM_OK;
+    return fail(ESIM_ENOMEM, "cudaMalloc(Algorithm 3 depth-rule workspace of " + std::to_string(need) + " bytes)");
 }
 
 // zsum(k) = sum_{l <= depth(k)} Z_l(k) for the nodes of the given depths (every other
@@ -647,7 +647,7 @@ esim_status alg3_zsums(Graph& g, const uint8_t* depth_dev, double c, double* zsu
 esim_status plan_alg3_paper(Graph& g, const Ws& w, double c, int* launches, uint64_t seed, bool* side) {
     esim_status a3 = ensure_a3pws(g);
     if (a3 != ESIM_OK) return a3;
-    ESIM_CUDA_TRY(alg3_paper_depths(g, w.R, c, g.alg3_max_depth, g.a3pws, w.depth, launches),
+    ESIM_CUDA_TRY(alg3_paper_depths(g, w.R, c, g.alg3_max_depth, g.a3pws, g.a3pws_bytes, w.depth, launches),
                   "Algorithm 3 depths (explored edges)");
     // Every node's walks are final now (the allocation's R(k) and offsets, the depths):
     // with a side stream they all run there while the first-meeting sums are computed,
@@ -1756,7 +1756,7 @@ esim_status esim_alg3_paper_depth(esim_graph* h, const uint64_t* R, double c, in
     ESIM_CUDA_TRY(cudaSetDevice(g.device), "cudaSetDevice");
     esim_status a3 = ensure_a3pws(g);
     if (a3 != ESIM_OK) return a3;
-    ESIM_CUDA_TRY(alg3_paper_depths(g, R, c, max_depth, g.a3pws, depth, nullptr), "Algorithm 3 depths (explored edges)");
+    ESIM_CUDA_TRY(alg3_paper_depths(g, R, c, max_depth, g.a3pws, g.a3pws_bytes, depth, nullptr), "Algorithm 3 depths (explored edges)");
     return ESIM_OK;
 }
 

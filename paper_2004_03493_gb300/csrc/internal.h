@@ -325,10 +325,11 @@ cudaError_t launch_dhat_alg3(const Graph& g, const uint64_t* counts, const uint6
 
 // alg3_paper.cu: the paper's adaptive depth (Algorithm 3).  depth[k] for every node with
 // R(k) > 0 (device arrays; the others get 0); synchronises g.stream once per level.
-size_t alg3_paper_bytes(int64_t n, int max_depth);
+// Workspace bytes: every level's sets kept as far as the budget goes, or the least (two of them).
+size_t alg3_paper_bytes(int64_t n, bool least);
 bool alg3_paper_fits(int64_t n);
-cudaError_t alg3_paper_depths(const Graph& g, const uint64_t* R, double c, int max_depth, void* ws, uint8_t* depth,
-                              int* launches);
+cudaError_t alg3_paper_depths(const Graph& g, const uint64_t* R, double c, int max_depth, void* ws, size_t ws_bytes,
+                              uint8_t* depth, int* launches);
 // zsum(k) = Z_1(k) = c / din(k) for the nodes of depth 1 (others untouched)
 cudaError_t alg3_paper_z1(const Graph& g, const uint8_t* depth, double c, double* zsum);
 // zsum(k) = Z_1(k) + Z_2(k) for the listed nodes (device ids), by the closed form of depth 2;
