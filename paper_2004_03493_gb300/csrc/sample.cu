@@ -332,6 +332,7 @@ constexpr uint32_t kRunMin = 128;        // shortest run of one segment that get
 constexpr uint32_t kChunkMin = 256;      // pairs per chunk where there are many
 constexpr uint32_t kChunkMax = 16384;    // few enough that the warps finish together
 constexpr uint32_t kChunksPerWarp = 8;
+constexpr int kSparseRuns = 8;           // segments of 32 with pairs
 constexpr uint32_t kPhiloxM0 = 0xD2511F53u, kPhiloxM1 = 0xCD9E8D57u;
 
 struct WalkArgs {
@@ -489,6 +490,11 @@ __device__ __forceinline__ uint64_t find_segment(const uint64_t* __restrict__ of
 
 // The pairs from g on, up to g1 or to the first segment with kRunMin pairs or more of the
 // chunk, over many segments; seg holds g.  Returns where it stopped (seg likewise).
+// A window of 32 segments with fewer than 32 pairs in fewer than kSparseRuns of them is one of
+// 32 pairs instead, and each lane finds the segment of its own: in a batch whose sources share an
+// eps most of a node's 64 segments have no pairs, and windows of segments took a turn for every
+// one or two of them (64 sources on a random graph of 50,000 nodes, eps = 1e-2: walks 572 us,
+// 107 now; one pair in every 64th of 4e6 nodes 98 and 34).
 template <bool kNarrow>
 __device__ __forceinline__ unsigned long long run_many(const WalkArgs& a, unsigned long long g, unsigned long long g1,
                                                     uint64_t& seg_io, const PhiloxKeys& K, uint32_t& steps) {
@@ -496,6 +502,7 @@ __device__ __forceinline__ unsigned long long run_many(const WalkArgs& a, unsign
     uint64_t wseg = seg_io;        // the window: segments wseg .. wseg + 31, one per lane
     uint32_t wend = 0, next = 0;   // pairs g + [next, wend) of the window are not taken yet
     uint32_t start = 0;            // pair number (from g) at which this lane's segment starts
+    bool sparse = false;           // the window is 32 pairs, start the segment (from wseg) of the lane's pair
     bool last = false;             // no window after this one
     bool active = false;
     uint32_t k = 0, rlo = 0, rhi = 0, t = 0, d = 0;
@@ -506,7 +513,7 @@ __device__ __forceinline__ unsigned long long run_many(const WalkArgs& a, unsign
         const uint32_t idle = __ballot_sync(0xffffffffu, !active);
         if (idle && next >= wend && !last) {  // the next window (uniform)
             if (!first) {
-                wseg += 32;
+                wseg += sparse ? __shfl_sync(0xffffffffu, start, (int)wend - 1) : 32u;
                 g += wend;
                 next = wend = 0;
             }
@@ -530,6 +537,32 @@ __device__ __forceinline__ unsigned long long run_many(const WalkArgs& a, unsign
                 start = (uint32_t)(lo - g);
                 const uint32_t all = (uint32_t)(__shfl_sync(0xffffffffu, hi, 31) - g);
                 wend = upto < 32 ? __shfl_sync(0xffffffffu, start, upto & 31) : all;
+                sparse = upto == 32 && all < 32 && all < g1 - g &&
+                         __popc(__ballot_sync(0xffffffffu, hi > lo)) < kSparseRuns;
+                if (sparse) {
+                    const unsigned long long p = g + lane;
+                    uint64_t width = 32;  // probes this far apart, until they reach past the 32 pairs
+                    unsigned long long probe;
+                    for (;; width *= 8) {
+                        const uint64_t at = wseg + width * (lane + 1);
+                        probe = at < a.nseg ? __ldg(a.off + at) : ~0ull;
+                        if (__shfl_sync(0xffffffffu, probe, 31) > g + 31) break;
+                    }
+                    uint32_t below = 0;  // probes at or before p
+#pragma unroll
+                    for (uint32_t s = 16; s > 0; s >>= 1)
+                        if (__shfl_sync(0xffffffffu, probe, below + s - 1) <= p) below += s;
+                    uint64_t in = wseg + width * below;  // off[in] <= p
+                    uint64_t end = in + width < a.nseg ? in + width : a.nseg;
+                    while (end - in > 1) {
+                        const uint64_t mid = (in + end) >> 1;
+                        if (__ldg(a.off + mid) <= p) in = mid; else end = mid;
+                    }
+                    // the first lane's segment lies in the window, or was searched for above
+                    const uint32_t out = __ballot_sync(0xffffffffu, p >= g1 || in - wseg > 0xffffffffull);
+                    start = (uint32_t)(in - wseg);
+                    wend = out ? (uint32_t)__ffs(out) - 1u : 32u;
+                }
                 if (upto < 32) {
                     last = true;
                     if ((int)lane >= upto) start = 0xffffffffu;
@@ -537,25 +570,26 @@ __device__ __forceinline__ unsigned long long run_many(const WalkArgs& a, unsign
                 }
             }
         }
-        // idle lanes take pairs: the segment is the last one that starts at or before it
+        // idle lanes take pairs: the segment is the last one that starts at or before it, or the found one
         if (idle) {
             const uint32_t i = next + __popc(idle & lanes_below());
             const bool take = !active && i < wend;
-            int j = 0;
+            uint32_t j = 0;
+            if (sparse) {
+                j = __shfl_sync(0xffffffffu, start, i & 31u);
+            } else {
 #pragma unroll
-            for (int s = 16; s > 0; s >>= 1) {
-                const uint32_t v = __shfl_sync(0xffffffffu, start, j + s);
-                if (v <= i) j += s;
+                for (int s = 16; s > 0; s >>= 1) {
+                    const uint32_t v = __shfl_sync(0xffffffffu, start, j + s);
+                    if (v <= i) j += s;
+                }
             }
-            const uint32_t sj = __shfl_sync(0xffffffffu, start, j);
             next += __popc(idle);
             if (next > wend) next = wend;
             if (take) {
-                seg = wseg + (uint32_t)j;
+                seg = wseg + j;
                 k = segment_node(seg, a.n, a.sh);
-                // pair number inside the segment: g + sj is where the window's share of it starts
                 const unsigned long long r = (a.sh.rbase ? __ldg(a.sh.rbase + seg) : 0ull) + (g + i - __ldg(a.off + seg));
-                (void)sj;
                 rlo = (uint32_t)r;
                 rhi = (uint32_t)(r >> 32);
                 d = a.depth ? a.depth[k] : 0u;
