@@ -117,12 +117,13 @@ struct BRevOp {
 // lane group into partial[seg * W + column].
 //
 // What bounds a level: the gathered rows (m x W values from L2) and, per lane group, the
-// chain of two-float additions, about 40 cycles an entry.  kU entries' rows are loaded
-// before they are added, and no chain is longer than kBatchSeg: with segments of 4096 and one
-// load in flight the longest segment alone took 460-770 us of every level with a hub.
-// 64 columns, n = 2^17, m = 3.75e6: 462 / 772 us forward / reverse before, 196 / 265 now;
-// 16 columns, n = 20,011, m = 2e5: 557 / 476 before, 18 / 23 at segments of 128.  The whole
-// query of five sources on that graph takes 0.87 ms at segments of 128, 0.76 at 64, 0.74 at
+// chain of two-float additions, about 40 cycles an entry.  No chain is longer than kBatchSeg: with
+// segments of 4096 the longest one alone took 460-770 us of every level with a hub.  The
+// plain loop keeps few registers and many warps: with eight entries' rows loaded before they are added
+// a level took a tenth to a third longer (64 columns, forward / reverse sweeps of a query,
+// random n = 400,000, m = 4.1e6: 2.74 / 5.44 ms, 2.19 / 5.08 now; R-MAT n = 2^17, m = 3.75e6: 2.03 / 3.14
+// and 1.73 / 2.44).
+// The query of five sources on n = 20,011, m = 2e5 took 0.87 ms at segments of 128, 0.76 at 64, 0.74 at
 // 32; the batch of 64 is fastest at 64 (a partial of 8 W bytes costs an eighth of the gathers
 // it stands for at 32).
 template <typename V, int LPR, int CPL, class Op>
@@ -132,7 +133,6 @@ __global__ void __launch_bounds__(kBlock) batch_rows_kernel(int64_t n, const uin
                                                             f2* __restrict__ partial, int seg_blocks) {
     constexpr int W = LPR * CPL;
     constexpr int RPW = 32 / LPR;  // rows (or segments) per warp per iteration
-    constexpr int kU = sizeof(V) * CPL <= 16 ? 8 : (sizeof(V) * CPL <= 32 ? 4 : 2);
     prior_done();
     const int lane = threadIdx.x & 31;
     const int sub = lane / LPR, cl = lane % LPR;
@@ -163,33 +163,18 @@ __global__ void __launch_bounds__(kBlock) batch_rows_kernel(int64_t n, const uin
         f2 acc[CPL];
 #pragma unroll
         for (int i = 0; i < CPL; ++i) acc[i] = f2{0.f, 0.f};
-        for (uint32_t p = b; p < e; p += kU) {
-            int32_t j[kU];
-#pragma unroll
-            for (int t = 0; t < kU; ++t)
-                if (p + t < e) j[t] = __ldg(col + p + t);
+        for (uint32_t p = b; p < e; ++p) {
+            const int64_t j = __ldg(col + p);
             if constexpr (sizeof(V) == 4) {
-                float v[kU][CPL];
+                float v[CPL];
+                load_f<CPL>(reinterpret_cast<const float*>(X) + j * W + c0, v);
 #pragma unroll
-                for (int t = 0; t < kU; ++t)
-                    if (p + t < e) load_f<CPL>(reinterpret_cast<const float*>(X) + (int64_t)j[t] * W + c0, v[t]);
-#pragma unroll
-                for (int t = 0; t < kU; ++t)
-                    if (p + t < e) {
-#pragma unroll
-                        for (int i = 0; i < CPL; ++i) acc[i] = f2_add_f(acc[i], v[t][i]);
-                    }
+                for (int i = 0; i < CPL; ++i) acc[i] = f2_add_f(acc[i], v[i]);
             } else {
-                f2 v[kU][CPL];
+                f2 v[CPL];
+                load_f2<CPL>(reinterpret_cast<const float2*>(X) + j * W + c0, v);
 #pragma unroll
-                for (int t = 0; t < kU; ++t)
-                    if (p + t < e) load_f2<CPL>(reinterpret_cast<const float2*>(X) + (int64_t)j[t] * W + c0, v[t]);
-#pragma unroll
-                for (int t = 0; t < kU; ++t)
-                    if (p + t < e) {
-#pragma unroll
-                        for (int i = 0; i < CPL; ++i) acc[i] = f2_add(acc[i], v[t][i]);
-                    }
+                for (int i = 0; i < CPL; ++i) acc[i] = f2_add(acc[i], v[i]);
             }
         }
         if (!mine) continue;
