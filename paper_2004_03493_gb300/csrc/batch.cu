@@ -10,7 +10,7 @@
 // (Algorithm 1, Eq. sL) gives each column exactly its own sum over l <= L_q.
 //
 // Every column accumulates a row's entries one after another in index order
-// (rows of kBatchSeg entries or more: segments of kBatchSeg, joined by four fixed
+// (rows of bseg_len entries or more: segments of bseg_len, joined by four fixed
 // strides over the segments), whatever the tile shape: a column's result does not depend on which other columns share the
 // batch nor on the tile chosen by the autotuner.
 #include "common.cuh"
@@ -117,7 +117,7 @@ struct BRevOp {
 // lane group into partial[seg * W + column].
 //
 // What bounds a level: the gathered rows (m x W values from L2) and, per lane group, the
-// chain of two-float additions, about 40 cycles an entry.  No chain is longer than kBatchSeg: with
+// chain of two-float additions, about 40 cycles an entry.  No chain is longer than seg_len: with
 // segments of 4096 the longest one alone took 460-770 us of every level with a hub.  The
 // plain loop keeps few registers and many warps: with eight entries' rows loaded before they are added
 // a level took a tenth to a third longer (64 columns, forward / reverse sweeps of a query,
@@ -130,7 +130,7 @@ template <typename V, int LPR, int CPL, class Op>
 __global__ void __launch_bounds__(kBlock) batch_rows_kernel(int64_t n, const uint32_t* __restrict__ rp,
                                                             const int32_t* __restrict__ col, const V* X,
                                                             Op op, int64_t nseg, const Segment* __restrict__ seg,
-                                                            f2* __restrict__ partial, int seg_blocks) {
+                                                            f2* __restrict__ partial, int seg_blocks, uint32_t seg_len) {
     constexpr int W = LPR * CPL;
     constexpr int RPW = 32 / LPR;  // rows (or segments) per warp per iteration
     prior_done();
@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(kBlock) batch_rows_kernel(int64_t n, const uin
             } else {
                 b = __ldg(rp + it);
                 e = __ldg(rp + it + 1);
-                mine = (e - b) < kBatchSeg;
+                mine = (e - b) < seg_len;
                 if (!mine) e = b;
             }
         }
@@ -328,7 +328,7 @@ cudaError_t batch_level(const Graph& g, const DevCsr& A, const V* X, const Op& o
     const int segb = A.bnseg ? grid_cap(g, A.bnseg, rows_per_block) : 0;
     const cudaError_t e = launch_after(g.stream, dim3((unsigned)(sb + segb)), kBlock, 0,
                                        batch_rows_kernel<V, LPR, CPL, Op>, g.n, A.rp, A.col, X, op, A.bnseg, A.bseg,
-                                       partial, segb);
+                                       partial, segb, A.bseg_len);
     if (e != cudaSuccess || A.bnlong == 0) return e;
     return launch_after(g.stream, dim3((unsigned)A.bnlong), 4 * W, 0, batch_long_rows_kernel<W, Op>, A.blong_rows,
                         A.blong_first, partial, op);

@@ -82,12 +82,26 @@ uint32_t sell_row_cap(int64_t n, const std::vector<uint32_t>& rp) {
     return kSmallRowCap;
 }
 
+// Entries that a lane group of the batched sweeps adds one after another, at most: 64, so that a hub
+// is not a level's longest chain; more on dense graphs, where cutting every row doubles the launches and
+// only adds partial sums, but never so much that there are fewer than 8192 pieces of that length, about
+// what the chip works on at once.  Sweeps of a query, 64 columns, forward + reverse, with 64 / 256:
+// random n = 20,000, m = 3.9e6 4.18 / 2.64 ms; R-MAT n = 2^17, m = 3.75e6 (mean degree 28; five columns)
+// 1.57 / 1.95, n = 3000, m = 9e5 with 64 / 128 0.92 / 1.04.
+uint32_t batch_seg_len(int64_t n, int64_t m) {
+    const int64_t most = std::min(4 * m / n, m / 8192);
+    uint32_t len = 64;
+    while (len < 4096 && 2 * (int64_t)len <= most) len *= 2;
+    return len;
+}
+
 // Upload a host CSR and build its row-split table.
 esim_status upload_csr(int64_t n, const std::vector<uint32_t>& rp, const int32_t* col, DevCsr& d,
                        bool with_info, const std::vector<uint32_t>& uses_rp, cudaStream_t stream) {
     const int64_t m = (int64_t)rp[n];
     d.long_min = kProbeLongMin;
     d.seg_len = kSegLen;
+    d.bseg_len = batch_seg_len(n, m);
     d.sell.row_cap = sell_row_cap(n, rp);
     std::vector<Segment> seg, bseg, pieces;
     std::vector<int32_t> piece_rows, piece_first;  // not kept: a piece names its row and its row's first piece
@@ -104,7 +118,7 @@ esim_status upload_csr(int64_t n, const std::vector<uint32_t>& rp, const int32_t
         const uint32_t len = rp[r + 1] - rp[r];
         if (len > kSegLen) cut(r, kSegLen, seg, long_rows, long_first);
         else if (len >= d.long_min) seg.push_back(Segment{(int32_t)r, rp[r], rp[r + 1], (uint32_t)seg.size()});
-        if (len >= kBatchSeg) cut(r, kBatchSeg, bseg, blong_rows, blong_first);
+        if (len >= d.bseg_len) cut(r, d.bseg_len, bseg, blong_rows, blong_first);
         if (len > d.sell.row_cap) cut(r, 32 * d.sell.row_cap, pieces, piece_rows, piece_first);
     }
     long_first.push_back((int32_t)seg.size());

@@ -88,16 +88,16 @@ struct DevCsr {
     uint32_t long_min = 0;
     uint32_t seg_len = 0;
     SellRows sell;
-    // The batched sweeps' segments: rows of kBatchSeg entries or more in pieces of kBatchSeg.
+    // The batched sweeps' segments: rows of bseg_len entries or more in pieces of bseg_len.
     Segment* bseg = nullptr;
     int32_t* blong_rows = nullptr;
     int32_t* blong_first = nullptr;
     int64_t bnseg = 0;
+    uint32_t bseg_len = 0;
     int64_t bnlong = 0;
     char* tables = nullptr;  // one allocation: every table above but rp and col
 };
 
-constexpr uint32_t kBatchSeg = 64;          // entries a lane group of the batched sweeps adds one after another, at most
 
 constexpr int kSampleSlots = 16;
 
