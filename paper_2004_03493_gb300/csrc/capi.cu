@@ -66,20 +66,27 @@ constexpr int64_t kLongRowsFrom = 4000000;  // from this many edges on a level i
 // (877 warps at 8), n = 20,001, m = 160,009 209 / 189 / 275 (709 and 8854), m = 400,021
 // 252 / 442 / 484 (16,303); skewed n = 20,001, m = 200,011 302 / 268 / 259 (4577), n = 50,001, m = 500,011
 // 345 / 313 / 423 (5940 and 11,381), n = 100,003, m = 1,000,031 397 / 441 / 627 (11,446).
-uint32_t sell_row_cap(int64_t n, const std::vector<uint32_t>& rp) {
-    constexpr int64_t kResidentWarps = 152 * 40;  // 48 registers a thread
+// Where 32 leaves many more warps than that and 64 clearly fewer, the warps are what takes the time:
+// forward + reverse, L = 20, FP64 with 32 / 64: random n = 50,000, m = 2.5e6 1175 / 764 us (51,500
+// and 2500 warps), n = 100,000, m = 3.9e6 1985 / 929, R-MAT n = 2^17, m = 3.75e6 937 / 739; but
+// R-MAT n = 2^16, m = 1.5e6 468 / 505 (14,000), random n = 20,000, m = 1.9e6 525 / 690 (nearly all rows
+// above 64: the few below it are the level's longest chains).
+uint32_t sell_row_cap(int64_t n, const std::vector<uint32_t>& rp, int sm_count) {
+    const int64_t resident = (int64_t)sm_count * 40;  // warps, at 48 registers a thread
     if ((int64_t)rp[n] >= kLongRowsFrom) return kLargeRowCap;
-    constexpr uint32_t kCaps[2] = {kLeastRowCap, 2 * kLeastRowCap};
-    static_assert(2 * kCaps[1] == kSmallRowCap, "a cap between would be left out");
-    int64_t warps[2];
-    warps[0] = warps[1] = (n + kSellWindow - 1) / kSellWindow * (kSellWindow / 32);
+    static_assert(kSmallRowCap == 4 * kLeastRowCap && kLargeRowCap == 2 * kSmallRowCap, "a cap between would be left out");
+    int64_t warps[4];
+    for (int64_t& w : warps) w = (n + kSellWindow - 1) / kSellWindow * (kSellWindow / 32);
     for (int64_t r = 0; r < n; ++r) {  // one pass without branches; lengths are below kLongRowsFrom
         const uint32_t len = rp[r + 1] - rp[r];
-        for (int i = 0; i < 2; ++i) warps[i] += len > kCaps[i] ? (len + 32 * kCaps[i] - 1) / (32 * kCaps[i]) : 0u;
+        for (int i = 0; i < 4; ++i) {
+            const uint32_t cap = kLeastRowCap << i;
+            warps[i] += len > cap ? (len + 32 * cap - 1) / (32 * cap) : 0u;
+        }
     }
-    for (int i = 0; i < 2; ++i)
-        if (warps[i] <= kResidentWarps) return kCaps[i];
-    return kSmallRowCap;
+    for (int i = 0; i < 3; ++i)
+        if (warps[i] <= resident) return kLeastRowCap << i;
+    return warps[2] > 4 * resident && 4 * warps[3] <= 3 * warps[2] ? kLargeRowCap : kSmallRowCap;
 }
 
 // Entries that a lane group of the batched sweeps adds one after another, at most: 64, so that a hub
@@ -97,12 +104,13 @@ uint32_t batch_seg_len(int64_t n, int64_t m) {
 
 // Upload a host CSR and build its row-split table.
 esim_status upload_csr(int64_t n, const std::vector<uint32_t>& rp, const int32_t* col, DevCsr& d,
-                       bool with_info, const std::vector<uint32_t>& uses_rp, cudaStream_t stream) {
+                       bool with_info, const std::vector<uint32_t>& uses_rp, int sm_count, cudaStream_t stream) {
     const int64_t m = (int64_t)rp[n];
     d.long_min = kProbeLongMin;
     d.seg_len = kSegLen;
     d.bseg_len = batch_seg_len(n, m);
-    d.sell.row_cap = sell_row_cap(n, rp);
+    d.sell.row_cap = sell_row_cap(n, rp, sm_count);
+    d.sell.few_in_flight = m >= kLongRowsFrom;
     std::vector<Segment> seg, bseg, pieces;
     std::vector<int32_t> piece_rows, piece_first;  // not kept: a piece names its row and its row's first piece
     std::vector<int32_t> long_rows, long_first, blong_rows, blong_first;
@@ -1368,8 +1376,8 @@ esim_status esim_load_graph(int64_t n, const int64_t* in_rowptr, const int32_t* 
             return fail(ESIM_ENOMEM, "device allocation for 1/din");
         }
     }
-    esim_status st = upload_csr(n, in_rp, in_col, g.in, true, out_rp, cudaStreamPerThread);
-    if (st == ESIM_OK) st = upload_csr(n, out_rp, out_c.data(), g.out, false, in_rp, cudaStreamPerThread);
+    esim_status st = upload_csr(n, in_rp, in_col, g.in, true, out_rp, g.sm_count, cudaStreamPerThread);
+    if (st == ESIM_OK) st = upload_csr(n, out_rp, out_c.data(), g.out, false, in_rp, g.sm_count, cudaStreamPerThread);
     if (st != ESIM_OK) {
         release(g);
         delete h;

@@ -65,6 +65,7 @@ struct SellRows {
     int64_t nslices = 0;
     int64_t npieces = 0;
     uint32_t row_cap = 64;
+    bool few_in_flight = false; // four gathers a lane instead of eight (sweep.cu)
     uint32_t* pos = nullptr;    // n, or NULL
 };
 

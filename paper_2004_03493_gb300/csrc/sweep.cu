@@ -198,8 +198,8 @@ struct ReverseOpD {
 // ones), kU gathers in flight, the next kU column numbers loaded before the gathers
 // are waited for.  No shared memory is used, so the L1 keeps the values of the nodes with
 // many edges; an entry costs about 16 instructions instead of 54.
-// Rows longer than row_cap (8 to 32 below four million edges, 64 from there on: a lane's chain is
-// most of a small level's time; capi.cu) are summed by a warp each, lanes side by side along the row,
+// Rows longer than row_cap (8 to 64, 64 from four million edges on: a lane's chain is most of
+// a small level's time; capi.cu) are summed by a warp each, lanes side by side along the row,
 // first in the grid; a row longer than 32 row_cap entries is cut into pieces, and the warp
 // that counts in the last of them adds their sums.  Both joins are fixed shuffle trees.
 // Every row's sum has a fixed order, so the sweeps are deterministic.
@@ -209,10 +209,11 @@ struct ReverseOpD {
 // (sparse history) 98 against 316 on eight or sixteen lanes a row.  n = 1e5, m = 1e6: 11-12
 // against 20-23.  What is left is the L2's rate of scattered sectors (tags 63 % busy, L1
 // path 66 %).
-// Gathers in flight per lane: eight where a level is one row's latency; four on large graphs, where
+// Gathers in flight per lane: eight where a level is one row's latency; four from four million edges on, where
 // the warps, not the lanes, have to cover it (half the registers a lane, for two-floats seven
 // blocks an SM).  n = 1e6, m = 1.75e7, L = 33, FP64 / FP32c sweeps: 4.60 / 4.08 ms with eight, 4.12 /
-// 3.85 with four; the FP32c query at n = 1e5 415 us with eight, 447 with four.
+// 3.85 with four; the FP32c query at n = 1e5 415 us with eight, 447 with four.  Below the line, at a cap
+// of 64 on both sides: random n = 100,000, m = 3.9e6 929 us with eight, 1092 with four.
 template <class Pol, int kU>
 constexpr int sell_min_blocks() {
     return kU == 4 && sizeof(typename Pol::V) == 8 && sizeof(typename Pol::A) == sizeof(f2) &&
@@ -517,7 +518,7 @@ cudaError_t sweep_level(const Graph& g, const DevCsr& A, const typename Pol::V* 
     Acc* partial = reinterpret_cast<Acc*>(g.partial);
     unsigned* arrived = call_counts(g).p;
     const int64_t blocks = (A.sell.nslices * 32 + kBlock - 1) / kBlock;
-    auto* kernel = A.sell.row_cap == kLargeRowCap ? sell_rows_kernel<Pol, 4, Op> : sell_rows_kernel<Pol, 8, Op>;
+    auto* kernel = A.sell.few_in_flight ? sell_rows_kernel<Pol, 4, Op> : sell_rows_kernel<Pol, 8, Op>;
     return launch_after(g.stream, dim3((unsigned)blocks), kBlock, 0, kernel, A.sell, A.rp, x, op, partial, arrived);
 }
 
