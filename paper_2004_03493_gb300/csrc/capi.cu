@@ -11,6 +11,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <memory>
 #include <new>
 #include <string>
 #include <thread>
@@ -46,13 +47,6 @@ cudaError_t dev_alloc(T** p, size_t count) {
     *p = nullptr;
     if (count == 0) count = 1;
     return cudaMalloc((void**)p, sizeof(T) * count);
-}
-
-void free_csr(DevCsr& c) {
-    cudaFree(c.rp);
-    cudaFree(c.col);
-    cudaFree(c.tables);
-    c = DevCsr{};
 }
 
 constexpr uint32_t kSegLen = 4096;         // probe sweeps: entries a block adds, an eighth of them each warp
@@ -102,91 +96,143 @@ uint32_t batch_seg_len(int64_t n, int64_t m) {
     return len;
 }
 
-// Upload a host CSR and build its row-split table.
-esim_status upload_csr(int64_t n, const std::vector<uint32_t>& rp, const int32_t* col, DevCsr& d,
-                       bool with_info, const std::vector<uint32_t>& uses_rp, int sm_count, cudaStream_t stream) {
+// A CSR's tables on the host.
+struct CsrTables {
+    std::vector<Segment> seg, bseg, pieces;
+    std::vector<int32_t> long_rows, long_first, blong_rows, blong_first;
+    std::vector<uint32_t> off, pos;
+};
+
+CsrTables plan_csr(int64_t n, const std::vector<uint32_t>& rp, const std::vector<uint32_t>& uses_rp, int sm_count,
+                   DevCsr& d) {
+    CsrTables t;
     const int64_t m = (int64_t)rp[n];
     d.long_min = kProbeLongMin;
     d.seg_len = kSegLen;
     d.bseg_len = batch_seg_len(n, m);
     d.sell.row_cap = sell_row_cap(n, rp, sm_count);
     d.sell.few_in_flight = m >= kLongRowsFrom;
-    std::vector<Segment> seg, bseg, pieces;
-    std::vector<int32_t> piece_rows, piece_first;  // not kept: a piece names its row and its row's first piece
-    std::vector<int32_t> long_rows, long_first, blong_rows, blong_first;
-    auto cut = [&](int64_t r, uint32_t len, std::vector<Segment>& sg, std::vector<int32_t>& rows,
-                   std::vector<int32_t>& firsts) {
-        rows.push_back((int32_t)r);
-        firsts.push_back((int32_t)sg.size());
-        const uint32_t first = (uint32_t)sg.size();
-        for (uint32_t s = rp[r]; s < rp[r + 1]; s += len)
-            sg.push_back(Segment{(int32_t)r, s, std::min(rp[r + 1], s + len), first});
+    auto cut = [&](int64_t r, uint32_t len, std::vector<Segment>& sg) {
+        const uint32_t first = (uint32_t)sg.size(), end = rp[r + 1];
+        for (uint32_t s = rp[r]; s < end; s += len) sg.push_back(Segment{(int32_t)r, s, std::min(end, s + len), first});
     };
+    const uint32_t cap = d.sell.row_cap, shortest = std::min(d.long_min, d.bseg_len);
+    int64_t wide = 0, longer = 0;  // rows above the cap, and those of the other tables
     for (int64_t r = 0; r < n; ++r) {
         const uint32_t len = rp[r + 1] - rp[r];
-        if (len > kSegLen) cut(r, kSegLen, seg, long_rows, long_first);
-        else if (len >= d.long_min) seg.push_back(Segment{(int32_t)r, rp[r], rp[r + 1], (uint32_t)seg.size()});
-        if (len >= d.bseg_len) cut(r, d.bseg_len, bseg, blong_rows, blong_first);
-        if (len > d.sell.row_cap) cut(r, 32 * d.sell.row_cap, pieces, piece_rows, piece_first);
+        wide += len > cap;
+        longer += len >= shortest;
     }
-    long_first.push_back((int32_t)seg.size());
-    blong_first.push_back((int32_t)bseg.size());
-    d.nseg = (int64_t)seg.size();
-    d.nlong = (int64_t)long_rows.size();
-    d.bnseg = (int64_t)bseg.size();
-    d.bnlong = (int64_t)blong_rows.size();
-    std::vector<uint32_t> off, pos;
-    plan_sell(n, rp, pieces, uses_rp, d.sell, off, pos);
-    // One allocation and one copy for the tables, and the space the device fills behind them:
-    // a load makes few calls of a size-independent cost.
+    t.pieces.reserve((size_t)(wide + m / (32 * (int64_t)cap)));
+    if (wide)
+        for (int64_t r = 0; r < n; ++r)
+            if (rp[r + 1] - rp[r] > cap) cut(r, 32 * cap, t.pieces);
+    if (longer)
+        for (int64_t r = 0; r < n; ++r) {
+            const uint32_t len = rp[r + 1] - rp[r];
+            if (len < shortest) continue;
+            if (len > kSegLen) {
+                t.long_rows.push_back((int32_t)r);
+                t.long_first.push_back((int32_t)t.seg.size());
+            }
+            if (len >= d.long_min) cut(r, kSegLen, t.seg);
+            if (len >= d.bseg_len) {
+                t.blong_rows.push_back((int32_t)r);
+                t.blong_first.push_back((int32_t)t.bseg.size());
+                cut(r, d.bseg_len, t.bseg);
+            }
+        }
+    t.long_first.push_back((int32_t)t.seg.size());
+    t.blong_first.push_back((int32_t)t.bseg.size());
+    d.nseg = (int64_t)t.seg.size();
+    d.nlong = (int64_t)t.long_rows.size();
+    d.bnseg = (int64_t)t.bseg.size();
+    d.bnlong = (int64_t)t.blong_rows.size();
+    plan_sell(n, rp, t.pieces, uses_rp, d.sell, t.off, t.pos);
+    return t;
+}
+
+size_t topk_stage_offset(int64_t n) { return (topk_workspace_bytes(n) + 255) / 256 * 256; }
+
+// The graph's device memory: one allocation, one copy of the small tables, and what the device
+// fills: a load makes few calls of a size-independent cost.  With allocations, copies and waits per table,
+// 1/din and its inverse made on the host, and repeated in-edges looked up by a mark per node, the
+// sliced rows had made it slower: n = 2000, m = 20,000 0.40 ms (0.32 without them, 0.30 now), n = 8000,
+// m = 80,001 1.00 (0.64, 0.62), n = 100,003, m = 1,000,003 7.2 (6.4, 5.9).
+esim_status upload_graph(Graph& g, const std::vector<uint32_t>& in_rp, const int32_t* in_col,
+                         const std::vector<uint32_t>& out_rp, const int32_t* out_col) {
+    const size_t n = (size_t)g.n, m = (size_t)g.m;
+    const CsrTables tables[2] = {plan_csr(g.n, in_rp, out_rp, g.sm_count, g.in), plan_csr(g.n, out_rp, in_rp, g.sm_count, g.out)};
+    struct Part {
+        void** to;
+        size_t at;
+        const void* from;
+        size_t bytes;
+    };
+    std::vector<Part> parts;
     size_t bytes = 0;
-    auto place = [&bytes](size_t b) {
-        const size_t at = bytes;
+    auto take = [&](auto*& to, size_t count, const void* from = nullptr) {
+        const size_t b = sizeof(*to) * count;
+        parts.push_back({(void**)&to, bytes, from, b});
         bytes += (b + 255) / 256 * 256;
-        return at;
     };
-    std::vector<char> stage;
-    auto put = [&](const auto& v) {
-        const size_t b = v.size() * sizeof(v[0]), at = place(b);
-        stage.resize(bytes);
-        if (b) memcpy(stage.data() + at, v.data(), b);
-        return at;
-    };
-    const size_t o_seg = put(seg), o_lr = put(long_rows), o_lf = put(long_first), o_bseg = put(bseg),
-                 o_br = put(blong_rows), o_bf = put(blong_first), o_off = put(off), o_piece = put(pieces), o_pos = put(pos);
-    const size_t entries = with_info ? (size_t)std::max(m, n) : 0;
-    const size_t o_rows = place(sizeof(int2) * 32 * (size_t)d.sell.nslices),
-                 o_col = place(sizeof(int32_t) * 32 * (size_t)off.back()),
-                 o_info = place(with_info ? sizeof(uint2) * (size_t)n : 0), o_walk = place(sizeof(uint2) * entries);
-    if (dev_alloc(&d.rp, (size_t)n + 1) != cudaSuccess || dev_alloc(&d.col, (size_t)m) != cudaSuccess ||
-        dev_alloc(&d.tables, bytes) != cudaSuccess) {
+    DevCsr* const csr[2] = {&g.in, &g.out};
+    for (int i = 0; i < 2; ++i) {
+        const CsrTables& t = tables[i];
+        DevCsr& d = *csr[i];
+        take(d.seg, t.seg.size(), t.seg.data());
+        take(d.long_rows, t.long_rows.size(), t.long_rows.data());
+        take(d.long_first, t.long_first.size(), t.long_first.data());
+        take(d.bseg, t.bseg.size(), t.bseg.data());
+        take(d.blong_rows, t.blong_rows.size(), t.blong_rows.data());
+        take(d.blong_first, t.blong_first.size(), t.blong_first.data());
+        take(d.sell.off, t.off.size(), t.off.data());
+        take(d.sell.piece, t.pieces.size(), t.pieces.data());
+        if (!t.pos.empty()) take(d.sell.pos, n, t.pos.data());
+    }
+    take(g.in.rp, n + 1, in_rp.data());
+    take(g.out.rp, n + 1, out_rp.data());
+    const size_t staged = bytes;
+    for (int i = 0; i < 2; ++i) {
+        take(csr[i]->col, m);
+        take(csr[i]->sell.rows, 32 * (size_t)csr[i]->sell.nslices);
+        take(csr[i]->sell.col, 32 * (size_t)tables[i].off.back());
+    }
+    take(g.in.info, n);                  // filled on the device, as the next three (launch_walk_table)
+    take(g.in.walk, std::max(m, n));     // the tail past m is never a position
+    take(g.inv_din, n);
+    take(g.din_magic, n);
+    take(g.status, 1);
+    take(g.sample_taken, kSampleSlots);
+    char* partial = nullptr;
+    char* topk = nullptr;
+    take(partial, scratch_bytes(g));
+    take(g.scan_part, (size_t)allocate_blocks(g.n));
+    take(g.norm_part, 2 * (size_t)allocate_blocks(g.n));
+    take(topk, topk_stage_offset(g.n) + (sizeof(double) + sizeof(int32_t)) * kTopkMax);
+    if (cudaMalloc((void**)&g.memory, bytes) != cudaSuccess) {
         cudaGetLastError();
-        return fail(ESIM_ENOMEM, "cudaMalloc(graph tables)");
+        g.memory = nullptr;
+        return fail(ESIM_ENOMEM, "cudaMalloc(graph tables of " + std::to_string(bytes) + " bytes)");
     }
-    d.seg = (Segment*)(d.tables + o_seg);
-    d.long_rows = (int32_t*)(d.tables + o_lr);
-    d.long_first = (int32_t*)(d.tables + o_lf);
-    d.bseg = (Segment*)(d.tables + o_bseg);
-    d.blong_rows = (int32_t*)(d.tables + o_br);
-    d.blong_first = (int32_t*)(d.tables + o_bf);
-    d.sell.off = (uint32_t*)(d.tables + o_off);
-    d.sell.piece = (Segment*)(d.tables + o_piece);
-    d.sell.pos = pos.empty() ? nullptr : (uint32_t*)(d.tables + o_pos);
-    d.sell.rows = (int2*)(d.tables + o_rows);
-    d.sell.col = (int32_t*)(d.tables + o_col);
-    if (with_info) {  // filled on the device (launch_walk_table); the tail past m is never a position
-        d.info = (uint2*)(d.tables + o_info);
-        d.walk = (uint2*)(d.tables + o_walk);
-    }
-    ESIM_CUDA_TRY(cudaMemcpyAsync(d.rp, rp.data(), sizeof(uint32_t) * ((size_t)n + 1), cudaMemcpyHostToDevice, stream),
-                  "upload rowptr");
-    if (m)
-        ESIM_CUDA_TRY(cudaMemcpyAsync(d.col, col, sizeof(int32_t) * (size_t)m, cudaMemcpyHostToDevice, stream),
+    for (const Part& p : parts) *p.to = g.memory + p.at;
+    g.partial = partial;
+    g.topk_ws = topk;
+    const std::unique_ptr<char[]> stage(new char[staged]);
+    for (const Part& p : parts)
+        if (p.from && p.bytes) memcpy(stage.get() + p.at, p.from, p.bytes);
+    const cudaStream_t stream = g.stream;
+    ESIM_CUDA_TRY(cudaMemcpyAsync(g.memory, stage.get(), staged, cudaMemcpyHostToDevice, stream), "upload graph tables");
+    if (m) {
+        ESIM_CUDA_TRY(cudaMemcpyAsync(g.in.col, in_col, sizeof(int32_t) * m, cudaMemcpyHostToDevice, stream), "upload col");
+        ESIM_CUDA_TRY(cudaMemcpyAsync(g.out.col, out_col, sizeof(int32_t) * m, cudaMemcpyHostToDevice, stream),
                       "upload col");
-    ESIM_CUDA_TRY(cudaMemcpyAsync(d.tables, stage.data(), stage.size(), cudaMemcpyHostToDevice, stream),
-                  "upload graph tables");
-    ESIM_CUDA_TRY(fill_sell(n, d, stream), "sliced rows");
-    ESIM_CUDA_TRY(cudaStreamSynchronize(stream), "graph tables");  // the host vectors are this call's
+    }
+    ESIM_CUDA_TRY(fill_sell(g.n, g.in, stream), "sliced rows");
+    ESIM_CUDA_TRY(fill_sell(g.n, g.out, stream), "sliced rows");
+    ESIM_CUDA_TRY(launch_walk_table(g), "walk table");
+    ESIM_CUDA_TRY(cudaMemsetAsync(g.status, 0, sizeof(Status), stream), "reset status");
+    ESIM_CUDA_TRY(cudaStreamSynchronize(stream), "graph tables");  // the host tables are this call's
     return ESIM_OK;
 }
 
@@ -244,12 +290,7 @@ void release(Graph& g) {
     if (g.own_stream) cudaStreamSynchronize(g.own_stream);
     if (g.side_stream) cudaStreamSynchronize(g.side_stream);
     free_a3workers(g);
-    free_csr(g.in);
-    free_csr(g.out);
-    cudaFree(g.inv_din);
-    cudaFree(g.din_magic);
-    cudaFree(g.status);
-    cudaFree(g.sample_taken);
+    cudaFree(g.memory);
     for (auto& ev : g.sample_ev)
         if (ev) cudaEventDestroy(ev);
     if (g.status_host) cudaFreeHost(g.status_host);
@@ -258,10 +299,6 @@ void release(Graph& g) {
     cudaFree(g.a3ws);
     cudaFree(g.a3pws);
     cudaFree(g.zstage);
-    cudaFree(g.partial);
-    cudaFree(g.scan_part);
-    cudaFree(g.norm_part);
-    cudaFree(g.topk_ws);
     for (auto& ev : g.ev)
         if (ev) cudaEventDestroy(ev);
     if (g.own_stream) cudaStreamDestroy(g.own_stream);
@@ -272,8 +309,6 @@ void release(Graph& g) {
         if (ev) cudaEventDestroy(ev);
     g = Graph{};
 }
-
-size_t topk_stage_offset(int64_t n) { return (topk_workspace_bytes(n) + 255) / 256 * 256; }
 
 bool valid_c_eps(double c, double eps) { return c > 0.0 && c < 1.0 && eps > 0.0 && eps < 1.0; }
 
@@ -1339,58 +1374,30 @@ esim_status esim_load_graph(int64_t n, const int64_t* in_rowptr, const int32_t* 
         for (int64_t j = 0; j < n; ++j)
             for (int64_t p = in_rowptr[j]; p < in_rowptr[j + 1]; ++p) out_c[cur[in_col[p]]++] = (int32_t)j;
     }
-    {
-        // repeated in-edges (Algorithm 3 needs a simple graph) and the host in-degrees
-        std::vector<int32_t> mark((size_t)n, -1);
-        auto din = std::make_shared<std::vector<uint32_t>>((size_t)n);
-        for (int64_t j = 0; j < n && !g.has_duplicates; ++j)
-            for (int64_t p = in_rowptr[j]; p < in_rowptr[j + 1]; ++p) {
-                if (mark[in_col[p]] == (int32_t)j) {
-                    g.has_duplicates = true;
-                    break;
-                }
-                mark[in_col[p]] = (int32_t)j;
-            }
-        for (int64_t j = 0; j < n; ++j) (*din)[j] = in_rp[j + 1] - in_rp[j];
-        g.din_host = din;
+    // repeated in-edges (Algorithm 3 needs a simple graph): a row of the out-CSR is ascending, so they
+    // are neighbours there; equal neighbours of two rows are taken off again
+    int64_t repeated = 0;
+    for (int64_t p = 1; p < m; ++p) repeated += out_c[(size_t)p] == out_c[(size_t)p - 1];
+    for (int64_t i = 0; i < n && repeated > 0; ++i) {
+        const uint32_t p = out_rp[(size_t)i];
+        if (p > 0 && p < out_rp[(size_t)i + 1]) repeated -= out_c[p] == out_c[p - 1];
     }
-    {
-        std::vector<double> inv((size_t)n);
-        for (int64_t j = 0; j < n; ++j) {
-            const int64_t d = in_rowptr[j + 1] - in_rowptr[j];
-            inv[j] = d ? 1.0 / (double)d : 0.0;
-        }
-        std::vector<unsigned long long> magic((size_t)n);
-        for (int64_t j = 0; j < n; ++j) {
-            const int64_t d = in_rowptr[j + 1] - in_rowptr[j];
-            magic[j] = d >= 2 ? ~0ull / (unsigned long long)d : 0ull;
-        }
-        if (dev_alloc(&g.inv_din, (size_t)n) != cudaSuccess ||
-            cudaMemcpy(g.inv_din, inv.data(), sizeof(double) * (size_t)n, cudaMemcpyHostToDevice) != cudaSuccess ||
-            dev_alloc(&g.din_magic, (size_t)n) != cudaSuccess ||
-            cudaMemcpy(g.din_magic, magic.data(), sizeof(unsigned long long) * (size_t)n, cudaMemcpyHostToDevice) !=
-                cudaSuccess) {
-            cudaGetLastError();
-            release(g);
-            delete h;
-            return fail(ESIM_ENOMEM, "device allocation for 1/din");
-        }
-    }
-    esim_status st = upload_csr(n, in_rp, in_col, g.in, true, out_rp, g.sm_count, cudaStreamPerThread);
-    if (st == ESIM_OK) st = upload_csr(n, out_rp, out_c.data(), g.out, false, in_rp, g.sm_count, cudaStreamPerThread);
+    g.has_duplicates = repeated > 0;
+    auto din = std::make_shared<std::vector<uint32_t>>((size_t)n);
+    for (int64_t j = 0; j < n; ++j) (*din)[j] = in_rp[j + 1] - in_rp[j];
+    g.din_host = din;
+    g.stream = cudaStreamPerThread;
+    const esim_status st = upload_graph(g, in_rp, in_col, out_rp, out_c.data());
     if (st != ESIM_OK) {
         release(g);
         delete h;
         return st;
     }
-    bool ok = dev_alloc(&g.status, 1) == cudaSuccess && dev_alloc(&g.sample_taken, kSampleSlots) == cudaSuccess &&
-              cudaMallocHost((void**)&g.status_host, sizeof(Status)) == cudaSuccess &&
-              alloc_scratch(g, &g.partial, &g.scan_part, &g.norm_part) &&
-              cudaMalloc(&g.topk_ws, topk_stage_offset(n) + (sizeof(double) + sizeof(int32_t)) * kTopkMax) == cudaSuccess &&
-              cudaStreamCreateWithFlags(&g.own_stream, cudaStreamNonBlocking) == cudaSuccess &&
-              cudaStreamCreateWithFlags(&g.side_stream, cudaStreamNonBlocking) == cudaSuccess &&
-              cudaEventCreateWithFlags(&g.side_ev[0], cudaEventDisableTiming) == cudaSuccess &&
-              cudaEventCreateWithFlags(&g.side_ev[1], cudaEventDisableTiming) == cudaSuccess;
+    const bool ok = cudaMallocHost((void**)&g.status_host, sizeof(Status)) == cudaSuccess &&
+                    cudaStreamCreateWithFlags(&g.own_stream, cudaStreamNonBlocking) == cudaSuccess &&
+                    cudaStreamCreateWithFlags(&g.side_stream, cudaStreamNonBlocking) == cudaSuccess &&
+                    cudaEventCreateWithFlags(&g.side_ev[0], cudaEventDisableTiming) == cudaSuccess &&
+                    cudaEventCreateWithFlags(&g.side_ev[1], cudaEventDisableTiming) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
         release(g);
@@ -1398,14 +1405,6 @@ esim_status esim_load_graph(int64_t n, const int64_t* in_rowptr, const int32_t* 
         return fail(ESIM_ENOMEM, "device allocation for graph workspace");
     }
     g.stream = g.own_stream;
-    cudaError_t we = cudaMemsetAsync(g.status, 0, sizeof(Status), g.stream);
-    if (we == cudaSuccess) we = launch_walk_table(g);
-    if (we == cudaSuccess) we = cudaStreamSynchronize(g.stream);
-    if (we != cudaSuccess) {
-        release(g);
-        delete h;
-        return cuda_fail(we, "walk table");
-    }
     *out = h;
     return ESIM_OK;
 }

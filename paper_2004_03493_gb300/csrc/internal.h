@@ -96,13 +96,13 @@ struct DevCsr {
     int64_t bnseg = 0;
     uint32_t bseg_len = 0;
     int64_t bnlong = 0;
-    char* tables = nullptr;  // one allocation: every table above but rp and col
 };
 
 
 constexpr int kSampleSlots = 16;
 
 struct Graph {
+    char* memory = nullptr;  // one allocation: all that a load makes on the device
     int device = 0;
     int sm_count = 0;
     int64_t n = 0, m = 0;
@@ -244,7 +244,7 @@ cudaError_t launch_reverse_sparse(const Graph& g, const SparseHist& h, int32_t L
                                   double* s_out, double* sa);
 
 // sample.cu
-// fills in.info and in.walk from the uploaded in-edge CSR
+// fills in.info, in.walk, inv_din and din_magic from the uploaded in-edge CSR
 cudaError_t launch_walk_table(const Graph& g);
 int64_t allocate_blocks(int64_t n);
 cudaError_t launch_allocate(const Graph& g, const double* hist, int32_t L, double R_b, int mode, double* pi_out,

@@ -737,11 +737,14 @@ __global__ void mark_kernel(const int32_t* __restrict__ ids, int count, uint8_t*
 }
 
 // (first in-edge, din) of every node, or (node, 0) without in-edges; positions times 8 in
-// a narrow table
-__global__ void walk_rows_kernel(int64_t n, const uint32_t* __restrict__ rp, int shift, uint2* __restrict__ row) {
+// a narrow table; and 1/din and floor((2^64 - 1) / din)
+__global__ void walk_rows_kernel(int64_t n, const uint32_t* __restrict__ rp, int shift, uint2* __restrict__ row,
+                                 double* __restrict__ inv_din, unsigned long long* __restrict__ magic) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t b = rp[i], d = rp[i + 1] - b;
         row[i] = make_uint2(((d ? b : (uint32_t)i) << shift) | (d || !shift ? 0u : 4u), d);
+        inv_din[i] = d ? 1.0 / (double)d : 0.0;
+        magic[i] = d >= 2 ? ~0ull / d : 0ull;
     }
 }
 
@@ -762,7 +765,8 @@ static int eb_cap(const Graph& g, int64_t n) {
 static bool walk_narrow(const Graph& g) { return (g.m > g.n ? g.m : g.n) < ((int64_t)1 << 29); }
 
 cudaError_t launch_walk_table(const Graph& g) {
-    walk_rows_kernel<<<eb_cap(g, g.n), kBlock, 0, g.stream>>>(g.n, g.in.rp, walk_narrow(g) ? 3 : 0, g.in.info);
+    walk_rows_kernel<<<eb_cap(g, g.n), kBlock, 0, g.stream>>>(g.n, g.in.rp, walk_narrow(g) ? 3 : 0, g.in.info, g.inv_din,
+                                                               g.din_magic);
     walk_edges_kernel<<<eb_cap(g, g.m), kBlock, 0, g.stream>>>(g.m, g.in.col, g.in.info, g.in.walk);
     return cudaGetLastError();
 }
