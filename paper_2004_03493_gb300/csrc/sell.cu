@@ -7,6 +7,8 @@
 // the 32 rows' t-th entries side by side, so a warp reads them with one coalesced load.
 // Rows of more than row_cap entries take slices of their own, before all others, the lanes
 // side by side along the row.
+// The layout is SELL-C-sigma (M. Kreutzer, G. Hager, G. Wellein, H. Fehske, A. R. Bishop, SIAM
+// J. Sci. Comput. 36(5), 2014) with C = 32 and sigma = kSellWindow; the cut rows are added to it.
 #include "common.cuh"
 #include "internal.h"
 

@@ -23,7 +23,7 @@
 //            integer conversions (f2conv.cuh).  Every stored value is within about
 //            2^-46 relative of an FP64 computation of the same sums (the step and query
 //            parity tests hold it to 1e-12 of the oracle).  The Lemma 5 sweeps of
-//            Algorithm 3 and the sparse history keep FP64 sums (Pol64);
+//            Algorithm 3 take the same form; the sparse history keeps FP64 sums (Pol64);
 //   FP32c -- the precision form: pi^l and x^l stored in FP32 with two-float
 //            (compensated) row sums; s^l stored and summed as two-floats; FP64
 //            only for the final s^L and the D^ ratio.  On GB300, whose FP64 issue
@@ -625,9 +625,9 @@ cudaError_t launch_reverse_sparse(const Graph& g, const SparseHist& h, int32_t L
 }
 
 // Algorithm 3 helpers: h_l = (P^T)^l(u, .), the distribution of a non-stop walk from
-// u (no decay, no stop), for l = 0..steps, into H[(steps+1) * n] (FP64 storage), on the
-// warp-tile kernel in the FP64 form's two-float arithmetic (x_l = h_l / din as two-floats
-// in xa/xb, n 8-byte entries each).
+// u (no decay, no stop), for l = 0..steps, into H[(steps+1) * n] (FP64 storage), in the
+// FP64 form's two-float arithmetic (x_l = h_l / din as two-floats in xa/xb, n 8-byte
+// entries each).
 cudaError_t launch_walk_distributions(const Graph& g, int64_t u, int steps, double* H, double* xa, double* xb) {
     const uint32_t din_u = (*g.din_host)[(size_t)u];
     const f2 x0 = din_u ? host_f2(1.0 / (double)din_u) : f2{0.f, 0.f};
