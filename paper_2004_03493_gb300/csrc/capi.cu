@@ -51,7 +51,15 @@ cudaError_t dev_alloc(T** p, size_t count) {
 
 constexpr uint32_t kSegLen = 4096;         // probe sweeps: entries a block adds, an eighth of them each warp
 constexpr uint32_t kProbeLongMin = 512;    // shortest row of a block; 1024/64, 2048/128, 1024/256 measured the same
-constexpr int64_t kLongRowsFrom = 4000000;  // from this many edges on a level is no longer one row's latency
+// From this many edges on a level is no longer one row's latency: rows of up to 64 entries a lane, four
+// gathers in flight.  Forward + reverse, L = 20, FP64, eight / four gathers at the rule's cap below the line
+// and at 64 above it: skewed (Chung-Lu, mean degree 10, exponent 2.2) m = 3e6 809 / 736 us, 4.1e6 983 / 968,
+// 6e6 1341 / 1289, 8e6 1766 / 1653, 1.2e7 2833 / 2397, 1.75e7 4053 / 3297; R-MAT n = 2^18 4.1e6 918 / 862,
+// 8e6 1335 / 1218; random of mean degree 10 2e6 538 / 684, 4.1e6 880 / 939, 8e6 1540 / 1571, 1.75e7 3371 /
+// 3301, of mean degree 40 3e6 684 / 707, 6e6 1006 / 1391, 8e6 1424 / 1816, 1.2e7 1908 / 1900.  The
+// skewed graphs decide.  The cap above the line, four gathers, 32 / 64: skewed 4.1e6 912 / 968, 8e6
+// 1629 / 1653, 1.75e7 3479 / 3297, random of mean degree 40 8e6 2987 / 1816.
+constexpr int64_t kLongRowsFrom = 4000000;
 
 // The longest row that one lane sums (SellRows, internal.h).  A lane's chain of gathers is most of
 // a small level's time and a warp per row shortens it, as long as all warps of the level are on
