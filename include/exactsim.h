@@ -145,7 +145,11 @@ int64_t esim_num_nodes(const esim_graph* g);
 int64_t esim_num_edges(const esim_graph* g);
 
 /* Run the graph's work on `stream` (a cudaStream_t of the graph's device; NULL
- * restores the library's own stream).  The library does not take ownership. */
+ * restores the library's own stream).  The library does not take ownership, and
+ * neither waits for work on the stream before nor orders the new one after it.
+ * esim_sample, esim_sample_depth, esim_dhat and esim_dhat_alg3 on buffers of their
+ * own may overlap on several streams; the other calls share the handle's scratch, so
+ * the caller orders them. */
 esim_status esim_set_stream(esim_graph* g, void* stream);
 
 /* Options (per graph handle):
