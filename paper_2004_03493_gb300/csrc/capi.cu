@@ -236,8 +236,7 @@ esim_status upload_graph(Graph& g, const std::vector<uint32_t>& in_rp, const int
         ESIM_CUDA_TRY(cudaMemcpyAsync(g.out.col, out_col, sizeof(int32_t) * m, cudaMemcpyHostToDevice, stream),
                       "upload col");
     }
-    ESIM_CUDA_TRY(fill_sell(g.n, g.in, stream), "sliced rows");
-    ESIM_CUDA_TRY(fill_sell(g.n, g.out, stream), "sliced rows");
+    ESIM_CUDA_TRY(fill_sell(g.n, g.in, g.out, stream), "sliced rows");
     ESIM_CUDA_TRY(launch_walk_table(g), "walk table");
     ESIM_CUDA_TRY(cudaMemsetAsync(g.status, 0, sizeof(Status), stream), "reset status");
     ESIM_CUDA_TRY(cudaStreamSynchronize(stream), "graph tables");  // the host tables are this call's

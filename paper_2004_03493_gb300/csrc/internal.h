@@ -205,8 +205,8 @@ struct Graph {
 void plan_sell(int64_t n, const std::vector<uint32_t>& rp, const std::vector<Segment>& pieces,
                const std::vector<uint32_t>& uses_rp, SellRows& out, std::vector<uint32_t>& off,
                std::vector<uint32_t>& pos);
-// Fills csr.sell.rows and .col from the uploaded CSR, offsets, pieces and positions.
-cudaError_t fill_sell(int64_t n, const DevCsr& csr, cudaStream_t stream);
+// Fills both CSRs' sell.rows and sell.col from the uploaded CSRs, offsets, pieces and positions.
+cudaError_t fill_sell(int64_t n, const DevCsr& in, const DevCsr& out, cudaStream_t stream);
 
 // sweep.cu
 // The scratch g.partial of work on one stream: 8 bytes per piece, then counts of arrivals: one
