@@ -160,13 +160,18 @@ CsrTables plan_csr(int64_t n, const std::vector<uint32_t>& rp, const std::vector
     return t;
 }
 
+// Up to here a CSR's entries go with the small tables in one copy: m = 20,000 0.281 -> 0.263 ms a load, 80,001
+// 0.547 and 0.546; above, the copy through the stage costs as much as the calls (156,071 0.794 -> 0.803).
+constexpr size_t kStagedEdges = 1 << 16;
+
 size_t topk_stage_offset(int64_t n) { return (topk_workspace_bytes(n) + 255) / 256 * 256; }
 
 // The graph's device memory: one allocation, one copy of the small tables, and what the device
-// fills: a load makes few calls of a size-independent cost.  With allocations, copies and waits per table,
-// 1/din and its inverse made on the host, and repeated in-edges looked up by a mark per node, the
-// sliced rows had made it slower: n = 2000, m = 20,000 0.40 ms (0.32 without them, 0.30 now), n = 8000,
-// m = 80,001 1.00 (0.64, 0.62), n = 100,003, m = 1,000,003 7.2 (6.4, 5.9).
+// fills, both CSRs' slices in one launch each: a load makes few calls of a size-independent cost.  With
+// allocations, copies and waits per table, 1/din and its inverse made on the host, and repeated in-edges
+// looked up by a mark per node, the sliced rows had made it slower: Chung-Lu n = 2000, m = 20,000 0.40 ms
+// (0.30 without them, 0.26 now), n = 8000, m = 80,001 0.89 (0.59, 0.55), n = 100,003, m = 1,000,003 7.4
+// (6.3, 5.9); random n = 2863, m = 22,047 0.35 (0.27, 0.28).
 esim_status upload_graph(Graph& g, const std::vector<uint32_t>& in_rp, const int32_t* in_col,
                          const std::vector<uint32_t>& out_rp, const int32_t* out_col) {
     const size_t n = (size_t)g.n, m = (size_t)g.m;
@@ -200,9 +205,13 @@ esim_status upload_graph(Graph& g, const std::vector<uint32_t>& in_rp, const int
     }
     take(g.in.rp, n + 1, in_rp.data());
     take(g.out.rp, n + 1, out_rp.data());
+    const bool stage_cols = m <= kStagedEdges;
+    const int32_t* const cols[2] = {in_col, out_col};
+    for (int i = 0; i < 2; ++i)
+        if (stage_cols) take(csr[i]->col, m, cols[i]);
     const size_t staged = bytes;
     for (int i = 0; i < 2; ++i) {
-        take(csr[i]->col, m);
+        if (!stage_cols) take(csr[i]->col, m);
         take(csr[i]->sell.rows, 32 * (size_t)csr[i]->sell.nslices);
         take(csr[i]->sell.col, 32 * (size_t)tables[i].off.back());
     }
@@ -231,11 +240,10 @@ esim_status upload_graph(Graph& g, const std::vector<uint32_t>& in_rp, const int
         if (p.from && p.bytes) memcpy(stage.get() + p.at, p.from, p.bytes);
     const cudaStream_t stream = g.stream;
     ESIM_CUDA_TRY(cudaMemcpyAsync(g.memory, stage.get(), staged, cudaMemcpyHostToDevice, stream), "upload graph tables");
-    if (m) {
-        ESIM_CUDA_TRY(cudaMemcpyAsync(g.in.col, in_col, sizeof(int32_t) * m, cudaMemcpyHostToDevice, stream), "upload col");
-        ESIM_CUDA_TRY(cudaMemcpyAsync(g.out.col, out_col, sizeof(int32_t) * m, cudaMemcpyHostToDevice, stream),
-                      "upload col");
-    }
+    for (int i = 0; i < 2; ++i)
+        if (!stage_cols)
+            ESIM_CUDA_TRY(cudaMemcpyAsync(csr[i]->col, cols[i], sizeof(int32_t) * m, cudaMemcpyHostToDevice, stream),
+                          "upload col");
     ESIM_CUDA_TRY(fill_sell(g.n, g.in, g.out, stream), "sliced rows");
     ESIM_CUDA_TRY(launch_walk_table(g), "walk table");
     ESIM_CUDA_TRY(cudaMemsetAsync(g.status, 0, sizeof(Status), stream), "reset status");
