@@ -494,7 +494,9 @@ __device__ __forceinline__ uint64_t find_segment(const uint64_t* __restrict__ of
 // 32 pairs instead, and each lane finds the segment of its own: in a batch whose sources share an
 // eps most of a node's 64 segments have no pairs, and windows of segments took a turn for every
 // one or two of them (64 sources on a random graph of 50,000 nodes, eps = 1e-2: walks 572 us,
-// 107 now; one pair in every 64th of 4e6 nodes 98 and 34).
+// 107 now; one pair in every 64th of 4e6 nodes 98 and 34).  The registers it takes cost the windows of
+// segments 2 % (random n = 400,003, m = 4,000,001, eps = 3e-4: walks 410 and 418 us).  Not inlined 2 % more; a
+// kernel without depths beside this one gets half of it back and loses 0.6 % on long runs (8.23 and 8.28 ms).
 template <bool kNarrow>
 __device__ __forceinline__ unsigned long long run_many(const WalkArgs& a, unsigned long long g, unsigned long long g1,
                                                     uint64_t& seg_io, const PhiloxKeys& K, uint32_t& steps) {
